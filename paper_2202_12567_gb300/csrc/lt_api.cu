@@ -259,6 +259,8 @@ extern "C" lt_status lt_scene_upload(lt_ctx* ctx, const float* boxes, int64_t nb
     g.bvh_aabb = nullptr;
     g.bvh_child = nullptr;
     g.bvh_tri = nullptr;
+    g.bvh_node = nullptr;
+    g.bvh_leaf = nullptr;
     g.box = ctx->d_boxes;
     g.cell_off = ctx->d_cell_off;
     g.cell_box = ctx->d_cell_box;

@@ -432,6 +432,24 @@ __global__ void k_bvh_up(int64_t nt, const int32_t* __restrict__ child, const in
     }
 }
 
+// the records the walk reads: both children's boxes and ids per internal node, and the
+// triangles in leaf order
+__global__ void k_bvh_pack(int64_t nt, const int32_t* __restrict__ child, const float* __restrict__ aabb,
+                           const int32_t* __restrict__ leaf_tri, const float4* __restrict__ rec,
+                           float4* __restrict__ node, float4* __restrict__ leaf) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nt; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t t = leaf_tri[i];
+        for (int k = 0; k < 3; ++k) leaf[3 * i + k] = rec[3 * t + k];
+        if (i == nt - 1) continue;
+        const int a = child[2 * i], b = child[2 * i + 1];
+        const float *A = aabb + 6 * (int64_t)a, *B = aabb + 6 * (int64_t)b;
+        node[4 * i] = make_float4(A[0], A[1], A[2], A[3]);
+        node[4 * i + 1] = make_float4(A[4], A[5], B[0], B[1]);
+        node[4 * i + 2] = make_float4(B[2], B[3], B[4], B[5]);
+        node[4 * i + 3] = make_float4(__int_as_float(a), __int_as_float(b), 0.f, 0.f);
+    }
+}
+
 }  // namespace
 
 // ------------------------------------------------------------------ tree
@@ -720,13 +738,15 @@ extern "C" lt_status lt_mesh_upload(lt_ctx* ctx, const float* tris, int64_t nt) 
     g.bvh_aabb = nullptr;
     g.bvh_child = nullptr;
     g.bvh_tri = nullptr;
+    g.bvh_node = nullptr;
+    g.bvh_leaf = nullptr;
     if (nt == 0) return LT_OK;
     const int64_t nn = 2 * nt - 1;
     auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
     const size_t b_rec = up((size_t)nt * 48), b_aabb = up((size_t)nn * 24), b_child = up((size_t)nn * 8),
-                 b_par = up((size_t)nn * 4), b_range = up((size_t)nn * 8), b_leaf = up((size_t)nt * 4);
+                 b_par = up((size_t)nn * 4), b_range = up((size_t)nn * 8), b_leaf = up((size_t)nt * 4), b_node = up((size_t)nt * 64);
     char* m = nullptr;
-    LT_CUDA(ctx, cudaMalloc(&m, b_rec + b_aabb + b_child + b_par + b_range + b_leaf));
+    LT_CUDA(ctx, cudaMalloc(&m, 2 * b_rec + b_aabb + b_child + b_par + b_range + b_leaf + b_node));
     ctx->d_mesh = m;
     float4* rec = (float4*)m;
     float* aabb = (float*)(m + b_rec);
@@ -734,6 +754,8 @@ extern "C" lt_status lt_mesh_upload(lt_ctx* ctx, const float* tris, int64_t nt) 
     int32_t* parent = (int32_t*)(m + b_rec + b_aabb + b_child);
     int32_t* range = (int32_t*)(m + b_rec + b_aabb + b_child + b_par);
     int32_t* leaf = (int32_t*)(m + b_rec + b_aabb + b_child + b_par + b_range);
+    float4* node_rec = (float4*)(m + b_rec + b_aabb + b_child + b_par + b_range + b_leaf);
+    float4* leaf_rec = (float4*)(m + b_rec + b_aabb + b_child + b_par + b_range + b_leaf + b_node);
     const int64_t npad = next_pow2(nt);
     lt_status st;
     char* p = (char*)lt_scratch(ctx, SCR_SORT, (size_t)npad * 8 + (size_t)nt * 4 + (size_t)nt * 16 + 1024, &st);
@@ -765,12 +787,16 @@ extern "C" lt_status lt_mesh_upload(lt_ctx* ctx, const float* tris, int64_t nt) 
         k_bvh_up<<<blocks, 256, 0, ctx->stream>>>(nt, child, parent, aabb, flags);
         LT_LAUNCH_CHECK(ctx, "k_bvh_up");
     }
+    k_bvh_pack<<<blocks, 256, 0, ctx->stream>>>(nt, child, aabb, leaf, rec, node_rec, leaf_rec);
+    LT_LAUNCH_CHECK(ctx, "k_bvh_pack");
     LT_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     g.nt = (int)nt;
     g.tri = rec;
     g.bvh_aabb = aabb;
     g.bvh_child = child;
     g.bvh_tri = leaf;
+    g.bvh_node = node_rec;
+    g.bvh_leaf = leaf_rec;
     return LT_OK;
 }
 
