@@ -552,84 +552,150 @@ __global__ void k_moff(lt_frame F, lt_samples smp, int64_t* __restrict__ moff) {
     if (threadIdx.x == 0) moff[F.S] = carry;
 }
 
-__global__ void __launch_bounds__(256) k_slice_matrix(lt_frame F, lt_samples smp, Grid g, float dmin2,
+// A thread keeps one column (its VPL record and scale in registers) and walks a run of
+// kMatRows rows, so that an entry costs one broadcast point record and its shadow ray.
+// Bound by the instructions of the entry model.
+constexpr int kMatRows = 32;
+
+__global__ void __launch_bounds__(128) k_slice_matrix(lt_frame F, lt_samples smp, Grid g, float dmin2,
                                                       const int64_t* __restrict__ moff, int64_t cap,
                                                       float* __restrict__ M, int32_t* status) {
     const float4* pts = reinterpret_cast<const float4*>(F.pts);
     const float4* vpls = reinterpret_cast<const float4*>(F.vpls);
     if (moff[F.S] > cap) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) latch(status, LT_ELIMIT);
+        if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) latch(status, LT_ELIMIT);
         return;
     }
     const int s = blockIdx.y;
     const int row0 = F.slice_off[s], ms = F.slice_off[s + 1] - row0, ns = smp.ncol[s];
+    const int tc = (ns + 127) / 128, tiles = tc * ((ms + kMatRows - 1) / kMatRows);
     float* out = M + moff[s];
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)ms * ns;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(e / ns), c = (int)(e % ns);
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const int c = (t % tc) * 128 + threadIdx.x, i0 = (t / tc) * kMatRows, i1 = min(i0 + kMatRows, ms);
+        if (c >= ns) continue;
         const int node = smp.col_node[(int64_t)s * F.C + c];
-        const int rep = F.tree.rep[node];
-        const PointRec P = load_rec(pts, F.m, row0 + i);
-        const PointRec L = load_rec(vpls, F.n, rep);
+        const PointRec L = load_rec(vpls, F.n, F.tree.rep[node]);
         // I_c / I_rep(c), I = flux * albedo, rounded as in the sampling passes
         const float scale = __fdiv_rn(F.tree.I[node], __fmul_rn(L.c.w, L.a.w));
-        out[e] = entry_value(P, L, scale, dmin2, g);
+        for (int i = i0; i < i1; ++i) {
+            const PointRec P = load_rec(pts, F.m, row0 + i);
+            out[(int64_t)i * ns + c] = entry_value(P, L, scale, dmin2, g);
+        }
     }
 }
 
 // G_s = M_s^T M_s (n' x n', float) at G + goff2[s] with goff2 the prefix of n'^2
-__global__ void k_goff(lt_samples smp, int S, int64_t* __restrict__ goff2) {
+constexpr int kGramTile = 128;
+constexpr int kGramStep = 16;
+
+// goff2 and the prefix of the tiles on or above the diagonal of every G_s
+__global__ void k_goff(lt_samples smp, int S, int64_t* __restrict__ goff2, int64_t* __restrict__ tpfx) {
     __shared__ int64_t ws[32];
-    int64_t carry = 0;
+    int64_t carry = 0, tcarry = 0;
     for (int c0 = 0; c0 < S; c0 += blockDim.x) {
         const int s = c0 + threadIdx.x;
-        const int64_t x = s < S ? (int64_t)smp.ncol[s] * smp.ncol[s] : 0;
+        const int64_t n = s < S ? smp.ncol[s] : 0, t = (n + kGramTile - 1) / kGramTile;
         int64_t tot;
-        const int64_t pre = block_exclusive_scan<int64_t>(x, ws, &tot);
+        int64_t pre = block_exclusive_scan<int64_t>(n * n, ws, &tot);
         if (s < S) goff2[s] = carry + pre;
         carry += tot;
+        pre = block_exclusive_scan<int64_t>(t * (t + 1) / 2, ws, &tot);
+        if (s < S) tpfx[s] = tcarry + pre;
+        tcarry += tot;
     }
-    if (threadIdx.x == 0) goff2[S] = carry;
+    if (threadIdx.x == 0) {
+        goff2[S] = carry;
+        tpfx[S] = tcarry;
+    }
 }
 
-// 32 x 32 output tiles, rows of M streamed through shared memory in steps of 32
-__global__ void __launch_bounds__(256) k_gram(lt_frame F, lt_samples smp, const float* __restrict__ M,
-                                              const int64_t* __restrict__ moff, const int64_t* __restrict__ goff2,
-                                              int64_t gcap, float* __restrict__ G) {
-    __shared__ float A[32][33], B[32][33];
+// G_s is symmetric: a persistent grid takes the 128 x 128 tiles on or above the diagonal
+// and writes each twice.  A thread holds 8 x 8 outputs; the rows of M stream through
+// shared memory 16 at a time, the next 16 loaded while these are added.  Every output
+// is one chain of multiply-adds over the rows in order.  Bound by the FP32 pipe.  With
+// this, k_slice_matrix and the split subspace iteration the training data of a scene of 65536
+// points (64 slices of about 630 columns, 30 rounds at rank 16) take 8.6 ms, 55.3 ms with
+// 32 x 32 tiles and one CTA per slice for the whole iteration.
+__global__ void __launch_bounds__(256, 2) k_gram(lt_frame F, lt_samples smp, const float* __restrict__ M,
+                                                 const int64_t* __restrict__ moff, const int64_t* __restrict__ goff2,
+                                                 const int64_t* __restrict__ tpfx, int64_t gcap,
+                                                 float* __restrict__ G) {
+    __shared__ __align__(16) float A[kGramStep][kGramTile], B[kGramStep][kGramTile];
     if (goff2[F.S] > gcap) return;
-    const int s = blockIdx.z;
-    const int ms = F.slice_off[s + 1] - F.slice_off[s], ns = smp.ncol[s];
-    const int ti = blockIdx.y * 32, tj = blockIdx.x * 32;
-    if (ti >= ns || tj >= ns) return;
-    const float* Ms = M + moff[s];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 8 rows of 4 outputs per thread
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int r0 = 0; r0 < ms; r0 += 32) {
-        for (int q = ty; q < 32; q += 8) {
-            const int r = r0 + q;
-            A[q][tx] = (r < ms && ti + tx < ns) ? Ms[(int64_t)r * ns + ti + tx] : 0.f;
-            B[q][tx] = (r < ms && tj + tx < ns) ? Ms[(int64_t)r * ns + tj + tx] : 0.f;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const int lc = threadIdx.x & 127, lr = threadIdx.x >> 7;  // the loads: column lc of rows lr, lr + 2, ...
+    for (int64_t w = blockIdx.x; w < tpfx[F.S]; w += gridDim.x) {
+        int lo = 0, hi = F.S;  // tpfx[lo] <= w < tpfx[lo + 1]
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (tpfx[mid] <= w) lo = mid;
+            else hi = mid;
         }
-        __syncthreads();
-        for (int k = 0; k < 32; ++k) {
-            const float b = B[k][tx];
+        const int s = lo;
+        const int ms = F.slice_off[s + 1] - F.slice_off[s], ns = smp.ncol[s];
+        int t = (int)(w - tpfx[s]), bi = 0;
+        for (int left = (ns + kGramTile - 1) / kGramTile; t >= left; --left, ++bi) t -= left;
+        const int ti = bi * kGramTile, tj = (bi + t) * kGramTile;
+        const float* Ms = M + moff[s];
+        float acc[8][8];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) acc[u] = fmaf(A[k][ty + 8 * u], b, acc[u]);
+        for (int u = 0; u < 8; ++u)
+#pragma unroll
+            for (int v = 0; v < 8; ++v) acc[u][v] = 0.f;
+        float pa[8], pb[8];
+        auto fetch = [&](int r0) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int r = r0 + lr + 2 * q;
+                pa[q] = (r < ms && ti + lc < ns) ? __ldg(Ms + (int64_t)r * ns + ti + lc) : 0.f;
+                pb[q] = (r < ms && tj + lc < ns) ? __ldg(Ms + (int64_t)r * ns + tj + lc) : 0.f;
+            }
+        };
+        fetch(0);
+        for (int r0 = 0; r0 < ms; r0 += kGramStep) {
+            __syncthreads();  // the last step's rows have been read
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                A[lr + 2 * q][lc] = pa[q];
+                B[lr + 2 * q][lc] = pb[q];
+            }
+            __syncthreads();
+            if (r0 + kGramStep < ms) fetch(r0 + kGramStep);
+#pragma unroll
+            for (int k = 0; k < kGramStep; ++k) {
+                float a[8], b[8];
+                *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(&A[k][4 * ty]);
+                *reinterpret_cast<float4*>(a + 4) = *reinterpret_cast<const float4*>(&A[k][64 + 4 * ty]);
+                *reinterpret_cast<float4*>(b) = *reinterpret_cast<const float4*>(&B[k][4 * tx]);
+                *reinterpret_cast<float4*>(b + 4) = *reinterpret_cast<const float4*>(&B[k][64 + 4 * tx]);
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+#pragma unroll
+                    for (int v = 0; v < 8; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
+            }
         }
-        __syncthreads();
-    }
-    float* Gs = G + goff2[s];
-    for (int u = 0; u < 4; ++u) {
-        const int i = ti + ty + 8 * u, j = tj + tx;
-        if (i < ns && j < ns) Gs[(int64_t)i * ns + j] = acc[u];
+        float* Gs = G + goff2[s];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+#pragma unroll
+            for (int v = 0; v < 8; ++v) {
+                const int i = ti + (u >> 2) * 64 + 4 * ty + (u & 3), j = tj + (v >> 2) * 64 + 4 * tx + (v & 3);
+                if (i < ns && j < ns) {
+                    Gs[(int64_t)i * ns + j] = acc[u][v];
+                    if (ti != tj) Gs[(int64_t)j * ns + i] = acc[u][v];
+                }
+            }
     }
 }
 
-// Subspace iteration per slice (one CTA): Q (n' x r, float, in global scratch) from
-// Philox, `iters` rounds of Q <- mgs(G Q), then p_c = (|Q_c|^2 + 1/n') / (r' + 1) with
-// r' the columns kept.  Modified Gram-Schmidt column by column, block reductions in a
-// fixed order.
+// Subspace iteration per slice: Q (n' x r, float, in global scratch) from Philox,
+// `iters` rounds of Q <- mgs(G Q), then p_c = (|Q_c|^2 + 1/n') / (r' + 1) with r' the
+// columns kept.  The product runs on the whole chip (k_lev_mult), the Gram-Schmidt one
+// CTA per slice (k_lev_mgs) with block reductions in a fixed order: one CTA per slice
+// for both spent 46.8 ms on the workload named above, most of it on 120 dependent block
+// reductions a round and on the product at 64 of 152 SMs.
+constexpr int kLevThreads = 512;
+
 __device__ float block_sum(float v, float* red) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     v = warp_sum(v);
@@ -641,6 +707,7 @@ __device__ float block_sum(float v, float* red) {
     return t;
 }
 
+// Modified Gram-Schmidt on the columns of Q in global memory (any n and r).
 __device__ void mgs_cols(float* Q, int n, int r, float* red) {
     for (int k = 0; k < r; ++k) {
         for (int j = 0; j < k; ++j) {
@@ -659,12 +726,89 @@ __device__ void mgs_cols(float* Q, int n, int r, float* red) {
     }
 }
 
-__global__ void __launch_bounds__(512) k_leverage(lt_samples smp, const int32_t* __restrict__ slice_id, int S, int C,
-                                                  const float* __restrict__ G,
-                                                  const int64_t* __restrict__ goff2, int64_t gcap, int r, int iters,
-                                                  uint64_t seed, float* __restrict__ Qall, float* __restrict__ Yall,
-                                                  const int32_t* __restrict__ goff, float* __restrict__ target) {
+// The same with every row in registers (thread t holds rows t + 512 p, p < NR; at most
+// 16 columns).  Column j, once normalised, is taken out of all later columns at once:
+// each of them meets the earlier ones in the same order and with the same sums as in
+// mgs_cols, so the bits are the same, with 2 block reductions per column in place of
+// one per pair of columns.  The sums of 16 values over a warp share their shuffles: a
+// lane hands on half of its values at each of the first four steps of the butterfly.
+template <int NR>
+__device__ void mgs_regs(float* __restrict__ Q, int n, int r, float* red, float (*part)[16], float* dots) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    float q[NR][16];
+#pragma unroll
+    for (int p = 0; p < NR; ++p) {
+        const int i = threadIdx.x + kLevThreads * p;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) q[p][k] = (i < n && k < r) ? Q[(int64_t)i * r + k] : 0.f;
+    }
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        if (j < r) {  // uniform
+            float q2 = 0.f;
+#pragma unroll
+            for (int p = 0; p < NR; ++p) q2 = fmaf(q[p][j], q[p][j], q2);
+            q2 = block_sum(q2, red);
+            const float inv = q2 > 0.f ? 1.f / sqrtf(q2) : 0.f;
+#pragma unroll
+            for (int p = 0; p < NR; ++p) q[p][j] *= inv;
+            if (j + 1 < r) {
+                float d[16];
+#pragma unroll
+                for (int k = 0; k < 16; ++k) {
+                    d[k] = 0.f;
+                    if (k > j) {
+#pragma unroll
+                        for (int p = 0; p < NR; ++p) d[k] = fmaf(q[p][j], q[p][k], d[k]);
+                    }
+                }
+#pragma unroll
+                for (int o = 16, h = 8; o > 1; o >>= 1, h >>= 1) {
+#pragma unroll
+                    for (int k = 0; k < h; ++k) {
+                        const bool up = lane & o;
+                        const float send = up ? d[k] : d[k + h], keep = up ? d[k + h] : d[k];
+                        d[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                    }
+                }
+                d[0] += __shfl_xor_sync(0xffffffffu, d[0], 1);
+                if (!(lane & 1)) part[w][lane >> 1] = d[0];  // lane bits 4..1 name the value
+                __syncthreads();
+                if (threadIdx.x < 16) {
+                    float t = 0.f;
+                    for (int x = 0; x < kLevThreads / 32; ++x) t += part[x][threadIdx.x];
+                    dots[threadIdx.x] = t;
+                }
+                __syncthreads();
+#pragma unroll
+                for (int k = j + 1; k < 16; ++k) {
+                    const float dk = dots[k];
+#pragma unroll
+                    for (int p = 0; p < NR; ++p) q[p][k] = fmaf(-dk, q[p][j], q[p][k]);
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int p = 0; p < NR; ++p) {
+        const int i = threadIdx.x + kLevThreads * p;
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+            if (i < n && k < r) Q[(int64_t)i * r + k] = q[p][k];
+    }
+    __syncthreads();
+}
+
+// Orthonormalises Q of every slice: from Philox first (start), else the product k_lev_mult
+// left there; after the last round also the targets.
+__global__ void __launch_bounds__(kLevThreads) k_lev_mgs(lt_samples smp, const int32_t* __restrict__ slice_id, int S,
+                                                         int C, const int64_t* __restrict__ goff2, int64_t gcap, int r,
+                                                         bool start, bool last, uint64_t seed, float* __restrict__ Qall,
+                                                         float* __restrict__ Yall, const int32_t* __restrict__ goff,
+                                                         float* __restrict__ target) {
     __shared__ float red[32];
+    __shared__ float part[kLevThreads / 32][16];
+    __shared__ float dots[16];
     if (goff2[S] > gcap) return;
     const int s = blockIdx.x;
     const int ns = smp.ncol[s];
@@ -672,27 +816,21 @@ __global__ void __launch_bounds__(512) k_leverage(lt_samples smp, const int32_t*
     const int rr = min(r, ns);
     float* Q = Qall + (int64_t)s * C * r;
     float* Y = Yall + (int64_t)s * C * r;
-    const float* Gs = G + goff2[s];
-    for (int e = threadIdx.x; e < ns * rr; e += blockDim.x) {
-        const int c = e / rr, k = e % rr;
-        Q[e] = (float)((double)philox((uint32_t)k, (uint32_t)c, slice_key(slice_id, s), kTagLeverage, seed).x *
-                           2.3283064365386963e-10 - 0.5);
-    }
-    __syncthreads();
-    mgs_cols(Q, ns, rr, red);
-    for (int it = 0; it < iters; ++it) {
+    if (start) {
         for (int e = threadIdx.x; e < ns * rr; e += blockDim.x) {
-            const int i = e / rr, k = e % rr;
-            const float* gi = Gs + (int64_t)i * ns;
-            float a = 0.f;
-            for (int j = 0; j < ns; ++j) a = fmaf(gi[j], Q[(int64_t)j * rr + k], a);
-            Y[e] = a;
+            const int c = e / rr, k = e % rr;
+            Q[e] = (float)((double)philox((uint32_t)k, (uint32_t)c, slice_key(slice_id, s), kTagLeverage, seed).x *
+                               2.3283064365386963e-10 - 0.5);
         }
         __syncthreads();
-        for (int e = threadIdx.x; e < ns * rr; e += blockDim.x) Q[e] = Y[e];
-        __syncthreads();
-        mgs_cols(Q, ns, rr, red);
     }
+    const int nr = (ns + kLevThreads - 1) / kLevThreads;
+    if (rr > 16 || nr > 4) mgs_cols(Q, ns, rr, red);
+    else if (nr == 1) mgs_regs<1>(Q, ns, rr, red, part, dots);
+    else if (nr == 2) mgs_regs<2>(Q, ns, rr, red, part, dots);
+    else if (nr == 3) mgs_regs<3>(Q, ns, rr, red, part, dots);
+    else mgs_regs<4>(Q, ns, rr, red, part, dots);
+    if (!last) return;
     float tot = 0.f;
     for (int c = threadIdx.x; c < ns; c += blockDim.x) {
         float l = 0.f;
@@ -702,6 +840,58 @@ __global__ void __launch_bounds__(512) k_leverage(lt_samples smp, const int32_t*
     }
     tot = block_sum(tot, red);
     for (int c = threadIdx.x; c < ns; c += blockDim.x) target[goff[s] + c] = Y[c] / tot;
+}
+
+// Y = G Q of every slice, a thread per row of G and 16 columns of Q at a time: row i of
+// G is read as column i (G is symmetric to the bit), so that a warp's loads are one line, the
+// rows of Q are broadcast from shared memory.  Sums over j in order.
+constexpr int kLevRows = 64, kLevTile = 64;
+
+__global__ void __launch_bounds__(kLevRows) k_lev_mult(lt_samples smp, int S, int C, const float* __restrict__ G,
+                                                       const int64_t* __restrict__ goff2, int64_t gcap, int r,
+                                                       const float* __restrict__ Qall, float* __restrict__ Yall) {
+    __shared__ __align__(16) float sq[kLevTile][16];
+    if (goff2[S] > gcap) return;
+    const int s = blockIdx.y;
+    const int ns = smp.ncol[s];
+    const int rr = min(r, ns), blocks = (ns + kLevRows - 1) / kLevRows, parts = (rr + 15) / 16;
+    const float* Q = Qall + (int64_t)s * C * r;
+    float* Y = Yall + (int64_t)s * C * r;
+    for (int b = blockIdx.x; b < blocks * parts; b += gridDim.x) {
+        const int i = (b % blocks) * kLevRows + threadIdx.x, k0 = (b / blocks) * 16;
+        const float* Gi = G + goff2[s] + min(i, ns - 1);
+        float a[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) a[k] = 0.f;
+        for (int j0 = 0; j0 < ns; j0 += kLevTile) {
+            __syncthreads();
+            for (int e = threadIdx.x; e < kLevTile * 16; e += kLevRows) {
+                const int j = j0 + (e >> 4), k = k0 + (e & 15);
+                sq[e >> 4][e & 15] = (j < ns && k < rr) ? Q[(int64_t)j * rr + k] : 0.f;
+            }
+            __syncthreads();
+            const int nj = min(kLevTile, ns - j0);
+            for (int jj = 0; jj < nj; jj += 16) {
+                float g[16];
+#pragma unroll
+                for (int u = 0; u < 16; ++u) g[u] = jj + u < nj ? __ldg(Gi + (int64_t)(j0 + jj + u) * ns) : 0.f;
+#pragma unroll
+                for (int u = 0; u < 16; ++u) {
+                    float x[16];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        *reinterpret_cast<float4*>(x + 4 * k) = *reinterpret_cast<const float4*>(&sq[jj + u][4 * k]);
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) a[k] = fmaf(g[u], x[k], a[k]);
+                }
+            }
+        }
+        if (i < ns) {
+#pragma unroll
+            for (int k = 0; k < 16; ++k)
+                if (k0 + k < rr) Y[(int64_t)i * rr + k0 + k] = a[k];
+        }
+    }
 }
 
 bool frame_ok3(const lt_frame* f) { return f && f->slice_off && f->S > 0 && f->S <= 1024 && f->C >= 1 && f->pts; }
@@ -760,7 +950,7 @@ extern "C" lt_status lt_slice_matrices(lt_ctx* ctx, const lt_frame* f, const lt_
     cudaSetDevice(ctx->device);
     k_moff<<<1, 1024, 0, ctx->stream>>>(*f, *smp, moff);
     LT_LAUNCH_CHECK(ctx, "k_moff");
-    k_slice_matrix<<<dim3(std::max(1, 4 * ctx->num_sms / f->S), f->S), 256, 0, ctx->stream>>>(
+    k_slice_matrix<<<dim3(std::max(1, 32 * ctx->num_sms / f->S), f->S), 128, 0, ctx->stream>>>(
         *f, *smp, ctx->grid, d_min * d_min, moff, cap, M, ctx->d_status);
     LT_LAUNCH_CHECK(ctx, "k_slice_matrix");
     return LT_OK;
@@ -780,20 +970,29 @@ extern "C" lt_status lt_leverage_targets(lt_ctx* ctx, const lt_frame* f, const l
     const int64_t gcap = (int64_t)S * nmax * nmax;
     lt_status st;
     char* p = (char*)lt_scratch(ctx, SCR_PROPOSAL_T,
-                                (size_t)gcap * 4 + (size_t)2 * S * C * r * 4 + (size_t)(S + 1) * 8 + 4 * 256, &st);
+                                (size_t)gcap * 4 + (size_t)2 * S * C * r * 4 + (size_t)(S + 1) * 16 + 4 * 256, &st);
     if (!p) return st;
     float* G = (float*)p;
     float* Q = (float*)(p + (((size_t)gcap * 4 + 255) & ~(size_t)255));
     float* Y = Q + (size_t)S * C * r;
     int64_t* goff2 = (int64_t*)((char*)Y + (((size_t)S * C * r * 4 + 255) & ~(size_t)255));
-    k_goff<<<1, 1024, 0, ctx->stream>>>(*smp, S, goff2);
+    int64_t* tpfx = goff2 + S + 1;
+    k_goff<<<1, 1024, 0, ctx->stream>>>(*smp, S, goff2, tpfx);
     LT_LAUNCH_CHECK(ctx, "k_goff");
-    const unsigned tiles = (unsigned)((nmax + 31) / 32);
-    k_gram<<<dim3(tiles, tiles, S), 256, 0, ctx->stream>>>(*f, *smp, M, moff, goff2, gcap, G);
+    k_gram<<<2 * ctx->num_sms, 256, 0, ctx->stream>>>(*f, *smp, M, moff, goff2, tpfx, gcap, G);
     LT_LAUNCH_CHECK(ctx, "k_gram");
-    k_leverage<<<S, 512, 0, ctx->stream>>>(*smp, f->slice_id, S, C, G, goff2, gcap, r, iters, seed, Q, Y, group_off,
-                                           target);
-    LT_LAUNCH_CHECK(ctx, "k_leverage");
+    // Q of a round is the product of the round before: the two buffers change roles
+    const unsigned rows = (unsigned)std::max(1, std::min((C + kLevRows - 1) / kLevRows, 12 * ctx->num_sms / S));
+    for (int it = 0; it <= iters; ++it) {
+        k_lev_mgs<<<S, kLevThreads, 0, ctx->stream>>>(*smp, f->slice_id, S, C, goff2, gcap, r, it == 0, it == iters, seed,
+                                                      Q, Y, group_off, target);
+        LT_LAUNCH_CHECK(ctx, "k_lev_mgs");
+        if (it < iters) {
+            k_lev_mult<<<dim3(rows, S), kLevRows, 0, ctx->stream>>>(*smp, S, C, G, goff2, gcap, r, Q, Y);
+            LT_LAUNCH_CHECK(ctx, "k_lev_mult");
+            std::swap(Q, Y);
+        }
+    }
     return LT_OK;
 }
 
