@@ -103,14 +103,17 @@ __global__ void __launch_bounds__(kP1Threads) k_pass1_plan(lt_frame F, float rat
 }
 
 // ------------------------------------------------------------------ pass 1: flat kernels
-// Every step below runs over all slices at once.  Per forest level: setup lays out
-// the union of each testable sibling pair and queues the entries it lacks (small
-// pairs by a thread, big ones by a CTA), rays evaluates the queue (one shadow ray
-// per thread), decide reduces eps, applies Eq. 2 and merges or rejects.  The levels
-// run either as separate launches per step (the default: on the 256x256, 16K-VPL
-// frame 2.07 ms) or inside one persistent cooperative launch with grid-wide
-// barriers between the steps (k_p1_walk, 2.52 ms there: the steps are chains of
-// dependent loads, and a grid barrier costs more than a launch inside a graph).
+// Every step below runs over all slices at once.  Per forest level a testable sibling
+// pair is handled from end to end by one group of lanes: the union of the two sorted
+// row lists (the slot of a row is its rank in its own list plus its rank in the other
+// less the rows in both), one shadow ray per row that only one child holds, eps over
+// the union, Eq. 2, and the merge.  Pairs of up to kSmallPair rows take 8 lanes, of up
+// to kMidPair a warp, bigger ones a CTA.  A level is two launches (small pairs, which
+// also list the others; then the others), or two steps of one persistent cooperative
+// launch with grid-wide barriers (k_p1_walk).  What bounds it: latency (dependent loads,
+// then the rays of a pair).  Against five launches a level with the missing entries in a
+// queue and a serial merge per small pair: the 64x64 frame 1.71 to 1.19 ms, the sampling of
+// the 512x512 scene with 1000 boxes 7.03 to 6.43 ms.
 
 struct P1Store {
     int32_t* rows;     // [total] row of each storage slot
@@ -124,14 +127,12 @@ struct P1Work {
     int64_t* kpfx;     // [S+1] prefix over slices of the initial entry counts
     float* leafmean;   // [S][C] mean of each cut node's initial entries
     float* thr;        // [S] tau * S_hat (-1 in a dark slice, S_hat = 0)
-    int64_t* mcount;   // [Hmax] queued missing entries per level
-    int64_t* bcount;   // [Hmax] big pairs per level
-    int64_t* mdst;     // [mcap] flat value index (v0 or v1) of a missing entry
-    int32_t* mpt;      // [mcap] slice-ordered point of the entry
-    int32_t* mnode;    // [mcap] tree node of the entry's column
-    int64_t* big;      // [bcap] flat pair index of a big pair
+    int64_t* mcount;   // [Hmax] pairs of a warp per level
+    int64_t* bcount;   // [Hmax] pairs of a CTA per level
+    int64_t* mid;      // [bcap] flat pair index of a warp's pair
+    int64_t* big;      // [bcap] flat pair index of a CTA's pair
     unsigned* bar;     // arrival counter of the persistent walk's grid barriers
-    int64_t mcap, bcap;
+    int64_t bcap;
 };
 
 // -- draws of the cut nodes and state of every forest node
@@ -391,217 +392,101 @@ __device__ __forceinline__ bool load_pair(const lt_frame& F, const P1Plan& pl, c
     return true;
 }
 
-// Reserve n queue slots for each lane of the warp with one atomic per warp; returns
-// this lane's first slot.  Every lane of the warp must call it.
-__device__ __forceinline__ long long warp_reserve(unsigned long long* counter, int n) {
-    const int lane = threadIdx.x & 31;
-    int incl = n;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    unsigned long long base = 0;
-    if (lane == 31 && total > 0) base = atomicAdd(counter, (unsigned long long)total);
-    base = __shfl_sync(0xffffffffu, base, 31);
-    return (long long)base + (incl - n);
-}
+// -- one level: pairs of a group of lanes
+constexpr int kSmallPair = 32;   // rows of both children: 8 lanes, at most 4 rows a lane
+constexpr int kMidPair = 256;    // a warp, at most 8 rows a lane
+constexpr int kGroup = 8;
 
-__device__ __forceinline__ void put_missing(const P1Work& w, long long q, int64_t dst, int pt, int node,
+__device__ __forceinline__ float pair_entry(const lt_frame& F, const Grid& g, float dmin2, int row, int node,
                                             int32_t* status) {
-    if (q < w.mcap) {
-        w.mdst[q] = dst;
-        w.mpt[q] = pt;
-        w.mnode[q] = node;
-    } else {
-        latch(status, LT_ELIMIT);
-    }
-}
-
-// -- level h, step 1: union layout of every testable pair, queue of missing entries.
-// A pair of at most kThreadPair rows is laid out by one thread (a serial merge of
-// the two sorted lists, once to count the rows that only one list holds and once to
-// write), a bigger one by a CTA (queued as big).
-constexpr int kThreadPair = 64;
-
-__device__ __forceinline__ bool pair_big(const PairCtx& pc) { return pc.na + pc.nb > kThreadPair; }
-
-__device__ __forceinline__ int serial_missing(const PairCtx& pc) {
-    int i = 0, j = 0, nmiss = 0;
-    while (i < pc.na || j < pc.nb) {
-        const int xa = i < pc.na ? pc.ra[i] : 0x7fffffff, xb = j < pc.nb ? pc.rb[j] : 0x7fffffff;
-        if (xa < xb) ++i, ++nmiss;
-        else if (xb < xa) ++j, ++nmiss;
-        else ++i, ++j;
-    }
-    return nmiss;
-}
-
-__device__ __forceinline__ void serial_write(const lt_frame& F, const P1Plan& pl, const P1Store& st, const P1Work& w,
-                                             const PairCtx& pc, long long q, int32_t* status) {
-    const int ta = F.forest[8 * pc.a], tb = F.forest[8 * pc.b];
-    int32_t* rf = st.rows + pc.iff;
-    float* fa = st.v0 + pc.iff;
-    float* fb = st.v1 + pc.iff;
-    int i = 0, j = 0, n = 0;
-    while (i < pc.na || j < pc.nb) {
-        const int xa = i < pc.na ? pc.ra[i] : 0x7fffffff, xb = j < pc.nb ? pc.rb[j] : 0x7fffffff;
-        if (xa < xb) {
-            rf[n] = xa;
-            fa[n] = st.v0[pc.ia + i++];
-            put_missing(w, q++, st.total + pc.iff + n, pc.row0 + xa, tb, status);   // V_b(xa)
-        } else if (xb < xa) {
-            rf[n] = xb;
-            fb[n] = st.v0[pc.ib + j++];
-            put_missing(w, q++, pc.iff + n, pc.row0 + xb, ta, status);              // V_a(xb)
-        } else {
-            rf[n] = xa;
-            fa[n] = st.v0[pc.ia + i++];
-            fb[n] = st.v0[pc.ib + j++];
-        }
-        ++n;
-    }
-    pl.cnt[(int64_t)pc.s * (2 * F.C - 1) + pc.f] = n;
-}
-
-__device__ __forceinline__ void p1_setup_body(const lt_frame& F, const P1Plan& pl, const P1Store& st, const P1Work& w,
-                                              int h, int32_t* status) {
-    const int np = F.level_off[h + 1] - F.level_off[h];
-    const int64_t npairs = (int64_t)F.S * np;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    // warp-uniform trip count so that every lane takes part in the reservations
-    for (int64_t t0 = blockIdx.x * (int64_t)blockDim.x; t0 < npairs; t0 += stride) {
-        const int64_t t = t0 + threadIdx.x;
-        PairCtx pc;
-        const bool active = t < npairs && load_pair(F, pl, st, h, t, pc);
-        const bool big = active && pair_big(pc);
-        const long long qb = warp_reserve((unsigned long long*)&w.bcount[h], big ? 1 : 0);
-        if (big) {
-            if (qb < w.bcap) w.big[qb] = t;
-            else latch(status, LT_ELIMIT);
-        }
-        const bool mine = active && !big;
-        const long long q = warp_reserve((unsigned long long*)&w.mcount[h], mine ? serial_missing(pc) : 0);
-        if (mine) serial_write(F, pl, st, w, pc, q, status);
-    }
-}
-
-// big pairs, one CTA per pair: both sorted row lists staged in shared memory (global
-// reads beyond kBigStage rows), the slot of a row from its rank in the other list
-// (binary search) and a block scan of the "in both" flags
-constexpr int kBigStage = 4096;
-
-__device__ __forceinline__ void p1_setup_big_body(const lt_frame& F, const P1Plan& pl, const P1Store& st,
-                                                  const P1Work& w, int h, int32_t* status) {
-    __shared__ int32_t sa[kBigStage], sb[kBigStage];
-    __shared__ int32_t ws[32];
-    const int NF = 2 * F.C - 1;
-    const int64_t nbig = min(w.bcount[h], w.bcap);
-    for (int64_t q = blockIdx.x; q < nbig; q += gridDim.x) {
-        PairCtx pc;
-        if (!load_pair(F, pl, st, h, w.big[q], pc)) continue;  // uniform in the block
-        const int ta = F.forest[8 * pc.a], tb = F.forest[8 * pc.b];
-        const bool staged = pc.na <= kBigStage && pc.nb <= kBigStage;
-        __syncthreads();  // the previous pair is done with the stage
-        if (staged) {
-            for (int i = threadIdx.x; i < pc.na; i += blockDim.x) sa[i] = pc.ra[i];
-            for (int j = threadIdx.x; j < pc.nb; j += blockDim.x) sb[j] = pc.rb[j];
-        }
-        __syncthreads();
-        const int32_t* A = staged ? sa : pc.ra;
-        const int32_t* B = staged ? sb : pc.rb;
-        int32_t* rf = st.rows + pc.iff;
-        float* fa = st.v0 + pc.iff;
-        float* fb = st.v1 + pc.iff;
-        int common = 0;
-        for (int i0 = 0; i0 < pc.na; i0 += blockDim.x) {
-            const int i = i0 + threadIdx.x;
-            int x = 0, pb = 0;
-            bool both = false;
-            if (i < pc.na) {
-                x = A[i];
-                pb = lower_bound<int32_t>(B, pc.nb, x);
-                both = pb < pc.nb && B[pb] == x;
-            }
-            int tot;
-            const int pre = block_exclusive_scan<int>(both ? 1 : 0, ws, &tot);
-            const long long m = warp_reserve((unsigned long long*)&w.mcount[h], (i < pc.na && !both) ? 1 : 0);
-            if (i < pc.na) {
-                const int slot = i + pb - (common + pre);
-                rf[slot] = x;
-                fa[slot] = st.v0[pc.ia + i];
-                if (both) fb[slot] = st.v0[pc.ib + pb];
-                else put_missing(w, m, st.total + pc.iff + slot, pc.row0 + x, tb, status);   // V_b(x)
-            }
-            common += tot;
-        }
-        int seen = 0;
-        for (int j0 = 0; j0 < pc.nb; j0 += blockDim.x) {
-            const int j = j0 + threadIdx.x;
-            int y = 0, pa = 0;
-            bool both = false;
-            if (j < pc.nb) {
-                y = B[j];
-                pa = lower_bound<int32_t>(A, pc.na, y);
-                both = pa < pc.na && A[pa] == y;
-            }
-            int tot;
-            const int pre = block_exclusive_scan<int>(both ? 1 : 0, ws, &tot);
-            const long long m = warp_reserve((unsigned long long*)&w.mcount[h], (j < pc.nb && !both) ? 1 : 0);
-            if (j < pc.nb && !both) {
-                const int slot = j + pa - (seen + pre);
-                rf[slot] = y;
-                fb[slot] = st.v0[pc.ib + j];
-                put_missing(w, m, pc.iff + slot, pc.row0 + y, ta, status);   // V_a(y)
-            }
-            seen += tot;
-        }
-        if (threadIdx.x == 0) pl.cnt[(int64_t)pc.s * NF + pc.f] = pc.na + pc.nb - common;
-    }
-}
-
-// -- level h, step 2: the queued entries, one shadow ray per thread
-__device__ __forceinline__ void p1_rays_body(const lt_frame& F, const Grid& g, float dmin2, const P1Store& st,
-                                             const P1Work& w, int h, int32_t* status) {
-    const float4* pts = reinterpret_cast<const float4*>(F.pts);
     const float4* vpls = reinterpret_cast<const float4*>(F.vpls);
-    const int64_t n = min(w.mcount[h], w.mcap);
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
-        const int node = w.mnode[q];
-        const PointRec P = load_rec(pts, F.m, w.mpt[q]);
-        const PointRec L = load_rec(vpls, F.n, F.tree.rep[node]);
-        const float v = entry_value(P, L, node_scale(F.tree, vpls, F.n, node), dmin2, g);
-        if (!isfinite(v)) latch(status, LT_ENUMERIC);
-        st.v0[w.mdst[q]] = v;
-    }
+    const PointRec P = load_rec(reinterpret_cast<const float4*>(F.pts), F.m, row);
+    const PointRec L = load_rec(vpls, F.n, F.tree.rep[node]);
+    const float v = entry_value(P, L, node_scale(F.tree, vpls, F.n, node), dmin2, g);
+    if (!isfinite(v)) latch(status, LT_ENUMERIC);
+    return v;
 }
 
-// -- level h, step 3: eps (Sec. 4), cost (Eq. 2), merge or reject
+// The ratios of a pair (Sec. 4): q is estimated from p, the child whose representative
+// the parent takes.
+struct PairRatio {
+    int ta, tb;
+    bool p_is_a;
+    float rq;   // I_q / I_p
+    float rfp;  // I_f / I_p
+};
+
+__device__ __forceinline__ PairRatio pair_ratio(const lt_frame& F, const PairCtx& pc) {
+    PairRatio r;
+    r.ta = F.forest[8 * pc.a];
+    r.tb = F.forest[8 * pc.b];
+    const float Ia = F.tree.I[r.ta], Ib = F.tree.I[r.tb], If = F.tree.I[F.forest[8 * pc.f]];
+    r.p_is_a = Ia >= Ib;
+    r.rq = r.p_is_a ? __fdiv_rn(Ib, Ia) : __fdiv_rn(Ia, Ib);
+    r.rfp = __fdiv_rn(If, r.p_is_a ? Ia : Ib);
+    return r;
+}
+
+// One row of the union: element t of the concatenated lists (t < na: row t of a, else row
+// t - na of b), its place p in the other list and whether the other holds it too.
+struct PairRow {
+    int x, p;
+    bool in_a, in_b, both;
+};
+
+__device__ __forceinline__ PairRow pair_row(const int32_t* A, int na, const int32_t* B, int nb, int t) {
+    PairRow r;
+    r.in_a = t < na;
+    r.in_b = !r.in_a && t < na + nb;
+    r.x = 0;
+    r.p = 0;
+    r.both = false;
+    if (r.in_a || r.in_b) {
+        const int32_t* O = r.in_a ? B : A;
+        const int no = r.in_a ? nb : na;
+        r.x = r.in_a ? A[t] : B[t - na];
+        r.p = lower_bound<int32_t>(O, no, r.x);
+        r.both = r.p < no && O[r.p] == r.x;
+    }
+    return r;
+}
+
+// Values of a row for both children (the missing one evaluated), stored at `slot`;
+// returns |V_q - V_p I_q / I_p|.
+__device__ __forceinline__ float pair_put(const lt_frame& F, const Grid& g, float dmin2, const P1Store& st,
+                                          const PairCtx& pc, const PairRatio& pr, const PairRow& r, int t, int slot,
+                                          int32_t* status) {
+    const float own = st.v0[r.in_a ? pc.ia + t : pc.ib + (t - pc.na)];
+    const float oth = r.both ? st.v0[pc.ib + r.p] : pair_entry(F, g, dmin2, pc.row0 + r.x, r.in_a ? pr.tb : pr.ta, status);
+    const float va = r.in_a ? own : oth, vb = r.in_a ? oth : own;
+    st.rows[pc.iff + slot] = r.x;
+    st.v0[pc.iff + slot] = va;
+    st.v1[pc.iff + slot] = vb;
+    const float vp = pr.p_is_a ? va : vb, vq = pr.p_is_a ? vb : va;
+    return fabsf(vq - vp * pr.rq);
+}
+
+// Cost (Eq. 2), merge or reject; `first`, `step`: this thread's slots of the union.
 __device__ __forceinline__ void decide_pair(const lt_frame& F, const P1Plan& pl, const P1Store& st, const float* thr,
-                                            const PairCtx& pc, float e_max, int first, int step, bool writer) {
+                                            const PairCtx& pc, const PairRatio& pr, int nf, float e_max, int first,
+                                            int step, bool writer) {
     const int NF = 2 * F.C - 1;
-    const int ta = F.forest[8 * pc.a], tb = F.forest[8 * pc.b], tf = F.forest[8 * pc.f];
-    const float Ia = F.tree.I[ta], Ib = F.tree.I[tb], If = F.tree.I[tf];
-    const bool p_is_a = Ia >= Ib;
     float* cost = pl.cost + (int64_t)pc.s * NF;
     int32_t* state = pl.state + (int64_t)pc.s * NF;
-    const int q = p_is_a ? pc.b : pc.a;
-    const float cf = e_max + cost[q];
+    const float cf = e_max + cost[pr.p_is_a ? pc.b : pc.a];
     const float th = thr[pc.s];
     const bool merge = th < 0.f ? cf == 0.f : cf < th;  // th < 0: a dark slice
-    const int nf = pl.cnt[(int64_t)pc.s * NF + pc.f];
     if (merge) {
-        const float rfp = __fdiv_rn(If, p_is_a ? Ia : Ib);
         float* fa = st.v0 + pc.iff;
         const float* fb = st.v1 + pc.iff;
         float* keep = st.v2 ? st.v2 + pc.iff : nullptr;
         for (int t = first; t < nf; t += step) {
             if (keep) keep[t] = fa[t];
-            fa[t] = (p_is_a ? fa[t] : fb[t]) * rfp;
+            fa[t] = (pr.p_is_a ? fa[t] : fb[t]) * pr.rfp;
         }
     }
     if (writer) {
+        pl.cnt[(int64_t)pc.s * NF + pc.f] = nf;
         cost[pc.f] = cf;
         state[pc.f] = merge ? kStAlive : kStRejected;
         if (merge) {
@@ -611,80 +496,135 @@ __device__ __forceinline__ void decide_pair(const lt_frame& F, const P1Plan& pl,
     }
 }
 
-__device__ __forceinline__ float pair_eps(const lt_frame& F, const P1Store& st, const PairCtx& pc, int nf, int lane,
-                                          int step) {
-    const int ta = F.forest[8 * pc.a], tb = F.forest[8 * pc.b];
-    const float Ia = F.tree.I[ta], Ib = F.tree.I[tb];
-    const bool p_is_a = Ia >= Ib;
-    const float rq = p_is_a ? __fdiv_rn(Ib, Ia) : __fdiv_rn(Ia, Ib);
-    const float* fa = st.v0 + pc.iff;
-    const float* fb = st.v1 + pc.iff;
+// One pair by each group of G lanes of the warp (every lane of the warp calls it; `live`
+// is uniform in a group).  The trip count is the warp's largest, so that the groups'
+// shadow rays run side by side.
+template <int G>
+__device__ __forceinline__ void group_pair(const lt_frame& F, const Grid& g, float dmin2, const P1Plan& pl,
+                                           const P1Store& st, const float* thr, const PairCtx& pc, bool live,
+                                           int32_t* status) {
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, gl = lane & (G - 1), sh = lane & ~(G - 1);
+    const unsigned gm = G == 32 ? FULL : (1u << G) - 1u, lt = (1u << gl) - 1u;
+    const int na = live ? pc.na : 0, nb = live ? pc.nb : 0;
+    PairRatio pr{};
+    if (live) pr = pair_ratio(F, pc);
+    const int trips = (__reduce_max_sync(FULL, na + nb) + G - 1) / G;
+    int ca = 0, cb = 0;  // rows of a (of b) so far that both children hold
     float e = 0.f;
-    for (int t = lane; t < nf; t += step) {
-        const float vp = p_is_a ? fa[t] : fb[t];
-        const float vq = p_is_a ? fb[t] : fa[t];
-        e = fmaxf(e, fabsf(vq - vp * rq));
+    for (int it = 0; it < trips; ++it) {
+        const int t = it * G + gl;
+        const PairRow r = pair_row(pc.ra, na, pc.rb, nb, t);
+        const unsigned ma = (__ballot_sync(FULL, r.in_a && r.both) >> sh) & gm;
+        const unsigned mb = (__ballot_sync(FULL, r.in_b && r.both) >> sh) & gm;
+        if (r.in_a || (r.in_b && !r.both)) {
+            const int slot = r.in_a ? t + r.p - (ca + __popc(ma & lt)) : t - na + r.p - (cb + __popc(mb & lt));
+            e = fmaxf(e, pair_put(F, g, dmin2, st, pc, pr, r, t, slot, status));
+        }
+        ca += __popc(ma);
+        cb += __popc(mb);
     }
-    return e;
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) e = fmaxf(e, __shfl_xor_sync(FULL, e, o));
+    __syncwarp();  // the group's stores are visible to the group
+    if (live) decide_pair(F, pl, st, thr, pc, pr, na + nb - ca, e, gl, G, gl == 0);
 }
 
-// pairs that are not big, one thread per pair
-__device__ __forceinline__ void p1_decide_body(const lt_frame& F, const P1Plan& pl, const P1Store& st,
-                                               const P1Work& w, int h) {
+// step 1: the pairs of at most kSmallPair rows, 8 lanes each; the others are listed
+__device__ __forceinline__ void p1_small_body(const lt_frame& F, const Grid& g, float dmin2, const P1Plan& pl,
+                                              const P1Store& st, const P1Work& w, int h, int32_t* status) {
     const int np = F.level_off[h + 1] - F.level_off[h];
-    const int NF = 2 * F.C - 1;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < (int64_t)F.S * np;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        PairCtx pc;
-        if (!load_pair(F, pl, st, h, t, pc)) continue;
-        if (pair_big(pc)) continue;
-        const int nf = pl.cnt[(int64_t)pc.s * NF + pc.f];
-        decide_pair(F, pl, st, w.thr, pc, pair_eps(F, st, pc, nf, 0, 1), 0, 1, true);
+    const int64_t npairs = (int64_t)F.S * np;
+    const int lane = threadIdx.x & 31;
+    const int per = blockDim.x / kGroup;
+    for (int64_t t0 = blockIdx.x * (int64_t)per; t0 < npairs; t0 += (int64_t)gridDim.x * per) {  // block-uniform
+        const int64_t t = t0 + threadIdx.x / kGroup;
+        PairCtx pc{};
+        const bool active = t < npairs && load_pair(F, pl, st, h, t, pc);
+        const int rows = pc.na + pc.nb;
+        const bool mid = active && rows > kSmallPair && rows <= kMidPair, big = active && rows > kMidPair;
+        const bool head = (lane & (kGroup - 1)) == 0;
+        const unsigned bm = __ballot_sync(0xffffffffu, mid && head), bb = __ballot_sync(0xffffffffu, big && head);
+        for (int kind = 0; kind < 2; ++kind) {
+            const unsigned b = kind ? bb : bm;
+            if (b == 0) continue;  // warp-uniform
+            unsigned long long base = 0;
+            if (lane == 0) base = atomicAdd((unsigned long long*)(kind ? w.bcount : w.mcount) + h,
+                                            (unsigned long long)__popc(b));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (head && (kind ? big : mid)) {
+                const int64_t q = (int64_t)base + __popc(b & ((1u << lane) - 1u));
+                if (q < w.bcap) (kind ? w.big : w.mid)[q] = t;
+                else latch(status, LT_ELIMIT);
+            }
+        }
+        group_pair<kGroup>(F, g, dmin2, pl, st, w.thr, pc, active && rows <= kSmallPair, status);
     }
 }
 
-// big pairs, one CTA per pair
-__device__ __forceinline__ void p1_decide_big_body(const lt_frame& F, const P1Plan& pl, const P1Store& st,
-                                                   const P1Work& w, int h) {
+// step 2: the listed pairs.  A CTA per pair of more than kMidPair rows (both row lists
+// staged in shared memory when they fit), then a warp per pair.
+constexpr int kBigStage = 4096;
+
+__device__ __forceinline__ void p1_rest_body(const lt_frame& F, const Grid& g, float dmin2, const P1Plan& pl,
+                                             const P1Store& st, const P1Work& w, int h, int32_t* status) {
+    __shared__ int32_t sa[kBigStage], sb[kBigStage];
+    __shared__ int32_t ws[32];
     __shared__ float red[32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int NF = 2 * F.C - 1;
-    const int64_t nbig = min(w.bcount[h], w.bcap);
+    const int64_t nbig = min(w.bcount[h], w.bcap), nmid = min(w.mcount[h], w.bcap);
     for (int64_t q = blockIdx.x; q < nbig; q += gridDim.x) {
         PairCtx pc;
         if (!load_pair(F, pl, st, h, w.big[q], pc)) continue;  // uniform in the block
-        const int nf = pl.cnt[(int64_t)pc.s * NF + pc.f];
-        const float e = warp_max(pair_eps(F, st, pc, nf, threadIdx.x, blockDim.x));
-        __syncthreads();  // red is free
-        if (lane == 0) red[wid] = e;
+        const PairRatio pr = pair_ratio(F, pc);
+        const bool staged = pc.na <= kBigStage && pc.nb <= kBigStage;
+        __syncthreads();  // the previous pair is done with the stage
+        if (staged) {
+            for (int i = threadIdx.x; i < pc.na; i += blockDim.x) sa[i] = pc.ra[i];
+            for (int j = threadIdx.x; j < pc.nb; j += blockDim.x) sb[j] = pc.rb[j];
+        }
         __syncthreads();
+        const int32_t* A = staged ? sa : pc.ra;
+        const int32_t* B = staged ? sb : pc.rb;
+        int ca = 0, cb = 0;
+        float e = 0.f;
+        for (int t0 = 0; t0 < pc.na + pc.nb; t0 += blockDim.x) {
+            const int t = t0 + threadIdx.x;
+            const PairRow r = pair_row(A, pc.na, B, pc.nb, t);
+            int tot;  // rows of a in the low half, of b in the high half (a block is at most 1024)
+            const int pre = block_exclusive_scan<int>(r.both ? (r.in_a ? 1 : 1 << 16) : 0, ws, &tot);
+            if (r.in_a || (r.in_b && !r.both)) {
+                const int slot = r.in_a ? t + r.p - (ca + (pre & 0xffff)) : t - pc.na + r.p - (cb + (pre >> 16));
+                e = fmaxf(e, pair_put(F, g, dmin2, st, pc, pr, r, t, slot, status));
+            }
+            ca += tot & 0xffff;
+            cb += tot >> 16;
+        }
+        e = warp_max(e);
+        if (lane == 0) red[wid] = e;
+        __syncthreads();  // also the block's stores before decide_pair reads them
         float em = 0.f;
         for (int k = 0; k < nw; ++k) em = fmaxf(em, red[k]);
-        decide_pair(F, pl, st, w.thr, pc, em, threadIdx.x, blockDim.x, threadIdx.x == 0);
+        decide_pair(F, pl, st, w.thr, pc, pr, pc.na + pc.nb - ca, em, threadIdx.x, blockDim.x, threadIdx.x == 0);
+    }
+    for (int64_t q = blockIdx.x * (int64_t)nw + wid; q < nmid; q += (int64_t)gridDim.x * nw) {
+        PairCtx pc;
+        if (!load_pair(F, pl, st, h, w.mid[q], pc)) continue;  // uniform in the warp
+        group_pair<32>(F, g, dmin2, pl, st, w.thr, pc, true, status);
     }
 }
 
 // Per-level form: each step of each level is its own launch.
-__global__ void __launch_bounds__(128) k_p1_setup(lt_frame F, P1Plan pl, P1Store st, P1Work w, int h,
-                                                  int32_t* status) {
-    p1_setup_body(F, pl, st, w, h, status);
+__global__ void __launch_bounds__(128, 6) k_p1_small(lt_frame F, Grid g, float dmin2, P1Plan pl, P1Store st, P1Work w,
+                                                  int h, int32_t* status) {
+    p1_small_body(F, g, dmin2, pl, st, w, h, status);
 }
-__global__ void __launch_bounds__(256) k_p1_setup_big(lt_frame F, P1Plan pl, P1Store st, P1Work w, int h,
-                                                      int32_t* status) {
-    p1_setup_big_body(F, pl, st, w, h, status);
-}
-__global__ void __launch_bounds__(128) k_p1_rays(lt_frame F, Grid g, float dmin2, P1Store st, P1Work w, int h,
-                                                 int32_t* status) {
-    p1_rays_body(F, g, dmin2, st, w, h, status);
-}
-__global__ void __launch_bounds__(128) k_p1_decide(lt_frame F, P1Plan pl, P1Store st, P1Work w, int h) {
-    p1_decide_body(F, pl, st, w, h);
-}
-__global__ void __launch_bounds__(256) k_p1_decide_big(lt_frame F, P1Plan pl, P1Store st, P1Work w, int h) {
-    p1_decide_big_body(F, pl, st, w, h);
+__global__ void __launch_bounds__(256, 3) k_p1_rest(lt_frame F, Grid g, float dmin2, P1Plan pl, P1Store st, P1Work w,
+                                                 int h, int32_t* status) {
+    p1_rest_body(F, g, dmin2, pl, st, w, h, status);
 }
 
-// Persistent form: one cooperative launch walks every level, the four steps of a level
+// Persistent form: one cooperative launch walks every level, the two steps of a level
 // separated by grid-wide barriers.  `bar` counts block arrivals (zeroed before the
 // launch); barrier k is passed when it reaches k * gridDim.x.  Every wait is bounded:
 // past the limit the block latches LT_ELIMIT and leaves the walk (so do the others at
@@ -726,14 +666,9 @@ __global__ void __launch_bounds__(256, 3) k_p1_walk(lt_frame F, Grid g, float dm
     unsigned k = 0;
     for (int h = 1; h <= F.H; ++h) {
         if (F.level_off[h + 1] == F.level_off[h]) continue;  // uniform over the grid
-        p1_setup_body(F, pl, st, w, h, status);
+        p1_small_body(F, g, dmin2, pl, st, w, h, status);
         if (!grid_barrier(w.bar, k, status, &s_ok)) return;
-        p1_setup_big_body(F, pl, st, w, h, status);
-        if (!grid_barrier(w.bar, k, status, &s_ok)) return;
-        p1_rays_body(F, g, dmin2, st, w, h, status);
-        if (!grid_barrier(w.bar, k, status, &s_ok)) return;
-        p1_decide_body(F, pl, st, w, h);
-        p1_decide_big_body(F, pl, st, w, h);
+        p1_rest_body(F, g, dmin2, pl, st, w, h, status);
         if (!grid_barrier(w.bar, k, status, &s_ok)) return;
     }
 }
@@ -1249,11 +1184,11 @@ lt_status sample_pass1(lt_ctx* ctx, const lt_frame* f, float rate1, float tau, i
     // storage: rows, then v0 and v1 back to back (a flat value index addresses both);
     // then the work arrays of the flat kernels
     const int Hn = f->H + 2;
-    const int64_t mcap = std::max<int64_t>(acc, 1024), bcap = std::max<int64_t>((int64_t)S * C, 1024);
+    const int64_t bcap = std::max<int64_t>((int64_t)S * C, 1024);
     const size_t store_bytes = (size_t)std::max<int64_t>(acc, 1) * (target > 0 ? 16 : 12) + 1024;
     const size_t eff_bytes = target > 0 ? (size_t)S * NF * 4 : 0;
     const size_t work_bytes = (size_t)(S + 1) * 8 + (size_t)S * C * 4 + (size_t)S * 4 + (size_t)Hn * 16 +
-                              (size_t)mcap * 16 + (size_t)bcap * 8 + eff_bytes + 17 * 256;
+                              (size_t)bcap * 16 + eff_bytes + 17 * 256;
     char* q = (char*)lt_scratch(ctx, SCR_P1_STORE, store_bytes + work_bytes, &st);
     if (!q) return st;
     P1Store store;
@@ -1274,12 +1209,9 @@ lt_status sample_pass1(lt_ctx* ctx, const lt_frame* f, float rate1, float tau, i
     w.thr = (float*)wtake((size_t)S * 4);
     w.mcount = (int64_t*)wtake((size_t)Hn * 8 + 8);
     w.bcount = (int64_t*)wtake((size_t)Hn * 8);
-    w.mdst = (int64_t*)wtake((size_t)mcap * 8);
-    w.mpt = (int32_t*)wtake((size_t)mcap * 4);
-    w.mnode = (int32_t*)wtake((size_t)mcap * 4);
+    w.mid = (int64_t*)wtake((size_t)bcap * 8);
     w.big = (int64_t*)wtake((size_t)bcap * 8);
     w.bar = (unsigned*)(w.mcount + Hn);  // shares the zeroing of the level counters
-    w.mcap = mcap;
     w.bcap = bcap;
     float* effs = target > 0 ? (float*)wtake(eff_bytes) : nullptr;
     if ((size_t)(wp - q) > ctx->scr_size[SCR_P1_STORE])
@@ -1344,16 +1276,11 @@ lt_status sample_pass1(lt_ctx* ctx, const lt_frame* f, float rate1, float tau, i
     for (int h = 1; h <= f->H && !walk; ++h) {
         const int64_t npairs = (int64_t)S * (loff[h + 1] - loff[h]);
         if (npairs == 0) continue;
-        k_p1_setup<<<grid_for(npairs, 128), 128, 0, ctx->stream>>>(*f, pl, store, w, h, ctx->d_status);
-        LT_LAUNCH_CHECK(ctx, "k_p1_setup");
-        k_p1_setup_big<<<4 * nsm, 256, 0, ctx->stream>>>(*f, pl, store, w, h, ctx->d_status);
-        LT_LAUNCH_CHECK(ctx, "k_p1_setup_big");
-        k_p1_rays<<<ray_grid, 128, 0, ctx->stream>>>(*f, ctx->grid, dmin2, store, w, h, ctx->d_status);
-        LT_LAUNCH_CHECK(ctx, "k_p1_rays");
-        k_p1_decide<<<grid_for(npairs, 128), 128, 0, ctx->stream>>>(*f, pl, store, w, h);
-        LT_LAUNCH_CHECK(ctx, "k_p1_decide");
-        k_p1_decide_big<<<4 * nsm, 256, 0, ctx->stream>>>(*f, pl, store, w, h);
-        LT_LAUNCH_CHECK(ctx, "k_p1_decide_big");
+        k_p1_small<<<grid_for(npairs * kGroup, 128), 128, 0, ctx->stream>>>(*f, ctx->grid, dmin2, pl, store, w, h,
+                                                                           ctx->d_status);
+        LT_LAUNCH_CHECK(ctx, "k_p1_small");
+        k_p1_rest<<<4 * nsm, 256, 0, ctx->stream>>>(*f, ctx->grid, dmin2, pl, store, w, h, ctx->d_status);
+        LT_LAUNCH_CHECK(ctx, "k_p1_rest");
     }
     if (target > 0) {
         k_p1_target<<<S, 1024, 0, ctx->stream>>>(*f, pl, effs, target);
