@@ -296,6 +296,20 @@ __global__ void k_om_sellpfx(int S, Omega om, int32_t* status) {
             if (carry > om.sell_cap) latch(status, LT_ELIMIT);
         }
         __syncthreads();
+        // warp tasks before each slice
+        int32_t* tp = side == 0 ? om.rtp : om.ctp;
+        const int32_t* cls = side == 0 ? om.rcls : om.ccls;
+        int64_t tasks = 0;
+        for (int i0 = 0; i0 < S; i0 += blockDim.x) {
+            const int i = i0 + threadIdx.x;
+            int64_t tot;
+            const int64_t pre = block_exclusive_scan<int64_t>(i < S ? cls[16 * i + 8 + kClasses] : 0, ws, &tot);
+            if (i < S) tp[i] = (int32_t)(tasks + pre);
+            tasks += tot;
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) tp[S] = (int32_t)tasks;
+        __syncthreads();
     }
 }
 
@@ -387,81 +401,178 @@ __global__ void k_als_init(lt_frame F, lt_samples smp, Omega om, int R, const in
     }
 }
 
-// ---- Gram of one line by one warp (ranks above 16) ---------------------------
+// ---- One line by one warp (ranks above 16) -----------------------------------
 // For one line (a row of U or of V) with observed entries e and factor rows x_e,
-// G = sum_e x_e x_e^T and b = sum_e a_e x_e.  Lane k accumulates row k of G (all RP
-// columns; G is symmetric) and b_k.  The entries are taken 32 at a time: lane l loads
-// the factor row of entry l with 16-byte loads and stages it in shared memory (the
-// line's Gram buffer, 16-byte chunk c of row l at chunk c ^ (l & 7) so that the
-// stores of eight lanes fill all banks), then for each staged row every lane reads
-// the whole row (broadcast loads) and its own component, and adds x_e[k] x_e and
-// a_e x_e[k].  The rows have stride R; components at or beyond R are zero.  At the
-// end rows k of G go to Gs[RP][RP+1] (over the stage) and b to bs[RP].
-template <int RP>  // RP == 32: lane k holds row k
+// G = sum_e x_e x_e^T and b = sum_e a_e x_e.  Lane k accumulates row k of G (all 32
+// columns; G is symmetric) and b_k, two columns per packed multiply-add.  The entries
+// are taken 32 at a time: eight lanes copy one factor row (128 contiguous bytes, so a
+// copy instruction touches 4 lines and not 32) into the warp's stage, 16-byte chunk c
+// of row q at chunk c ^ (q & 7), and the next 32 rows are on their way (cp.async)
+// while these are added.  Rows have stride R; components at or beyond R are zero.
+constexpr int kWarpStage = 32 * 32;    // floats of one stage: 32 rows of 32
+constexpr int kWarpCol = 36;           // stride of a column of L (16-byte aligned, odd in 16-byte chunks)
+
+__device__ __forceinline__ void copy16(float* dst, const float* src, bool full) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    const int n = full ? 16 : 0;  // 0: the 16 bytes are zeroed and nothing is read
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+}
+
+// starts the copies of rows idx[e0 ..] (at most 32, the rest zero) into st
+__device__ __forceinline__ void stage_entries(int len, int e0, int j, const float* __restrict__ src, int R, bool vec,
+                                              float* st) {
+    const int lane = threadIdx.x & 31, c = lane & 7;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int q = 4 * i + (lane >> 3);
+        const int jq = __shfl_sync(0xffffffffu, j, q);
+        const bool live = e0 + q < len && 4 * c < R;
+        const float* p = src + (live ? (int64_t)jq * R + 4 * c : 0);
+        float* d = st + q * 32 + 4 * (c ^ (q & 7));
+        if (vec) {
+            copy16(d, p, live);
+        } else {  // R not a multiple of 4, or rows not on 16 bytes
+#pragma unroll
+            for (int k = 0; k < 4; ++k) d[k] = live && 4 * c + k < R ? __ldg(p + k) : 0.f;
+        }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
 __device__ __forceinline__ void gram_warp(int len, const uint16_t* __restrict__ idx, const float* __restrict__ val,
-                                          const float* __restrict__ src, int R, float* Gs, float* bs) {
-    static_assert(RP == 32, "one lane per Gram row");
+                                          const float* __restrict__ src, int R, float* st0, float (&g)[32], float& b) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const bool vec = (R & 3) == 0 && ((uintptr_t)src & 15) == 0;
-    float4* xs4 = reinterpret_cast<float4*>(Gs);  // 32 staged rows of 8 chunks (4 KB <= the Gram buffer)
-    const float* xsf = Gs;
-    float g[RP];
+    F32x2 g2[16];
 #pragma unroll
-    for (int c = 0; c < RP; ++c) g[c] = 0.f;
-    float b = 0.f;
-    for (int e0 = 0; e0 < len; e0 += 32) {
-        const int n = min(32, len - e0);
-        const bool mine = lane < n;
-        const int j = mine ? (int)idx[e0 + lane] : 0;
-        const float av = mine ? val[e0 + lane] : 0.f;
-        const float* xr = src + (int64_t)j * R;
-        float4 t[RP / 4];
-#pragma unroll
-        for (int c = 0; c < RP / 4; ++c) {
-            t[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (mine) {
-                if (vec) {
-                    if (4 * c < R) t[c] = __ldg(reinterpret_cast<const float4*>(xr) + c);
-                } else {
-                    t[c].x = 4 * c < R ? __ldg(xr + 4 * c) : 0.f;
-                    t[c].y = 4 * c + 1 < R ? __ldg(xr + 4 * c + 1) : 0.f;
-                    t[c].z = 4 * c + 2 < R ? __ldg(xr + 4 * c + 2) : 0.f;
-                    t[c].w = 4 * c + 3 < R ? __ldg(xr + 4 * c + 3) : 0.f;
-                }
-            }
+    for (int c = 0; c < 16; ++c) g2[c] = 0ull;
+    b = 0.f;
+    const int kc = lane >> 2, kw = lane & 3;
+    int j = lane < len ? (int)idx[lane] : 0;
+    float av = lane < len ? val[lane] : 0.f;
+    __syncwarp();  // the stage is free
+    if (len > 0) stage_entries(len, 0, j, src, R, vec, st0);
+    for (int e0 = 0, h = 0; e0 < len; e0 += 32, h ^= 1) {
+        const float a_now = av;
+        const float* st = st0 + h * kWarpStage;
+        if (e0 + 32 < len) {  // warp-uniform
+            const int e = e0 + 32 + lane;
+            j = e < len ? (int)idx[e] : 0;
+            av = e < len ? val[e] : 0.f;
+            stage_entries(len, e0 + 32, j, src, R, vec, st0 + (h ^ 1) * kWarpStage);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
-        __syncwarp();  // the previous chunk's rows have been read
-#pragma unroll
-        for (int c = 0; c < RP / 4; ++c) xs4[lane * 8 + (c ^ (lane & 7))] = t[c];
         __syncwarp();
-        const int kc = lane >> 2, kw = lane & 3;
-        for (int q = 0; q < n; ++q) {  // n is warp-uniform
-            const float a = __shfl_sync(FULL, av, q);
-            float x[RP];
-#pragma unroll
-            for (int c = 0; c < RP / 4; ++c) {
-                const float4 u = xs4[q * 8 + (c ^ (q & 7))];
-                x[4 * c] = u.x;
-                x[4 * c + 1] = u.y;
-                x[4 * c + 2] = u.z;
-                x[4 * c + 3] = u.w;
-            }
-            const float xk = xsf[(q * 8 + (kc ^ (q & 7))) * 4 + kw];
+        const int n = min(32, len - e0);
+#pragma unroll 2
+        for (int q = 0; q < n; ++q) {
+            const float a = __shfl_sync(FULL, a_now, q);
+            const float xk = st[q * 32 + 4 * (kc ^ (q & 7)) + kw];
+            const F32x2 xx = pack2(xk, xk);
             b = fmaf(a, xk, b);
 #pragma unroll
-            for (int c = 0; c < RP; ++c) g[c] = fmaf(xk, x[c], g[c]);
+            for (int c = 0; c < 8; ++c) {
+                const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(st + q * 32 + 4 * (c ^ (q & 7)));
+                g2[2 * c] = fma2(xx, u.x, g2[2 * c]);
+                g2[2 * c + 1] = fma2(xx, u.y, g2[2 * c + 1]);
+            }
         }
+        __syncwarp();  // the stage after next is this one
     }
-    __syncwarp();  // every lane is done with the staged rows
 #pragma unroll
-    for (int c = 0; c < RP; ++c) Gs[lane * (RP + 1) + c] = g[c];
-    bs[lane] = b;
+    for (int c = 0; c < 16; ++c) unpack2(g2[c], g[2 * c], g[2 * c + 1]);
 }
 
-// A group of G lanes solves (Gram + ridge) u = b for one line: lane k holds row k of
-// the Gram in acc and b_k in rhs.  Returns false when the float factorisation is not
-// acceptable (a non-positive pivot, or pivots spread by more than 1/kPivotRatio).
+// Column J of the Cholesky of a line whose row k lane k holds, and the columns after
+// it.  A column of L goes through shared memory (one store, then 16-byte broadcast
+// loads of its rows below J, a quarter as many instructions as a shuffle per row) and
+// stays there for the backward substitution.  Entries above the diagonal are not
+// used, so every lane updates its whole row.
+template <int J>
+__device__ __forceinline__ void chol_col32(float (&acc)[32], int k, int r, bool& ok, float& dmin, float& dmax,
+                                           float& my_inv, float* Lc) {
+    if constexpr (J < 32) {
+        const float djj = __shfl_sync(0xffffffffu, acc[J], J);
+        if (J < r) {
+            ok &= (djj > 0.f);
+            dmin = djj < dmin ? djj : dmin;
+            dmax = djj > dmax ? djj : dmax;
+        }
+        const float dpos = djj > 0.f ? djj : 1.f;
+        const float ljj = sqrtf(dpos);
+        const float inv = 1.f / ljj;
+        if (k == J) my_inv = inv;
+        const float lij = (k > J) ? acc[J] * inv : (k == J ? ljj : 0.f);
+        acc[J] = lij;
+        Lc[J * kWarpCol + k] = lij;
+        __syncwarp();
+#pragma unroll
+        for (int q = (J + 1) / 4; q < 8; ++q) {
+            const float4 l = *reinterpret_cast<const float4*>(Lc + J * kWarpCol + 4 * q);
+            if (4 * q > J) acc[4 * q] = fmaf(-lij, l.x, acc[4 * q]);
+            if (4 * q + 1 > J) acc[4 * q + 1] = fmaf(-lij, l.y, acc[4 * q + 1]);
+            if (4 * q + 2 > J) acc[4 * q + 2] = fmaf(-lij, l.z, acc[4 * q + 2]);
+            if (4 * q + 3 > J) acc[4 * q + 3] = fmaf(-lij, l.w, acc[4 * q + 3]);
+        }
+        chol_col32<J + 1>(acc, k, r, ok, dmin, dmax, my_inv, Lc);
+    }
+}
+
+// Solves (G + ridge) u = b for one line in one warp: lane k holds row k of G in acc
+// and b_k in rhs and receives u_k.  Returns false when the float factorisation is not
+// acceptable (a non-positive pivot, or pivots spread by more than 1 / kPivotRatio).
+// Lc: 32 columns of kWarpCol floats.
+__device__ __forceinline__ bool warp_solve32(float (&acc)[32], float rhs, int len, int r, float lam_rel, int k,
+                                             float* out_k, float* Lc) {
+    const unsigned FULL = 0xffffffffu;
+    float tr = 0.f;
+#pragma unroll
+    for (int c = 0; c < 32; ++c)
+        if (c == k) tr = acc[c];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(FULL, tr, o);
+    const bool zero = !(tr > 0.f) || len == 0;
+    const float lam = lam_rel * tr / (float)r;
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+        const float d = (k < r) ? acc[c] + lam : 1.f;
+        acc[c] = c == k ? d : (k >= r ? 0.f : acc[c]);
+    }
+    if (k >= r) rhs = 0.f;
+    float dmin = 3.0e38f, dmax = 0.f, inv = 1.f;
+    bool ok = true;
+    chol_col32<0>(acc, k, r, ok, dmin, dmax, inv, Lc);
+    if (!zero && (!ok || dmin < kPivotRatio * dmax)) return false;
+    float y = rhs;  // L y = b: lane k has its row of L in acc
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+        const float yj = __shfl_sync(FULL, y * inv, j);
+        if (k == j) y = yj;
+        else if (k > j) y = fmaf(-acc[j], yj, y);
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {  // L^T x = y: lane k takes its column of L
+        const float4 l = *reinterpret_cast<const float4*>(Lc + k * kWarpCol + 4 * q);
+        acc[4 * q] = l.x;
+        acc[4 * q + 1] = l.y;
+        acc[4 * q + 2] = l.z;
+        acc[4 * q + 3] = l.w;
+    }
+    float x = y;
+#pragma unroll
+    for (int j = 31; j >= 0; --j) {
+        const float xj = __shfl_sync(FULL, x * inv, j);
+        if (k == j) x = xj;
+        else if (k < j) x = fmaf(-acc[j], xj, x);
+    }
+    *out_k = (zero || k >= r) ? 0.f : x;
+    return true;
+}
+
+// ---- Float64 factor and solve of one line in one warp (the retry above rank 16) ----
 // Column J of the in-warp Cholesky and the columns after it, unrolled at compile
 // time (a loop whose inner bound depends on the outer index is not fully unrolled
 // by the compiler, and acc then lives in local memory)
@@ -505,11 +616,11 @@ __device__ __forceinline__ void back_col(const T (&acc)[G], int k, T& x) {
     }
 }
 
-template <int G, typename T, bool SMEM_L>
-__device__ __forceinline__ bool factor_solve_rows(T (&acc)[G], T rhs, bool live, int len, int r, float lam_rel,
-                                                  int k, T* out_k, bool check, float* Lsh) {
+// Lane k holds row k of the Gram in acc and b_k in rhs and receives u_k.
+template <int G, typename T>
+__device__ __forceinline__ void factor_solve_rows(T (&acc)[G], T rhs, int len, int r, float lam_rel, int k,
+                                                  T* out_k) {
     const unsigned FULL = 0xffffffffu;
-    if (!live) len = 0;
     T tr = T(0);
 #pragma unroll
     for (int c = 0; c < G; ++c)
@@ -531,38 +642,6 @@ __device__ __forceinline__ bool factor_solve_rows(T (&acc)[G], T rhs, bool live,
     T dmin = T(3.0e38), dmax = T(0);
     bool ok = true;
     chol_col<G, T, 0>(acc, k, r, ok, dmin, dmax);
-    if (check && !zero && (!ok || dmin < (T)kPivotRatio * dmax)) return false;
-    if (SMEM_L) {
-        // triangular solves through shared memory (Lsh may alias this line's Gram:
-        // every lane has read its row before any lane writes here)
-        __syncwarp();
-        // row k of L; the diagonal slot holds 1 / L[k][k]
-        T dk = T(1);
-#pragma unroll
-        for (int c = 0; c < G; ++c)
-            if (c == k) dk = acc[c];
-#pragma unroll
-        for (int c = 0; c < G; ++c) Lsh[k * G + c] = (c == k) ? (float)(T(1) / dk) : (float)acc[c];
-        __syncwarp();
-        T y = rhs;
-#pragma unroll
-        for (int j = 0; j < G; ++j) {
-            const T yj = __shfl_sync(FULL, y, j, G) * (T)Lsh[j * G + j];
-            if (k == j) y = yj;
-            else if (k > j) y -= (T)Lsh[k * G + j] * yj;
-        }
-        T x = y;
-#pragma unroll
-        for (int j = G - 1; j >= 0; --j) {
-            const T xj = __shfl_sync(FULL, x, j, G) * (T)Lsh[j * G + j];
-            if (k == j) x = xj;
-            else if (k < j) x -= (T)Lsh[j * G + k] * xj;
-        }
-        __syncwarp();
-        *out_k = (zero || k >= r) ? T(0) : x;
-        return true;
-    }
-    if (SMEM_L) return true;  // not reached
     // forward L y = b: lane k holds L[k][0..k] in acc[0..k]
     T y = rhs;
 #pragma unroll
@@ -575,108 +654,82 @@ __device__ __forceinline__ bool factor_solve_rows(T (&acc)[G], T rhs, bool live,
     T x = y;
     back_col<G, T, G - 1>(acc, k, x);
     *out_k = (zero || k >= r) ? T(0) : x;
-    return true;
 }
 
-// the same with row k of the Gram and b_k read from Gs [G][G + 1] and bs
-template <int G, typename T, bool SMEM_L>
-__device__ __forceinline__ bool factor_solve(const float* Gs, const float* bs, bool live, int len, int r,
-                                             float lam_rel, int k, T* out_k, bool check, float* Lsh) {
-    T acc[G];
-#pragma unroll
-    for (int c = 0; c < G; ++c) acc[c] = live ? (T)Gs[k * (G + 1) + c] : T(0);
-    const T rhs = live ? (T)bs[k] : T(0);
-    return factor_solve_rows<G, T, SMEM_L>(acc, rhs, live, len, r, lam_rel, k, out_k, check, Lsh);
-}
+// One half-step for ranks above 16: rows of U (rows_side) or columns of V, a warp per
+// line.  A persistent grid: warps take the frame's lines in order, two at a time, from
+// a counter (lines of one slice run side by side and share its factor rows in L1), so
+// that no CTA waits for another's share.  A line whose pivots fail the check goes to
+// the float64 pass (k_als_retry).
+// What bounds it: the stage reads of the Gram (9 shared-memory wavefronts per entry)
+// and the latency of the 32 dependent columns of the solve.  Completion of the 200-box
+// scene (5.7 M entries, ranks 8 to 32 per slice, 10 sweeps; the lane-group kernel has the
+// slices up to rank 16): 23.9 ms with a lane per factor row in the copies, a shuffle
+// per element in the Cholesky and 32-way bank conflicts in the solves; 16.3 ms so.
+constexpr int kHalfWarps = 8;
+constexpr int kHalfSmem = kHalfWarps * 2 * kWarpStage * 4;  // the columns of L use the stage after the Gram
+static_assert(32 * kWarpCol <= 2 * kWarpStage, "the columns of L fit the stage");
 
-// One half-step for ranks above 16: rows of U (rows_side) or columns of V, slice by
-// slice.  CTA (p, s) takes the p-th of P equal parts of the lines of slice s; a warp
-// builds the Gram of one line at a time (gram_warp, the other side's factor rows
-// read from L2) and factors and solves it in the warp in float32; a line whose
-// pivots fail the check goes to the float64 pass (k_als_retry).
-template <int RP>
-__host__ __device__ constexpr int als_warps() { return RP == 32 ? 8 : 16; }
-
-template <int RP>
-__global__ void __launch_bounds__(32 * als_warps<RP>(), 2) k_als_half(lt_frame F, lt_samples smp, Omega om, int R,
-                                                                   const int32_t* __restrict__ rk,
-                                                                   float lam_rel, bool rows_side,
-                                                                   const float* __restrict__ Fin,
-                                                                   float* __restrict__ Fout, AlsQueue<RP> aq) {
-    constexpr int LPW = 32 / RP;  // lines per warp
-    constexpr int NW = als_warps<RP>();
-    __shared__ __align__(16) float Gs_all[NW][LPW][RP * (RP + 1)];
-    __shared__ float bs_all[NW][LPW][RP];
-    const int s = blockIdx.y, P = gridDim.x, p = blockIdx.x;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int grp = lane / RP, k = lane % RP;
-    const int r = slice_rank(rk, s, R);  // the slice's rank (factor rows have stride R)
-    if (rk && r <= 16) return;           // per-slice ranks: the lane-group kernel has these slices
-    const int row0 = F.slice_off[s], ms = F.slice_off[s + 1] - row0;
-    const int ns = smp.ncol[s];
-    const int nlines = rows_side ? ms : ns;
-    const int l0 = (int)((int64_t)nlines * p / P), l1 = (int)((int64_t)nlines * (p + 1) / P);
-    if (l0 >= l1) return;
-    const float* src = rows_side ? Fin + (int64_t)s * F.C * R : Fin + (int64_t)row0 * R;
-    const int64_t o = smp.off[s];
-    for (int base = l0 + wid * LPW; base < l1; base += NW * LPW) {
-        int my_len = 0;
-        int64_t my_dst = 0, my_pos = 0;
-#pragma unroll
-        for (int q = 0; q < LPW; ++q) {
-            const int line = base + q;
-            if (line >= l1) break;  // warp-uniform
-            int len, b;
-            const uint16_t* idx;
-            const float* vv;
-            int64_t dst;
-            if (rows_side) {
-                const int32_t* rp = om.rp + row0 + s;
-                b = rp[line];
-                len = rp[line + 1] - b;
-                idx = om.cidx + o + b;
-                vv = om.cval + o + b;
-                dst = (int64_t)(row0 + line) * R;           // U row
-            } else {
-                const int32_t* cp = om.cp + (int64_t)s * (F.C + 1);
-                b = cp[line];
-                len = cp[line + 1] - b;
-                idx = om.ridx + o + b;
-                vv = om.rval + o + b;
-                dst = ((int64_t)s * F.C + line) * R;        // V row
+__global__ void __launch_bounds__(32 * kHalfWarps, 2) k_als_half(lt_frame F, lt_samples smp, Omega om, int R,
+                                                                const int32_t* __restrict__ rk, float lam_rel,
+                                                                bool rows_side, const float* __restrict__ Fin,
+                                                                float* __restrict__ Fout, AlsQueue<32> aq,
+                                                                int32_t* __restrict__ next) {
+    extern __shared__ __align__(16) float wst[];
+    const int lane = threadIdx.x & 31, k = lane;
+    float* st = wst + (threadIdx.x >> 5) * 2 * kWarpStage;
+    const int S = F.S;
+    const int64_t total = rows_side ? (int64_t)F.slice_off[S] : om.line_pfx[S];
+    int s = -1;
+    int64_t s_lo = 0, s_hi = 0;  // lines of slice s
+    for (;;) {
+        int64_t L0 = 0;
+        if (lane == 0) L0 = 2 * (int64_t)atomicAdd(next, 1);
+        L0 = __shfl_sync(0xffffffffu, L0, 0);
+        if (L0 >= total) break;
+        for (int64_t L = L0; L < min(L0 + 2, total); ++L) {
+            if (L >= s_hi) {  // the slice with s_lo <= L < s_hi, at or after the last one's
+                int x = s < 0 ? 0 : s + 1, y = S - 1;
+                while (x < y) {
+                    const int m = (x + y) >> 1;
+                    if (L >= (rows_side ? (int64_t)F.slice_off[m + 1] : om.line_pfx[m + 1])) x = m + 1;
+                    else y = m;
+                }
+                s = x;
+                s_lo = rows_side ? (int64_t)F.slice_off[s] : om.line_pfx[s];
+                s_hi = rows_side ? (int64_t)F.slice_off[s + 1] : om.line_pfx[s + 1];
             }
-            gram_warp<RP>(len, idx, vv, src, R, &Gs_all[wid][q][0], &bs_all[wid][q][0]);
-            if (grp == q) {
-                my_len = len;
-                my_dst = dst;
-                my_pos = o + b;
+            const int r = slice_rank(rk, s, R);  // the slice's rank (factor rows have stride R)
+            if (rk && r <= 16) continue;         // per-slice ranks: the lane-group kernel has these slices
+            const int line = (int)(L - s_lo);
+            const int row0 = F.slice_off[s];
+            const int64_t o = smp.off[s];
+            const float* src = rows_side ? Fin + (int64_t)s * F.C * R : Fin + (int64_t)row0 * R;
+            const int32_t* ptr = rows_side ? om.rp + row0 + s : om.cp + (int64_t)s * (F.C + 1);
+            const int b0 = ptr[line], len = ptr[line + 1] - b0;
+            const int64_t dst = rows_side ? (int64_t)(row0 + line) * R : ((int64_t)s * F.C + line) * R;
+            float g[32], b, x = 0.f;
+            gram_warp(len, (rows_side ? om.cidx : om.ridx) + o + b0, (rows_side ? om.cval : om.rval) + o + b0, src, R,
+                      st, g, b);
+            const bool ok = warp_solve32(g, b, len, r, lam_rel, k, &x, st);
+            if (k < R) Fout[dst + k] = (ok && k < r) ? x : 0.f;
+            if (!ok && k == 0) {
+                // rare: the float pivots were not acceptable; k_als_retry forms the line's
+                // Gram again in float64 from the factor rows (a Gram summed in float32 would
+                // carry its rounding into the solve)
+                const int qs = atomicAdd(aq.count, 1);
+                if (qs < aq.cap) {
+                    aq.dst[qs] = dst;
+                    aq.slot[qs] = o + b0;
+                    aq.src[qs] = src - Fin;
+                    aq.len[qs] = len;
+                    aq.grp[qs] = 0;  // contiguous in CSR / CSC
+                    aq.rank[qs] = r;
+                } else {
+                    latch(aq.status, LT_ELIMIT);
+                }
             }
         }
-        __syncwarp();
-        const bool live = base + grp < l1;
-        const float* Gs = &Gs_all[wid][grp][0];
-        const float* bs = &bs_all[wid][grp][0];
-        float xf = 0.f;
-        const bool okf = factor_solve<RP, float, true>(Gs, bs, live, my_len, r, lam_rel, k, &xf, true,
-                                                 &Gs_all[wid][grp][0]);
-        if (live && k < R) Fout[my_dst + k] = (okf && k < r) ? xf : 0.f;
-        if (live && !okf && k == 0) {
-            // rare: the float pivots were not acceptable; the line goes to the float64
-            // pass (k_als_retry), which forms its Gram again in float64 from the factor
-            // rows (a Gram summed in float32 would carry its rounding into the solve)
-            const int qs = atomicAdd(aq.count, 1);
-            if (qs < aq.cap) {
-                aq.dst[qs] = my_dst;
-                aq.slot[qs] = my_pos;
-                aq.src[qs] = src - Fin;
-                aq.len[qs] = my_len;
-                aq.grp[qs] = 0;  // contiguous in CSR / CSC
-                aq.rank[qs] = r;
-            } else {
-                latch(aq.status, LT_ELIMIT);
-            }
-        }
-        __syncwarp();
     }
 }
 
@@ -701,57 +754,91 @@ __device__ __forceinline__ int stage_slot(int j, int q) {
     return j * NQ + (q ^ ((j / RPB) % NQ));
 }
 
+// A factor row, from the staged rows or, for a slice of more rows than the stage holds,
+// from memory (row -1: zeros).
+template <int RP>
+__device__ __forceinline__ void load_row(float (&x)[RP], int j, int r, int R, const float* __restrict__ src,
+                                         bool staged, bool vec, const float4* stage4) {
+    if (staged) {
+#pragma unroll
+        for (int q = 0; q < RP / 4; ++q) {
+            const float4 t = stage4[stage_slot<RP>(j, q)];
+            x[4 * q] = t.x;
+            x[4 * q + 1] = t.y;
+            x[4 * q + 2] = t.z;
+            x[4 * q + 3] = t.w;
+        }
+    } else if (vec) {  // R and r multiples of 4, rows on 16 bytes
+#pragma unroll
+        for (int q = 0; q < RP / 4; ++q) {
+            float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (j >= 0 && 4 * q < r) t = __ldg(reinterpret_cast<const float4*>(src + (int64_t)j * R) + q);
+            x[4 * q] = t.x;
+            x[4 * q + 1] = t.y;
+            x[4 * q + 2] = t.z;
+            x[4 * q + 3] = t.w;
+        }
+    } else {
+#pragma unroll
+        for (int c = 0; c < RP; ++c) x[c] = j >= 0 && c < r ? __ldg(src + (int64_t)j * R + c) : 0.f;
+    }
+}
+
+template <int RP>
+__device__ __forceinline__ void add_entry(const float (&x)[RP], float av, float (&a)[RP * (RP + 1) / 2],
+                                          float (&bb)[RP]) {
+#pragma unroll
+    for (int i = 0; i < RP; ++i) {
+        bb[i] = fmaf(av, x[i], bb[i]);
+#pragma unroll
+        for (int k = 0; k <= i; ++k) a[i * (i + 1) / 2 + k] = fmaf(x[i], x[k], a[i * (i + 1) / 2 + k]);
+    }
+}
+
 // Adds x_e x_e^T (lower triangle) and a_e x_e for the nk entries of one lane's
 // stream (chunks of 4 at idx4[32 c], vv4[32 c]) to a and bb, in stream order.
+// The row of the next entry is loaded before this one is added, so that the
+// shared-memory reads (bank conflicts of random rows) run under the arithmetic.  Every lane
+// runs to the longest stream of the warp; past its own end it adds zeros (row zrow),
+// which leave the sums as they are.  Two entries per round of the inner loop: the
+// whole chunk unrolled is more code than the instruction caches hold.
 template <int RP>
 __device__ __forceinline__ void stream_gram(int nk, const uint2* __restrict__ idx4, const float4* __restrict__ vv4,
-                                            int r, int R, const float* __restrict__ src, bool staged,
-                                            const float4* stage4, float (&a)[RP * (RP + 1) / 2], float (&bb)[RP]) {
-    constexpr int NQ = RP / 4;
-    const int nc = (nk + 3) >> 2;
-    // the next two chunks' loads are in flight during this chunk's four entries
-    uint2 ic = nc > 0 ? idx4[0] : make_uint2(0u, 0u), in = nc > 1 ? idx4[32] : ic;
-    float4 vc = nc > 0 ? vv4[0] : make_float4(0.f, 0.f, 0.f, 0.f), vn = nc > 1 ? vv4[32] : vc;
+                                            int r, int R, const float* __restrict__ src, bool staged, bool vec,
+                                            int zrow, const float4* stage4, float (&a)[RP * (RP + 1) / 2],
+                                            float (&bb)[RP]) {
+#pragma unroll
+    for (int i = 0; i < RP * (RP + 1) / 2; ++i) a[i] = 0.f;
+#pragma unroll
+    for (int i = 0; i < RP; ++i) bb[i] = 0.f;
+    const int nc = (__reduce_max_sync(0xffffffffu, nk) + 3) >> 2;
+    uint2 ic = make_uint2(0u, 0u);
+    float4 vc = make_float4(0.f, 0.f, 0.f, 0.f);
+    float x[RP], y[RP];
+    if (nc > 0) {
+        ic = idx4[0];
+        vc = vv4[0];
+        load_row<RP>(x, nk > 0 ? (int)(ic.x & 0xffffu) : zrow, r, R, src, staged, vec, stage4);
+    }
     for (int c = 0; c < nc; ++c) {
-        uint2 in2 = in;
-        float4 vn2 = vn;
-        if (c + 2 < nc) {
-            in2 = idx4[32 * (c + 2)];
-            vn2 = vv4[32 * (c + 2)];
+        uint2 in = ic;
+        float4 vn = vc;
+        if (c + 1 < nc) {
+            in = idx4[32 * (c + 1)];
+            vn = vv4[32 * (c + 1)];
         }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            if (4 * c + q < nk) {
-                const uint32_t w = q < 2 ? ic.x : ic.y;
-                const int j = (int)((w >> (16 * (q & 1))) & 0xffffu);
-                const float av = q == 0 ? vc.x : q == 1 ? vc.y : q == 2 ? vc.z : vc.w;
-                float x[RP];
-                if (staged) {
-#pragma unroll
-                    for (int c4 = 0; c4 < NQ; ++c4) {
-                        const float4 t = stage4[stage_slot<RP>(j, c4)];
-                        x[4 * c4] = t.x;
-                        x[4 * c4 + 1] = t.y;
-                        x[4 * c4 + 2] = t.z;
-                        x[4 * c4 + 3] = t.w;
-                    }
-                } else {
-#pragma unroll
-                    for (int cc = 0; cc < RP; ++cc) x[cc] = cc < r ? __ldg(src + (int64_t)j * R + cc) : 0.f;
-                }
-#pragma unroll
-                for (int i = 0; i < RP; ++i) {
-                    bb[i] = fmaf(av, x[i], bb[i]);
-#pragma unroll
-                    for (int k = 0; k <= i; ++k)
-                        a[i * (i + 1) / 2 + k] = fmaf(x[i], x[k], a[i * (i + 1) / 2 + k]);
-                }
-            }
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            const int e = 4 * c + 2 * h;
+            const uint32_t w0 = h ? ic.y : ic.x, w1 = h ? in.x : ic.y;
+            const float v0 = h ? vc.z : vc.x, v1 = h ? vc.w : vc.y;
+            load_row<RP>(y, e + 1 < nk ? (int)(w0 >> 16) : zrow, r, R, src, staged, vec, stage4);
+            add_entry<RP>(x, e < nk ? v0 : 0.f, a, bb);
+            load_row<RP>(x, e + 2 < nk ? (int)(w1 & 0xffffu) : zrow, r, R, src, staged, vec, stage4);
+            add_entry<RP>(y, e + 1 < nk ? v1 : 0.f, a, bb);
         }
         ic = in;
         vc = vn;
-        in = in2;
-        vn = vn2;
     }
 }
 
@@ -760,7 +847,7 @@ __device__ __forceinline__ void stream_gram(int nk, const uint2* __restrict__ id
 template <int RP>
 __device__ __forceinline__ void als_line(const lt_frame& F, const Omega& om, int r, int R, bool rows_side,
                                          const float* __restrict__ src_base, const float* __restrict__ src,
-                                         bool staged, const float4* stage4,
+                                         bool staged, bool vec, int zrow, const float4* stage4,
                                          float* __restrict__ Fout, float lam_rel, const AlsQueue<RP>& q, int s,
                                          int line, int sub, int G, int64_t slot) {
     constexpr int NA = RP * (RP + 1) / 2;
@@ -778,13 +865,9 @@ __device__ __forceinline__ void als_line(const lt_frame& F, const Omega& om, int
     const uint16_t* sidx = rows_side ? om.sidx_r : om.sidx_c;
     const float* sval = rows_side ? om.sval_r : om.sval_c;
     float a[NA], bb[RP];
-#pragma unroll
-    for (int i = 0; i < NA; ++i) a[i] = 0.f;
-#pragma unroll
-    for (int i = 0; i < RP; ++i) bb[i] = 0.f;
     const int nk = sub < len ? (len - sub + G - 1) / G : 0;
     stream_gram<RP>(nk, reinterpret_cast<const uint2*>(sidx + slot), reinterpret_cast<const float4*>(sval + slot), r,
-                    R, src, staged, stage4, a, bb);
+                    R, src, staged, vec, zrow, stage4, a, bb);
     if (G > 1) {  // the group's partial sums into its first lane (G is warp-uniform)
         for (int m = G >> 1; m > 0; m >>= 1) {
 #pragma unroll
@@ -817,133 +900,159 @@ __device__ __forceinline__ void als_line(const lt_frame& F, const Omega& om, int
 }
 
 // stage the slice's source factor rows (nsrc rows of stride R, the first r values,
-// zero-padded to RP) in shared memory
+// zero-padded to RP) in shared memory, and a row of zeros after them
 template <int RP>
-__device__ __forceinline__ void stage_factors(const float* __restrict__ src, int nsrc, int r, int R, float4* stage4) {
+__device__ __forceinline__ void stage_factors(const float* __restrict__ src, int nsrc, int r, int R, bool vec,
+                                              float4* stage4) {
     constexpr int NQ = RP / 4;
-    if (r == RP && R == RP) {
-        const float4* src4 = reinterpret_cast<const float4*>(src);
-        for (int i = threadIdx.x; i < nsrc * NQ; i += blockDim.x)
-            stage4[stage_slot<RP>(i / NQ, i % NQ)] = __ldg(src4 + i);
-    } else {
-        for (int i = threadIdx.x; i < nsrc * NQ; i += blockDim.x) {
-            const int row = i / NQ, q4 = i % NQ;
-            float v[4];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) v[c] = 4 * q4 + c < r ? __ldg(src + (int64_t)row * R + 4 * q4 + c) : 0.f;
-            stage4[stage_slot<RP>(row, q4)] = make_float4(v[0], v[1], v[2], v[3]);
+    for (int i = threadIdx.x; i < (nsrc + 1) * NQ; i += blockDim.x) {
+        const int row = i / NQ, q4 = i % NQ;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (row < nsrc) {
+            const float* p = src + (int64_t)row * R + 4 * q4;
+            if (vec) {
+                if (4 * q4 < r) v = __ldg(reinterpret_cast<const float4*>(p));
+            } else {
+                v.x = 4 * q4 < r ? __ldg(p) : 0.f;
+                v.y = 4 * q4 + 1 < r ? __ldg(p + 1) : 0.f;
+                v.z = 4 * q4 + 2 < r ? __ldg(p + 2) : 0.f;
+                v.w = 4 * q4 + 3 < r ? __ldg(p + 3) : 0.f;
+            }
         }
+        stage4[stage_slot<RP>(row, q4)] = v;
     }
 }
 
 // Persistent half-step: one CTA per SM.  CTA c owns the warp tasks (all slices, in
-// slice order) whose first slot lies in its equal share [lo, hi) of all the slots
-// of the side; for each slice it touches it stages the source factor rows once and
-// its warps take that slice's tasks from a shared counter.
+// slice order) whose start lies in its equal share [lo, hi) of the side's work, a task
+// counting its slots and kTaskCost for its solve.  It stages the source factor rows of
+// the slices it touches, as many at once as fit (most shares lie in two or three
+// slices), and its warps take all their tasks from one shared counter.
+// What bounds it: latency at two warps per scheduler (the registers of a lane's Gram) and
+// the bank conflicts of random factor rows.  Completion of 7.2 M entries in 64 slices,
+// rank 16, 10 sweeps: 4.24 ms with 110 KB of stage, one slice staged at a time, shares
+// that count slots only and no row loaded ahead; 3.39 ms so.  With three times the rows
+// (slices over the old stage, read from memory by scalar loads): 11.57 to 7.88 ms.
+// Packed multiply-adds (two elements an instruction) run at the rate of single ones
+// here and cost register moves: 4.58 ms.
+constexpr int kTaskCost = 512;   // slots worth a task's reduction and Cholesky (32 lanes x 16 entries)
+constexpr int kSegs = 8;
+
+struct AlsSeg {
+    int s, t0, t1;      // tasks [t0, t1) of slice s
+    int row;            // first staged row, or -1: not staged
+    int end;            // tasks of the batch up to and with this segment
+};
+
 template <int RP>
-__global__ void __launch_bounds__(256, 1) k_als_line(lt_frame F, lt_samples smp, Omega om, int R,
+__global__ void __launch_bounds__(256, RP == 8 ? 2 : 1) k_als_line(lt_frame F, lt_samples smp, Omega om, int R,
                                                     const int32_t* __restrict__ rk, bool rows_side,
                                                     const float* __restrict__ Fin, float* __restrict__ Fout,
                                                     float lam_rel, AlsQueue<RP> q, int stage_rows) {
     extern __shared__ float4 stage4[];
-    __shared__ int s_next, s_t0, s_t1, s_slice;
+    __shared__ int s_next, s_n;
+    __shared__ AlsSeg seg[kSegs];
     const int S = F.S;
     const int64_t* base = rows_side ? om.rbase : om.cbase;
-    const int64_t total = base[S];
+    const int32_t* tpfx = rows_side ? om.rtp : om.ctp;
+    const int32_t* cls_all = rows_side ? om.rcls : om.ccls;
+    const int32_t* tb_all = rows_side ? om.rtb : om.ctb;
     // a layout over its capacity was latched as LT_ELIMIT and not written: read nothing
-    if (total > om.sell_cap) return;
+    if (base[S] > om.sell_cap) return;
+    const int64_t total = base[S] + (int64_t)kTaskCost * tpfx[S];
     const int64_t lo = total * blockIdx.x / gridDim.x;
     const int64_t hi = blockIdx.x + 1 == gridDim.x ? INT64_MAX : total * (blockIdx.x + 1) / gridDim.x;
+    // work before task t of slice x
+    auto before = [&](int x, int t) {
+        return base[x] + tb_all[(int64_t)x * om.tcap + t] + (int64_t)kTaskCost * (tpfx[x] + t);
+    };
+    // first task in [t, T) of slice x that starts at or after `at`
+    auto first_task = [&](int x, int t, int T, int64_t at) {
+        while (t < T) {
+            const int m = (t + T) >> 1;
+            if (before(x, m) < at) t = m + 1; else T = m;
+        }
+        return t;
+    };
     const int lane = threadIdx.x & 31;
-    int s = -1, t = 0;  // next task to consider (thread 0's view, shared through s_*)
+    int s = -1, t = 0;  // next task to consider (thread 0's view, shared through seg)
     if (threadIdx.x == 0) {
         // Task starts are non-decreasing in (slice, task) order and every task of slice
-        // s starts at or before base[s + 1]: the first slice with base[s + 1] >= lo holds
-        // the first task at or after lo, if it has one, else a later slice does.
+        // s starts at or before the end of slice s: the first slice that ends at or after
+        // lo holds the first task at or after lo, if it has one, else a later slice does.
         int x = 0, y = S;
         while (x < y) {
             const int m = (x + y) >> 1;
-            if (base[m + 1] < lo) x = m + 1; else y = m;
+            if (base[m + 1] + (int64_t)kTaskCost * tpfx[m + 1] < lo) x = m + 1; else y = m;
         }
         s = x;
-        t = 0;
-        if (s < S) {
-            const int32_t* cls = (rows_side ? om.rcls : om.ccls) + (int64_t)s * 16;
-            const int32_t* tb = (rows_side ? om.rtb : om.ctb) + (int64_t)s * om.tcap;
-            int a = 0, b = cls[8 + kClasses];
-            while (a < b) {
-                const int m = (a + b) >> 1;
-                if (base[s] + tb[m] < lo) a = m + 1; else b = m;
-            }
-            t = a;
-        }
+        t = s < S ? first_task(s, 0, tpfx[s + 1] - tpfx[s], lo) : 0;
     }
     for (;;) {
         if (threadIdx.x == 0) {
-            // the next slice segment of this CTA: tasks [t, t1) of slice s starting before hi
-            int seg = -1, t0 = 0, t1 = 0;
-            while (s < S) {
-                const int32_t* cls = (rows_side ? om.rcls : om.ccls) + (int64_t)s * 16;
-                const int32_t* tb = (rows_side ? om.rtb : om.ctb) + (int64_t)s * om.tcap;
-                const int T = cls[8 + kClasses];
-                if (t < T && base[s] + tb[t] < hi) {
-                    int x = t, y = T;  // first task at or after hi
-                    while (x < y) {
-                        const int m = (x + y) >> 1;
-                        if (base[s] + tb[m] < hi) x = m + 1; else y = m;
-                    }
-                    seg = s;
-                    t0 = t;
-                    t1 = x;
-                    if (x < T) {
-                        s = S;  // the share ends inside this slice
-                    } else {
-                        ++s;
-                        t = 0;
-                    }
-                    break;
+            // the next slice segments of this CTA (tasks starting before hi), while their rows fit
+            int n = 0, used = 0, tasks = 0;
+            while (s < S && n < kSegs) {
+                const int T = tpfx[s + 1] - tpfx[s];
+                if (t < T && before(s, t) >= hi) s = S;  // the share ends here
+                if (s >= S) break;
+                const int r = slice_rank(rk, s, R);
+                const int t1 = first_task(s, t, T, hi);
+                if (t < t1 && r <= RP) {  // per-slice ranks above RP are the warp-per-line kernel's
+                    const int need = (rows_side ? smp.ncol[s] : F.slice_off[s + 1] - F.slice_off[s]) + 1;
+                    const bool fits = need <= stage_rows;
+                    if (fits && used + need > stage_rows) break;  // in the next batch
+                    tasks += t1 - t;
+                    seg[n++] = AlsSeg{s, t, t1, fits ? used : -1, tasks};
+                    if (fits) used += need;
                 }
-                if (t < T) {  // the next task of this slice is past hi: done
-                    s = S;
-                    break;
+                if (t1 < T) {
+                    s = S;  // the share ends inside this slice
+                } else {
+                    ++s;
+                    t = 0;
                 }
-                ++s;
-                t = 0;
             }
-            s_slice = seg;
-            s_t0 = t0;
-            s_t1 = t1;
-            s_next = t0;
+            s_n = n;
+            s_next = 0;
         }
         __syncthreads();
-        const int sl = s_slice;
-        if (sl < 0) break;
-        const int row0 = F.slice_off[sl], ms = F.slice_off[sl + 1] - row0, ns = smp.ncol[sl];
-        const int r = slice_rank(rk, sl, R);  // the slice's rank (factor rows have stride R)
-        const bool mine = r <= RP;      // per-slice ranks above RP are the warp-group kernel's
-        const float* src = rows_side ? Fin + (int64_t)sl * F.C * R : Fin + (int64_t)row0 * R;
-        const int nsrc = rows_side ? ns : ms;
-        const bool staged = nsrc <= stage_rows;
-        if (staged && mine) stage_factors<RP>(src, nsrc, r, R, stage4);
+        const int n = s_n;
+        if (n == 0) break;
+        for (int k = 0; k < n; ++k) {
+            if (seg[k].row < 0) continue;
+            const int sl = seg[k].s, row0 = F.slice_off[sl], r = slice_rank(rk, sl, R);
+            const float* src = rows_side ? Fin + (int64_t)sl * F.C * R : Fin + (int64_t)row0 * R;
+            const bool vec = (R & 3) == 0 && (r & 3) == 0 && ((uintptr_t)src & 15) == 0;
+            stage_factors<RP>(src, rows_side ? smp.ncol[sl] : F.slice_off[sl + 1] - row0, r, R, vec,
+                              stage4 + seg[k].row * (RP / 4));
+        }
         __syncthreads();
-        const int32_t* ord = rows_side ? om.rord + row0 : om.cord + (int64_t)sl * F.C;
-        const int32_t* cls = (rows_side ? om.rcls : om.ccls) + (int64_t)sl * 16;
-        const int32_t* tb = (rows_side ? om.rtb : om.ctb) + (int64_t)sl * om.tcap;
-        const int t1 = mine ? s_t1 : 0;
         for (;;) {
             int tk = 0;
             if (lane == 0) tk = atomicAdd(&s_next, 1);
             tk = __shfl_sync(0xffffffffu, tk, 0);
-            if (tk >= t1) break;
+            if (tk >= seg[n - 1].end) break;
             int k = 0;
-            while (k + 1 < kClasses && tk >= cls[8 + k + 1]) ++k;
-            const int g = kClasses - 1 - k, G = 1 << g;
-            const int li = cls[k] + (tk - cls[8 + k]) * (32 >> g) + (lane >> g);
-            const bool live = li < cls[k + 1];
-            als_line<RP>(F, om, r, R, rows_side, Fin, src, staged, stage4, Fout, lam_rel, q, sl, live ? ord[li] : -1,
-                         lane & (G - 1), G, base[sl] + tb[tk] + 4 * lane);
+            while (tk >= seg[k].end) ++k;
+            tk = seg[k].t1 - (seg[k].end - tk);
+            const int sl = seg[k].s, row0 = F.slice_off[sl], r = slice_rank(rk, sl, R);
+            const bool staged = seg[k].row >= 0;
+            const int nsrc = rows_side ? smp.ncol[sl] : F.slice_off[sl + 1] - row0;
+            const float* src = rows_side ? Fin + (int64_t)sl * F.C * R : Fin + (int64_t)row0 * R;
+            const bool vec = (R & 3) == 0 && (r & 3) == 0 && ((uintptr_t)src & 15) == 0;
+            const int32_t* ord = rows_side ? om.rord + row0 : om.cord + (int64_t)sl * F.C;
+            const int32_t* cls = cls_all + (int64_t)sl * 16;
+            int c = 0;
+            while (c + 1 < kClasses && tk >= cls[8 + c + 1]) ++c;
+            const int g = kClasses - 1 - c, G = 1 << g;
+            const int li = cls[c] + (tk - cls[8 + c]) * (32 >> g) + (lane >> g);
+            const bool live = li < cls[c + 1];
+            als_line<RP>(F, om, r, R, rows_side, Fin, src, staged, vec, staged ? nsrc : -1,
+                         stage4 + (staged ? seg[k].row * (RP / 4) : 0), Fout, lam_rel, q, sl, live ? ord[li] : -1,
+                         lane & (G - 1), G, base[sl] + tb_all[(int64_t)sl * om.tcap + tk] + 4 * lane);
         }
-        __syncthreads();  // the stage is reused by the next segment
+        __syncthreads();  // the stage and the segments are reused by the next batch
     }
 }
 
@@ -1028,8 +1137,7 @@ __global__ void __launch_bounds__(128) k_als_retry(AlsQueue<RP> q, Omega om, boo
             for (int c = 0; c < 32; ++c)
                 row[c] = c <= lane ? gs[w][lane * (lane + 1) / 2 + c] : gs[w][c * (c + 1) / 2 + lane];
             double xd = 0.0;
-            factor_solve_rows<32, double, false>(row, gs[w][NA + lane], true, len, r, lam_rel, lane, &xd, false,
-                                                 nullptr);
+            factor_solve_rows<32, double>(row, gs[w][NA + lane], len, r, lam_rel, lane, &xd);
             if (lane < r) Fout[q.dst[t] + lane] = (float)xd;
             if (lane == 0) atomicAdd(n_fp64, 1);
         } else if (lane == 0) {
@@ -1137,8 +1245,8 @@ lt_status omega_build(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, int
     char* p = (char*)lt_scratch(ctx, SCR_OMEGA,
                                 (size_t)(f->m + S) * 4 + (size_t)S * (C + 1) * 4 + e_csr * 16 + e_sell * 12 + S * 8 +
                                     (size_t)S * (om.bm_stride + om.bt_stride) * 8 + (S + 1) * 8 + (size_t)f->m * 8 +
-                                    (size_t)S * C * 8 + (size_t)S * 128 + t_sell * 8 + (size_t)(S + 1) * 16 +
-                                    (size_t)S * kOmParts * 4 + 34 * 256,
+                                    (size_t)S * C * 8 + (size_t)S * 128 + (size_t)(S + 1) * 8 + t_sell * 8 + (size_t)(S + 1) * 16 +
+                                    (size_t)S * kOmParts * 4 + 36 * 256,
                                 &st);
     if (!p) return st;
     auto take = [&](size_t nbytes) {
@@ -1169,6 +1277,8 @@ lt_status omega_build(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, int
     om.ctb = (int32_t*)take(t_sell * 4);
     om.rbase = (int64_t*)take((size_t)(S + 1) * 8);
     om.cbase = (int64_t*)take((size_t)(S + 1) * 8);
+    om.rtp = (int32_t*)take((size_t)(S + 1) * 4);
+    om.ctp = (int32_t*)take((size_t)(S + 1) * 4);
     om.sidx_r = (uint16_t*)take(e_sell * 2);
     om.sval_r = (float*)take(e_sell * 4);
     om.sidx_c = (uint16_t*)take(e_sell * 2);
@@ -1267,12 +1377,13 @@ lt_status complete_impl(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, i
     // float64 count
     const bool high = R > 16;
     const int nq = std::max(1, 2 * iters);
-    char* sp = (char*)lt_scratch(ctx, SCR_ALS, (size_t)(2 * nq + 64) * 4 + 256, &st);
+    char* sp = (char*)lt_scratch(ctx, SCR_ALS, (size_t)(3 * nq + 64) * 4 + 256, &st);
     if (!sp) return st;
     int32_t* n64 = (int32_t*)sp;
     int32_t* qcount = n64 + 64;
     int32_t* qcount_hi = qcount + nq;
-    LT_CUDA(ctx, cudaMemsetAsync(n64, 0, (size_t)(2 * nq + 64) * 4, ctx->stream));
+    int32_t* next_hi = qcount + 2 * nq;  // line counters of the warp-per-line kernel
+    LT_CUDA(ctx, cudaMemsetAsync(n64, 0, (size_t)(3 * nq + 64) * 4, ctx->stream));
     const int nsm = ctx->num_sms;
     k_als_init<<<dim3(8, S), 256, 0, ctx->stream>>>(*f, *smp, om, R, rk, seed_ref(ctx, seed), uv->V);
     LT_LAUNCH_CHECK(ctx, "k_als_init");
@@ -1283,10 +1394,12 @@ lt_status complete_impl(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, i
         k_als_warm<<<S, 256, shm, ctx->stream>>>(*f, *smp, R, rk, *warm, uv->V);
         LT_LAUNCH_CHECK(ctx, "k_als_warm");
     }
-    // lane-group kernel: one thread (group) per line; one 256-thread CTA per SM stages
-    // the slice's factor rows (up to 110 KB) and leaves the rest of the SM to L1
+    // lane-group kernel: one thread (group) per line; one 256-thread CTA per SM (its
+    // registers fill the SM) stages the factor rows of its slices, each with a row of
+    // zeros, up to 208 KB (3328 rows at rank 16)
     const size_t row_bytes = (size_t)RP * 4;
-    const int stage_rows = (int)std::min<int64_t>((110 * 1024) / row_bytes, std::max<int64_t>(mr, C));
+    const int per_sm = RP == 8 ? 2 : 1;  // rank 8 needs half the registers: two CTAs of 104 KB
+    const int stage_rows = (int)((208 * 1024 / per_sm) / row_bytes);
     const size_t dyn = (size_t)stage_rows * row_bytes;
     const int64_t cap = std::min<int64_t>(std::max<int64_t>(f->m, (int64_t)S * C), 1 << 18);
     int64_t *qdst = nullptr, *qslot = nullptr, *qsrc = nullptr;
@@ -1314,9 +1427,7 @@ lt_status complete_impl(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, i
         else
             LT_CUDA(ctx, cudaFuncSetAttribute(k_als_line<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
     }
-    // warp-per-line kernel for ranks above 16: each slice's lines split over P CTAs
-    // (about 16 CTAs per SM in all, so that uneven slices balance)
-    const int P = std::max(1, (16 * ctx->num_sms + S - 1) / S);
+    if (high) LT_CUDA(ctx, cudaFuncSetAttribute(k_als_half, cudaFuncAttributeMaxDynamicSharedMemorySize, kHalfSmem));
     TcPlan tcp{};
     if (tc) {
         st = als_tc_plan(ctx, f, smp, om, E, R, rk, RP, 2 * iters, &tcp);
@@ -1342,7 +1453,7 @@ lt_status complete_impl(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, i
                 LT_LAUNCH_CHECK(ctx, "k_als_retry");
             } else if (om.sell && RP == 8) {
                 AlsQueue<8> q{cnt, qdst, qslot, qsrc, qlen, qgrp, qrank, cap, ctx->d_status};
-                k_als_line<8><<<nsm, 256, dyn, ctx->stream>>>(*f, *smp, om, R, rk, rows, fin, fout, lam_rel, q,
+                k_als_line<8><<<per_sm * nsm, 256, dyn, ctx->stream>>>(*f, *smp, om, R, rk, rows, fin, fout, lam_rel, q,
                                                               stage_rows);
                 LT_LAUNCH_CHECK(ctx, "k_als_line");
                 k_als_retry<8><<<nsm, 128, 0, ctx->stream>>>(q, om, rows, fin, R, lam_rel, fout, n64);
@@ -1358,8 +1469,8 @@ lt_status complete_impl(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, i
             if (high) {
                 AlsQueue<32> q = qhi;
                 q.count = qcount_hi + 2 * it + side;
-                k_als_half<32><<<dim3(P, S), 32 * als_warps<32>(), 0, ctx->stream>>>(
-                    *f, *smp, om, R, rk, lam_rel, rows, fin, fout, q);
+                k_als_half<<<2 * nsm, 32 * kHalfWarps, kHalfSmem, ctx->stream>>>(*f, *smp, om, R, rk, lam_rel, rows, fin, fout,
+                                                                            q, next_hi + 2 * it + side);
                 LT_LAUNCH_CHECK(ctx, "k_als_half");
                 k_als_retry<32><<<nsm, 128, 0, ctx->stream>>>(q, om, rows, fin, R, lam_rel, fout, n64);
                 LT_LAUNCH_CHECK(ctx, "k_als_retry");

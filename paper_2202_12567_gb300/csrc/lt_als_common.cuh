@@ -11,6 +11,26 @@ namespace {
 // min pivot >= kPivotRatio * max pivot (pivots are the squared diagonal of L)
 constexpr float kPivotRatio = 1e-6f;
 
+// Two float32 values in one 64-bit register: one packed fused multiply-add does two
+// of them (each rounded as fmaf rounds).
+typedef unsigned long long F32x2;
+
+__device__ __forceinline__ F32x2 pack2(float lo, float hi) {
+    F32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+
+__device__ __forceinline__ void unpack2(F32x2 v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+
+__device__ __forceinline__ F32x2 fma2(F32x2 a, F32x2 b, F32x2 c) {
+    F32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
 template <int RP>
 struct AlsQueue {
     int32_t* count;     // [1] lines queued by this half-step
@@ -52,11 +72,14 @@ __device__ __forceinline__ bool chol_solve(T (&a)[RP * (RP + 1) / 2], T (&b)[RP]
     }
     T dmin = T(3.0e38), dmax = T(0);
     bool ok = true;
+    // every loop runs to RP under a condition: bounds that depend on an outer index are not
+    // always unrolled, and the array then lives in local memory
 #pragma unroll
     for (int j = 0; j < RP; ++j) {
         T d = a[j * (j + 1) / 2 + j];
 #pragma unroll
-        for (int k = 0; k < j; ++k) d -= a[j * (j + 1) / 2 + k] * a[j * (j + 1) / 2 + k];
+        for (int k = 0; k < RP; ++k)
+            if (k < j) d -= a[j * (j + 1) / 2 + k] * a[j * (j + 1) / 2 + k];
         if (j < r) {
             ok &= d > T(0);
             dmin = d < dmin ? d : dmin;
@@ -66,10 +89,12 @@ __device__ __forceinline__ bool chol_solve(T (&a)[RP * (RP + 1) / 2], T (&b)[RP]
         const T inv = T(1) / ljj;
         a[j * (j + 1) / 2 + j] = ljj;
 #pragma unroll
-        for (int i = j + 1; i < RP; ++i) {
+        for (int i = 0; i < RP; ++i) {
+            if (i <= j) continue;
             T t = a[i * (i + 1) / 2 + j];
 #pragma unroll
-            for (int k = 0; k < j; ++k) t -= a[i * (i + 1) / 2 + k] * a[j * (j + 1) / 2 + k];
+            for (int k = 0; k < RP; ++k)
+                if (k < j) t -= a[i * (i + 1) / 2 + k] * a[j * (j + 1) / 2 + k];
             a[i * (i + 1) / 2 + j] = t * inv;
         }
     }
@@ -78,14 +103,16 @@ __device__ __forceinline__ bool chol_solve(T (&a)[RP * (RP + 1) / 2], T (&b)[RP]
     for (int i = 0; i < RP; ++i) {  // L y = b
         T t = b[i];
 #pragma unroll
-        for (int k = 0; k < i; ++k) t -= a[i * (i + 1) / 2 + k] * b[k];
+        for (int k = 0; k < RP; ++k)
+            if (k < i) t -= a[i * (i + 1) / 2 + k] * b[k];
         b[i] = t / a[i * (i + 1) / 2 + i];
     }
 #pragma unroll
     for (int i = RP - 1; i >= 0; --i) {  // L^T x = y
         T t = b[i];
 #pragma unroll
-        for (int k = i + 1; k < RP; ++k) t -= a[k * (k + 1) / 2 + i] * b[k];
+        for (int k = 0; k < RP; ++k)
+            if (k > i) t -= a[k * (k + 1) / 2 + i] * b[k];
         b[i] = t / a[i * (i + 1) / 2 + i];
     }
     return true;

@@ -46,6 +46,8 @@ struct Omega {
     int32_t* ctb;       // [S][tcap]
     int64_t* rbase;     // [S + 1]      region start of each slice, rows side ([S] = total)
     int64_t* cbase;     // [S + 1]
+    int32_t* rtp;       // [S + 1]      warp tasks of the slices before each, rows side
+    int32_t* ctp;       // [S + 1]
     uint16_t* sidx_r;   // [sell_cap]   column of each rows-side slot
     float* sval_r;
     uint16_t* sidx_c;   // [sell_cap]   row of each columns-side slot
