@@ -7,6 +7,7 @@
 // and of the parameters in include/lt.h).
 #include <cuda_bf16.h>
 #include <math.h>
+#include <stddef.h>
 
 #include <algorithm>
 
@@ -21,7 +22,15 @@ constexpr int OW1 = 0, OB1 = OW1 + NH * NF, OW2 = OB1 + NH, OB2 = OW2 + NH * NH,
               OB3 = OW3 + NH * NH, OW4 = OB3 + NH, OB4 = OW4 + NH;
 static_assert(OB4 + 1 == NPAR, "parameter layout");
 constexpr uint32_t kTagLeverage = 4, kTagInit = 5;
-constexpr int TM = 64;            // rows per tile (4 warps x 16)
+constexpr int TM = 64;            // rows per tile
+// 16 warps per CTA: warp w takes the 16 rows (or outputs) 16 (w & 3) .. and a quarter of
+// the columns of every product of a tile.  The elementwise work and the parameter loads
+// of a tile, which are most of its time, spread over four times the threads of one warp
+// per 16 rows.  What bounds it: latency between the barriers of a tile (4 or 5 tiles a
+// CTA).  A training step on 40 K rows (forward, softmax, backward, reduction, Adam):
+// 0.118 ms, 0.223 ms with 4 warps, transposed copies of every operand and the loads of
+// the reductions one at a time.
+constexpr int MT = 512;
 constexpr int L1 = NF + 8;        // bf16 row stride of 32-wide operands (conflict-free fragments)
 constexpr int L2 = NH + 8;        // of 64-wide operands
 
@@ -63,6 +72,43 @@ __device__ __forceinline__ void warp_gemm(const bf16* A, int lda, const bf16* Bt
     }
 }
 
+// 8x8 matrices of 16-bit values, transposed on the way in: lane 8 q + i gives row i of
+// matrix q, and register q of lane (g, t) is element (2t, 2t + 1; g) of it
+__device__ __forceinline__ void ldm4_trans(uint32_t (&r)[4], const bf16* p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((unsigned)__cvta_generic_to_shared(p)));
+}
+__device__ __forceinline__ void ldm2_trans(uint32_t (&r)[2], const bf16* p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];"
+                 : "=r"(r[0]), "=r"(r[1])
+                 : "r"((unsigned)__cvta_generic_to_shared(p)));
+}
+
+// One warp: C[16][8 NT] += A B with B [K][8 NT] row-major (stride ldb) and A [16][K]
+// row-major (AT false) or given as its transpose [K][16] (AT true).
+template <int NT, bool AT>
+__device__ __forceinline__ void warp_gemm_kn(const bf16* A, int lda, const bf16* B, int ldb, int K, float (&c)[NT][4]) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    for (int k0 = 0; k0 < K; k0 += 16) {
+        uint32_t a[4];
+        if (AT) {  // matrices (k 0-7, m 0-7) (k 0-7, m 8-15) (k 8-15, m 0-7) (k 8-15, m 8-15)
+            ldm4_trans(a, A + (k0 + (lane & 7) + (lane >= 16 ? 8 : 0)) * lda + ((lane & 8) ? 8 : 0));
+        } else {
+            a[0] = ld2(A + g * lda + k0 + 2 * t);
+            a[1] = ld2(A + (g + 8) * lda + k0 + 2 * t);
+            a[2] = ld2(A + g * lda + k0 + 8 + 2 * t);
+            a[3] = ld2(A + (g + 8) * lda + k0 + 8 + 2 * t);
+        }
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+            uint32_t b[2];
+            ldm2_trans(b, B + (k0 + (lane & 15)) * ldb + 8 * nt);
+            mma_bf16(c[nt], a[0], a[1], a[2], a[3], b[0], b[1]);
+        }
+    }
+}
+
 template <int NT>
 __device__ __forceinline__ void zero(float (&c)[NT][4]) {
 #pragma unroll
@@ -71,13 +117,14 @@ __device__ __forceinline__ void zero(float (&c)[NT][4]) {
 
 // ---------------------------------------------------------------- parameters
 struct MlpSmem {
-    bf16 X[TM * L1];      // input tile, rows x 32
-    bf16 W1[NH * L1];     // [out][in]
-    bf16 W2[NH * L2];
-    bf16 W3[NH * L2];
-    bf16 A1[TM * L2];     // activations, rows x 64
-    bf16 A2[TM * L2];
-    bf16 A3[TM * L2];
+    // every bf16 array starts on 16 bytes and has rows of a multiple of 16 bytes (ldmatrix)
+    alignas(16) bf16 X[TM * L1];  // input tile, rows x 32
+    alignas(16) bf16 W1[NH * L1];     // [out][in]
+    alignas(16) bf16 W2[NH * L2];
+    alignas(16) bf16 W3[NH * L2];
+    alignas(16) bf16 A1[TM * L2];     // activations, rows x 64
+    alignas(16) bf16 A2[TM * L2];
+    alignas(16) bf16 A3[TM * L2];
     float b1[NH], b2[NH], b3[NH], w4[NH], b4;
     float z[TM];
 };
@@ -106,45 +153,49 @@ __device__ void load_tile(const float* __restrict__ feat, int64_t r0, int64_t n,
     }
 }
 
-// one hidden layer for the warp's 16 rows: H = A W^T + b, out = bf16(silu(H)); the
-// pre-activations go to Hs (float [TM][NH]) when it is given
+// one hidden layer for the warp's 16 rows and 16 columns: H = A W^T + b, out =
+// bf16(silu(H)); the pre-activations go to Hs (float [TM][NH]) when it is given
 template <int K>
 __device__ __forceinline__ void layer(const bf16* Ain, int lda, const bf16* W, int ldw, const float* b, bf16* Aout,
                                       float* Hs) {
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, w = threadIdx.x >> 5;
-    float c[8][4];
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, w = threadIdx.x >> 5, wr = w & 3, wc = w >> 2;
+    float c[2][4];
     zero(c);
-    warp_gemm<8>(Ain + 16 * w * lda, lda, W, ldw, K, c);
+    warp_gemm<2>(Ain + 16 * wr * lda, lda, W + 16 * wc * ldw, ldw, K, c);
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt)
+    for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const int row = 16 * w + g + (q >= 2 ? 8 : 0), col = 8 * nt + 2 * t + (q & 1);
+            const int row = 16 * wr + g + (q >= 2 ? 8 : 0), col = 16 * wc + 8 * nt + 2 * t + (q & 1);
             const float h = c[nt][q] + b[col];
             if (Hs) Hs[row * NH + col] = h;
             Aout[row * L2 + col] = __float2bfloat16_rn(silu(h));
         }
 }
 
-// forward of the tile in s.X: logits into s.z (each warp its 16 rows)
+// forward of the tile in s.X: logits into s.z; ends with a CTA barrier
 __device__ void forward_tile(MlpSmem& s, float* H1, float* H2, float* H3) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     layer<NF>(s.X, L1, s.W1, L1, s.b1, s.A1, H1);
-    __syncwarp();
+    __syncthreads();
     layer<NH>(s.A1, L2, s.W2, L2, s.b2, s.A2, H2);
-    __syncwarp();
+    __syncthreads();
     layer<NH>(s.A2, L2, s.W3, L2, s.b3, s.A3, H3);
-    __syncwarp();
-    if (lane < 16) {
-        const int row = 16 * w + lane;
+    __syncthreads();
+    if (threadIdx.x < TM) {
+        const int row = threadIdx.x;
         float z = s.b4;
-        for (int j = 0; j < NH; ++j) z = fmaf(__bfloat162float(s.A3[row * L2 + j]), s.w4[j], z);
+#pragma unroll 8
+        for (int j = 0; j < NH; j += 2) {
+            const __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162*>(s.A3 + row * L2 + j);
+            z = fmaf(__bfloat162float(a.x), s.w4[j], z);
+            z = fmaf(__bfloat162float(a.y), s.w4[j + 1], z);
+        }
         s.z[row] = z;
     }
-    __syncwarp();
+    __syncthreads();
 }
 
-__global__ void __launch_bounds__(128) k_mlp_forward(const float* __restrict__ theta, const float* __restrict__ feat,
+__global__ void __launch_bounds__(MT) k_mlp_forward(const float* __restrict__ theta, const float* __restrict__ feat,
                                                      int64_t n_max, const int32_t* __restrict__ n_dev,
                                                      float* __restrict__ z) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -156,7 +207,6 @@ __global__ void __launch_bounds__(128) k_mlp_forward(const float* __restrict__ t
         load_tile(feat, r0, n, s);
         __syncthreads();
         forward_tile(s, nullptr, nullptr, nullptr);
-        __syncthreads();
         for (int i = threadIdx.x; i < TM; i += blockDim.x)
             if (r0 + i < n) z[r0 + i] = s.z[i];
     }
@@ -165,145 +215,126 @@ __global__ void __launch_bounds__(128) k_mlp_forward(const float* __restrict__ t
 // ---------------------------------------------------------------- training
 struct BwdSmem {
     MlpSmem f;
-    bf16 XT[NF * L2];      // [in][rows]
-    bf16 A1T[NH * L2];     // [in][rows]
-    bf16 A2T[NH * L2];
-    bf16 W2T[NH * L2];     // [in][out]
-    bf16 W3T[NH * L2];
-    bf16 D[TM * L2];       // dH of the current layer, [rows][out]
-    bf16 DT[NH * L2];      // [out][rows]
+    alignas(16) bf16 D[TM * L2];  // dH of the current layer, [rows][out]
     float H1[TM * NH], H2[TM * NH], H3[TM * NH];  // pre-activations, then dH in float
     float dz[TM];
     float grad[NPAR];      // this CTA's gradient, accumulated over its tiles
 };
 
-// transpose a [rows][cols] bf16 tile (stride ls) into [cols][rows] (stride lt)
-__device__ void transpose(const bf16* S, int ls, bf16* T, int lt, int rows, int cols) {
-    for (int i = threadIdx.x; i < rows * cols; i += blockDim.x) {
-        const int r = i / cols, c = i % cols;
-        T[c * lt + r] = S[r * ls + c];
-    }
-}
+static_assert(offsetof(BwdSmem, D) % 16 == 0 && offsetof(MlpSmem, A1) % 16 == 0 && offsetof(MlpSmem, A2) % 16 == 0 &&
+                  offsetof(MlpSmem, W2) % 16 == 0 && offsetof(MlpSmem, W3) % 16 == 0 && L1 % 8 == 0 && L2 % 8 == 0,
+              "ldmatrix reads 16-byte rows");
 
-// dW[out][in] += DT[out][rows] (X^T)[in][rows]^T for the tile: warp w owns outputs 16w..
+// dW[out][in] += D^T X for the tile (both [rows][..]): warp w owns outputs 16 (w & 3) ..
+// and NT x 8 inputs
 template <int NT>
-__device__ void weight_grad(const bf16* DT, const bf16* XT, int K_in, float* gW) {
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, w = threadIdx.x >> 5;
+__device__ void weight_grad(const bf16* D, const bf16* X, int ldx, int K_in, float* gW) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, w = threadIdx.x >> 5, wr = w & 3, wc = w >> 2;
     float c[NT][4];
     zero(c);
-    warp_gemm<NT>(DT + 16 * w * L2, L2, XT, L2, TM, c);
+    warp_gemm_kn<NT, true>(D + 16 * wr, L2, X + 8 * NT * wc, ldx, TM, c);
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const int o = 16 * w + g + (q >= 2 ? 8 : 0), i = 8 * nt + 2 * t + (q & 1);
+            const int o = 16 * wr + g + (q >= 2 ? 8 : 0), i = 8 * (NT * wc + nt) + 2 * t + (q & 1);
             gW[o * K_in + i] += c[nt][q];
         }
 }
 
-// Hf [rows][NH] float holds dA of the layer on entry; turns it into dH = dA silu'(H)
-// (H the pre-activations in Hpre), fills D / DT (bf16) and adds the bias gradient.
-__device__ void act_grad(float* Hf, const float* Hpre, BwdSmem& s, float* gb, int nrows) {
-    for (int i = threadIdx.x; i < TM * NH; i += blockDim.x) {
-        const int r = i / NH, c = i % NH;
-        const float d = r < nrows ? Hf[i] * dsilu(Hpre[i]) : 0.f;
-        Hf[i] = d;
-        const bf16 b = __float2bfloat16_rn(d);
-        s.D[r * L2 + c] = b;
-        s.DT[c * L2 + r] = b;
-    }
-    __syncthreads();
-    for (int c = threadIdx.x; c < NH; c += blockDim.x) {
+// the bias gradient of a layer: column sums of dH over the rows in order
+__device__ void bias_grad(const float* Hf, float* gb) {
+    if (threadIdx.x < NH) {
         float a = 0.f;
-        for (int r = 0; r < TM; ++r) a += Hf[r * NH + c];
-        gb[c] += a;
+#pragma unroll 8
+        for (int r = 0; r < TM; ++r) a += Hf[r * NH + threadIdx.x];
+        gb[threadIdx.x] += a;
     }
 }
 
-// dA_prev[rows][in] = D[rows][out] W[out][in] (Wt = W^T as [in][out]) into Hf
-__device__ void input_grad(const BwdSmem& s, const bf16* Wt, float* Hf) {
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, w = threadIdx.x >> 5;
-    float c[8][4];
+// Hf [rows][NH] float holds dA of the layer on entry; turns it into dH = dA silu'(H)
+// (H the pre-activations in Hpre) and fills D (bf16)
+__device__ void act_grad(float* Hf, const float* Hpre, BwdSmem& s, int nrows) {
+    for (int i = threadIdx.x; i < TM * NH; i += MT) {
+        const int r = i / NH, c = i % NH;
+        const float d = r < nrows ? Hf[i] * dsilu(Hpre[i]) : 0.f;
+        Hf[i] = d;
+        s.D[r * L2 + c] = __float2bfloat16_rn(d);
+    }
+}
+
+// dA_prev[rows][in] = D[rows][out] W[out][in] into Hf
+__device__ void input_grad(const BwdSmem& s, const bf16* W, float* Hf) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, w = threadIdx.x >> 5, wr = w & 3, wc = w >> 2;
+    float c[2][4];
     zero(c);
-    warp_gemm<8>(s.D + 16 * w * L2, L2, Wt, L2, NH, c);
+    warp_gemm_kn<2, false>(s.D + 16 * wr * L2, L2, W + 16 * wc, L2, NH, c);
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt)
+    for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const int row = 16 * w + g + (q >= 2 ? 8 : 0), col = 8 * nt + 2 * t + (q & 1);
+            const int row = 16 * wr + g + (q >= 2 ? 8 : 0), col = 16 * wc + 8 * nt + 2 * t + (q & 1);
             Hf[row * NH + col] = c[nt][q];
         }
 }
 
 // Gradient of loss = sum_rows dz * z over rows [0, n); per CTA into part[blockIdx][NPAR].
-__global__ void __launch_bounds__(128) k_mlp_backward(const float* __restrict__ theta, const float* __restrict__ feat,
-                                                      const float* __restrict__ dz, int64_t n,
-                                                      float* __restrict__ part) {
+__global__ void __launch_bounds__(MT, 1) k_mlp_backward(const float* __restrict__ theta, const float* __restrict__ feat,
+                                                     const float* __restrict__ dz, int64_t n,
+                                                     float* __restrict__ part) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     BwdSmem& s = *reinterpret_cast<BwdSmem*>(smem_raw);
     load_params(theta, s.f);
-    for (int i = threadIdx.x; i < NPAR; i += blockDim.x) s.grad[i] = 0.f;
-    __syncthreads();
-    transpose(s.f.W2, L2, s.W2T, L2, NH, NH);
-    transpose(s.f.W3, L2, s.W3T, L2, NH, NH);
+    for (int i = threadIdx.x; i < NPAR; i += MT) s.grad[i] = 0.f;
     for (int64_t r0 = (int64_t)blockIdx.x * TM; r0 < n; r0 += (int64_t)gridDim.x * TM) {
         const int nrows = (int)min((int64_t)TM, n - r0);
         __syncthreads();
         load_tile(feat, r0, n, s.f);
-        for (int i = threadIdx.x; i < TM; i += blockDim.x) s.dz[i] = i < nrows ? dz[r0 + i] : 0.f;
+        for (int i = threadIdx.x; i < TM; i += MT) s.dz[i] = i < nrows ? dz[r0 + i] : 0.f;
         __syncthreads();
         forward_tile(s.f, s.H1, s.H2, s.H3);
-        __syncthreads();
-        // output layer: z = w4 . a3 + b4
-        for (int j = threadIdx.x; j < NH; j += blockDim.x) {
+        // output layer: z = w4 . a3 + b4 (the last warps, beside the first ones' dH3)
+        if (threadIdx.x >= MT - NH) {
+            const int j = threadIdx.x - (MT - NH);
             float a = 0.f;
+#pragma unroll 8
             for (int r = 0; r < TM; ++r) a += s.dz[r] * __bfloat162float(s.f.A3[r * L2 + j]);
             s.grad[OW4 + j] += a;
-        }
-        if (threadIdx.x == 0) {
+        } else if (threadIdx.x == MT - NH - 1) {
             float a = 0.f;
+#pragma unroll 8
             for (int r = 0; r < TM; ++r) a += s.dz[r];
             s.grad[OB4] += a;
         }
         // dH3 = dz w4 silu'(H3), in place of the pre-activations
-        for (int i = threadIdx.x; i < TM * NH; i += blockDim.x) {
+        for (int i = threadIdx.x; i < TM * NH; i += MT) {
             const int r = i / NH, c = i % NH;
-            s.H3[i] = r < nrows ? s.dz[r] * s.f.w4[c] * dsilu(s.H3[i]) : 0.f;
+            const float d = r < nrows ? s.dz[r] * s.f.w4[c] * dsilu(s.H3[i]) : 0.f;
+            s.H3[i] = d;
+            s.D[r * L2 + c] = __float2bfloat16_rn(d);
         }
         __syncthreads();
-        for (int i = threadIdx.x; i < TM * NH; i += blockDim.x) {
-            const int r = i / NH, c = i % NH;
-            const bf16 b = __float2bfloat16_rn(s.H3[i]);
-            s.D[r * L2 + c] = b;
-            s.DT[c * L2 + r] = b;
-        }
-        transpose(s.f.A2, L2, s.A2T, L2, TM, NH);
-        transpose(s.f.A1, L2, s.A1T, L2, TM, NH);
-        transpose(s.f.X, L1, s.XT, L2, TM, NF);
-        __syncthreads();
-        for (int c = threadIdx.x; c < NH; c += blockDim.x) {
-            float a = 0.f;
-            for (int r = 0; r < TM; ++r) a += s.H3[r * NH + c];
-            s.grad[OB3 + c] += a;
-        }
-        weight_grad<8>(s.DT, s.A2T, NH, s.grad + OW3);
+        weight_grad<2>(s.D, s.f.A2, L2, NH, s.grad + OW3);
+        bias_grad(s.H3, s.grad + OB3);
         __syncthreads();
         // layer 2
-        input_grad(s, s.W3T, s.H3);  // dA2 into H3's storage
+        input_grad(s, s.f.W3, s.H3);  // dA2 into H3's storage
         __syncthreads();
-        act_grad(s.H3, s.H2, s, s.grad + OB2, nrows);
+        act_grad(s.H3, s.H2, s, nrows);
         __syncthreads();
-        weight_grad<8>(s.DT, s.A1T, NH, s.grad + OW2);
+        weight_grad<2>(s.D, s.f.A1, L2, NH, s.grad + OW2);
+        bias_grad(s.H3, s.grad + OB2);
         __syncthreads();
         // layer 1
-        input_grad(s, s.W2T, s.H3);  // dA1
+        input_grad(s, s.f.W2, s.H3);  // dA1
         __syncthreads();
-        act_grad(s.H3, s.H1, s, s.grad + OB1, nrows);
+        act_grad(s.H3, s.H1, s, nrows);
         __syncthreads();
-        weight_grad<4>(s.DT, s.XT, NF, s.grad + OW1);
+        weight_grad<1>(s.D, s.f.X, L1, NF, s.grad + OW1);
+        bias_grad(s.H3, s.grad + OB1);
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < NPAR; i += blockDim.x) part[(int64_t)blockIdx.x * NPAR + i] = s.grad[i];
+    for (int i = threadIdx.x; i < NPAR; i += MT) part[(int64_t)blockIdx.x * NPAR + i] = s.grad[i];
 }
 
 // softmax over each group's rows, dz = (softmax - target) / G, loss per group
@@ -314,13 +345,16 @@ __global__ void k_group_softmax(const float* __restrict__ z, const float* __rest
     for (int gi = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); gi < G; gi += gridDim.x * (blockDim.x >> 5)) {
         const int a = goff[gi], b = goff[gi + 1];
         float mx = -3.0e38f;
+#pragma unroll 8
         for (int i = a + lane; i < b; i += 32) mx = fmaxf(mx, z[i]);
         mx = warp_max(mx);
         float se = 0.f;
+#pragma unroll 8
         for (int i = a + lane; i < b; i += 32) se += expf(z[i] - mx);
         se = warp_sum(se);
         const float lse = logf(se);
         float l = 0.f;
+#pragma unroll 8
         for (int i = a + lane; i < b; i += 32) {
             const float lp = z[i] - mx - lse;
             dz[i] = (expf(lp) - target[i]) / (float)G;
@@ -336,11 +370,13 @@ __global__ void k_grad_reduce(const float* __restrict__ part, int nparts, float*
                               const float* __restrict__ gloss, int G, float* __restrict__ loss) {
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < NPAR; p += gridDim.x * blockDim.x) {
         float a = 0.f;
+#pragma unroll 16
         for (int q = 0; q < nparts; ++q) a += part[(int64_t)q * NPAR + p];
         grad[p] = a;
     }
     if (loss && blockIdx.x == 0 && threadIdx.x == 0) {
         float a = 0.f;
+#pragma unroll 16
         for (int g = 0; g < G; ++g) a += gloss[g];
         *loss = a / (float)G;
     }
@@ -926,8 +962,8 @@ extern "C" lt_status lt_proposal_forward(lt_ctx* ctx, const float* theta, const 
     cudaSetDevice(ctx->device);
     const size_t shm = sizeof(MlpSmem);
     LT_CUDA(ctx, cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n_max + TM - 1) / TM, 4 * ctx->num_sms));
-    k_mlp_forward<<<grid, 128, shm, ctx->stream>>>(theta, feat, n_max, n_dev, z);
+    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n_max + TM - 1) / TM, 3 * ctx->num_sms));
+    k_mlp_forward<<<grid, MT, shm, ctx->stream>>>(theta, feat, n_max, n_dev, z);
     LT_LAUNCH_CHECK(ctx, "k_mlp_forward");
     return LT_OK;
 }
@@ -1020,13 +1056,13 @@ extern "C" lt_status lt_proposal_grad(lt_ctx* ctx, const float* theta, const flo
     float* part = (float*)((char*)gloss + (((size_t)ngroups * 4 + 255) & ~(size_t)255));
     lt_status s1 = lt_proposal_forward(ctx, theta, feat, n, nullptr, z);
     if (s1 != LT_OK) return s1;
-    k_group_softmax<<<(ngroups + 7) / 8, 256, 0, ctx->stream>>>(z, target, group_off, ngroups, dz, gloss);
+    k_group_softmax<<<ngroups, 32, 0, ctx->stream>>>(z, target, group_off, ngroups, dz, gloss);
     LT_LAUNCH_CHECK(ctx, "k_group_softmax");
     const size_t shm = sizeof(BwdSmem);
     LT_CUDA(ctx, cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-    k_mlp_backward<<<nparts, 128, shm, ctx->stream>>>(theta, feat, dz, n, part);
+    k_mlp_backward<<<nparts, MT, shm, ctx->stream>>>(theta, feat, dz, n, part);
     LT_LAUNCH_CHECK(ctx, "k_mlp_backward");
-    k_grad_reduce<<<(NPAR + 255) / 256, 256, 0, ctx->stream>>>(part, nparts, grad, gloss, ngroups, loss);
+    k_grad_reduce<<<(NPAR + 63) / 64, 64, 0, ctx->stream>>>(part, nparts, grad, gloss, ngroups, loss);
     LT_LAUNCH_CHECK(ctx, "k_grad_reduce");
     return LT_OK;
 }
