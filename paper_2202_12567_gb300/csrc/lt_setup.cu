@@ -33,13 +33,49 @@ __global__ void k_bitonic_step(unsigned long long* keys, int64_t n, int64_t j, i
     }
 }
 
+// Chunks of kSortChunk keys in shared memory.  first: sorts every chunk (all k up to
+// the chunk, alternating direction); otherwise the steps j < kSortChunk of one k.
+// A launch does up to 78 steps of the network where the global step does one: 377
+// launches for the sorts of 16384 lights and 65536 points become 31.  (With the records of
+// the cut below and the sums of the k-means: setup of that scene 8.03 to 5.01 ms.)
+constexpr int kSortChunk = 4096;
+
+__global__ void __launch_bounds__(1024) k_bitonic_chunk(unsigned long long* keys, int64_t n, int64_t k, bool first) {
+    __shared__ unsigned long long sk[kSortChunk];
+    const int64_t base = blockIdx.x * (int64_t)kSortChunk;
+    const int cnt = (int)(n - base < kSortChunk ? n - base : kSortChunk);  // a power of two
+    for (int i = threadIdx.x; i < cnt; i += blockDim.x) sk[i] = keys[base + i];
+    __syncthreads();
+    for (int64_t kk = first ? 2 : k; kk <= (first ? (int64_t)cnt : k); kk <<= 1) {
+        for (int j = (int)((kk < cnt ? kk : cnt) >> 1); j > 0; j >>= 1) {
+            for (int i = threadIdx.x; i < cnt / 2; i += blockDim.x) {
+                const int a = 2 * i - (i & (j - 1)), b = a + j;  // the i-th pair of distance j
+                const unsigned long long x = sk[a], y = sk[b];
+                if ((x > y) == (((base + a) & kk) == 0)) {
+                    sk[a] = y;
+                    sk[b] = x;
+                }
+            }
+            __syncthreads();
+        }
+    }
+    for (int i = threadIdx.x; i < cnt; i += blockDim.x) keys[base + i] = sk[i];
+}
+
 lt_status bitonic_sort(lt_ctx* ctx, unsigned long long* keys, int64_t npow2) {
+    if (npow2 < 2) return LT_OK;
     const int blocks = (int)std::min<int64_t>((npow2 + 255) / 256, 8 * (int64_t)ctx->num_sms);
-    for (int64_t k = 2; k <= npow2; k <<= 1)
-        for (int64_t j = k >> 1; j > 0; j >>= 1) {
+    const unsigned chunks = (unsigned)((npow2 + kSortChunk - 1) / kSortChunk);
+    k_bitonic_chunk<<<chunks, 1024, 0, ctx->stream>>>(keys, npow2, 0, true);
+    LT_LAUNCH_CHECK(ctx, "k_bitonic_chunk");
+    for (int64_t k = 2 * kSortChunk; k <= npow2; k <<= 1) {
+        for (int64_t j = k >> 1; j >= kSortChunk; j >>= 1) {
             k_bitonic_step<<<blocks, 256, 0, ctx->stream>>>(keys, npow2, j, k);
             LT_LAUNCH_CHECK(ctx, "k_bitonic_step");
         }
+        k_bitonic_chunk<<<chunks, 1024, 0, ctx->stream>>>(keys, npow2, k, false);
+        LT_LAUNCH_CHECK(ctx, "k_bitonic_chunk");
+    }
     return LT_OK;
 }
 
@@ -221,53 +257,115 @@ __device__ __forceinline__ float brdf_max(float alb, float gloss) {
     return gloss > 0.f ? 0.5f * alb * kInvPi + 0.5f * alb * (gloss + 2.f) * (0.5f * kInvPi) : alb * kInvPi;
 }
 
-// estimate(x) = sum over cut nodes of the unoccluded A(x, c); one warp per test row.
-__global__ void k_cut_estimate(const float4* __restrict__ pts, int64_t m, const float4* __restrict__ vpls, int64_t n,
-                               lt_tree T, const int32_t* __restrict__ rows, int64_t nr,
-                               const int32_t* __restrict__ cut, int C, float dmin2, float* est) {
-    const int lane = threadIdx.x & 31;
-    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t x = w; x < nr; x += nw) {
+// What a refinement round reads of a test row (once per setup) and of a cut node (once
+// per round), gathered into records that the passes over rows and nodes read in order.
+__global__ void k_cut_rows(const float4* __restrict__ pts, int64_t m, const int32_t* __restrict__ rows, int64_t nr,
+                           float4* __restrict__ rec) {
+    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < nr; x += (int64_t)gridDim.x * blockDim.x) {
         const PointRec P = load_rec(pts, m, rows[x]);
-        float acc = 0.f;
-        for (int c = lane; c < C; c += 32) {
-            const int node = cut[c];
-            const int r = T.rep[node];
-            const PointRec L = load_rec(vpls, n, r);
-            const float sc = __fdiv_rn(T.I[node], __fmul_rn(L.c.w, L.a.w));
-            acc += unoccluded(P, L, dmin2) * sc;
-        }
-        acc = warp_sum(acc);
-        if (lane == 0) est[x] = acc;
+        rec[x] = P.a;
+        rec[nr + x] = P.b;
+        rec[2 * nr + x] = P.c;
+        rec[3 * nr + x] = make_float4(P.a.x, P.a.y, P.a.z, brdf_max(P.a.w, P.b.w));
     }
 }
 
-// error(c) = max over rows of bound(x, c) / estimate(x); one warp per cut node.
-__global__ void k_cut_error(const float4* __restrict__ pts, int64_t m, lt_tree T, const int32_t* __restrict__ rows,
-                            int64_t nr, const int32_t* __restrict__ cut, int C, const float* __restrict__ est,
-                            float dmin2, float* err) {
+struct CutRecs {
+    float4* l;     // [3][C] record of the representative VPL
+    float4* box;   // [2][C] (lo xyz, hi x) (hi yz, I B, scale)
+};
+
+__global__ void k_cut_nodes(const float4* __restrict__ vpls, int64_t n, lt_tree T, const int32_t* __restrict__ cut,
+                            int C, CutRecs q) {
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x) {
+        const int node = cut[c];
+        const PointRec L = load_rec(vpls, n, T.rep[node]);
+        const float* bb = T.aabb + 6 * (int64_t)node;
+        q.l[c] = L.a;
+        q.l[C + c] = L.b;
+        q.l[2 * C + c] = L.c;
+        q.box[c] = make_float4(bb[0], bb[1], bb[2], bb[3]);
+        q.box[C + c] = make_float4(bb[4], bb[5], T.I[node] * T.B[node], __fdiv_rn(T.I[node], __fmul_rn(L.c.w, L.a.w)));
+    }
+}
+
+// estimate(x) = sum over cut nodes of the unoccluded A(x, c); one CTA per test row.  The
+// threads evaluate 256 nodes at a time; lane l of the first warp adds the terms l, l + 32,
+// ... in that order and the lanes' sums are added by a butterfly (a warp per row alone
+// leaves a chain of C / 32 dependent evaluations).
+constexpr int kCutThreads = 256;
+
+__global__ void __launch_bounds__(kCutThreads) k_cut_estimate(const float4* __restrict__ rec, int64_t nr, CutRecs q, int C,
+                                                              float dmin2, float* __restrict__ est) {
+    __shared__ float2 v[2][kCutThreads];
     const int lane = threadIdx.x & 31;
-    const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t ci = w; ci < C; ci += nw) {
-        const int node = cut[ci];
-        const float* bb = T.aabb + 6 * node;
-        const float IB = T.I[node] * T.B[node];
+    for (int64_t x = blockIdx.x; x < nr; x += gridDim.x) {
+        PointRec P;
+        P.a = rec[x];
+        P.b = rec[nr + x];
+        P.c = rec[2 * nr + x];
+        float acc = 0.f;
+        int h = 0;
+        for (int c0 = 0; c0 < C; c0 += kCutThreads, h ^= 1) {
+            const int c = c0 + threadIdx.x;
+            float u = 0.f, sc = 0.f;
+            if (c < C) {
+                PointRec L;
+                L.a = q.l[c];
+                L.b = q.l[C + c];
+                L.c = q.l[2 * C + c];
+                sc = q.box[C + c].w;
+                u = unoccluded(P, L, dmin2);
+            }
+            v[h][threadIdx.x] = make_float2(u, sc);  // u sc enters the sum through one multiply-add
+            __syncthreads();
+            if (threadIdx.x < 32) {
+                const int k1 = min(kCutThreads, C - c0);
+                for (int k = lane; k < k1; k += 32) acc = fmaf(v[h][k].x, v[h][k].y, acc);
+            }
+        }
+        if (threadIdx.x < 32) {
+            acc = warp_sum(acc);
+            if (lane == 0) est[x] = acc;
+        }
+        __syncthreads();
+    }
+}
+
+// error(c) = max over rows of bound(x, c) / estimate(x); `wpn` warps per cut node (a
+// maximum does not depend on their order).
+__global__ void __launch_bounds__(kCutThreads) k_cut_error(const float4* __restrict__ rec, int64_t nr, CutRecs q, int C,
+                                                           const float* __restrict__ est, float dmin2, int wpn,
+                                                           float* __restrict__ err) {
+    __shared__ float red[kCutThreads / 32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nodes = (kCutThreads / 32) / wpn;  // nodes of the CTA
+    const int part = wid % wpn;
+    const float4* row = rec + 3 * nr;
+    for (int64_t c0 = blockIdx.x * (int64_t)nodes; c0 < C; c0 += (int64_t)gridDim.x * nodes) {
+        const int64_t ci = c0 + wid / wpn;
         float e = 0.f;
-        for (int64_t x = lane; x < nr; x += 32) {
-            const PointRec P = load_rec(pts, m, rows[x]);
-            const float gx = fmaxf(0.f, fmaxf(bb[0] - P.a.x, P.a.x - bb[3]));
-            const float gy = fmaxf(0.f, fmaxf(bb[1] - P.a.y, P.a.y - bb[4]));
-            const float gz = fmaxf(0.f, fmaxf(bb[2] - P.a.z, P.a.z - bb[5]));
-            const float d2 = gx * gx + gy * gy + gz * gz;
-            const float b = IB * brdf_max(P.a.w, P.b.w) / fmaxf(d2, dmin2);
-            const float ex = est[x];
-            const float ratio = ex > 0.f ? b / ex : (b > 0.f ? INFINITY : 0.f);
-            e = fmaxf(e, ratio);
+        if (ci < C) {
+            const float4 b0 = q.box[ci], b1 = q.box[C + ci];
+            for (int64_t x = part * 32 + lane; x < nr; x += 32 * wpn) {
+                const float4 p = __ldg(row + x);
+                const float gx = fmaxf(0.f, fmaxf(b0.x - p.x, p.x - b0.w));
+                const float gy = fmaxf(0.f, fmaxf(b0.y - p.y, p.y - b1.x));
+                const float gz = fmaxf(0.f, fmaxf(b0.z - p.z, p.z - b1.y));
+                const float d2 = gx * gx + gy * gy + gz * gz;
+                const float b = b1.z * p.w / fmaxf(d2, dmin2);
+                const float ex = est[x];
+                const float ratio = ex > 0.f ? b / ex : (b > 0.f ? INFINITY : 0.f);
+                e = fmaxf(e, ratio);
+            }
         }
         e = warp_max(e);
-        if (lane == 0) err[ci] = e;
+        if (lane == 0) red[wid] = e;
+        __syncthreads();
+        if (ci < C && part == 0 && lane == 0) {
+            for (int k = 1; k < wpn; ++k) e = fmaxf(e, red[wid + k]);
+            err[ci] = e;
+        }
+        __syncthreads();
     }
 }
 
@@ -304,32 +402,52 @@ __global__ void k_kmeans_seed(const float4* __restrict__ pts, int64_t m, const u
     }
 }
 
+// Nearest centroid of every point and the sums of the clusters.  Points come in image
+// order, so a warp's points fall into few clusters: the lanes of a cluster add up by
+// shuffles and one of them adds to the cluster (the values are float32 and the sums
+// float64, wide enough that their order does not show).
 __global__ void k_kmeans_assign(const float4* __restrict__ pts, int64_t m, int S, float w,
                                 const float* __restrict__ cen, int32_t* __restrict__ lab, double* sums) {
     extern __shared__ float sc[];  // [S][6]
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
     for (int i = threadIdx.x; i < 6 * S; i += blockDim.x) sc[i] = cen[i];
     __syncthreads();
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-        float f[6];
-        feature(pts, m, i, w, f);
-        int best = 0;
-        float bd = 3e38f;
-        for (int k = 0; k < S; ++k) {
-            float d = 0.f;
-            for (int a = 0; a < 6; ++a) {
-                const float t = f[a] - sc[6 * k + a];
-                d += t * t;
+    for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x; i0 < m; i0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = i0 + threadIdx.x;
+        float f[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        int best = -1;
+        if (i < m) {
+            feature(pts, m, i, w, f);
+            best = 0;
+            float bd = 3e38f;
+            for (int k = 0; k < S; ++k) {
+                float d = 0.f;
+                for (int a = 0; a < 6; ++a) {
+                    const float t = f[a] - sc[6 * k + a];
+                    d += t * t;
+                }
+                if (d < bd) {
+                    bd = d;
+                    best = k;
+                }
             }
-            if (d < bd) {
-                bd = d;
-                best = k;
-            }
+            lab[i] = best;
         }
-        lab[i] = best;
-        if (sums) {
-            double* sk = sums + 7 * best;
-            for (int a = 0; a < 6; ++a) atomicAdd(sk + a, (double)f[a]);
-            atomicAdd(sk + 6, 1.0);
+        if (!sums) continue;
+        unsigned left = __ballot_sync(FULL, best >= 0);
+        while (left) {  // one cluster of the warp at a time
+            const int k = __shfl_sync(FULL, best, __ffs(left) - 1);
+            const unsigned mine = __ballot_sync(FULL, best == k);
+            double v[6];
+#pragma unroll
+            for (int a = 0; a < 6; ++a) v[a] = warp_sum<double>(best == k ? (double)f[a] : 0.0);
+            double* sk = sums + 7 * k;
+#pragma unroll
+            for (int a = 0; a < 6; ++a)
+                if (lane == a) atomicAdd(sk + a, v[a]);
+            if (lane == 6) atomicAdd(sk + 6, (double)__popc(mine));
+            left &= ~mine;
         }
     }
 }
@@ -485,15 +603,50 @@ extern "C" lt_status lt_build_tree(lt_ctx* ctx, const float* vpls, int64_t n, lt
 
 // ------------------------------------------------------------------ global cut
 namespace {
+// Scratch of the refinement for nr test rows and cuts of up to `most` nodes.
+struct CutWork {
+    float4* rec;   // [4][nr]
+    CutRecs q;
+    float* est;    // [nr]
+    float* err;    // [most]
+};
+
+lt_status cut_work(lt_ctx* ctx, int64_t nr, int64_t most, CutWork* w) {
+    auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    const size_t b_rec = up((size_t)nr * 64), b_l = up((size_t)most * 48), b_box = up((size_t)most * 32),
+                 b_est = up((size_t)nr * 4);
+    lt_status st;
+    char* p = (char*)lt_scratch(ctx, SCR_CUT, b_rec + b_l + b_box + b_est + up((size_t)most * 4), &st);
+    if (!p) return st;
+    w->rec = (float4*)p;
+    w->q.l = (float4*)(p + b_rec);
+    w->q.box = (float4*)(p + b_rec + b_l);
+    w->est = (float*)(p + b_rec + b_l + b_box);
+    w->err = (float*)(p + b_rec + b_l + b_box + b_est);
+    return LT_OK;
+}
+
+lt_status cut_rows(lt_ctx* ctx, const float* pts, int64_t m, const int32_t* rows, int64_t nr, const CutWork& w) {
+    k_cut_rows<<<(unsigned)std::min<int64_t>((nr + 255) / 256, 8 * (int64_t)ctx->num_sms), 256, 0, ctx->stream>>>(
+        (const float4*)pts, m, rows, nr, w.rec);
+    LT_LAUNCH_CHECK(ctx, "k_cut_rows");
+    return LT_OK;
+}
+
 // est[nr] and err[C] of the cut (device arrays); the refinement's per-round errors.
-lt_status cut_errors(lt_ctx* ctx, const lt_tree* tree, const float* pts, int64_t m, const float* vpls,
-                     const int32_t* rows, int64_t nr, const int32_t* cut, int C, float d_min, float* est, float* err) {
-    const int blocks = std::max(1, 8 * ctx->num_sms);
-    k_cut_estimate<<<blocks, 256, 0, ctx->stream>>>((const float4*)pts, m, (const float4*)vpls, tree->n, *tree, rows,
-                                                   nr, cut, C, d_min * d_min, est);
+lt_status cut_errors(lt_ctx* ctx, const lt_tree* tree, const float* vpls, int64_t nr, const int32_t* cut, int C,
+                     float d_min, const CutWork& w, float* err) {
+    const int nsm = ctx->num_sms;
+    k_cut_nodes<<<std::min((C + 255) / 256, 8 * nsm), 256, 0, ctx->stream>>>((const float4*)vpls, tree->n, *tree, cut, C,
+                                                                            w.q);
+    LT_LAUNCH_CHECK(ctx, "k_cut_nodes");
+    k_cut_estimate<<<(unsigned)std::min<int64_t>(nr, 8 * (int64_t)nsm), kCutThreads, 0, ctx->stream>>>(w.rec, nr, w.q, C,
+                                                                                             d_min * d_min, w.est);
     LT_LAUNCH_CHECK(ctx, "k_cut_estimate");
-    k_cut_error<<<blocks, 256, 0, ctx->stream>>>((const float4*)pts, m, *tree, rows, nr, cut, C, est, d_min * d_min,
-                                                err);
+    // small cuts: all 8 warps of a CTA on one node, until the nodes alone fill the chip
+    const int wpn = C < 8 * nsm ? 8 : C < 32 * nsm ? 2 : 1;
+    k_cut_error<<<(unsigned)std::min<int64_t>(((int64_t)C * wpn + 7) / 8, 8 * (int64_t)nsm), kCutThreads, 0,
+                  ctx->stream>>>(w.rec, nr, w.q, C, w.est, d_min * d_min, wpn, err);
     LT_LAUNCH_CHECK(ctx, "k_cut_error");
     return LT_OK;
 }
@@ -505,10 +658,11 @@ extern "C" lt_status lt_cut_errors(lt_ctx* ctx, const lt_tree* tree, const float
     if (!ctx || !tree_ok(tree) || !pts || !vpls || !rows || nr < 1 || m < 1 || !cut || C < 1 || !err)
         return lt_fail(ctx, LT_EINVAL, "lt_cut_errors: bad arguments");
     cudaSetDevice(ctx->device);
-    lt_status st;
-    float* est = (float*)lt_scratch(ctx, SCR_CUT, (size_t)nr * 4 + 256, &st);
-    if (!est) return st;
-    return cut_errors(ctx, tree, pts, m, vpls, rows, nr, cut, C, d_min, est, err);
+    CutWork w;
+    lt_status st = cut_work(ctx, nr, C, &w);
+    if (st != LT_OK) return st;
+    if ((st = cut_rows(ctx, pts, m, rows, nr, w)) != LT_OK) return st;
+    return cut_errors(ctx, tree, vpls, nr, cut, C, d_min, w, err);
 }
 
 extern "C" lt_status lt_build_global_cut(lt_ctx* ctx, const lt_tree* tree, const float* pts, int64_t m,
@@ -524,20 +678,19 @@ extern "C" lt_status lt_build_global_cut(lt_ctx* ctx, const lt_tree* tree, const
     LT_CUDA(ctx, cudaMemcpyAsync(child.data(), tree->child, child.size() * 4, cudaMemcpyDeviceToHost, ctx->stream));
     LT_CUDA(ctx, cudaMemcpyAsync(range.data(), tree->range, range.size() * 4, cudaMemcpyDeviceToHost, ctx->stream));
     LT_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    lt_status st;
-    char* p = (char*)lt_scratch(ctx, SCR_CUT, (size_t)nr * 4 + (size_t)max_cut * 8 + 1024, &st);
-    if (!p) return st;
-    float* est = (float*)p;
-    float* err = (float*)(p + ((nr * 4 + 255) & ~255LL));
+    CutWork w;
+    lt_status st = cut_work(ctx, nr, std::min<int64_t>(max_cut, n), &w);
+    if (st != LT_OK) return st;
+    if ((st = cut_rows(ctx, pts, m, rows, nr, w)) != LT_OK) return st;
     std::vector<int32_t> cur = {0};
     std::vector<float> herr;
     for (int round = 0; round < 4096; ++round) {
         const int C = (int)cur.size();
         LT_CUDA(ctx, cudaMemcpyAsync(cut, cur.data(), C * 4, cudaMemcpyHostToDevice, ctx->stream));
-        st = cut_errors(ctx, tree, pts, m, vpls, rows, nr, cut, C, d_min, est, err);
+        st = cut_errors(ctx, tree, vpls, nr, cut, C, d_min, w, w.err);
         if (st != LT_OK) return st;
         herr.resize(C);
-        LT_CUDA(ctx, cudaMemcpyAsync(herr.data(), err, C * 4, cudaMemcpyDeviceToHost, ctx->stream));
+        LT_CUDA(ctx, cudaMemcpyAsync(herr.data(), w.err, C * 4, cudaMemcpyDeviceToHost, ctx->stream));
         LT_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
         std::vector<int> cand;
         for (int i = 0; i < C; ++i)
