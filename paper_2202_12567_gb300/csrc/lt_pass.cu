@@ -135,50 +135,95 @@ struct P1Work {
     int64_t bcap;
 };
 
-// -- draws of the cut nodes and state of every forest node
-__global__ void k_p1_draws(lt_frame F, SeedRef sr, P1Plan pl, P1Store st, int32_t* status) {
+// -- draws of the cut nodes and state of every forest node.  A node's rows are the first
+// k distinct draws, ascending.  Up to kSerialDraws rows a thread draws for its node; for
+// more the warp does it, 32 draws at a time (a serial search and an insertion sort of
+// up to 64 rows cost 0.65 ms on the 512x512 scene with about 30 rows a node).
+constexpr int kSerialDraws = 4;
+
+__global__ void __launch_bounds__(256) k_p1_draws(lt_frame F, SeedRef sr, P1Plan pl, P1Store st, int32_t* status) {
+    __shared__ int32_t got_rows[8][kMaxRowsPerNode];
+    const unsigned FULL = 0xffffffffu;
     const int C = F.C, NF = 2 * C - 1;
     const uint64_t seed = sr.get();
-    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < (int64_t)F.S * NF;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int s = (int)(idx / NF), x = (int)(idx % NF);
+    const int lane = threadIdx.x & 31;
+    int32_t* mine = got_rows[threadIdx.x >> 5];
+    const int64_t total = (int64_t)F.S * NF;
+    for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x; i0 < total; i0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t idx = i0 + threadIdx.x;
+        const bool in = idx < total;
+        const int s = in ? (int)(idx / NF) : 0, x = in ? (int)(idx % NF) : 0;
         const int ms = F.slice_off[s + 1] - F.slice_off[s];
-        int32_t* cnt = pl.cnt + (int64_t)s * NF;
-        int32_t* state = pl.state + (int64_t)s * NF;
-        float* cost = pl.cost + (int64_t)s * NF;
-        cost[x] = 0.f;
-        if (x >= C) {
-            cnt[x] = 0;
-            state[x] = kStNot;
-            continue;
+        const int k = in && x < C ? pl.k[(int64_t)s * C + x] : 0;
+        int32_t* r = st.rows;
+        if (in) {
+            pl.cost[(int64_t)s * NF + x] = 0.f;
+            pl.state[(int64_t)s * NF + x] = x < C && ms > 0 ? kStAlive : kStNot;
+            if (x < C) r += pl.base[s] + pl.off[(int64_t)s * NF + x];
+            else pl.cnt[(int64_t)s * NF + x] = 0;
         }
-        const int k = pl.k[(int64_t)s * C + x];
-        int32_t* r = st.rows + pl.base[s] + pl.off[(int64_t)s * NF + x];
-        int got = 0;
-        if (k >= ms) {
-            for (int t = 0; t < ms; ++t) r[t] = t;
-            got = ms;
-        } else {
-            for (int t = 0; got < k && t < kMaxDraws; ++t) {
-                const int v = (int)uniform_index(philox((uint32_t)t, (uint32_t)x, slice_key(F.slice_id, s), kTagPass1, seed).x,
-                                                 (uint32_t)ms);
-                bool dup = false;
-                for (int q = 0; q < got; ++q) dup |= (r[q] == v);
-                if (!dup) r[got++] = v;
-            }
-            if (got < k) latch(status, LT_ELIMIT);
-            for (int a = 1; a < got; ++a) {  // insertion sort, got <= 64
-                const int v = r[a];
-                int b = a - 1;
-                while (b >= 0 && r[b] > v) {
-                    r[b + 1] = r[b];
-                    --b;
+        const bool node = in && x < C;
+        const bool wide = node && k < ms && k > kSerialDraws;
+        if (node && !wide) {
+            int got = 0;
+            if (k >= ms) {
+                for (int t = 0; t < ms; ++t) r[t] = t;
+                got = ms;
+            } else {
+                int v[kSerialDraws];  // ascending
+                for (int t = 0; got < k && t < kMaxDraws; ++t) {
+                    int u = (int)uniform_index(
+                        philox((uint32_t)t, (uint32_t)x, slice_key(F.slice_id, s), kTagPass1, seed).x, (uint32_t)ms);
+                    bool dup = false;
+#pragma unroll
+                    for (int q = 0; q < kSerialDraws; ++q) dup |= q < got && v[q] == u;
+                    if (dup) continue;
+                    ++got;
+#pragma unroll
+                    for (int q = 0; q < kSerialDraws; ++q) {
+                        if (q >= got) continue;
+                        if (q == got - 1 || u < v[q]) {  // insert u, carry what it displaces
+                            const int w = q == got - 1 ? u : v[q];
+                            v[q] = u;
+                            u = w;
+                        }
+                    }
                 }
-                r[b + 1] = v;
+                if (got < k) latch(status, LT_ELIMIT);
+#pragma unroll
+                for (int q = 0; q < kSerialDraws; ++q)
+                    if (q < got) r[q] = v[q];
             }
+            pl.cnt[(int64_t)s * NF + x] = got;
         }
-        cnt[x] = got;
-        state[x] = ms > 0 ? kStAlive : kStNot;
+        for (unsigned left = __ballot_sync(FULL, wide); left; left &= left - 1) {
+            const int src = __ffs(left) - 1;
+            const int ws = __shfl_sync(FULL, s, src), wx = __shfl_sync(FULL, x, src), wk = __shfl_sync(FULL, k, src);
+            const uint32_t wm = (uint32_t)__shfl_sync(FULL, ms, src);
+            int got = 0;
+            for (int t0 = 0; got < wk && t0 < kMaxDraws; t0 += 32) {
+                const int v = (int)uniform_index(
+                    philox((uint32_t)(t0 + lane), (uint32_t)wx, slice_key(F.slice_id, ws), kTagPass1, seed).x, wm);
+                bool fresh = __ffs(__match_any_sync(FULL, v)) - 1 == lane;  // the first of its value in the batch
+                for (int q = 0; q < got; ++q) fresh &= mine[q] != v;
+                const unsigned b = __ballot_sync(FULL, fresh);
+                const int pos = got + __popc(b & ((1u << lane) - 1u));
+                __syncwarp();  // every lane has read the list
+                if (fresh && pos < wk) mine[pos] = v;
+                got = min(wk, got + __popc(b));
+                __syncwarp();
+            }
+            if (got < wk && lane == 0) latch(status, LT_ELIMIT);
+            int32_t* wr = st.rows + pl.base[ws] + pl.off[(int64_t)ws * NF + wx];
+            for (int e = lane; e < got; e += 32) {  // a row's place is the number of smaller ones
+                const int v = mine[e];
+                int rank = 0;
+                for (int q = 0; q < got; ++q) rank += mine[q] < v;
+                wr[rank] = v;
+            }
+            if (lane == 0) pl.cnt[(int64_t)ws * NF + wx] = got;
+            __syncwarp();
+        }
     }
 }
 
