@@ -59,6 +59,8 @@ struct AdmArgs {
     const int32_t* ordr;  // [m]        rows of each slice ordered by class (k_adm_order)
     const int32_t* ordc;  // [S][C]     columns of each slice ordered by class
     const int32_t* ncls;  // [S][2][8]  lines per class, rows then columns
+    const int32_t* sord;  // [S]        slices by decreasing entry count
+    int parts;            // CTAs of a slice whose Gram parts are added (the cluster has 1 or 2 times as many)
     int R;
     const int32_t* rk;
     int iters;
@@ -97,10 +99,19 @@ __device__ __forceinline__ int adm_class(int len) {
 // index within a class (a stable counting sort, so the order is deterministic), and
 // the count of each class.  Block (s, side): side 0 the rows, 1 the columns.
 __global__ void k_adm_order(lt_frame F, lt_samples smp, Omega om, int32_t* __restrict__ ordr,
-                            int32_t* __restrict__ ordc, int32_t* __restrict__ ncls) {
+                            int32_t* __restrict__ ordc, int32_t* __restrict__ ncls, int32_t* __restrict__ sord) {
     __shared__ int32_t ws[32];
     __shared__ int32_t cnt[kAdmClasses], base[kAdmClasses];
     const int s = blockIdx.x, side = blockIdx.y;
+    if (side == 0) {  // the slice's place by entry count
+        const int mine = smp.cnt[s];
+        int before = 0;
+        for (int q = threadIdx.x; q < F.S; q += blockDim.x)
+            before += smp.cnt[q] > mine || (smp.cnt[q] == mine && q < s);
+        int32_t tot;
+        block_exclusive_scan<int32_t>(before, ws, &tot);
+        if (threadIdx.x == 0) sord[tot] = s;
+    }
     const int row0 = F.slice_off[s];
     const int n = side ? smp.ncol[s] : F.slice_off[s + 1] - row0;
     const int32_t* ptr = side ? om.cp + (int64_t)s * (F.C + 1) : om.rp + row0 + s;
@@ -218,12 +229,12 @@ __device__ void gj_inverse(const float* __restrict__ M, float add, float* __rest
     }
 }
 
-// sum over the cluster's CTAs, in rank order, of the partial matrices at `part`
-// (n floats each) into `out` (this CTA's shared memory)
-__device__ __forceinline__ void cluster_sum(cg::cluster_group& cl, int K, float* part, float* out, int n) {
+// sum over K of the cluster's CTAs (ranks r0, r0 + 1, ...), in rank order, of the partial
+// matrices at `part` (n floats each) into `out` (this CTA's shared memory)
+__device__ __forceinline__ void cluster_sum(cg::cluster_group& cl, int r0, int K, float* part, float* out, int n) {
     for (int e = threadIdx.x; e < n; e += blockDim.x) {
         float t = 0.f;
-        for (int q = 0; q < K; ++q) t += cl.map_shared_rank(part, q)[e];
+        for (int q = 0; q < K; ++q) t += cl.map_shared_rank(part, r0 + q)[e];
         out[e] = t;
     }
 }
@@ -238,30 +249,40 @@ __device__ __forceinline__ void tile_gram(const float* __restrict__ N, const flo
         if (e < RP * RP) {
             const int a = e / RP, b = e % RP;
             float t = g[q];
+#pragma unroll 8
             for (int i = 0; i < nt; ++i) t = fmaf(N[i * RP + a], (O ? O : N)[i * RP + b], t);
             g[q] = t;
         }
     }
 }
 
-// g1 += N^T N and, when O is given, g2 += N^T O over n factor rows of stride R (row
-// l at N + line(l) R), staged through `buf` (2 kAdmChunk RP floats of shared memory)
-// in chunks; every thread of the CTA calls it
+// g1 += N^T N (unless skip1) and, when O is given, g2 += N^T O over n factor rows of
+// stride R (row l at N + line(l) R), staged through `buf` (2 kAdmChunk RP floats of
+// shared memory) in chunks; every thread of the CTA calls it
 template <int RP, int NE, class Line>
 __device__ void gram_rows(const float* N, const float* O, int n, int R, Line line, float* __restrict__ buf,
-                          float (&g1)[NE], float (&g2)[NE]) {
+                          float (&g1)[NE], float (&g2)[NE], bool skip1 = false) {
     float* bn = buf;
     float* bo = buf + kAdmChunk * RP;
     for (int base = 0; base < n; base += kAdmChunk) {
         const int nt = min(kAdmChunk, n - base);
-        for (int e = threadIdx.x; e < nt * RP; e += kAdmThreads) {
-            const int i = e / RP, c = e % RP;
-            const int64_t at = (int64_t)line(base + i) * R + c;
-            bn[e] = c < R ? __ldcg(N + at) : 0.f;
-            if (O) bo[e] = c < R ? __ldcg(O + at) : 0.f;
+        if (R == RP && ((uintptr_t)N & 15) == 0 && ((uintptr_t)O & 15) == 0) {  // 16 bytes at a time
+            for (int e = threadIdx.x; e < nt * (RP / 4); e += kAdmThreads) {
+                const int i = e / (RP / 4), c = e % (RP / 4);
+                const int64_t at = (int64_t)line(base + i) * (RP / 4) + c;
+                reinterpret_cast<float4*>(bn)[e] = __ldcg(reinterpret_cast<const float4*>(N) + at);
+                if (O) reinterpret_cast<float4*>(bo)[e] = __ldcg(reinterpret_cast<const float4*>(O) + at);
+            }
+        } else {
+            for (int e = threadIdx.x; e < nt * RP; e += kAdmThreads) {
+                const int i = e / RP, c = e % RP;
+                const int64_t at = (int64_t)line(base + i) * R + c;
+                bn[e] = c < R ? __ldcg(N + at) : 0.f;
+                if (O) bo[e] = c < R ? __ldcg(O + at) : 0.f;
+            }
         }
         __syncthreads();
-        tile_gram<RP, NE>(bn, nullptr, nt, g1);
+        if (!skip1) tile_gram<RP, NE>(bn, nullptr, nt, g1);
         if (O) tile_gram<RP, NE>(bn, bo, nt, g2);
         __syncthreads();
     }
@@ -303,9 +324,16 @@ __device__ __forceinline__ void group_reduce(float (&acc)[RP], int G, unsigned g
 // stage n factor rows of stride R into shared memory, swizzled
 template <int RP>
 __device__ __forceinline__ void stage_rows(float* sm, const float* src, int n, int R) {
+    if (R == RP && ((uintptr_t)src & 15) == 0) {
+        for (int e = threadIdx.x; e < n * (RP / 4); e += kAdmThreads) {
+            const int j = e / (RP / 4), q = e % (RP / 4);
+            *reinterpret_cast<float4*>(sm + sy_chunk<RP>(j, q)) = __ldcg(reinterpret_cast<const float4*>(src) + e);
+        }
+        return;
+    }
     for (int e = threadIdx.x; e < n * RP; e += kAdmThreads) {
         const int j = e / RP, c = e % RP;
-        sm[sy_chunk<RP>(j, c >> 2) + (c & 3)] = c < R ? src[(int64_t)j * R + c] : 0.f;
+        sm[sy_chunk<RP>(j, c >> 2) + (c & 3)] = c < R ? __ldcg(src + (int64_t)j * R + c) : 0.f;
     }
 }
 
@@ -332,11 +360,12 @@ __device__ __forceinline__ void load_f(bool staged, const float* sm, const float
     }
 }
 
-constexpr int kAdmBatch = 8;  // entries whose indices a lane loads at once
+constexpr int kAdmBatch = 4;  // entries whose indices a lane loads at once, one batch ahead
 
 template <int RP>
 __global__ void __launch_bounds__(kAdmThreads, 2) k_adm(lt_frame F, lt_samples smp, Omega om, AdmArgs a, SeedRef sr) {
     constexpr int NE = (RP * RP + kAdmThreads - 1) / kAdmThreads;
+    constexpr int PU = RP <= 16 ? 2 : 1;  // entries whose dot products run side by side
     __shared__ __align__(16) float sInv[RP * RP];   // (A + alpha I)^-1, then (B + beta I)^-1
     __shared__ __align__(16) float sD[RP * RP];     // (B + beta I)^-1 C
     __shared__ __align__(16) float sM[2 * RP * RP]; // reduced A, or B and C
@@ -350,7 +379,12 @@ __global__ void __launch_bounds__(kAdmThreads, 2) k_adm(lt_frame F, lt_samples s
     cg::cluster_group cl = cg::this_cluster();
     const int K = (int)cl.dim_blocks().x;
     const int k = (int)cl.block_rank();
-    const int s = blockIdx.x / K;
+    // The Gram parts are those of K0 CTAs whatever the cluster's size (their sums are
+    // added in rank order): rank k adds up the lines of part k % K0, the first K0 ranks
+    // for X'^T X' and Y^T Y, the others for X'^T X.
+    const int K0 = a.parts, kg = k % K0, second = k / K0;
+    const bool split = K > K0;
+    const int s = a.sord[blockIdx.x / K];  // the longest slices start first
     const int tid = threadIdx.x;
     const int R = a.R;
     const int row0 = F.slice_off[s], ms = F.slice_off[s + 1] - row0;
@@ -358,8 +392,9 @@ __global__ void __launch_bounds__(kAdmThreads, 2) k_adm(lt_frame F, lt_samples s
     const int64_t o = smp.off[s];
     const int r = slice_rank(a.rk, s, R);
     const float mu = om.mu[s];
-    const int rlo = (int)((int64_t)k * ms / K), rhi = (int)((int64_t)(k + 1) * ms / K);
-    const int clo = (int)((int64_t)k * ns / K), chi = (int)((int64_t)(k + 1) * ns / K);
+    // lines of the start (the ranks past K0 have none)
+    const int rlo = second ? 0 : (int)((int64_t)k * ms / K0), rhi = second ? 0 : (int)((int64_t)(k + 1) * ms / K0);
+    const int clo = second ? 0 : (int)((int64_t)k * ns / K0), chi = second ? 0 : (int)((int64_t)(k + 1) * ns / K0);
     float* Yb = a.Y + (int64_t)s * F.C * R;
     float* Vb = a.Vp + (int64_t)s * F.C * R;
     float* Pb = a.Pi + (int64_t)s * F.C * R;
@@ -420,7 +455,7 @@ __global__ void __launch_bounds__(kAdmThreads, 2) k_adm(lt_frame F, lt_samples s
     if (tid == 0) sPartA[RP * RP] = ssx;
     __threadfence();
     cl.sync();
-    cluster_sum(cl, K, sPartA, sM, RP * RP + 1);
+    cluster_sum(cl, 0, K0, sPartA, sM, RP * RP + 1);
     __syncthreads();
     if (tid == 0) {
         float tr = 0.f;
@@ -435,9 +470,12 @@ __global__ void __launch_bounds__(kAdmThreads, 2) k_adm(lt_frame F, lt_samples s
     __syncthreads();
 
     __shared__ AdmSched shr, shc;  // the CTA's rows and columns
+    __shared__ AdmSched ghr, ghc;  // the lines of its Gram part
     if (tid == 0) {
         make_sched(a.ncls + (int64_t)s * 16, k, K, shr);
         make_sched(a.ncls + (int64_t)s * 16 + 8, k, K, shc);
+        make_sched(a.ncls + (int64_t)s * 16, kg, K0, ghr);
+        make_sched(a.ncls + (int64_t)s * 16 + 8, kg, K0, ghc);
     }
     __syncthreads();
     const int32_t* ordr = a.ordr + row0;
@@ -461,27 +499,50 @@ __global__ void __launch_bounds__(kAdmThreads, 2) k_adm(lt_frame F, lt_samples s
 #pragma unroll
             for (int c = 0; c < RP; ++c) acc[c] = 0.f;
             const int e1 = rp[i + 1];
-            for (int e0 = rp[i] + lane; e0 < e1; e0 += kAdmBatch * G) {
-                int jj[kAdmBatch], ss[kAdmBatch];
-                float mm[kAdmBatch];
+            // batches of kAdmBatch entries, the next batch's indices on their way; past the end
+            // an entry repeats the batch's first row with a zero residual
+            int e0 = rp[i] + lane;
+            int jj[kAdmBatch], ss[kAdmBatch];
+            float mm[kAdmBatch];
+            auto fetch = [&](int e, int (&j)[kAdmBatch], int (&sl)[kAdmBatch], float (&m)[kAdmBatch]) {
 #pragma unroll
                 for (int u = 0; u < kAdmBatch; ++u) {
-                    const int e = e0 + u * G;
-                    jj[u] = e < e1 ? cidx[e] : -1;
-                    mm[u] = e < e1 ? cval[e] : 0.f;
-                    ss[u] = e < e1 ? r2c[e] : 0;
+                    const int f = e + u * G;
+                    j[u] = f < e1 ? (int)cidx[f] : -1;
+                    m[u] = f < e1 ? cval[f] : 0.f;
+                    sl[u] = f < e1 ? r2c[f] : 0;
+                }
+            };
+            if (e0 < e1) fetch(e0, jj, ss, mm);
+            for (; e0 < e1; e0 += kAdmBatch * G) {
+                int jn[kAdmBatch], sn[kAdmBatch];
+                float mn[kAdmBatch];
+                fetch(e0 + kAdmBatch * G, jn, sn, mn);
+#pragma unroll
+                for (int u = 0; u < kAdmBatch; u += PU) {
+                    float y[PU][RP], d[PU];
+#pragma unroll
+                    for (int v = 0; v < PU; ++v) {
+                        load_f<RP>(staged, sY, Yb, jj[u + v] >= 0 ? jj[u + v] : jj[0], R, y[v]);
+                        d[v] = mm[u + v];
+                    }
+#pragma unroll
+                    for (int c = 0; c < RP; ++c)
+#pragma unroll
+                        for (int v = 0; v < PU; ++v) d[v] = fmaf(-xo[c], y[v][c], d[v]);
+#pragma unroll
+                    for (int v = 0; v < PU; ++v) {
+                        if (jj[u + v] >= 0) Sr[ss[u + v]] = d[v];
+                        else d[v] = 0.f;
+#pragma unroll
+                        for (int c = 0; c < RP; ++c) acc[c] = fmaf(d[v], y[v][c], acc[c]);
+                    }
                 }
 #pragma unroll
                 for (int u = 0; u < kAdmBatch; ++u) {
-                    if (jj[u] < 0) break;
-                    float y[RP];
-                    load_f<RP>(staged, sY, Yb, jj[u], R, y);
-                    float d = mm[u];
-#pragma unroll
-                    for (int c = 0; c < RP; ++c) d = fmaf(-xo[c], y[c], d);
-                    Sr[ss[u]] = d;
-#pragma unroll
-                    for (int c = 0; c < RP; ++c) acc[c] = fmaf(d, y[c], acc[c]);
+                    jj[u] = jn[u];
+                    ss[u] = sn[u];
+                    mm[u] = mn[u];
                 }
             }
             if (lane == 0) {  // alpha (U_k - X_k) - Lambda_k, once per row
@@ -504,18 +565,23 @@ __global__ void __launch_bounds__(kAdmThreads, 2) k_adm(lt_frame F, lt_samples s
             }
         }
         __syncthreads();  // the CTA's new rows are written; sY is free
+        if (split) {      // a Gram part has rows of two CTAs
+            __threadfence();
+            cl.sync();
+        }
         {
 #pragma unroll
             for (int q = 0; q < NE; ++q) gB[q] = gC[q] = 0.f;
-            auto line = [&](int l) { return row0 + ordr[sched_pos(shr, l, k, K)]; };
-            gram_rows<RP, NE>(Xn, Xc, shr.lines, R, line, sY, gB, gC);
+            auto line = [&](int l) { return row0 + ordr[sched_pos(ghr, l, kg, K0)]; };
+            gram_rows<RP, NE>(Xn, split && !second ? nullptr : Xc, ghr.lines, R, line, sY, gB, gC, second != 0);
             store_part<RP, NE>(sPartBC, gB);
             store_part<RP, NE>(sPartBC + RP * RP, gC);
         }
         __threadfence();
         cl.sync();
         // ---- (B + beta I)^-1 and D = (B + beta I)^-1 C ----------------------------
-        cluster_sum(cl, K, sPartBC, sM, 2 * RP * RP);
+        cluster_sum(cl, 0, K0, sPartBC, sM, RP * RP);
+        cluster_sum(cl, split ? K0 : 0, K0, sPartBC + RP * RP, sM + RP * RP, RP * RP);
         __syncthreads();
         if (tid < 32) gj_inverse<RP>(sM, beta, sInv, tid);
         __syncthreads();
@@ -545,22 +611,33 @@ __global__ void __launch_bounds__(kAdmThreads, 2) k_adm(lt_frame F, lt_samples s
             for (int c = 0; c < RP; ++c) acc[c] = 0.f;
             const int e1 = cp[j + 1];
             const float* Xs = Xn + (int64_t)row0 * R;
-            for (int e0 = cp[j] + lane; e0 < e1; e0 += kAdmBatch * G) {
-                int ii[kAdmBatch];
-                float sv[kAdmBatch];
+            int e0 = cp[j] + lane;
+            int ii[kAdmBatch];
+            float sv[kAdmBatch];
+            auto fetch = [&](int e, int (&i)[kAdmBatch], float (&v)[kAdmBatch]) {
 #pragma unroll
                 for (int u = 0; u < kAdmBatch; ++u) {
-                    const int e = e0 + u * G;
-                    ii[u] = e < e1 ? ridx[e] : -1;
-                    sv[u] = e < e1 ? Sr[e] : 0.f;
+                    const int f = e + u * G;
+                    i[u] = f < e1 ? (int)ridx[f] : -1;
+                    v[u] = f < e1 ? __ldcg(Sr + f) : 0.f;
+                }
+            };
+            if (e0 < e1) fetch(e0, ii, sv);
+            for (; e0 < e1; e0 += kAdmBatch * G) {
+                int in[kAdmBatch];
+                float vn[kAdmBatch];
+                fetch(e0 + kAdmBatch * G, in, vn);
+#pragma unroll
+                for (int u = 0; u < kAdmBatch; ++u) {
+                    float x[RP];
+                    load_f<RP>(staged_x, sY, Xs, ii[u] >= 0 ? ii[u] : ii[0], R, x);
+#pragma unroll
+                    for (int c = 0; c < RP; ++c) acc[c] = fmaf(sv[u], x[c], acc[c]);
                 }
 #pragma unroll
                 for (int u = 0; u < kAdmBatch; ++u) {
-                    if (ii[u] < 0) break;
-                    float x[RP];
-                    load_f<RP>(staged_x, sY, Xs, ii[u], R, x);
-#pragma unroll
-                    for (int c = 0; c < RP; ++c) acc[c] = fmaf(sv[u], x[c], acc[c]);
+                    ii[u] = in[u];
+                    sv[u] = vn[u];
                 }
             }
             if (lane == 0) {  // beta V_k - Pi_k, once per column
@@ -585,18 +662,22 @@ __global__ void __launch_bounds__(kAdmThreads, 2) k_adm(lt_frame F, lt_samples s
             }
         }
         __syncthreads();
-        {
+        if (split) {
+            __threadfence();
+            cl.sync();
+        }
+        if (!second) {
 #pragma unroll
             for (int q = 0; q < NE; ++q) gA[q] = 0.f;
-            auto line = [&](int l) { return ordc[sched_pos(shc, l, k, K)]; };
-            gram_rows<RP, NE>(Yb, nullptr, shc.lines, R, line, sY, gA, gA);
+            auto line = [&](int l) { return ordc[sched_pos(ghc, l, kg, K0)]; };
+            gram_rows<RP, NE>(Yb, nullptr, ghc.lines, R, line, sY, gA, gA);
             store_part<RP, NE>(sPartA, gA);
         }
         __threadfence();
         cl.sync();
         if (it + 1 < a.iters) {
             // ---- next (A + alpha I)^-1 and the staged Y ------------------------------
-            cluster_sum(cl, K, sPartA, sM, RP * RP);
+            cluster_sum(cl, 0, K0, sPartA, sM, RP * RP);
             __syncthreads();
             if (tid < 32) gj_inverse<RP>(sM, alpha, sInv, tid);
             if (staged) stage_rows<RP>(sY, Yb, ns, R);
@@ -613,13 +694,19 @@ __global__ void __launch_bounds__(kAdmThreads, 2) k_adm(lt_frame F, lt_samples s
 }
 
 template <int RP>
-lt_status launch_adm(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, const Omega& om, const AdmArgs& a,
-                     SeedRef sr) {
+lt_status launch_adm(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, const Omega& om, AdmArgs a, SeedRef sr) {
     const size_t dyn = (size_t)std::max(2 * kAdmChunk, a.stage_cap) * RP * 4;
     LT_CUDA(ctx, cudaFuncSetAttribute(k_adm<RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
-    // the largest cluster (8, 4 or 2 CTAs) with which all slices fit at two CTAs per SM
-    int K = kAdmMaxK;
-    while (K > 2 && (int64_t)f->S * K > 2 * (int64_t)ctx->num_sms) K >>= 1;
+    // Gram parts: 8, 4 or 2, as many as let all slices run at once at two CTAs per SM.
+    // The cluster is twice as large where it can be: slices are uneven (a factor of four in
+    // entries on the bench workload), every slice runs all iterations, and with all
+    // of them resident the chip waits for the longest.  100 iterations at rank 16 on 6 M
+    // entries: 33.9 ms with clusters of the parts' size in slice order, a batch of indices
+    // loaded when the one before is done and one dot product at a time; 24.3 ms so.
+    int K0 = kAdmMaxK;
+    while (K0 > 2 && (int64_t)f->S * K0 > 2 * (int64_t)ctx->num_sms) K0 >>= 1;
+    const int K = std::min(kAdmMaxK, 2 * K0);
+    a.parts = K0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(f->S * K));
     cfg.blockDim = dim3(kAdmThreads);
@@ -662,7 +749,7 @@ extern "C" lt_status lt_complete_adm(lt_ctx* ctx, const lt_frame* f, const lt_sa
     auto up = [](size_t n) { return (n * 4 + 255) & ~(size_t)255; };
     char* p = (char*)lt_scratch(ctx, SCR_ADM,
                                 3 * up(nx) + 2 * up(ny) + up((size_t)E) + up((size_t)f->m) + up((size_t)S * C) +
-                                    up((size_t)S * 16),
+                                    up((size_t)S * 16) + up((size_t)S),
                                 &st);
     if (!p) return st;
     AdmArgs a;
@@ -680,7 +767,9 @@ extern "C" lt_status lt_complete_adm(lt_ctx* ctx, const lt_frame* f, const lt_sa
     a.ordr = ordr;
     a.ordc = ordc;
     a.ncls = ncls;
-    k_adm_order<<<dim3(S, 2), 1024, 0, ctx->stream>>>(*f, *smp, om, ordr, ordc, ncls);
+    int32_t* sord = (int32_t*)((char*)ncls + up((size_t)S * 16));
+    a.sord = sord;
+    k_adm_order<<<dim3(S, 2), 1024, 0, ctx->stream>>>(*f, *smp, om, ordr, ordc, ncls, sord);
     LT_LAUNCH_CHECK(ctx, "k_adm_order");
     a.R = R;
     a.rk = uv->rank;
