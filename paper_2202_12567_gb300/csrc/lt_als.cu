@@ -42,31 +42,30 @@ __host__ __device__ inline int line_class(int len, int lane_entries) {
     return g;
 }
 
-// Omega build in five passes over the whole GPU (slice = blockIdx.y):
-//  1. clear the used words of both bitmaps;  2. set the bit of every entry and sum
-//  the values (one partial per block, fixed order);  3. one warp per row (column):
-//  popcount of each bitmap word, warp scan into the per-word prefix, line count;
-//  4. one block per slice: exclusive scan of the line counts into row / column
-//  pointers, mean value;  5. one thread per entry: slot = pointer + bits before.
+// Omega build in six passes over the whole GPU (slice = blockIdx.y):
+//  1. clear the used words of the row-major bitmap;  2. set the bit of every entry and
+//  sum the values (one partial per block, fixed order);  3. the column-major bitmap by
+//  32 x 32 bit transposes (a second scattered atomic per entry costs more);  4. one warp
+//  per row (column): popcount of each bitmap word, warp scan into the per-word prefix,
+//  line count;  5. one block per slice: exclusive scan of the line counts into row /
+//  column pointers, mean value;  6. one thread per entry: slot = pointer + bits before.
+// A word and its prefix sit side by side, so that an entry finds its index in a line
+// with one 8-byte load.
 __global__ void k_om_clear(lt_frame F, lt_samples smp, Omega om) {
     const int s = blockIdx.y;
     const int ms = F.slice_off[s + 1] - F.slice_off[s], ns = smp.ncol[s];
-    const int64_t nbm = (int64_t)ms * ((ns + 31) >> 5), nbt = (int64_t)ns * ((ms + 31) >> 5);
-    uint32_t* bm = om.bm + (int64_t)s * om.bm_stride;
-    uint32_t* bt = om.bt + (int64_t)s * om.bt_stride;
+    const int64_t nbm = (int64_t)ms * ((ns + 31) >> 5);
+    uint2* wr = om.wr + (int64_t)s * om.bm_stride;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nbm; i += (int64_t)gridDim.x * blockDim.x)
-        bm[i] = 0u;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nbt; i += (int64_t)gridDim.x * blockDim.x)
-        bt[i] = 0u;
+        wr[i] = make_uint2(0u, 0u);
 }
 
 __global__ void k_om_bits(lt_frame F, lt_samples smp, Omega om, float* __restrict__ part, int32_t* status) {
     __shared__ float red[32];
     const int s = blockIdx.y;
     const int ms = F.slice_off[s + 1] - F.slice_off[s], ns = smp.ncol[s], ne = smp.cnt[s];
-    const int W = (ns + 31) >> 5, WT = (ms + 31) >> 5;
-    uint32_t* bm = om.bm + (int64_t)s * om.bm_stride;
-    uint32_t* bt = om.bt + (int64_t)s * om.bt_stride;
+    const int W = (ns + 31) >> 5;
+    uint2* wr = om.wr + (int64_t)s * om.bm_stride;
     const uint32_t* key = smp.key + smp.off[s];
     const float* val = smp.val + smp.off[s];
     float sum = 0.f;
@@ -77,8 +76,7 @@ __global__ void k_om_bits(lt_frame F, lt_samples smp, Omega om, float* __restric
             latch(status, LT_EINVAL);
             continue;
         }
-        atomicOr(bm + (int64_t)r * W + (c >> 5), 1u << (c & 31));
-        atomicOr(bt + (int64_t)c * WT + (r >> 5), 1u << (r & 31));
+        atomicOr(&wr[(int64_t)r * W + (c >> 5)].y, 1u << (c & 31));
         sum += val[e];
     }
     sum = warp_sum(sum);
@@ -91,21 +89,49 @@ __global__ void k_om_bits(lt_frame F, lt_samples smp, Omega om, float* __restric
     }
 }
 
-// one warp per line: word prefixes of one bitmap row, the line's count into cnt_out
-__device__ __forceinline__ void om_line_words(const uint32_t* __restrict__ bits, uint32_t* __restrict__ pfx,
-                                              int nw, int32_t* cnt_out) {
+// one warp per 32 rows: lane i holds a word of row i; bit b of the 32 words is word b's
+// transpose, which lane b writes
+__global__ void k_om_transpose(lt_frame F, lt_samples smp, Omega om) {
+    const int s = blockIdx.y;
+    const int ms = F.slice_off[s + 1] - F.slice_off[s], ns = smp.ncol[s];
+    const int W = (ns + 31) >> 5, WT = (ms + 31) >> 5;
+    const uint2* wr = om.wr + (int64_t)s * om.bm_stride;
+    uint2* wc = om.wc + (int64_t)s * om.bt_stride;
+    const int lane = threadIdx.x & 31;
+    const int nwarps = gridDim.x * (blockDim.x >> 5);
+    for (int64_t t = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); t < (int64_t)W * WT; t += nwarps) {
+        const int rb = (int)(t / W), cw = (int)(t % W), r = 32 * rb + lane, c = 32 * cw + lane;
+        const uint32_t w = r < ms ? wr[(int64_t)r * W + cw].y : 0u;
+        uint32_t mine = 0u;
+#pragma unroll
+        for (int b = 0; b < 32; ++b) {
+            const uint32_t x = __ballot_sync(0xffffffffu, (w >> b) & 1u);
+            if (lane == b) mine = x;
+        }
+        if (c < ns) wc[(int64_t)c * WT + rb] = make_uint2(0u, mine);
+    }
+}
+
+// one warp per line: the word prefixes of one bitmap row, the line's count into cnt_out, and
+// the plain words into `bits` where they are wanted
+__device__ __forceinline__ void om_line_words(uint2* __restrict__ words, uint32_t* __restrict__ bits, int nw,
+                                              int32_t* cnt_out) {
     const int lane = threadIdx.x & 31;
     int carry = 0;
     for (int w0 = 0; w0 < nw; w0 += 32) {
         const int w = w0 + lane;
-        const int c = w < nw ? __popc(bits[w]) : 0;
+        const uint32_t b = w < nw ? words[w].y : 0u;
+        const int c = __popc(b);
         int incl = c;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int y = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += y;
         }
-        if (w < nw) pfx[w] = (uint32_t)(carry + incl - c);
+        if (w < nw) {
+            words[w].x = (uint32_t)(carry + incl - c);
+            if (bits) bits[w] = b;
+        }
         carry += __shfl_sync(0xffffffffu, incl, 31);
     }
     if (lane == 0) *cnt_out = carry;
@@ -120,11 +146,11 @@ __global__ void k_om_lines(lt_frame F, lt_samples smp, Omega om) {
     for (int l = gw; l < ms + ns; l += nwarps) {
         if (l < ms) {
             const int64_t o = (int64_t)s * om.bm_stride + (int64_t)l * W;
-            om_line_words(om.bm + o, om.wr + o, W, om.rp + row0 + s + l + 1);
+            om_line_words(om.wr + o, om.bm ? om.bm + o : nullptr, W, om.rp + row0 + s + l + 1);
         } else {
             const int c = l - ms;
             const int64_t o = (int64_t)s * om.bt_stride + (int64_t)c * WT;
-            om_line_words(om.bt + o, om.wc + o, WT, om.cp + (int64_t)s * (F.C + 1) + c + 1);
+            om_line_words(om.wc + o, om.bt ? om.bt + o : nullptr, WT, om.cp + (int64_t)s * (F.C + 1) + c + 1);
         }
     }
 }
@@ -328,10 +354,8 @@ __global__ void k_om_scatter(lt_frame F, lt_samples smp, Omega om) {
     const int s = blockIdx.y;
     const int row0 = F.slice_off[s], ms = F.slice_off[s + 1] - row0, ns = smp.ncol[s], ne = smp.cnt[s];
     const int W = (ns + 31) >> 5, WT = (ms + 31) >> 5;
-    const uint32_t* bm = om.bm + (int64_t)s * om.bm_stride;
-    const uint32_t* bt = om.bt + (int64_t)s * om.bt_stride;
-    const uint32_t* wr = om.wr + (int64_t)s * om.bm_stride;
-    const uint32_t* wc = om.wc + (int64_t)s * om.bt_stride;
+    const uint2* wr = om.wr + (int64_t)s * om.bm_stride;
+    const uint2* wc = om.wc + (int64_t)s * om.bt_stride;
     const int32_t* rp = om.rp + row0 + s;
     const int32_t* cp = om.cp + (int64_t)s * (F.C + 1);
     const int64_t o = smp.off[s];
@@ -342,8 +366,9 @@ __global__ void k_om_scatter(lt_frame F, lt_samples smp, Omega om) {
         const int r = (int)(k >> 16), c = (int)(k & 0xffffu);
         if (r >= ms || c >= ns) continue;
         const int64_t iw = (int64_t)r * W + (c >> 5), jw = (int64_t)c * WT + (r >> 5);
-        const int kr = (int)wr[iw] + __popc(bm[iw] & ((1u << (c & 31)) - 1u));  // index in its row
-        const int kc = (int)wc[jw] + __popc(bt[jw] & ((1u << (r & 31)) - 1u));  // index in its column
+        const uint2 a = __ldg(wr + iw), b = __ldg(wc + jw);
+        const int kr = (int)a.x + __popc(a.y & ((1u << (c & 31)) - 1u));  // index in its row
+        const int kc = (int)b.x + __popc(b.y & ((1u << (r & 31)) - 1u));  // index in its column
         const float v = val[e];
         if (om.csr) {
             om.cidx[o + rp[r] + kr] = (uint16_t)c;
@@ -1217,10 +1242,10 @@ __global__ void k_slice_ranks(lt_samples smp, int S, int R, int cols, int32_t* _
 
 namespace ltk {
 
-lt_status omega_build(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, int64_t E, bool sell, bool csr,
+lt_status omega_build(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, int64_t E, bool sell, bool csr, bool bits,
                       Omega* omp) {
     const int S = f->S, C = f->C;
-    constexpr int kOmParts = 8;
+    constexpr int kOmParts = 8;   // fixes the order of the mean value's sum
     const int64_t mr = std::max(f->max_rows, 1);
     Omega& om = *omp;
     om.bm_stride = mr * ((C + 31) / 32);
@@ -1244,7 +1269,7 @@ lt_status omega_build(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, int
     lt_status st;
     char* p = (char*)lt_scratch(ctx, SCR_OMEGA,
                                 (size_t)(f->m + S) * 4 + (size_t)S * (C + 1) * 4 + e_csr * 16 + e_sell * 12 + S * 8 +
-                                    (size_t)S * (om.bm_stride + om.bt_stride) * 8 + (S + 1) * 8 + (size_t)f->m * 8 +
+                                    (size_t)S * (om.bm_stride + om.bt_stride) * (bits ? 12 : 8) + (S + 1) * 8 + (size_t)f->m * 8 +
                                     (size_t)S * C * 8 + (size_t)S * 128 + (size_t)(S + 1) * 8 + t_sell * 8 + (size_t)(S + 1) * 16 +
                                     (size_t)S * kOmParts * 4 + 36 * 256,
                                 &st);
@@ -1262,10 +1287,10 @@ lt_status omega_build(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, int
     om.rval = (float*)take(e_csr * 4);
     om.r2c = (int32_t*)take(e_csr * 4);
     om.mu = (float*)take(S * 4);
-    om.bm = (uint32_t*)take((size_t)S * om.bm_stride * 4);
-    om.bt = (uint32_t*)take((size_t)S * om.bt_stride * 4);
-    om.wr = (uint32_t*)take((size_t)S * om.bm_stride * 4);
-    om.wc = (uint32_t*)take((size_t)S * om.bt_stride * 4);
+    om.bm = bits ? (uint32_t*)take((size_t)S * om.bm_stride * 4) : nullptr;
+    om.bt = bits ? (uint32_t*)take((size_t)S * om.bt_stride * 4) : nullptr;
+    om.wr = (uint2*)take((size_t)S * om.bm_stride * 8);
+    om.wc = (uint2*)take((size_t)S * om.bt_stride * 8);
     om.line_pfx = (int64_t*)take((S + 1) * 8);
     om.rord = (int32_t*)take((size_t)f->m * 4);
     om.cord = (int32_t*)take((size_t)S * C * 4);
@@ -1291,6 +1316,8 @@ lt_status omega_build(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, int
     LT_LAUNCH_CHECK(ctx, "k_om_clear");
     k_om_bits<<<dim3(kOmParts, S), 256, 0, ctx->stream>>>(*f, *smp, om, part, ctx->d_status);
     LT_LAUNCH_CHECK(ctx, "k_om_bits");
+    k_om_transpose<<<dim3(std::max(1, 8 * nsm / S), S), 256, 0, ctx->stream>>>(*f, *smp, om);
+    LT_LAUNCH_CHECK(ctx, "k_om_transpose");
     k_om_lines<<<dim3(std::max(1, 4 * nsm / S), S), 256, 0, ctx->stream>>>(*f, *smp, om);
     LT_LAUNCH_CHECK(ctx, "k_om_lines");
     k_om_scan<<<S, 1024, 0, ctx->stream>>>(*f, *smp, om, part, kOmParts);
@@ -1370,7 +1397,7 @@ lt_status complete_impl(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, i
     const bool low = R <= 16 || rk != nullptr;
     const bool tc = low && ctx->tune.als_form == 1;
     Omega om;
-    lt_status st = omega_build(ctx, f, smp, E, low && !tc, R > 16 || tc, &om);
+    lt_status st = omega_build(ctx, f, smp, E, low && !tc, R > 16 || tc, tc, &om);
     if (st != LT_OK) return st;
     const int RP = R <= 8 ? 8 : 16;  // the low-rank kernels cover ranks up to RP
     // per half-step retry counters (one set for ranks <= 16, one above) and the
@@ -1506,7 +1533,7 @@ extern "C" lt_status lt_als_gram(lt_ctx* ctx, const lt_frame* f, const lt_sample
     LT_CUDA(ctx, cudaMemcpyAsync(&E, smp->off + f->S, sizeof(int64_t), cudaMemcpyDeviceToHost, ctx->stream));
     LT_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     Omega om;
-    lt_status st = omega_build(ctx, f, smp, E, false, true, &om);
+    lt_status st = omega_build(ctx, f, smp, E, false, true, true, &om);
     if (st != LT_OK) return st;
     const int R = uv->r, RP = R <= 8 ? 8 : 16;
     TcPlan tcp{};

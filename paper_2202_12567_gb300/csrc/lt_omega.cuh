@@ -26,10 +26,10 @@ struct Omega {
     float* rval;        // [off[S]]
     int32_t* r2c;       // [off[S]]     CSC slot (within the slice) of each CSR entry
     float* mu;          // [S] mean observed value
-    uint32_t* bm;       // row-major bitmaps
+    uint32_t* bm;       // row-major bitmaps, where wanted (else null)
     uint32_t* bt;       // column-major bitmaps
-    uint32_t* wr;       // per word of bm: set bits before it in its row
-    uint32_t* wc;       // per word of bt: set bits before it in its column
+    uint2* wr;          // per word of the row-major bitmap: set bits before it in its row, the word
+    uint2* wc;          // the same of the column-major bitmap
     int64_t bm_stride, bt_stride;
     int64_t* line_pfx;  // [S + 1] prefix of n'_s (V-step lines)
     int32_t* rord;      // [m]          rows of each slice by decreasing entry count
@@ -62,8 +62,8 @@ struct Omega {
 // Builds Omega for the frame's samples (E = total entry count, known to the host):
 // bitmaps, per-word prefixes, line counts, row / column pointers, sorted line orders,
 // mean observed value per slice, and the sliced layout (sell) and / or CSR / CSC
-// (csr), in scratch slot SCR_OMEGA.
-lt_status omega_build(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, int64_t E, bool sell, bool csr,
+// (csr), and the plain bitmaps (bits), in scratch slot SCR_OMEGA.
+lt_status omega_build(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, int64_t E, bool sell, bool csr, bool bits,
                       Omega* om);
 
 }  // namespace ltk
