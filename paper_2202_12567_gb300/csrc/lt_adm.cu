@@ -743,7 +743,7 @@ extern "C" lt_status lt_complete_adm(lt_ctx* ctx, const lt_frame* f, const lt_sa
         ctx->plan.entries = E;
     }
     Omega om;
-    lt_status st = omega_build(ctx, f, smp, E, false, true, false, &om);
+    lt_status st = omega_build(ctx, f, smp, E, false, true, false, uv->rank, R, &om);
     if (st != LT_OK) return st;
     const size_t nx = (size_t)f->m * R, ny = (size_t)S * C * R;
     auto up = [](size_t n) { return (n * 4 + 255) & ~(size_t)255; };

@@ -60,15 +60,12 @@ __global__ void k_om_clear(lt_frame F, lt_samples smp, Omega om) {
         wr[i] = make_uint2(0u, 0u);
 }
 
-__global__ void k_om_bits(lt_frame F, lt_samples smp, Omega om, float* __restrict__ part, int32_t* status) {
-    __shared__ float red[32];
+__global__ void k_om_bits(lt_frame F, lt_samples smp, Omega om, int32_t* status) {
     const int s = blockIdx.y;
     const int ms = F.slice_off[s + 1] - F.slice_off[s], ns = smp.ncol[s], ne = smp.cnt[s];
     const int W = (ns + 31) >> 5;
     uint2* wr = om.wr + (int64_t)s * om.bm_stride;
     const uint32_t* key = smp.key + smp.off[s];
-    const float* val = smp.val + smp.off[s];
-    float sum = 0.f;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < ne; e += gridDim.x * blockDim.x) {
         const uint32_t k = key[e];
         const int r = (int)(k >> 16), c = (int)(k & 0xffffu);
@@ -77,23 +74,41 @@ __global__ void k_om_bits(lt_frame F, lt_samples smp, Omega om, float* __restric
             continue;
         }
         atomicOr(&wr[(int64_t)r * W + (c >> 5)].y, 1u << (c & 31));
-        sum += val[e];
+    }
+}
+
+// Part p of the sum of a slice's values: thread t of kOmParts blocks of 256 adds every
+// 256 kOmParts-th value, then the block adds its threads, in a fixed order.  (Entries out
+// of range are not in the layout nor in its sum.)
+constexpr int kOmParts = 8;
+
+__device__ __forceinline__ void om_sum(const lt_samples& smp, int s, int ms, int ns, int p, float* __restrict__ part) {
+    __shared__ float red[32];
+    const int ne = smp.cnt[s];
+    const uint32_t* key = smp.key + smp.off[s];
+    const float* val = smp.val + smp.off[s];
+    float sum = 0.f;
+#pragma unroll 8
+    for (int e = p * 256 + threadIdx.x; e < ne; e += kOmParts * 256) {
+        const uint32_t k = key[e];
+        if ((int)(k >> 16) < ms && (int)(k & 0xffffu) < ns) sum += val[e];
     }
     sum = warp_sum(sum);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
     __syncthreads();
     if (threadIdx.x == 0) {
         float t = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-        part[(int64_t)s * gridDim.x + blockIdx.x] = t;
+        for (int w = 0; w < 8; ++w) t += red[w];
+        part[(int64_t)s * kOmParts + p] = t;
     }
 }
 
 // one warp per 32 rows: lane i holds a word of row i; bit b of the 32 words is word b's
-// transpose, which lane b writes
-__global__ void k_om_transpose(lt_frame F, lt_samples smp, Omega om) {
+// transpose, which lane b writes.  The first kOmParts blocks of a slice also sum its values.
+__global__ void __launch_bounds__(256) k_om_transpose(lt_frame F, lt_samples smp, Omega om, float* __restrict__ part) {
     const int s = blockIdx.y;
     const int ms = F.slice_off[s + 1] - F.slice_off[s], ns = smp.ncol[s];
+    if (blockIdx.x < kOmParts) om_sum(smp, s, ms, ns, blockIdx.x, part);
     const int W = (ns + 31) >> 5, WT = (ms + 31) >> 5;
     const uint2* wr = om.wr + (int64_t)s * om.bm_stride;
     uint2* wc = om.wc + (int64_t)s * om.bt_stride;
@@ -283,16 +298,18 @@ __global__ void k_om_scan(lt_frame F, lt_samples smp, Omega om, const float* __r
     int32_t* cord = om.cord + (int64_t)s * F.C;
     int32_t* rcls = om.rcls + (int64_t)s * 16;
     int32_t* ccls = om.ccls + (int64_t)s * 16;
-    om_order(rc1, ms, rord, key);
-    om_classes(rc1, ms, rord, ms <= kOrdMax, om.lane_entries, rcls);
+    if (blockIdx.y == 0) {
+        om_order(rc1, ms, rord, key);
+        om_classes(rc1, ms, rord, ms <= kOrdMax, om.lane_entries, rcls);
+        if (om.sell)
+            om_tasks(rc1, ms, rord, rcls, om.rpos + row0, om.rtb + (int64_t)s * om.tcap, om.rbase + s + 1, ws);
+        om_scan_counts(om.rp + row0 + s, ms, ws);
+        return;
+    }
     om_order(cc1, ns, cord, key);
     om_classes(cc1, ns, cord, ns <= kOrdMax, om.lane_entries, ccls);
-    if (om.sell) {
-        om_tasks(rc1, ms, rord, rcls, om.rpos + row0, om.rtb + (int64_t)s * om.tcap, om.rbase + s + 1, ws);
-        om_tasks(cc1, ns, cord, ccls, om.cpos + (int64_t)s * F.C, om.ctb + (int64_t)s * om.tcap, om.cbase + s + 1,
-                 ws);
-    }
-    om_scan_counts(om.rp + row0 + s, ms, ws);
+    if (om.sell)
+        om_tasks(cc1, ns, cord, ccls, om.cpos + (int64_t)s * F.C, om.ctb + (int64_t)s * om.tcap, om.cbase + s + 1, ws);
     om_scan_counts(om.cp + (int64_t)s * (F.C + 1), ns, ws);
     if (threadIdx.x == 0) {
         float t = 0.f;
@@ -303,7 +320,11 @@ __global__ void k_om_scan(lt_frame F, lt_samples smp, Omega om, const float* __r
 
 // region starts of the sliced layouts: in place, x[1..S] sizes -> x[0..S] prefix;
 // a total beyond the capacity latches LT_ELIMIT (the scatter then skips slots past it)
-__global__ void k_om_sellpfx(int S, Omega om, int32_t* status) {
+// (with the work before each slice: slots and kTaskCost per warp task of the slices whose
+// rank the lane-group kernel has)
+constexpr int kTaskCost = 512;   // slots worth a task's reduction and Cholesky (32 lanes x 16 entries)
+
+__global__ void k_om_sellpfx(int S, Omega om, const int32_t* __restrict__ rk, int R, int32_t* status) {
     __shared__ int64_t ws[32];
     for (int side = 0; side < 2; ++side) {
         int64_t* x = side == 0 ? om.rbase : om.cbase;
@@ -322,19 +343,21 @@ __global__ void k_om_sellpfx(int S, Omega om, int32_t* status) {
             if (carry > om.sell_cap) latch(status, LT_ELIMIT);
         }
         __syncthreads();
-        // warp tasks before each slice
-        int32_t* tp = side == 0 ? om.rtp : om.ctp;
+        int64_t* wk = side == 0 ? om.rwk : om.cwk;
         const int32_t* cls = side == 0 ? om.rcls : om.ccls;
-        int64_t tasks = 0;
+        int64_t work = 0;
         for (int i0 = 0; i0 < S; i0 += blockDim.x) {
             const int i = i0 + threadIdx.x;
+            int64_t c = 0;
+            if (i < S && slice_rank(rk, i, R) <= 16)
+                c = x[i + 1] - x[i] + (int64_t)kTaskCost * cls[16 * i + 8 + kClasses];
             int64_t tot;
-            const int64_t pre = block_exclusive_scan<int64_t>(i < S ? cls[16 * i + 8 + kClasses] : 0, ws, &tot);
-            if (i < S) tp[i] = (int32_t)(tasks + pre);
-            tasks += tot;
+            const int64_t pre = block_exclusive_scan<int64_t>(c, ws, &tot);
+            if (i < S) wk[i] = work + pre;
+            work += tot;
             __syncthreads();
         }
-        if (threadIdx.x == 0) tp[S] = (int32_t)tasks;
+        if (threadIdx.x == 0) wk[S] = work;
         __syncthreads();
     }
 }
@@ -435,7 +458,7 @@ __global__ void k_als_init(lt_frame F, lt_samples smp, Omega om, int R, const in
 // of row q at chunk c ^ (q & 7), and the next 32 rows are on their way (cp.async)
 // while these are added.  Rows have stride R; components at or beyond R are zero.
 constexpr int kWarpStage = 32 * 32;    // floats of one stage: 32 rows of 32
-constexpr int kWarpCol = 36;           // stride of a column of L (16-byte aligned, odd in 16-byte chunks)
+constexpr int kWarpCol = 36;           // stride of a column of L (16-byte aligned)
 
 __device__ __forceinline__ void copy16(float* dst, const float* src, bool full) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
@@ -511,16 +534,22 @@ __device__ __forceinline__ void gram_warp(int len, const uint16_t* __restrict__ 
     for (int c = 0; c < 16; ++c) unpack2(g2[c], g[2 * c], g[2 * c + 1]);
 }
 
-// Column J of the Cholesky of a line whose row k lane k holds, and the columns after
-// it.  A column of L goes through shared memory (one store, then 16-byte broadcast
-// loads of its rows below J, a quarter as many instructions as a shuffle per row) and
-// stays there for the backward substitution.  Entries above the diagonal are not
-// used, so every lane updates its whole row.
-template <int J>
-__device__ __forceinline__ void chol_col32(float (&acc)[32], int k, int r, bool& ok, float& dmin, float& dmax,
-                                           float& my_inv, float* Lc) {
-    if constexpr (J < 32) {
-        const float djj = __shfl_sync(0xffffffffu, acc[J], J);
+// Eight columns (8 P ..) of the Cholesky of a line whose row k lane k holds, and the
+// forward substitution with them.  acc[0] is the current column and the registers move
+// down by one per column, so that one loop body serves the eight (all 32 unrolled are
+// more code than the instruction caches hold: 41% of the stall cycles).  A column of L
+// goes through shared memory (one store, then 16-byte broadcast loads, a quarter as many
+// instructions as a shuffle per row) and stays there for the backward substitution.
+// Entries above the diagonal are not used, so every lane updates its whole row.
+template <int P>
+__device__ __forceinline__ void chol_block32(float (&acc)[32], float& y, int k, int r, bool& ok, float& dmin,
+                                             float& dmax, float& my_inv, float* Lc) {
+    constexpr int W = 32 - 8 * P;  // columns left at the start of the block
+    const unsigned FULL = 0xffffffffu;
+#pragma unroll 1
+    for (int t = 0; t < 8; ++t) {
+        const int J = 8 * P + t;
+        const float djj = __shfl_sync(FULL, acc[0], J);
         if (J < r) {
             ok &= (djj > 0.f);
             dmin = djj < dmin ? djj : dmin;
@@ -529,20 +558,22 @@ __device__ __forceinline__ void chol_col32(float (&acc)[32], int k, int r, bool&
         const float dpos = djj > 0.f ? djj : 1.f;
         const float ljj = sqrtf(dpos);
         const float inv = 1.f / ljj;
+        const float lij = (k > J) ? acc[0] * inv : (k == J ? ljj : 0.f);
+        float* col = Lc + J * kWarpCol;  // row J + c of the column at col[c]
+        if (k >= J) col[k - J] = lij;
         if (k == J) my_inv = inv;
-        const float lij = (k > J) ? acc[J] * inv : (k == J ? ljj : 0.f);
-        acc[J] = lij;
-        Lc[J * kWarpCol + k] = lij;
+        const float yj = __shfl_sync(FULL, y * my_inv, J);  // L y = b: y_J is final
+        if (k == J) y = yj;
+        else if (k > J) y = fmaf(-lij, yj, y);
         __syncwarp();
 #pragma unroll
-        for (int q = (J + 1) / 4; q < 8; ++q) {
-            const float4 l = *reinterpret_cast<const float4*>(Lc + J * kWarpCol + 4 * q);
-            if (4 * q > J) acc[4 * q] = fmaf(-lij, l.x, acc[4 * q]);
-            if (4 * q + 1 > J) acc[4 * q + 1] = fmaf(-lij, l.y, acc[4 * q + 1]);
-            if (4 * q + 2 > J) acc[4 * q + 2] = fmaf(-lij, l.z, acc[4 * q + 2]);
-            if (4 * q + 3 > J) acc[4 * q + 3] = fmaf(-lij, l.w, acc[4 * q + 3]);
+        for (int q = 0; q < W / 4; ++q) {  // (columns past the last hold anything and are never read)
+            const float4 l = *reinterpret_cast<const float4*>(col + 4 * q);
+            if (q > 0) acc[4 * q - 1] = fmaf(-lij, l.x, acc[4 * q]);
+            acc[4 * q] = fmaf(-lij, l.y, acc[4 * q + 1]);
+            acc[4 * q + 1] = fmaf(-lij, l.z, acc[4 * q + 2]);
+            acc[4 * q + 2] = fmaf(-lij, l.w, acc[4 * q + 3]);
         }
-        chol_col32<J + 1>(acc, k, r, ok, dmin, dmax, my_inv, Lc);
     }
 }
 
@@ -567,31 +598,20 @@ __device__ __forceinline__ bool warp_solve32(float (&acc)[32], float rhs, int le
         acc[c] = c == k ? d : (k >= r ? 0.f : acc[c]);
     }
     if (k >= r) rhs = 0.f;
-    float dmin = 3.0e38f, dmax = 0.f, inv = 1.f;
+    float dmin = 3.0e38f, dmax = 0.f, inv = 1.f, y = rhs;
     bool ok = true;
-    chol_col32<0>(acc, k, r, ok, dmin, dmax, inv, Lc);
+    chol_block32<0>(acc, y, k, r, ok, dmin, dmax, inv, Lc);
+    chol_block32<1>(acc, y, k, r, ok, dmin, dmax, inv, Lc);
+    chol_block32<2>(acc, y, k, r, ok, dmin, dmax, inv, Lc);
+    chol_block32<3>(acc, y, k, r, ok, dmin, dmax, inv, Lc);
     if (!zero && (!ok || dmin < kPivotRatio * dmax)) return false;
-    float y = rhs;  // L y = b: lane k has its row of L in acc
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-        const float yj = __shfl_sync(FULL, y * inv, j);
-        if (k == j) y = yj;
-        else if (k > j) y = fmaf(-acc[j], yj, y);
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {  // L^T x = y: lane k takes its column of L
-        const float4 l = *reinterpret_cast<const float4*>(Lc + k * kWarpCol + 4 * q);
-        acc[4 * q] = l.x;
-        acc[4 * q + 1] = l.y;
-        acc[4 * q + 2] = l.z;
-        acc[4 * q + 3] = l.w;
-    }
-    float x = y;
-#pragma unroll
+    float x = y;  // L^T x = y: lane k reads its column of L (35 k + j: no bank conflicts)
+#pragma unroll 4
     for (int j = 31; j >= 0; --j) {
+        const float l = Lc[k * (kWarpCol - 1) + j];
         const float xj = __shfl_sync(FULL, x * inv, j);
         if (k == j) x = xj;
-        else if (k < j) x = fmaf(-acc[j], xj, x);
+        else if (k < j) x = fmaf(-l, xj, x);
     }
     *out_k = (zero || k >= r) ? 0.f : x;
     return true;
@@ -690,7 +710,7 @@ __device__ __forceinline__ void factor_solve_rows(T (&acc)[G], T rhs, int len, i
 // and the latency of the 32 dependent columns of the solve.  Completion of the 200-box
 // scene (5.7 M entries, ranks 8 to 32 per slice, 10 sweeps; the lane-group kernel has the
 // slices up to rank 16): 23.9 ms with a lane per factor row in the copies, a shuffle
-// per element in the Cholesky and 32-way bank conflicts in the solves; 16.3 ms so.
+// per element in the Cholesky and 32-way bank conflicts in the solves; 14.1 ms so.
 constexpr int kHalfWarps = 8;
 constexpr int kHalfSmem = kHalfWarps * 2 * kWarpStage * 4;  // the columns of L use the stage after the Gram
 static_assert(32 * kWarpCol <= 2 * kWarpStage, "the columns of L fit the stage");
@@ -820,38 +840,56 @@ __device__ __forceinline__ void add_entry(const float (&x)[RP], float av, float 
     }
 }
 
+// The entry streams of a warp's lanes on their way: a ring of kRing chunks of 4 entries
+// (8 bytes of indices, 16 of values a lane), filled by cp.async so that no register
+// holds them.  Every lane reads what it copied itself.
+constexpr int kRing = 4;
+constexpr int kRingBytes = kRing * 32 * 24;  // of a warp
+
+__device__ __forceinline__ void ring_copy(unsigned char* ring, int slot, const uint2* idx, const float4* val) {
+    const int lane = threadIdx.x & 31;
+    const unsigned di = (unsigned)__cvta_generic_to_shared(ring + slot * 256 + lane * 8);
+    const unsigned dv = (unsigned)__cvta_generic_to_shared(ring + kRing * 256 + slot * 512 + lane * 16);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(di), "l"(idx) : "memory");
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dv), "l"(val) : "memory");
+}
+
 // Adds x_e x_e^T (lower triangle) and a_e x_e for the nk entries of one lane's
 // stream (chunks of 4 at idx4[32 c], vv4[32 c]) to a and bb, in stream order.
 // The row of the next entry is loaded before this one is added, so that the
-// shared-memory reads (bank conflicts of random rows) run under the arithmetic.  Every lane
-// runs to the longest stream of the warp; past its own end it adds zeros (row zrow),
-// which leave the sums as they are.  Two entries per round of the inner loop: the
-// whole chunk unrolled is more code than the instruction caches hold.
+// shared-memory reads (bank conflicts of random rows) run under the arithmetic, and the
+// stream is three chunks ahead.  Every lane runs to the longest stream of the warp; past
+// its own end it adds zeros (row zrow), which leave the sums as they are.  Two entries per
+// round of the inner loop: the whole chunk unrolled is more code than the instruction
+// caches hold.
 template <int RP>
 __device__ __forceinline__ void stream_gram(int nk, const uint2* __restrict__ idx4, const float4* __restrict__ vv4,
                                             int r, int R, const float* __restrict__ src, bool staged, bool vec,
-                                            int zrow, const float4* stage4, float (&a)[RP * (RP + 1) / 2],
-                                            float (&bb)[RP]) {
+                                            int zrow, const float4* stage4, unsigned char* ring,
+                                            float (&a)[RP * (RP + 1) / 2], float (&bb)[RP]) {
+    const int lane = threadIdx.x & 31;
 #pragma unroll
     for (int i = 0; i < RP * (RP + 1) / 2; ++i) a[i] = 0.f;
 #pragma unroll
     for (int i = 0; i < RP; ++i) bb[i] = 0.f;
     const int nc = (__reduce_max_sync(0xffffffffu, nk) + 3) >> 2;
-    uint2 ic = make_uint2(0u, 0u);
-    float4 vc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (nc == 0) return;
+    auto ring_idx = [&](int c) { return *reinterpret_cast<const uint2*>(ring + (c & (kRing - 1)) * 256 + lane * 8); };
+    auto fill = [&](int c) {
+        if (c < nc) ring_copy(ring, c & (kRing - 1), idx4 + 32 * c, vv4 + 32 * c);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int c = 0; c < kRing - 1; ++c) fill(c);
+    asm volatile("cp.async.wait_group %0;" ::"n"(kRing - 2) : "memory");  // chunk 0
     float x[RP], y[RP];
-    if (nc > 0) {
-        ic = idx4[0];
-        vc = vv4[0];
-        load_row<RP>(x, nk > 0 ? (int)(ic.x & 0xffffu) : zrow, r, R, src, staged, vec, stage4);
-    }
+    uint2 ic = ring_idx(0);
+    load_row<RP>(x, nk > 0 ? (int)(ic.x & 0xffffu) : zrow, r, R, src, staged, vec, stage4);
     for (int c = 0; c < nc; ++c) {
-        uint2 in = ic;
-        float4 vn = vc;
-        if (c + 1 < nc) {
-            in = idx4[32 * (c + 1)];
-            vn = vv4[32 * (c + 1)];
-        }
+        fill(c + kRing - 1);
+        asm volatile("cp.async.wait_group %0;" ::"n"(kRing - 2) : "memory");  // chunks up to c + 1
+        const float4 vc = *reinterpret_cast<const float4*>(ring + kRing * 256 + (c & (kRing - 1)) * 512 + lane * 16);
+        const uint2 in = ring_idx(c + 1);  // (past the last chunk: not used)
 #pragma unroll 1
         for (int h = 0; h < 2; ++h) {
             const int e = 4 * c + 2 * h;
@@ -863,8 +901,8 @@ __device__ __forceinline__ void stream_gram(int nk, const uint2* __restrict__ id
             add_entry<RP>(y, e + 1 < nk ? v1 : 0.f, a, bb);
         }
         ic = in;
-        vc = vn;
     }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
 // One lane of a warp task: `line` (or -1) is its line, `sub` its rank among the G
@@ -873,7 +911,7 @@ template <int RP>
 __device__ __forceinline__ void als_line(const lt_frame& F, const Omega& om, int r, int R, bool rows_side,
                                          const float* __restrict__ src_base, const float* __restrict__ src,
                                          bool staged, bool vec, int zrow, const float4* stage4,
-                                         float* __restrict__ Fout, float lam_rel, const AlsQueue<RP>& q, int s,
+                                         unsigned char* ring, float* __restrict__ Fout, float lam_rel, const AlsQueue<RP>& q, int s,
                                          int line, int sub, int G, int64_t slot) {
     constexpr int NA = RP * (RP + 1) / 2;
     const int row0 = F.slice_off[s];
@@ -892,7 +930,7 @@ __device__ __forceinline__ void als_line(const lt_frame& F, const Omega& om, int
     float a[NA], bb[RP];
     const int nk = sub < len ? (len - sub + G - 1) / G : 0;
     stream_gram<RP>(nk, reinterpret_cast<const uint2*>(sidx + slot), reinterpret_cast<const float4*>(sval + slot), r,
-                    R, src, staged, vec, zrow, stage4, a, bb);
+                    R, src, staged, vec, zrow, stage4, ring, a, bb);
     if (G > 1) {  // the group's partial sums into its first lane (G is warp-uniform)
         for (int m = G >> 1; m > 0; m >>= 1) {
 #pragma unroll
@@ -956,11 +994,11 @@ __device__ __forceinline__ void stage_factors(const float* __restrict__ src, int
 // What bounds it: latency at two warps per scheduler (the registers of a lane's Gram) and
 // the bank conflicts of random factor rows.  Completion of 7.2 M entries in 64 slices,
 // rank 16, 10 sweeps: 4.24 ms with 110 KB of stage, one slice staged at a time, shares
-// that count slots only and no row loaded ahead; 3.39 ms so.  With three times the rows
-// (slices over the old stage, read from memory by scalar loads): 11.57 to 7.88 ms.
+// that count slots only, no row loaded ahead and the stream one chunk ahead; 2.83 ms so
+// (with the Omega build below it).  With three times the rows (slices over the old
+// stage, read from memory by scalar loads): 11.57 to 6.53 ms.
 // Packed multiply-adds (two elements an instruction) run at the rate of single ones
 // here and cost register moves: 4.58 ms.
-constexpr int kTaskCost = 512;   // slots worth a task's reduction and Cholesky (32 lanes x 16 entries)
 constexpr int kSegs = 8;
 
 struct AlsSeg {
@@ -977,19 +1015,24 @@ __global__ void __launch_bounds__(256, RP == 8 ? 2 : 1) k_als_line(lt_frame F, l
     extern __shared__ float4 stage4[];
     __shared__ int s_next, s_n;
     __shared__ AlsSeg seg[kSegs];
+    unsigned char* ring = reinterpret_cast<unsigned char*>(stage4 + (int64_t)stage_rows * (RP / 4)) +
+                          (threadIdx.x >> 5) * kRingBytes;
     const int S = F.S;
     const int64_t* base = rows_side ? om.rbase : om.cbase;
-    const int32_t* tpfx = rows_side ? om.rtp : om.ctp;
+    const int64_t* wk = rows_side ? om.rwk : om.cwk;
     const int32_t* cls_all = rows_side ? om.rcls : om.ccls;
     const int32_t* tb_all = rows_side ? om.rtb : om.ctb;
     // a layout over its capacity was latched as LT_ELIMIT and not written: read nothing
     if (base[S] > om.sell_cap) return;
-    const int64_t total = base[S] + (int64_t)kTaskCost * tpfx[S];
+    const int64_t total = wk[S];
     const int64_t lo = total * blockIdx.x / gridDim.x;
     const int64_t hi = blockIdx.x + 1 == gridDim.x ? INT64_MAX : total * (blockIdx.x + 1) / gridDim.x;
-    // work before task t of slice x
+    // tasks of slice x (none where its rank is the warp-per-line kernel's) and the work before task t
+    auto tasks_of = [&](int x) {
+        return slice_rank(rk, x, R) <= RP ? cls_all[(int64_t)x * 16 + 8 + kClasses] : 0;
+    };
     auto before = [&](int x, int t) {
-        return base[x] + tb_all[(int64_t)x * om.tcap + t] + (int64_t)kTaskCost * (tpfx[x] + t);
+        return wk[x] + tb_all[(int64_t)x * om.tcap + t] + (int64_t)kTaskCost * t;
     };
     // first task in [t, T) of slice x that starts at or after `at`
     auto first_task = [&](int x, int t, int T, int64_t at) {
@@ -1008,22 +1051,21 @@ __global__ void __launch_bounds__(256, RP == 8 ? 2 : 1) k_als_line(lt_frame F, l
         int x = 0, y = S;
         while (x < y) {
             const int m = (x + y) >> 1;
-            if (base[m + 1] + (int64_t)kTaskCost * tpfx[m + 1] < lo) x = m + 1; else y = m;
+            if (wk[m + 1] < lo) x = m + 1; else y = m;
         }
         s = x;
-        t = s < S ? first_task(s, 0, tpfx[s + 1] - tpfx[s], lo) : 0;
+        t = s < S ? first_task(s, 0, tasks_of(s), lo) : 0;
     }
     for (;;) {
         if (threadIdx.x == 0) {
             // the next slice segments of this CTA (tasks starting before hi), while their rows fit
             int n = 0, used = 0, tasks = 0;
             while (s < S && n < kSegs) {
-                const int T = tpfx[s + 1] - tpfx[s];
+                const int T = tasks_of(s);
                 if (t < T && before(s, t) >= hi) s = S;  // the share ends here
                 if (s >= S) break;
-                const int r = slice_rank(rk, s, R);
                 const int t1 = first_task(s, t, T, hi);
-                if (t < t1 && r <= RP) {  // per-slice ranks above RP are the warp-per-line kernel's
+                if (t < t1) {
                     const int need = (rows_side ? smp.ncol[s] : F.slice_off[s + 1] - F.slice_off[s]) + 1;
                     const bool fits = need <= stage_rows;
                     if (fits && used + need > stage_rows) break;  // in the next batch
@@ -1074,7 +1116,7 @@ __global__ void __launch_bounds__(256, RP == 8 ? 2 : 1) k_als_line(lt_frame F, l
             const int li = cls[c] + (tk - cls[8 + c]) * (32 >> g) + (lane >> g);
             const bool live = li < cls[c + 1];
             als_line<RP>(F, om, r, R, rows_side, Fin, src, staged, vec, staged ? nsrc : -1,
-                         stage4 + (staged ? seg[k].row * (RP / 4) : 0), Fout, lam_rel, q, sl, live ? ord[li] : -1,
+                         stage4 + (staged ? seg[k].row * (RP / 4) : 0), ring, Fout, lam_rel, q, sl, live ? ord[li] : -1,
                          lane & (G - 1), G, base[sl] + tb_all[(int64_t)sl * om.tcap + tk] + 4 * lane);
         }
         __syncthreads();  // the stage and the segments are reused by the next batch
@@ -1243,9 +1285,8 @@ __global__ void k_slice_ranks(lt_samples smp, int S, int R, int cols, int32_t* _
 namespace ltk {
 
 lt_status omega_build(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, int64_t E, bool sell, bool csr, bool bits,
-                      Omega* omp) {
+                      const int32_t* rk, int R, Omega* omp) {
     const int S = f->S, C = f->C;
-    constexpr int kOmParts = 8;   // fixes the order of the mean value's sum
     const int64_t mr = std::max(f->max_rows, 1);
     Omega& om = *omp;
     om.bm_stride = mr * ((C + 31) / 32);
@@ -1270,7 +1311,7 @@ lt_status omega_build(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, int
     char* p = (char*)lt_scratch(ctx, SCR_OMEGA,
                                 (size_t)(f->m + S) * 4 + (size_t)S * (C + 1) * 4 + e_csr * 16 + e_sell * 12 + S * 8 +
                                     (size_t)S * (om.bm_stride + om.bt_stride) * (bits ? 12 : 8) + (S + 1) * 8 + (size_t)f->m * 8 +
-                                    (size_t)S * C * 8 + (size_t)S * 128 + (size_t)(S + 1) * 8 + t_sell * 8 + (size_t)(S + 1) * 16 +
+                                    (size_t)S * C * 8 + (size_t)S * 128 + (size_t)(S + 1) * 16 + t_sell * 8 + (size_t)(S + 1) * 16 +
                                     (size_t)S * kOmParts * 4 + 36 * 256,
                                 &st);
     if (!p) return st;
@@ -1302,8 +1343,8 @@ lt_status omega_build(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, int
     om.ctb = (int32_t*)take(t_sell * 4);
     om.rbase = (int64_t*)take((size_t)(S + 1) * 8);
     om.cbase = (int64_t*)take((size_t)(S + 1) * 8);
-    om.rtp = (int32_t*)take((size_t)(S + 1) * 4);
-    om.ctp = (int32_t*)take((size_t)(S + 1) * 4);
+    om.rwk = (int64_t*)take((size_t)(S + 1) * 8);
+    om.cwk = (int64_t*)take((size_t)(S + 1) * 8);
     om.sidx_r = (uint16_t*)take(e_sell * 2);
     om.sval_r = (float*)take(e_sell * 4);
     om.sidx_c = (uint16_t*)take(e_sell * 2);
@@ -1312,21 +1353,24 @@ lt_status omega_build(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, int
     if ((size_t)(p - (char*)ctx->scr[SCR_OMEGA]) > ctx->scr_size[SCR_OMEGA])
         return lt_fail(ctx, LT_ENOMEM, "omega_build: layout overflow");
     const int nsm = ctx->num_sms;
+    // (a thread's chain of dependent loads is what these passes wait for: grids of up to 16
+    // CTAs per SM; 4 took 0.31 ms for the scatter of 7.2 M entries)
+    const unsigned wide = (unsigned)std::max(1, 16 * nsm / S);
     k_om_clear<<<dim3(std::max(1, 2 * nsm / S), S), 256, 0, ctx->stream>>>(*f, *smp, om);
     LT_LAUNCH_CHECK(ctx, "k_om_clear");
-    k_om_bits<<<dim3(kOmParts, S), 256, 0, ctx->stream>>>(*f, *smp, om, part, ctx->d_status);
+    k_om_bits<<<dim3(wide, S), 256, 0, ctx->stream>>>(*f, *smp, om, ctx->d_status);
     LT_LAUNCH_CHECK(ctx, "k_om_bits");
-    k_om_transpose<<<dim3(std::max(1, 8 * nsm / S), S), 256, 0, ctx->stream>>>(*f, *smp, om);
+    k_om_transpose<<<dim3(std::max(kOmParts, 8 * nsm / S), S), 256, 0, ctx->stream>>>(*f, *smp, om, part);
     LT_LAUNCH_CHECK(ctx, "k_om_transpose");
     k_om_lines<<<dim3(std::max(1, 4 * nsm / S), S), 256, 0, ctx->stream>>>(*f, *smp, om);
     LT_LAUNCH_CHECK(ctx, "k_om_lines");
-    k_om_scan<<<S, 1024, 0, ctx->stream>>>(*f, *smp, om, part, kOmParts);
+    k_om_scan<<<dim3(S, 2), 1024, 0, ctx->stream>>>(*f, *smp, om, part, kOmParts);
     LT_LAUNCH_CHECK(ctx, "k_om_scan");
     if (om.sell) {
-        k_om_sellpfx<<<1, 1024, 0, ctx->stream>>>(S, om, ctx->d_status);
+        k_om_sellpfx<<<1, 1024, 0, ctx->stream>>>(S, om, rk, R, ctx->d_status);
         LT_LAUNCH_CHECK(ctx, "k_om_sellpfx");
     }
-    k_om_scatter<<<dim3(std::max(1, 4 * nsm / S), S), 256, 0, ctx->stream>>>(*f, *smp, om);
+    k_om_scatter<<<dim3(wide, S), 256, 0, ctx->stream>>>(*f, *smp, om);
     LT_LAUNCH_CHECK(ctx, "k_om_scatter");
     k_line_prefix<<<1, 1024, 0, ctx->stream>>>(*smp, S, om.line_pfx);
     LT_LAUNCH_CHECK(ctx, "k_line_prefix");
@@ -1397,7 +1441,7 @@ lt_status complete_impl(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, i
     const bool low = R <= 16 || rk != nullptr;
     const bool tc = low && ctx->tune.als_form == 1;
     Omega om;
-    lt_status st = omega_build(ctx, f, smp, E, low && !tc, R > 16 || tc, tc, &om);
+    lt_status st = omega_build(ctx, f, smp, E, low && !tc, R > 16 || tc, tc, rk, R, &om);
     if (st != LT_OK) return st;
     const int RP = R <= 8 ? 8 : 16;  // the low-rank kernels cover ranks up to RP
     // per half-step retry counters (one set for ranks <= 16, one above) and the
@@ -1423,11 +1467,12 @@ lt_status complete_impl(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, i
     }
     // lane-group kernel: one thread (group) per line; one 256-thread CTA per SM (its
     // registers fill the SM) stages the factor rows of its slices, each with a row of
-    // zeros, up to 208 KB (3328 rows at rank 16)
+    // zeros, and the streams' rings: up to 216 KB (3072 rows at rank 16)
     const size_t row_bytes = (size_t)RP * 4;
-    const int per_sm = RP == 8 ? 2 : 1;  // rank 8 needs half the registers: two CTAs of 104 KB
-    const int stage_rows = (int)((208 * 1024 / per_sm) / row_bytes);
-    const size_t dyn = (size_t)stage_rows * row_bytes;
+    const int per_sm = RP == 8 ? 2 : 1;  // rank 8 needs half the registers: two CTAs of 108 KB
+    const size_t ring_bytes = 8 * kRingBytes;
+    const int stage_rows = (int)((216 * 1024 / per_sm - ring_bytes) / row_bytes);
+    const size_t dyn = (size_t)stage_rows * row_bytes + ring_bytes;
     const int64_t cap = std::min<int64_t>(std::max<int64_t>(f->m, (int64_t)S * C), 1 << 18);
     int64_t *qdst = nullptr, *qslot = nullptr, *qsrc = nullptr;
     int32_t *qlen = nullptr, *qgrp = nullptr, *qrank = nullptr;
@@ -1533,7 +1578,7 @@ extern "C" lt_status lt_als_gram(lt_ctx* ctx, const lt_frame* f, const lt_sample
     LT_CUDA(ctx, cudaMemcpyAsync(&E, smp->off + f->S, sizeof(int64_t), cudaMemcpyDeviceToHost, ctx->stream));
     LT_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     Omega om;
-    lt_status st = omega_build(ctx, f, smp, E, false, true, true, &om);
+    lt_status st = omega_build(ctx, f, smp, E, false, true, true, nullptr, uv->r, &om);
     if (st != LT_OK) return st;
     const int R = uv->r, RP = R <= 8 ? 8 : 16;
     TcPlan tcp{};

@@ -46,8 +46,8 @@ struct Omega {
     int32_t* ctb;       // [S][tcap]
     int64_t* rbase;     // [S + 1]      region start of each slice, rows side ([S] = total)
     int64_t* cbase;     // [S + 1]
-    int32_t* rtp;       // [S + 1]      warp tasks of the slices before each, rows side
-    int32_t* ctp;       // [S + 1]
+    int64_t* rwk;       // [S + 1]      lane-group work of the slices before each, rows side
+    int64_t* cwk;       // [S + 1]
     uint16_t* sidx_r;   // [sell_cap]   column of each rows-side slot
     float* sval_r;
     uint16_t* sidx_c;   // [sell_cap]   row of each columns-side slot
@@ -62,8 +62,9 @@ struct Omega {
 // Builds Omega for the frame's samples (E = total entry count, known to the host):
 // bitmaps, per-word prefixes, line counts, row / column pointers, sorted line orders,
 // mean observed value per slice, and the sliced layout (sell) and / or CSR / CSC
-// (csr), and the plain bitmaps (bits), in scratch slot SCR_OMEGA.
+// (csr), and the plain bitmaps (bits), in scratch slot SCR_OMEGA; rk and R: the ranks
+// (see slice_rank), which say whose lines the lane-group kernel has.
 lt_status omega_build(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, int64_t E, bool sell, bool csr, bool bits,
-                      Omega* om);
+                      const int32_t* rk, int R, Omega* om);
 
 }  // namespace ltk
