@@ -424,6 +424,7 @@ __global__ void k_feat_slice(lt_frame F, lt_samples smp, float* __restrict__ st)
     for (int k = 6; k < 9; ++k) acc[k] = 3.0e38f;
     for (int k = 9; k < 12; ++k) acc[k] = -3.0e38f;
     acc[12] = 0.f;
+#pragma unroll 4
     for (int i = threadIdx.x; i < ms; i += blockDim.x) {
         const float4 p = P0[row0 + i], nn = P1[row0 + i];
         acc[0] += p.x;
@@ -441,6 +442,7 @@ __global__ void k_feat_slice(lt_frame F, lt_samples smp, float* __restrict__ st)
     }
     const int n1 = smp.n1[s];
     const float* val = smp.val + smp.off[s];
+#pragma unroll 16
     for (int e = threadIdx.x; e < n1; e += blockDim.x) acc[12] += val[e];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int k = 0; k < 13; ++k) {
@@ -493,15 +495,13 @@ __device__ __forceinline__ int first_col_at_least(const uint32_t* key, int n1, i
 __global__ void k_feat_cols(lt_frame F, lt_samples smp, const float* __restrict__ st,
                             const int32_t* __restrict__ goff, float* __restrict__ feat) {
     const int lane = threadIdx.x & 31;
-    const int S = F.S, C = F.C;
+    const int C = F.C;
     const float4* V0 = reinterpret_cast<const float4*>(F.vpls);
     const float4* V1 = V0 + F.n;
     const float iroot = F.tree.I[0];
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t x = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); x < (int64_t)S * C; x += nwarps) {
-        const int s = (int)(x / C), j = (int)(x % C);
-        const int ns = smp.ncol[s];
-        if (j >= ns) continue;
+    const int s = blockIdx.y;
+    const int ns = smp.ncol[s];
+    for (int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); j < ns; j += gridDim.x * (blockDim.x >> 5)) {
         const uint32_t* key = smp.key + smp.off[s];
         const float* val = smp.val + smp.off[s];
         const int n1 = smp.n1[s];
@@ -650,7 +650,7 @@ __global__ void k_goff(lt_samples smp, int S, int64_t* __restrict__ goff2, int64
 // shared memory 16 at a time, the next 16 loaded while these are added.  Every output
 // is one chain of multiply-adds over the rows in order.  Bound by the FP32 pipe.  With
 // this, k_slice_matrix and the split subspace iteration the training data of a scene of 65536
-// points (64 slices of about 630 columns, 30 rounds at rank 16) take 8.6 ms, 55.3 ms with
+// points (64 slices of about 630 columns, 30 rounds at rank 16) take 6.4 ms, 54.1 ms with
 // 32 x 32 tiles and one CTA per slice for the whole iteration.
 __global__ void __launch_bounds__(256, 2) k_gram(lt_frame F, lt_samples smp, const float* __restrict__ M,
                                                  const int64_t* __restrict__ moff, const int64_t* __restrict__ goff2,
@@ -771,12 +771,24 @@ __device__ void mgs_cols(float* Q, int n, int r, float* red) {
 template <int NR>
 __device__ void mgs_regs(float* __restrict__ Q, int n, int r, float* red, float (*part)[16], float* dots) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const bool vec = r == 16 && ((uintptr_t)Q & 15) == 0;  // rows of 64 bytes
     float q[NR][16];
 #pragma unroll
     for (int p = 0; p < NR; ++p) {
         const int i = threadIdx.x + kLevThreads * p;
+        if (vec && i < n) {
 #pragma unroll
-        for (int k = 0; k < 16; ++k) q[p][k] = (i < n && k < r) ? Q[(int64_t)i * r + k] : 0.f;
+            for (int k = 0; k < 4; ++k) {
+                const float4 t = *reinterpret_cast<const float4*>(Q + (int64_t)i * 16 + 4 * k);
+                q[p][4 * k] = t.x;
+                q[p][4 * k + 1] = t.y;
+                q[p][4 * k + 2] = t.z;
+                q[p][4 * k + 3] = t.w;
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) q[p][k] = (i < n && k < r) ? Q[(int64_t)i * r + k] : 0.f;
+        }
     }
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
@@ -784,7 +796,12 @@ __device__ void mgs_regs(float* __restrict__ Q, int n, int r, float* red, float 
             float q2 = 0.f;
 #pragma unroll
             for (int p = 0; p < NR; ++p) q2 = fmaf(q[p][j], q[p][j], q2);
-            q2 = block_sum(q2, red);
+            q2 = warp_sum(q2);
+            if (lane == 0) red[w] = q2;
+            __syncthreads();  // (the next write of red is two barriers away)
+            q2 = 0.f;
+#pragma unroll
+            for (int x = 0; x < kLevThreads / 32; ++x) q2 += red[x];
             const float inv = q2 > 0.f ? 1.f / sqrtf(q2) : 0.f;
 #pragma unroll
             for (int p = 0; p < NR; ++p) q[p][j] *= inv;
@@ -812,6 +829,7 @@ __device__ void mgs_regs(float* __restrict__ Q, int n, int r, float* red, float 
                 __syncthreads();
                 if (threadIdx.x < 16) {
                     float t = 0.f;
+#pragma unroll
                     for (int x = 0; x < kLevThreads / 32; ++x) t += part[x][threadIdx.x];
                     dots[threadIdx.x] = t;
                 }
@@ -828,9 +846,16 @@ __device__ void mgs_regs(float* __restrict__ Q, int n, int r, float* red, float 
 #pragma unroll
     for (int p = 0; p < NR; ++p) {
         const int i = threadIdx.x + kLevThreads * p;
+        if (vec && i < n) {
 #pragma unroll
-        for (int k = 0; k < 16; ++k)
-            if (i < n && k < r) Q[(int64_t)i * r + k] = q[p][k];
+            for (int k = 0; k < 4; ++k)
+                *reinterpret_cast<float4*>(Q + (int64_t)i * 16 + 4 * k) =
+                    make_float4(q[p][4 * k], q[p][4 * k + 1], q[p][4 * k + 2], q[p][4 * k + 3]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 16; ++k)
+                if (i < n && k < r) Q[(int64_t)i * r + k] = q[p][k];
+        }
     }
     __syncthreads();
 }
@@ -899,6 +924,13 @@ __global__ void __launch_bounds__(kLevRows) k_lev_mult(lt_samples smp, int S, in
         float a[16];
 #pragma unroll
         for (int k = 0; k < 16; ++k) a[k] = 0.f;
+        float g[16], gn[16];
+        auto fetch = [&](int j) {
+            if (j >= ns) return;
+#pragma unroll
+            for (int u = 0; u < 16; ++u) gn[u] = __ldg(Gi + (int64_t)min(j + u, ns - 1) * ns);
+        };
+        fetch(0);
         for (int j0 = 0; j0 < ns; j0 += kLevTile) {
             __syncthreads();
             for (int e = threadIdx.x; e < kLevTile * 16; e += kLevRows) {
@@ -906,11 +938,14 @@ __global__ void __launch_bounds__(kLevRows) k_lev_mult(lt_samples smp, int S, in
                 sq[e >> 4][e & 15] = (j < ns && k < rr) ? Q[(int64_t)j * rr + k] : 0.f;
             }
             __syncthreads();
-            const int nj = min(kLevTile, ns - j0);
-            for (int jj = 0; jj < nj; jj += 16) {
-                float g[16];
+            // 16 rows' loads in flight, the next 16 issued before these are added; rows past the
+            // last are the last one again, against zeros of Q
+#pragma unroll 1
+            for (int jj = 0; jj < kLevTile; jj += 16) {
+                if (j0 + jj >= ns) break;
 #pragma unroll
-                for (int u = 0; u < 16; ++u) g[u] = jj + u < nj ? __ldg(Gi + (int64_t)(j0 + jj + u) * ns) : 0.f;
+                for (int u = 0; u < 16; ++u) g[u] = gn[u];
+                fetch(j0 + jj + 16);
 #pragma unroll
                 for (int u = 0; u < 16; ++u) {
                     float x[16];
@@ -948,9 +983,8 @@ extern "C" lt_status lt_proposal_features(lt_ctx* ctx, const lt_frame* f, const 
     LT_LAUNCH_CHECK(ctx, "k_feat_slice");
     k_group_prefix<<<1, 1024, 0, ctx->stream>>>(smp->ncol, f->S, group_off);
     LT_LAUNCH_CHECK(ctx, "k_group_prefix");
-    const int64_t warps = (int64_t)f->S * f->C;
-    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((warps + 7) / 8, 16 * ctx->num_sms));
-    k_feat_cols<<<grid, 256, 0, ctx->stream>>>(*f, *smp, stats, group_off, feat);
+    const unsigned grid = (unsigned)std::max(1, std::min((f->C + 7) / 8, 8 * ctx->num_sms / f->S));
+    k_feat_cols<<<dim3(grid, f->S), 256, 0, ctx->stream>>>(*f, *smp, stats, group_off, feat);
     LT_LAUNCH_CHECK(ctx, "k_feat_cols");
     return LT_OK;
 }
