@@ -112,8 +112,9 @@ __global__ void __launch_bounds__(kP1Threads) k_pass1_plan(lt_frame F, float rat
 // also list the others; then the others), or two steps of one persistent cooperative
 // launch with grid-wide barriers (k_p1_walk).  What bounds it: latency (dependent loads,
 // then the rays of a pair).  Against five launches a level with the missing entries in a
-// queue and a serial merge per small pair: the 64x64 frame 1.71 to 1.19 ms, the sampling of
-// the 512x512 scene with 1000 boxes 7.03 to 6.43 ms.
+// queue and a serial merge per small pair: the 64x64 frame 1.71 to 1.19 ms (1.01 ms with
+// a CTA per listed pair where they are few), the sampling of the 512x512 scene with 1000
+// boxes 7.1 to 5.1 ms.
 
 struct P1Store {
     int32_t* rows;     // [total] row of each storage slot
@@ -608,8 +609,11 @@ __device__ __forceinline__ void p1_small_body(const lt_frame& F, const Grid& g, 
 }
 
 // step 2: the listed pairs.  A CTA per pair of more than kMidPair rows (both row lists
-// staged in shared memory when they fit), then a warp per pair.
+// staged in shared memory when they fit), then a warp per pair; where a level has few
+// pairs (at most kFewPairs per CTA), a CTA each for those too: with a warp, a level waits
+// for eight shadow rays one after the other.
 constexpr int kBigStage = 4096;
+constexpr int kFewPairs = 4;
 
 __device__ __forceinline__ void p1_rest_body(const lt_frame& F, const Grid& g, float dmin2, const P1Plan& pl,
                                              const P1Store& st, const P1Work& w, int h, int32_t* status) {
@@ -618,9 +622,10 @@ __device__ __forceinline__ void p1_rest_body(const lt_frame& F, const Grid& g, f
     __shared__ float red[32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int64_t nbig = min(w.bcount[h], w.bcap), nmid = min(w.mcount[h], w.bcap);
-    for (int64_t q = blockIdx.x; q < nbig; q += gridDim.x) {
+    const bool few = nmid <= (int64_t)kFewPairs * gridDim.x;
+    for (int64_t q = blockIdx.x; q < nbig + (few ? nmid : 0); q += gridDim.x) {
         PairCtx pc;
-        if (!load_pair(F, pl, st, h, w.big[q], pc)) continue;  // uniform in the block
+        if (!load_pair(F, pl, st, h, q < nbig ? w.big[q] : w.mid[q - nbig], pc)) continue;  // uniform in the block
         const PairRatio pr = pair_ratio(F, pc);
         const bool staged = pc.na <= kBigStage && pc.nb <= kBigStage;
         __syncthreads();  // the previous pair is done with the stage
@@ -652,6 +657,7 @@ __device__ __forceinline__ void p1_rest_body(const lt_frame& F, const Grid& g, f
         for (int k = 0; k < nw; ++k) em = fmaxf(em, red[k]);
         decide_pair(F, pl, st, w.thr, pc, pr, pc.na + pc.nb - ca, em, threadIdx.x, blockDim.x, threadIdx.x == 0);
     }
+    if (few) return;
     for (int64_t q = blockIdx.x * (int64_t)nw + wid; q < nmid; q += (int64_t)gridDim.x * nw) {
         PairCtx pc;
         if (!load_pair(F, pl, st, h, w.mid[q], pc)) continue;  // uniform in the warp
@@ -660,11 +666,13 @@ __device__ __forceinline__ void p1_rest_body(const lt_frame& F, const Grid& g, f
 }
 
 // Per-level form: each step of each level is its own launch.
+constexpr int kRestThreads = 512;
+
 __global__ void __launch_bounds__(128, 6) k_p1_small(lt_frame F, Grid g, float dmin2, P1Plan pl, P1Store st, P1Work w,
                                                   int h, int32_t* status) {
     p1_small_body(F, g, dmin2, pl, st, w, h, status);
 }
-__global__ void __launch_bounds__(256, 3) k_p1_rest(lt_frame F, Grid g, float dmin2, P1Plan pl, P1Store st, P1Work w,
+__global__ void __launch_bounds__(kRestThreads, 2) k_p1_rest(lt_frame F, Grid g, float dmin2, P1Plan pl, P1Store st, P1Work w,
                                                  int h, int32_t* status) {
     p1_rest_body(F, g, dmin2, pl, st, w, h, status);
 }
@@ -719,10 +727,12 @@ __global__ void __launch_bounds__(256, 3) k_p1_walk(lt_frame F, Grid g, float dm
 }
 
 // -- the coarsened cut of every slice in leaf order and its observed entries
-__global__ void __launch_bounds__(kP1Threads) k_p1_output(lt_frame F, P1Plan pl, P1Store st, lt_samples smp,
+constexpr int kOutThreads = 1024;
+
+__global__ void __launch_bounds__(kOutThreads) k_p1_output(lt_frame F, P1Plan pl, P1Store st, lt_samples smp,
                                                           int32_t* status) {
     extern __shared__ int32_t mark[];  // [C] forest node whose first leaf is c, else -1
-    __shared__ int32_t ws[32];
+    __shared__ long long ws[32];
     __shared__ float red[32];
     const int s = blockIdx.x;
     const int C = F.C, NF = 2 * C - 1;
@@ -750,32 +760,27 @@ __global__ void __launch_bounds__(kP1Threads) k_p1_output(lt_frame F, P1Plan pl,
     __syncthreads();
     int32_t* colx = pl.colx + (int64_t)s * C;
     int32_t* eoff = pl.eoff + (int64_t)s * C;
-    int ncol = 0;
-    for (int c0 = 0; c0 < C; c0 += blockDim.x) {
-        const int c = c0 + threadIdx.x;
-        const int x = c < C ? mark[c] : -1;
-        int tot;
-        const int pre = block_exclusive_scan<int>(x >= 0 ? 1 : 0, ws, &tot);
-        if (x >= 0) {
-            const int j = ncol + pre;
-            colx[j] = x;
-            const int par = F.forest[8 * x + 3];
-            const bool from_par = par >= 0 && state[par] == kStRejected;
-            eoff[j] = from_par ? cnt[par] : cnt[x];
-            smp.col_node[(int64_t)s * C + j] = F.forest[8 * x];
-        }
-        ncol += tot;
+    // each thread has a run of cut nodes: one scan for the columns and their entry counts
+    const int run = (C + blockDim.x - 1) / blockDim.x, c_lo = min(C, (int)threadIdx.x * run), c_hi = min(C, c_lo + run);
+    auto entries = [&](int x) {
+        const int par = F.forest[8 * x + 3];
+        return par >= 0 && state[par] == kStRejected ? cnt[par] : cnt[x];
+    };
+    long long cols = 0;  // columns in the high half, entries in the low half
+    for (int c = c_lo; c < c_hi; ++c)
+        if (mark[c] >= 0) cols += (1ll << 40) + entries(mark[c]);
+    long long tot;
+    long long at = block_exclusive_scan<long long>(cols, ws, &tot);
+    for (int c = c_lo; c < c_hi; ++c) {
+        const int x = mark[c];
+        if (x < 0) continue;
+        const int j = (int)(at >> 40);
+        colx[j] = x;
+        eoff[j] = (int)(at & ((1ll << 40) - 1));
+        smp.col_node[(int64_t)s * C + j] = F.forest[8 * x];
+        at += (1ll << 40) + entries(x);
     }
-    __syncthreads();
-    int n1 = 0;
-    for (int c0 = 0; c0 < ncol; c0 += blockDim.x) {
-        const int j = c0 + threadIdx.x;
-        const int x = j < ncol ? eoff[j] : 0;
-        int tot;
-        const int pre = block_exclusive_scan<int>(x, ws, &tot);
-        if (j < ncol) eoff[j] = n1 + pre;
-        n1 += tot;
-    }
+    const int ncol = (int)(tot >> 40), n1 = (int)(tot & ((1ll << 40) - 1));
     __syncthreads();
     const int64_t capacity = smp.off[s + 1] - smp.off[s];
     const bool over = (int64_t)n1 > capacity;
@@ -1380,7 +1385,7 @@ lt_status sample_pass1(lt_ctx* ctx, const lt_frame* f, float rate1, float tau, i
         k_p1_small<<<grid_for(npairs * kGroup, 128), 128, 0, ctx->stream>>>(*f, ctx->grid, dmin2, pl, store, w, h,
                                                                            ctx->d_status);
         LT_LAUNCH_CHECK(ctx, "k_p1_small");
-        k_p1_rest<<<4 * nsm, 256, 0, ctx->stream>>>(*f, ctx->grid, dmin2, pl, store, w, h, ctx->d_status);
+        k_p1_rest<<<2 * nsm, kRestThreads, 0, ctx->stream>>>(*f, ctx->grid, dmin2, pl, store, w, h, ctx->d_status);
         LT_LAUNCH_CHECK(ctx, "k_p1_rest");
     }
     if (target > 0) {
@@ -1390,7 +1395,7 @@ lt_status sample_pass1(lt_ctx* ctx, const lt_frame* f, float rate1, float tau, i
     const size_t shm = (size_t)C * 4;
     if (shm > 16 * 1024)
         LT_CUDA(ctx, cudaFuncSetAttribute(k_p1_output, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-    k_p1_output<<<S, kP1Threads, shm, ctx->stream>>>(*f, pl, store, *smp, ctx->d_status);
+    k_p1_output<<<S, kOutThreads, shm, ctx->stream>>>(*f, pl, store, *smp, ctx->d_status);
     LT_LAUNCH_CHECK(ctx, "k_p1_output");
     return LT_OK;
 }
