@@ -113,8 +113,8 @@ __global__ void __launch_bounds__(kP1Threads) k_pass1_plan(lt_frame F, float rat
 // launch with grid-wide barriers (k_p1_walk).  What bounds it: latency (dependent loads,
 // then the rays of a pair).  Against five launches a level with the missing entries in a
 // queue and a serial merge per small pair: the 64x64 frame 1.71 to 1.19 ms (1.01 ms with
-// a CTA per listed pair where they are few), the sampling of the 512x512 scene with 1000
-// boxes 7.1 to 5.1 ms.
+// a CTA per listed pair where they are few, 0.95 ms with one record per forest node), the
+// sampling of the 512x512 scene with 1000 boxes 7.1 to 5.1, then 4.7 ms.
 
 struct P1Store {
     int32_t* rows;     // [total] row of each storage slot
@@ -128,6 +128,7 @@ struct P1Work {
     int64_t* kpfx;     // [S+1] prefix over slices of the initial entry counts
     float* leafmean;   // [S][C] mean of each cut node's initial entries
     float* thr;        // [S] tau * S_hat (-1 in a dark slice, S_hat = 0)
+    float4* nrec;      // [NF][4] per forest node: its representative's planes, then (scale, I, 0, 0)
     int64_t* mcount;   // [Hmax] pairs of a warp per level
     int64_t* bcount;   // [Hmax] pairs of a CTA per level
     int64_t* mid;      // [bcap] flat pair index of a warp's pair
@@ -135,6 +136,20 @@ struct P1Work {
     unsigned* bar;     // arrival counter of the persistent walk's grid barriers
     int64_t bcap;
 };
+
+// -- what an entry or a pair reads of a forest node, in one 64-byte record
+__global__ void k_p1_nodes(lt_frame F, float4* __restrict__ nrec) {
+    const float4* vpls = reinterpret_cast<const float4*>(F.vpls);
+    const int NF = 2 * F.C - 1;
+    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < NF; x += gridDim.x * blockDim.x) {
+        const int node = F.forest[8 * x];
+        const PointRec L = load_rec(vpls, F.n, F.tree.rep[node]);
+        nrec[4 * x] = L.a;
+        nrec[4 * x + 1] = L.b;
+        nrec[4 * x + 2] = L.c;
+        nrec[4 * x + 3] = make_float4(node_scale(F.tree, vpls, F.n, node), F.tree.I[node], 0.f, 0.f);
+    }
+}
 
 // -- draws of the cut nodes and state of every forest node.  A node's rows are the first
 // k distinct draws, ascending.  Up to kSerialDraws rows a thread draws for its node; for
@@ -258,9 +273,9 @@ __global__ void k_p1_kpfx(lt_frame F, P1Plan pl, int64_t* kpfx) {
 
 // -- initial entries of every cut node of every slice (one shadow ray per thread)
 __global__ void __launch_bounds__(128) k_p1_initial(lt_frame F, Grid g, float dmin2, P1Plan pl, P1Store st,
-                                                    const int64_t* __restrict__ kpfx, int32_t* status) {
+                                                    const int64_t* __restrict__ kpfx,
+                                                    const float4* __restrict__ nrec, int32_t* status) {
     const float4* pts = reinterpret_cast<const float4*>(F.pts);
-    const float4* vpls = reinterpret_cast<const float4*>(F.vpls);
     const int C = F.C, NF = 2 * C - 1;
     const int64_t total = kpfx[F.S];
     for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
@@ -282,10 +297,9 @@ __global__ void __launch_bounds__(128) k_p1_initial(lt_frame F, Grid g, float dm
         }
         const int c = a, t = e - pf[c];
         const int64_t slot = pl.base[s] + pl.off[(int64_t)s * NF + c] + t;
-        const int node = F.forest[8 * c];
         const PointRec P = load_rec(pts, F.m, F.slice_off[s] + st.rows[slot]);
-        const PointRec L = load_rec(vpls, F.n, F.tree.rep[node]);
-        const float v = entry_value(P, L, node_scale(F.tree, vpls, F.n, node), dmin2, g);
+        const PointRec L = {nrec[4 * c], nrec[4 * c + 1], nrec[4 * c + 2]};
+        const float v = entry_value(P, L, nrec[4 * c + 3].x, dmin2, g);
         if (!isfinite(v)) latch(status, LT_ENUMERIC);  // a non-finite input (flux, albedo, position)
         st.v0[slot] = v;
     }
@@ -418,8 +432,16 @@ __device__ __forceinline__ bool load_pair(const lt_frame& F, const P1Plan& pl, c
                                           PairCtx& pc) {
     const int l0 = F.level_off[h], np = F.level_off[h + 1] - l0;
     const int NF = 2 * F.C - 1;
-    pc.s = (int)(t / np);
-    pc.f = F.level_nodes[l0 + (int)(t % np)];
+    // (a frame has fewer than 2^32 pairs a level: S <= 1024 where the completions take it, C <= 16384;
+    // larger S goes the long way)
+    if (t <= 0xffffffffll) {
+        const uint32_t q = (uint32_t)t / (uint32_t)np;
+        pc.s = (int)q;
+        pc.f = F.level_nodes[l0 + (int)((uint32_t)t - q * (uint32_t)np)];
+    } else {
+        pc.s = (int)(t / np);
+        pc.f = F.level_nodes[l0 + (int)(t % np)];
+    }
     pc.a = F.forest[8 * pc.f + 1];
     pc.b = F.forest[8 * pc.f + 2];
     const int32_t* state = pl.state + (int64_t)pc.s * NF;
@@ -439,16 +461,18 @@ __device__ __forceinline__ bool load_pair(const lt_frame& F, const P1Plan& pl, c
 }
 
 // -- one level: pairs of a group of lanes
-constexpr int kSmallPair = 32;   // rows of both children: 8 lanes, at most 4 rows a lane
+// (64x64 frame / sampling of the 512x512 scene, ms: small pairs up to 8 rows 0.95 / 4.64,
+// 16: 0.96 / 4.64, 32: 1.00 / 4.77, 64: 1.02 / 5.0; warp pairs up to 128 rows 5% slower on the
+// latter than 256, 512 2%)
+constexpr int kSmallPair = 16;   // rows of both children: 8 lanes, at most 2 rows a lane
 constexpr int kMidPair = 256;    // a warp, at most 8 rows a lane
 constexpr int kGroup = 8;
 
-__device__ __forceinline__ float pair_entry(const lt_frame& F, const Grid& g, float dmin2, int row, int node,
+__device__ __forceinline__ float pair_entry(const lt_frame& F, const Grid& g, float dmin2, int row, const float4* rec,
                                             int32_t* status) {
-    const float4* vpls = reinterpret_cast<const float4*>(F.vpls);
     const PointRec P = load_rec(reinterpret_cast<const float4*>(F.pts), F.m, row);
-    const PointRec L = load_rec(vpls, F.n, F.tree.rep[node]);
-    const float v = entry_value(P, L, node_scale(F.tree, vpls, F.n, node), dmin2, g);
+    const PointRec L = {rec[0], rec[1], rec[2]};
+    const float v = entry_value(P, L, rec[3].x, dmin2, g);
     if (!isfinite(v)) latch(status, LT_ENUMERIC);
     return v;
 }
@@ -456,17 +480,14 @@ __device__ __forceinline__ float pair_entry(const lt_frame& F, const Grid& g, fl
 // The ratios of a pair (Sec. 4): q is estimated from p, the child whose representative
 // the parent takes.
 struct PairRatio {
-    int ta, tb;
     bool p_is_a;
     float rq;   // I_q / I_p
     float rfp;  // I_f / I_p
 };
 
-__device__ __forceinline__ PairRatio pair_ratio(const lt_frame& F, const PairCtx& pc) {
+__device__ __forceinline__ PairRatio pair_ratio(const float4* __restrict__ nrec, const PairCtx& pc) {
     PairRatio r;
-    r.ta = F.forest[8 * pc.a];
-    r.tb = F.forest[8 * pc.b];
-    const float Ia = F.tree.I[r.ta], Ib = F.tree.I[r.tb], If = F.tree.I[F.forest[8 * pc.f]];
+    const float Ia = nrec[4 * pc.a + 3].y, Ib = nrec[4 * pc.b + 3].y, If = nrec[4 * pc.f + 3].y;
     r.p_is_a = Ia >= Ib;
     r.rq = r.p_is_a ? __fdiv_rn(Ib, Ia) : __fdiv_rn(Ia, Ib);
     r.rfp = __fdiv_rn(If, r.p_is_a ? Ia : Ib);
@@ -500,10 +521,11 @@ __device__ __forceinline__ PairRow pair_row(const int32_t* A, int na, const int3
 // Values of a row for both children (the missing one evaluated), stored at `slot`;
 // returns |V_q - V_p I_q / I_p|.
 __device__ __forceinline__ float pair_put(const lt_frame& F, const Grid& g, float dmin2, const P1Store& st,
-                                          const PairCtx& pc, const PairRatio& pr, const PairRow& r, int t, int slot,
-                                          int32_t* status) {
+                                          const PairCtx& pc, const PairRatio& pr, const float4* rec_a,
+                                          const float4* rec_b, const PairRow& r, int t, int slot, int32_t* status) {
     const float own = st.v0[r.in_a ? pc.ia + t : pc.ib + (t - pc.na)];
-    const float oth = r.both ? st.v0[pc.ib + r.p] : pair_entry(F, g, dmin2, pc.row0 + r.x, r.in_a ? pr.tb : pr.ta, status);
+    const float oth = r.both ? st.v0[pc.ib + r.p]
+                             : pair_entry(F, g, dmin2, pc.row0 + r.x, r.in_a ? rec_b : rec_a, status);
     const float va = r.in_a ? own : oth, vb = r.in_a ? oth : own;
     st.rows[pc.iff + slot] = r.x;
     st.v0[pc.iff + slot] = va;
@@ -547,14 +569,14 @@ __device__ __forceinline__ void decide_pair(const lt_frame& F, const P1Plan& pl,
 // shadow rays run side by side.
 template <int G>
 __device__ __forceinline__ void group_pair(const lt_frame& F, const Grid& g, float dmin2, const P1Plan& pl,
-                                           const P1Store& st, const float* thr, const PairCtx& pc, bool live,
+                                           const P1Store& st, const P1Work& w, const PairCtx& pc, bool live,
                                            int32_t* status) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, gl = lane & (G - 1), sh = lane & ~(G - 1);
     const unsigned gm = G == 32 ? FULL : (1u << G) - 1u, lt = (1u << gl) - 1u;
     const int na = live ? pc.na : 0, nb = live ? pc.nb : 0;
     PairRatio pr{};
-    if (live) pr = pair_ratio(F, pc);
+    if (live) pr = pair_ratio(w.nrec, pc);
     const int trips = (__reduce_max_sync(FULL, na + nb) + G - 1) / G;
     int ca = 0, cb = 0;  // rows of a (of b) so far that both children hold
     float e = 0.f;
@@ -565,7 +587,7 @@ __device__ __forceinline__ void group_pair(const lt_frame& F, const Grid& g, flo
         const unsigned mb = (__ballot_sync(FULL, r.in_b && r.both) >> sh) & gm;
         if (r.in_a || (r.in_b && !r.both)) {
             const int slot = r.in_a ? t + r.p - (ca + __popc(ma & lt)) : t - na + r.p - (cb + __popc(mb & lt));
-            e = fmaxf(e, pair_put(F, g, dmin2, st, pc, pr, r, t, slot, status));
+            e = fmaxf(e, pair_put(F, g, dmin2, st, pc, pr, w.nrec + 4 * pc.a, w.nrec + 4 * pc.b, r, t, slot, status));
         }
         ca += __popc(ma);
         cb += __popc(mb);
@@ -573,7 +595,7 @@ __device__ __forceinline__ void group_pair(const lt_frame& F, const Grid& g, flo
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) e = fmaxf(e, __shfl_xor_sync(FULL, e, o));
     __syncwarp();  // the group's stores are visible to the group
-    if (live) decide_pair(F, pl, st, thr, pc, pr, na + nb - ca, e, gl, G, gl == 0);
+    if (live) decide_pair(F, pl, st, w.thr, pc, pr, na + nb - ca, e, gl, G, gl == 0);
 }
 
 // step 1: the pairs of at most kSmallPair rows, 8 lanes each; the others are listed
@@ -604,14 +626,15 @@ __device__ __forceinline__ void p1_small_body(const lt_frame& F, const Grid& g, 
                 else latch(status, LT_ELIMIT);
             }
         }
-        group_pair<kGroup>(F, g, dmin2, pl, st, w.thr, pc, active && rows <= kSmallPair, status);
+        group_pair<kGroup>(F, g, dmin2, pl, st, w, pc, active && rows <= kSmallPair, status);
     }
 }
 
 // step 2: the listed pairs.  A CTA per pair of more than kMidPair rows (both row lists
 // staged in shared memory when they fit), then a warp per pair; where a level has few
 // pairs (at most kFewPairs per CTA), a CTA each for those too: with a warp, a level waits
-// for eight shadow rays one after the other.
+// for eight shadow rays one after the other.  (64x64 frame 1.08 ms with kFewPairs 0, 1.01
+// with 4, 1.02 with 16.)
 constexpr int kBigStage = 4096;
 constexpr int kFewPairs = 4;
 
@@ -620,15 +643,24 @@ __device__ __forceinline__ void p1_rest_body(const lt_frame& F, const Grid& g, f
     __shared__ int32_t sa[kBigStage], sb[kBigStage];
     __shared__ int32_t ws[32];
     __shared__ float red[32];
+    // the CTA's pair: in shared memory, the registers are for the rays
+    __shared__ PairCtx pc;
+    __shared__ PairRatio pr;
+    __shared__ float4 rec[8];
+    __shared__ int s_live;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int64_t nbig = min(w.bcount[h], w.bcap), nmid = min(w.mcount[h], w.bcap);
     const bool few = nmid <= (int64_t)kFewPairs * gridDim.x;
     for (int64_t q = blockIdx.x; q < nbig + (few ? nmid : 0); q += gridDim.x) {
-        PairCtx pc;
-        if (!load_pair(F, pl, st, h, q < nbig ? w.big[q] : w.mid[q - nbig], pc)) continue;  // uniform in the block
-        const PairRatio pr = pair_ratio(F, pc);
+        __syncthreads();  // the previous pair is done with the shared state
+        if (threadIdx.x == 0) {
+            s_live = load_pair(F, pl, st, h, q < nbig ? w.big[q] : w.mid[q - nbig], pc);
+            if (s_live) pr = pair_ratio(w.nrec, pc);
+        }
+        __syncthreads();
+        if (!s_live) continue;
         const bool staged = pc.na <= kBigStage && pc.nb <= kBigStage;
-        __syncthreads();  // the previous pair is done with the stage
+        if (threadIdx.x < 8) rec[threadIdx.x] = w.nrec[4 * (threadIdx.x < 4 ? pc.a : pc.b) + (threadIdx.x & 3)];
         if (staged) {
             for (int i = threadIdx.x; i < pc.na; i += blockDim.x) sa[i] = pc.ra[i];
             for (int j = threadIdx.x; j < pc.nb; j += blockDim.x) sb[j] = pc.rb[j];
@@ -645,7 +677,7 @@ __device__ __forceinline__ void p1_rest_body(const lt_frame& F, const Grid& g, f
             const int pre = block_exclusive_scan<int>(r.both ? (r.in_a ? 1 : 1 << 16) : 0, ws, &tot);
             if (r.in_a || (r.in_b && !r.both)) {
                 const int slot = r.in_a ? t + r.p - (ca + (pre & 0xffff)) : t - pc.na + r.p - (cb + (pre >> 16));
-                e = fmaxf(e, pair_put(F, g, dmin2, st, pc, pr, r, t, slot, status));
+                e = fmaxf(e, pair_put(F, g, dmin2, st, pc, pr, rec, rec + 4, r, t, slot, status));
             }
             ca += tot & 0xffff;
             cb += tot >> 16;
@@ -659,9 +691,9 @@ __device__ __forceinline__ void p1_rest_body(const lt_frame& F, const Grid& g, f
     }
     if (few) return;
     for (int64_t q = blockIdx.x * (int64_t)nw + wid; q < nmid; q += (int64_t)gridDim.x * nw) {
-        PairCtx pc;
-        if (!load_pair(F, pl, st, h, w.mid[q], pc)) continue;  // uniform in the warp
-        group_pair<32>(F, g, dmin2, pl, st, w.thr, pc, true, status);
+        PairCtx wpc;
+        if (!load_pair(F, pl, st, h, w.mid[q], wpc)) continue;  // uniform in the warp
+        group_pair<32>(F, g, dmin2, pl, st, w, wpc, true, status);
     }
 }
 
@@ -1294,7 +1326,7 @@ lt_status sample_pass1(lt_ctx* ctx, const lt_frame* f, float rate1, float tau, i
     const size_t store_bytes = (size_t)std::max<int64_t>(acc, 1) * (target > 0 ? 16 : 12) + 1024;
     const size_t eff_bytes = target > 0 ? (size_t)S * NF * 4 : 0;
     const size_t work_bytes = (size_t)(S + 1) * 8 + (size_t)S * C * 4 + (size_t)S * 4 + (size_t)Hn * 16 +
-                              (size_t)bcap * 16 + eff_bytes + 17 * 256;
+                              (size_t)bcap * 16 + (size_t)NF * 64 + eff_bytes + 18 * 256;
     char* q = (char*)lt_scratch(ctx, SCR_P1_STORE, store_bytes + work_bytes, &st);
     if (!q) return st;
     P1Store store;
@@ -1315,6 +1347,7 @@ lt_status sample_pass1(lt_ctx* ctx, const lt_frame* f, float rate1, float tau, i
     w.thr = (float*)wtake((size_t)S * 4);
     w.mcount = (int64_t*)wtake((size_t)Hn * 8 + 8);
     w.bcount = (int64_t*)wtake((size_t)Hn * 8);
+    w.nrec = (float4*)wtake((size_t)NF * 64);
     w.mid = (int64_t*)wtake((size_t)bcap * 8);
     w.big = (int64_t*)wtake((size_t)bcap * 8);
     w.bar = (unsigned*)(w.mcount + Hn);  // shares the zeroing of the level counters
@@ -1332,10 +1365,12 @@ lt_status sample_pass1(lt_ctx* ctx, const lt_frame* f, float rate1, float tau, i
     k_p1_draws<<<grid_for((int64_t)S * NF, 256), 256, 0, ctx->stream>>>(*f, seed_ref(ctx, seed), pl, store,
                                                                         ctx->d_status);
     LT_LAUNCH_CHECK(ctx, "k_p1_draws");
+    k_p1_nodes<<<(NF + 255) / 256, 256, 0, ctx->stream>>>(*f, w.nrec);
+    LT_LAUNCH_CHECK(ctx, "k_p1_nodes");
     k_p1_kpfx<<<1, 1024, 0, ctx->stream>>>(*f, pl, w.kpfx);
     LT_LAUNCH_CHECK(ctx, "k_p1_kpfx");
     const int ray_grid = ctx->tune.ray_ctas_per_sm * nsm;
-    k_p1_initial<<<ray_grid, 128, 0, ctx->stream>>>(*f, ctx->grid, dmin2, pl, store, w.kpfx, ctx->d_status);
+    k_p1_initial<<<ray_grid, 128, 0, ctx->stream>>>(*f, ctx->grid, dmin2, pl, store, w.kpfx, w.nrec, ctx->d_status);
     LT_LAUNCH_CHECK(ctx, "k_p1_initial");
     k_p1_leafmean<<<grid_for((int64_t)S * C, 256), 256, 0, ctx->stream>>>(*f, pl, store, w.leafmean);
     LT_LAUNCH_CHECK(ctx, "k_p1_leafmean");

@@ -1,6 +1,6 @@
 """Sizes at which the kernels and their dispatch rules change path.
 
-* shadow rays: 8 boxes (tested one by one) and 9 (grid walk), one and few triangles;
+* shadow rays: 16 boxes (tested one by one) and 17 (grid walk), one and few triangles;
 * brute force: points and lights around the 32-point CTA, the 256-light tile and the
   16-warp rule, against the float64 oracle;
 * sorts around one 4096-key chunk, and the cut errors of small and large cuts;
@@ -53,7 +53,7 @@ def _segments(k, seed):
     return o, e
 
 
-@pytest.mark.parametrize("nb", [1, 7, 8, 9])
+@pytest.mark.parametrize("nb", [1, 8, 16, 17])
 def test_few_boxes(lt, ctx, nb):
     cfg = get_config("room256_vpl16k_200box", n_small_boxes=nb, width=8, height=8, n_vpl=8)
     boxes = make_scene(cfg).boxes
@@ -63,7 +63,7 @@ def test_few_boxes(lt, ctx, nb):
     exp = shading.segment_blocked(o.astype(np.float64), e.astype(np.float64), boxes)
     assert np.mean(got != exp) <= 1e-4
     # the other path on the same boxes: copies of the first box change no answer
-    n = 8 if nb > 8 else 9
+    n = 17
     if n > nb:
         lt.lt_scene_upload(ctx, _cuda(np.concatenate([boxes, np.repeat(boxes[:1], n - nb, 0)])))
         again = lt.lt_shadow_test(ctx, _cuda(o), _cuda(e)).cpu().numpy().astype(bool)
