@@ -456,7 +456,9 @@ __global__ void k_als_init(lt_frame F, lt_samples smp, Omega om, int R, const in
 // are taken 32 at a time: eight lanes copy one factor row (128 contiguous bytes, so a
 // copy instruction touches 4 lines and not 32) into the warp's stage, 16-byte chunk c
 // of row q at chunk c ^ (q & 7), and the next 32 rows are on their way (cp.async)
-// while these are added.  Rows have stride R; components at or beyond R are zero.
+// while these are added.  Rows have stride R; components at or beyond the rank are zero.  RB = 3 (ranks
+// up to 24) or 4: only the first 8 RB components are copied, added and solved for; lanes
+// past them idle.
 constexpr int kWarpStage = 32 * 32;    // floats of one stage: 32 rows of 32
 constexpr int kWarpCol = 36;           // stride of a column of L (16-byte aligned)
 
@@ -467,13 +469,14 @@ __device__ __forceinline__ void copy16(float* dst, const float* src, bool full) 
 }
 
 // starts the copies of rows idx[e0 ..] (at most 32, the rest zero) into st
-__device__ __forceinline__ void stage_entries(int len, int e0, int j, const float* __restrict__ src, int R, bool vec,
-                                              float* st) {
+__device__ __forceinline__ void stage_entries(int len, int e0, int j, const float* __restrict__ src, int R, int rmax,
+                                              bool vec, float* st) {
     const int lane = threadIdx.x & 31, c = lane & 7;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const int q = 4 * i + (lane >> 3);
         const int jq = __shfl_sync(0xffffffffu, j, q);
+        if (4 * c >= rmax) continue;
         const bool live = e0 + q < len && 4 * c < R;
         const float* p = src + (live ? (int64_t)jq * R + 4 * c : 0);
         float* d = st + q * 32 + 4 * (c ^ (q & 7));
@@ -487,20 +490,22 @@ __device__ __forceinline__ void stage_entries(int len, int e0, int j, const floa
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
+template <int RB>
 __device__ __forceinline__ void gram_warp(int len, const uint16_t* __restrict__ idx, const float* __restrict__ val,
-                                          const float* __restrict__ src, int R, float* st0, float (&g)[32], float& b) {
+                                          const float* __restrict__ src, int R, float* st0, float (&g)[8 * RB],
+                                          float& b) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const bool vec = (R & 3) == 0 && ((uintptr_t)src & 15) == 0;
-    F32x2 g2[16];
+    F32x2 g2[4 * RB];
 #pragma unroll
-    for (int c = 0; c < 16; ++c) g2[c] = 0ull;
+    for (int c = 0; c < 4 * RB; ++c) g2[c] = 0ull;
     b = 0.f;
-    const int kc = lane >> 2, kw = lane & 3;
+    const int kc = min(lane, 8 * RB - 1) >> 2, kw = lane & 3;
     int j = lane < len ? (int)idx[lane] : 0;
     float av = lane < len ? val[lane] : 0.f;
     __syncwarp();  // the stage is free
-    if (len > 0) stage_entries(len, 0, j, src, R, vec, st0);
+    if (len > 0) stage_entries(len, 0, j, src, R, 8 * RB, vec, st0);
     for (int e0 = 0, h = 0; e0 < len; e0 += 32, h ^= 1) {
         const float a_now = av;
         const float* st = st0 + h * kWarpStage;
@@ -508,7 +513,7 @@ __device__ __forceinline__ void gram_warp(int len, const uint16_t* __restrict__ 
             const int e = e0 + 32 + lane;
             j = e < len ? (int)idx[e] : 0;
             av = e < len ? val[e] : 0.f;
-            stage_entries(len, e0 + 32, j, src, R, vec, st0 + (h ^ 1) * kWarpStage);
+            stage_entries(len, e0 + 32, j, src, R, 8 * RB, vec, st0 + (h ^ 1) * kWarpStage);
             asm volatile("cp.async.wait_group 1;" ::: "memory");
         } else {
             asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -522,7 +527,7 @@ __device__ __forceinline__ void gram_warp(int len, const uint16_t* __restrict__ 
             const F32x2 xx = pack2(xk, xk);
             b = fmaf(a, xk, b);
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
+            for (int c = 0; c < 2 * RB; ++c) {
                 const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(st + q * 32 + 4 * (c ^ (q & 7)));
                 g2[2 * c] = fma2(xx, u.x, g2[2 * c]);
                 g2[2 * c + 1] = fma2(xx, u.y, g2[2 * c + 1]);
@@ -531,20 +536,20 @@ __device__ __forceinline__ void gram_warp(int len, const uint16_t* __restrict__ 
         __syncwarp();  // the stage after next is this one
     }
 #pragma unroll
-    for (int c = 0; c < 16; ++c) unpack2(g2[c], g[2 * c], g[2 * c + 1]);
+    for (int c = 0; c < 4 * RB; ++c) unpack2(g2[c], g[2 * c], g[2 * c + 1]);
 }
 
 // Eight columns (8 P ..) of the Cholesky of a line whose row k lane k holds, and the
 // forward substitution with them.  acc[0] is the current column and the registers move
-// down by one per column, so that one loop body serves the eight (all 32 unrolled are
+// down by one per column, so that one loop body serves the eight (all of them unrolled are
 // more code than the instruction caches hold: 41% of the stall cycles).  A column of L
 // goes through shared memory (one store, then 16-byte broadcast loads, a quarter as many
 // instructions as a shuffle per row) and stays there for the backward substitution.
 // Entries above the diagonal are not used, so every lane updates its whole row.
-template <int P>
-__device__ __forceinline__ void chol_block32(float (&acc)[32], float& y, int k, int r, bool& ok, float& dmin,
+template <int P, int RB>
+__device__ __forceinline__ void chol_block32(float (&acc)[8 * RB], float& y, int k, int r, bool& ok, float& dmin,
                                              float& dmax, float& my_inv, float* Lc) {
-    constexpr int W = 32 - 8 * P;  // columns left at the start of the block
+    constexpr int W = 8 * (RB - P);  // columns left at the start of the block
     const unsigned FULL = 0xffffffffu;
 #pragma unroll 1
     for (int t = 0; t < 8; ++t) {
@@ -581,33 +586,34 @@ __device__ __forceinline__ void chol_block32(float (&acc)[32], float& y, int k, 
 // and b_k in rhs and receives u_k.  Returns false when the float factorisation is not
 // acceptable (a non-positive pivot, or pivots spread by more than 1 / kPivotRatio).
 // Lc: 32 columns of kWarpCol floats.
-__device__ __forceinline__ bool warp_solve32(float (&acc)[32], float rhs, int len, int r, float lam_rel, int k,
+template <int RB>
+__device__ __forceinline__ bool warp_solve32(float (&acc)[8 * RB], float rhs, int len, int r, float lam_rel, int k,
                                              float* out_k, float* Lc) {
     const unsigned FULL = 0xffffffffu;
     float tr = 0.f;
 #pragma unroll
-    for (int c = 0; c < 32; ++c)
+    for (int c = 0; c < 8 * RB; ++c)
         if (c == k) tr = acc[c];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(FULL, tr, o);
     const bool zero = !(tr > 0.f) || len == 0;
     const float lam = lam_rel * tr / (float)r;
 #pragma unroll
-    for (int c = 0; c < 32; ++c) {
+    for (int c = 0; c < 8 * RB; ++c) {
         const float d = (k < r) ? acc[c] + lam : 1.f;
         acc[c] = c == k ? d : (k >= r ? 0.f : acc[c]);
     }
     if (k >= r) rhs = 0.f;
     float dmin = 3.0e38f, dmax = 0.f, inv = 1.f, y = rhs;
     bool ok = true;
-    chol_block32<0>(acc, y, k, r, ok, dmin, dmax, inv, Lc);
-    chol_block32<1>(acc, y, k, r, ok, dmin, dmax, inv, Lc);
-    chol_block32<2>(acc, y, k, r, ok, dmin, dmax, inv, Lc);
-    chol_block32<3>(acc, y, k, r, ok, dmin, dmax, inv, Lc);
+    chol_block32<0, RB>(acc, y, k, r, ok, dmin, dmax, inv, Lc);
+    chol_block32<1, RB>(acc, y, k, r, ok, dmin, dmax, inv, Lc);
+    chol_block32<2, RB>(acc, y, k, r, ok, dmin, dmax, inv, Lc);
+    if constexpr (RB > 3) chol_block32<3, RB>(acc, y, k, r, ok, dmin, dmax, inv, Lc);
     if (!zero && (!ok || dmin < kPivotRatio * dmax)) return false;
     float x = y;  // L^T x = y: lane k reads its column of L (35 k + j: no bank conflicts)
 #pragma unroll 4
-    for (int j = 31; j >= 0; --j) {
+    for (int j = 8 * RB - 1; j >= 0; --j) {
         const float l = Lc[k * (kWarpCol - 1) + j];
         const float xj = __shfl_sync(FULL, x * inv, j);
         if (k == j) x = xj;
@@ -701,6 +707,15 @@ __device__ __forceinline__ void factor_solve_rows(T (&acc)[G], T rhs, int len, i
     *out_k = (zero || k >= r) ? T(0) : x;
 }
 
+template <int RB>
+__device__ __forceinline__ bool warp_line(int len, const uint16_t* __restrict__ idx, const float* __restrict__ val,
+                                          const float* __restrict__ src, int R, int r, float lam_rel, float* st,
+                                          float* x) {
+    float g[8 * RB], b;
+    gram_warp<RB>(len, idx, val, src, R, st, g, b);
+    return warp_solve32<RB>(g, b, len, r, lam_rel, threadIdx.x & 31, x, st);
+}
+
 // One half-step for ranks above 16: rows of U (rows_side) or columns of V, a warp per
 // line.  A persistent grid: warps take the frame's lines in order, two at a time, from
 // a counter (lines of one slice run side by side and share its factor rows in L1), so
@@ -710,7 +725,8 @@ __device__ __forceinline__ void factor_solve_rows(T (&acc)[G], T rhs, int len, i
 // and the latency of the 32 dependent columns of the solve.  Completion of the 200-box
 // scene (5.7 M entries, ranks 8 to 32 per slice, 10 sweeps; the lane-group kernel has the
 // slices up to rank 16): 23.9 ms with a lane per factor row in the copies, a shuffle
-// per element in the Cholesky and 32-way bank conflicts in the solves; 14.1 ms so.
+// per element in the Cholesky and 32-way bank conflicts in the solves; 14.1 ms so, 12.6
+// with the components past rank 24 left out where they are zero.
 constexpr int kHalfWarps = 8;
 constexpr int kHalfSmem = kHalfWarps * 2 * kWarpStage * 4;  // the columns of L use the stage after the Gram
 static_assert(32 * kWarpCol <= 2 * kWarpStage, "the columns of L fit the stage");
@@ -753,10 +769,11 @@ __global__ void __launch_bounds__(32 * kHalfWarps, 2) k_als_half(lt_frame F, lt_
             const int32_t* ptr = rows_side ? om.rp + row0 + s : om.cp + (int64_t)s * (F.C + 1);
             const int b0 = ptr[line], len = ptr[line + 1] - b0;
             const int64_t dst = rows_side ? (int64_t)(row0 + line) * R : ((int64_t)s * F.C + line) * R;
-            float g[32], b, x = 0.f;
-            gram_warp(len, (rows_side ? om.cidx : om.ridx) + o + b0, (rows_side ? om.cval : om.rval) + o + b0, src, R,
-                      st, g, b);
-            const bool ok = warp_solve32(g, b, len, r, lam_rel, k, &x, st);
+            const uint16_t* idx = (rows_side ? om.cidx : om.ridx) + o + b0;
+            const float* val = (rows_side ? om.cval : om.rval) + o + b0;
+            float x = 0.f;
+            const bool ok = r <= 24 ? warp_line<3>(len, idx, val, src, R, r, lam_rel, st, &x)
+                                    : warp_line<4>(len, idx, val, src, R, r, lam_rel, st, &x);
             if (k < R) Fout[dst + k] = (ok && k < r) ? x : 0.f;
             if (!ok && k == 0) {
                 // rare: the float pivots were not acceptable; k_als_retry forms the line's
