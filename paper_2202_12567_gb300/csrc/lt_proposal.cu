@@ -420,10 +420,8 @@ __global__ void k_feat_slice(lt_frame F, lt_samples smp, float* __restrict__ st)
     const float4* P0 = reinterpret_cast<const float4*>(F.pts);
     const float4* P1 = P0 + F.m;
     float acc[13];
-    for (int k = 0; k < 6; ++k) acc[k] = 0.f;
-    for (int k = 6; k < 9; ++k) acc[k] = 3.0e38f;
-    for (int k = 9; k < 12; ++k) acc[k] = -3.0e38f;
-    acc[12] = 0.f;
+#pragma unroll
+    for (int k = 0; k < 13; ++k) acc[k] = k < 6 || k == 12 ? 0.f : k < 9 ? 3.0e38f : -3.0e38f;
 #pragma unroll 4
     for (int i = threadIdx.x; i < ms; i += blockDim.x) {
         const float4 p = P0[row0 + i], nn = P1[row0 + i];
@@ -445,7 +443,8 @@ __global__ void k_feat_slice(lt_frame F, lt_samples smp, float* __restrict__ st)
 #pragma unroll 16
     for (int e = threadIdx.x; e < n1; e += blockDim.x) acc[12] += val[e];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int k = 0; k < 13; ++k) {
+#pragma unroll
+    for (int k = 0; k < 13; ++k) {  // (unrolled: acc must not live in local memory)
         float v = acc[k];
         v = (k >= 6 && k < 9) ? warp_min(v) : (k >= 9 && k < 12) ? warp_max(v) : warp_sum(v);
         if (lane == 0) red[k][w] = v;
@@ -482,11 +481,16 @@ __global__ void k_group_prefix(const int32_t* __restrict__ ncol, int S, int32_t*
 }
 
 // first pass-1 entry of the slice (keys grouped by column, ascending) whose column >= j
+// by one warp: 32 probes a step (a binary search is a chain of 15 loads)
 __device__ __forceinline__ int first_col_at_least(const uint32_t* key, int n1, int j) {
-    int a = 0, b = n1;
+    const int lane = threadIdx.x & 31;
+    int a = 0, b = n1;  // the answer is in [a, b]
     while (a < b) {
-        const int m = (a + b) >> 1;
-        if ((int)(key[m] & 0xffffu) < j) a = m + 1; else b = m;
+        const int step = (b - a + 31) / 32, p = a + step * (lane + 1) - 1;
+        const int c = __popc(__ballot_sync(0xffffffffu, p < b && (int)(key[p] & 0xffffu) < j));
+        a += c * step;  // the probes below are a prefix
+        b = min(b, a + step - 1);
+        if (a > b) a = b;
     }
     return a;
 }
@@ -620,7 +624,10 @@ __global__ void __launch_bounds__(128) k_slice_matrix(lt_frame F, lt_samples smp
     }
 }
 
-// G_s = M_s^T M_s (n' x n', float) at G + goff2[s] with goff2 the prefix of n'^2
+// G_s = M_s^T M_s (n' rows of gram_ld(n') floats, so that every row starts on 16 bytes) at
+// G + goff2[s], goff2 the prefix of their sizes
+__host__ __device__ __forceinline__ int gram_ld(int n) { return (n + 3) & ~3; }
+
 constexpr int kGramTile = 128;
 constexpr int kGramStep = 16;
 
@@ -632,7 +639,7 @@ __global__ void k_goff(lt_samples smp, int S, int64_t* __restrict__ goff2, int64
         const int s = c0 + threadIdx.x;
         const int64_t n = s < S ? smp.ncol[s] : 0, t = (n + kGramTile - 1) / kGramTile;
         int64_t tot;
-        int64_t pre = block_exclusive_scan<int64_t>(n * n, ws, &tot);
+        int64_t pre = block_exclusive_scan<int64_t>(n * gram_ld((int)n), ws, &tot);
         if (s < S) goff2[s] = carry + pre;
         carry += tot;
         pre = block_exclusive_scan<int64_t>(t * (t + 1) / 2, ws, &tot);
@@ -711,14 +718,15 @@ __global__ void __launch_bounds__(256, 2) k_gram(lt_frame F, lt_samples smp, con
             }
         }
         float* Gs = G + goff2[s];
+        const int ld = gram_ld(ns);
 #pragma unroll
         for (int u = 0; u < 8; ++u)
 #pragma unroll
             for (int v = 0; v < 8; ++v) {
                 const int i = ti + (u >> 2) * 64 + 4 * ty + (u & 3), j = tj + (v >> 2) * 64 + 4 * tx + (v & 3);
                 if (i < ns && j < ns) {
-                    Gs[(int64_t)i * ns + j] = acc[u][v];
-                    if (ti != tj) Gs[(int64_t)j * ns + i] = acc[u][v];
+                    Gs[(int64_t)i * ld + j] = acc[u][v];
+                    if (ti != tj) Gs[(int64_t)j * ld + i] = acc[u][v];
                 }
             }
     }
@@ -903,60 +911,86 @@ __global__ void __launch_bounds__(kLevThreads) k_lev_mgs(lt_samples smp, const i
     for (int c = threadIdx.x; c < ns; c += blockDim.x) target[goff[s] + c] = Y[c] / tot;
 }
 
-// Y = G Q of every slice, a thread per row of G and 16 columns of Q at a time: row i of
-// G is read as column i (G is symmetric to the bit), so that a warp's loads are one line, the
-// rows of Q are broadcast from shared memory.  Sums over j in order.
-constexpr int kLevRows = 64, kLevTile = 64;
+// Y = G Q of every slice, a thread per row of G and 16 columns of Q at a time.  Row i of G
+// is read as column i (G is symmetric to the bit): the CTA's 128 columns of 16 rows at a
+// time go through a ring of kLevStages tiles in shared memory (cp.async, 16 bytes), the rows
+// of Q beside them.  Sums over j in order.  Bound by the memory system: G (115 MB on the
+// workload named above) is read every round, and a load per row of G in registers, 16
+// rows ahead, kept too few bytes on their way (0.13 ms a round).
+constexpr int kLevRows = 128, kLevTile = 16, kLevStages = 6;
+
+struct LevStage {
+    float g[kLevTile][kLevRows];
+    float q[kLevTile][16];
+};
 
 __global__ void __launch_bounds__(kLevRows) k_lev_mult(lt_samples smp, int S, int C, const float* __restrict__ G,
                                                        const int64_t* __restrict__ goff2, int64_t gcap, int r,
                                                        const float* __restrict__ Qall, float* __restrict__ Yall) {
-    __shared__ __align__(16) float sq[kLevTile][16];
+    extern __shared__ __align__(16) unsigned char lev_raw[];
+    LevStage* ring = reinterpret_cast<LevStage*>(lev_raw);
     if (goff2[S] > gcap) return;
     const int s = blockIdx.y;
     const int ns = smp.ncol[s];
-    const int rr = min(r, ns), blocks = (ns + kLevRows - 1) / kLevRows, parts = (rr + 15) / 16;
+    const int rr = min(r, ns), ld = gram_ld(ns), blocks = (ns + kLevRows - 1) / kLevRows, parts = (rr + 15) / 16;
+    const int steps = (ns + kLevTile - 1) / kLevTile;
+    const float* Gs = G + goff2[s];
     const float* Q = Qall + (int64_t)s * C * r;
     float* Y = Yall + (int64_t)s * C * r;
     for (int b = blockIdx.x; b < blocks * parts; b += gridDim.x) {
-        const int i = (b % blocks) * kLevRows + threadIdx.x, k0 = (b / blocks) * 16;
-        const float* Gi = G + goff2[s] + min(i, ns - 1);
+        const int i0 = (b % blocks) * kLevRows, k0 = (b / blocks) * 16;
+        // tile t: rows 16 t .. of G, columns i0 .. (zeros past the last row and past column ld)
+        auto fill = [&](int t) {
+            if (t < steps) {
+                LevStage& st = ring[t % kLevStages];
+                const int j0 = t * kLevTile;
+#pragma unroll
+                for (int e = threadIdx.x; e < kLevTile * (kLevRows / 4); e += kLevRows) {
+                    const int j = e / (kLevRows / 4), c = 4 * (e % (kLevRows / 4));
+                    const bool live = j0 + j < ns && i0 + c < ld;
+                    const float* p = live ? Gs + (int64_t)(j0 + j) * ld + i0 + c : Gs;
+                    const unsigned d = (unsigned)__cvta_generic_to_shared(&st.g[j][c]);
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(p), "r"(live ? 16 : 0)
+                                 : "memory");
+                }
+#pragma unroll
+                for (int e = threadIdx.x; e < kLevTile * 16; e += kLevRows) {
+                    const int j = e >> 4, k = e & 15;
+                    const bool live = j0 + j < ns && k0 + k < rr;
+                    const float* p = live ? Q + (int64_t)(j0 + j) * rr + k0 + k : Q;
+                    const unsigned d = (unsigned)__cvta_generic_to_shared(&st.q[j][k]);
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(p), "r"(live ? 4 : 0)
+                                 : "memory");
+                }
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
         float a[16];
 #pragma unroll
         for (int k = 0; k < 16; ++k) a[k] = 0.f;
-        float g[16], gn[16];
-        auto fetch = [&](int j) {
-            if (j >= ns) return;
-#pragma unroll
-            for (int u = 0; u < 16; ++u) gn[u] = __ldg(Gi + (int64_t)min(j + u, ns - 1) * ns);
-        };
-        fetch(0);
-        for (int j0 = 0; j0 < ns; j0 += kLevTile) {
-            __syncthreads();
-            for (int e = threadIdx.x; e < kLevTile * 16; e += kLevRows) {
-                const int j = j0 + (e >> 4), k = k0 + (e & 15);
-                sq[e >> 4][e & 15] = (j < ns && k < rr) ? Q[(int64_t)j * rr + k] : 0.f;
-            }
-            __syncthreads();
-            // 16 rows' loads in flight, the next 16 issued before these are added; rows past the
-            // last are the last one again, against zeros of Q
 #pragma unroll 1
-            for (int jj = 0; jj < kLevTile; jj += 16) {
-                if (j0 + jj >= ns) break;
+        for (int t = 0; t < kLevStages - 1; ++t) fill(t);
+        for (int t = 0; t < steps; ++t) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(kLevStages - 2) : "memory");
+            __syncthreads();  // tile t is here for every thread, tile t - 1 has been read
+            fill(t + kLevStages - 1);
+            const LevStage& st = ring[t % kLevStages];
 #pragma unroll
-                for (int u = 0; u < 16; ++u) g[u] = gn[u];
-                fetch(j0 + jj + 16);
+            for (int j = 0; j < kLevTile; ++j) {
+                const float g = st.g[j][threadIdx.x];
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
-                    float x[16];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        *reinterpret_cast<float4*>(x + 4 * k) = *reinterpret_cast<const float4*>(&sq[jj + u][4 * k]);
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) a[k] = fmaf(g[u], x[k], a[k]);
+                for (int k = 0; k < 4; ++k) {
+                    const float4 x = *reinterpret_cast<const float4*>(&st.q[j][4 * k]);
+                    a[4 * k] = fmaf(g, x.x, a[4 * k]);
+                    a[4 * k + 1] = fmaf(g, x.y, a[4 * k + 1]);
+                    a[4 * k + 2] = fmaf(g, x.z, a[4 * k + 2]);
+                    a[4 * k + 3] = fmaf(g, x.w, a[4 * k + 3]);
                 }
             }
         }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();  // the ring is free for the next block
+        const int i = i0 + threadIdx.x;
         if (i < ns) {
 #pragma unroll
             for (int k = 0; k < 16; ++k)
@@ -1037,7 +1071,7 @@ extern "C" lt_status lt_leverage_targets(lt_ctx* ctx, const lt_frame* f, const l
     // Gram capacity: sum of n'^2 <= S * min(C, 4096)^2 floats is bounded by the
     // largest coarsened cut the slices can have; slices beyond it are skipped
     const int64_t nmax = std::min<int64_t>(C, 4096);
-    const int64_t gcap = (int64_t)S * nmax * nmax;
+    const int64_t gcap = (int64_t)S * nmax * gram_ld((int)nmax);
     lt_status st;
     char* p = (char*)lt_scratch(ctx, SCR_PROPOSAL_T,
                                 (size_t)gcap * 4 + (size_t)2 * S * C * r * 4 + (size_t)(S + 1) * 16 + 4 * 256, &st);
@@ -1052,13 +1086,15 @@ extern "C" lt_status lt_leverage_targets(lt_ctx* ctx, const lt_frame* f, const l
     k_gram<<<2 * ctx->num_sms, 256, 0, ctx->stream>>>(*f, *smp, M, moff, goff2, tpfx, gcap, G);
     LT_LAUNCH_CHECK(ctx, "k_gram");
     // Q of a round is the product of the round before: the two buffers change roles
-    const unsigned rows = (unsigned)std::max(1, std::min((C + kLevRows - 1) / kLevRows, 12 * ctx->num_sms / S));
+    const unsigned rows = (unsigned)std::max(1, std::min((C + kLevRows - 1) / kLevRows, 8 * ctx->num_sms / S));
+    const size_t shm = kLevStages * sizeof(LevStage);
+    LT_CUDA(ctx, cudaFuncSetAttribute(k_lev_mult, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
     for (int it = 0; it <= iters; ++it) {
         k_lev_mgs<<<S, kLevThreads, 0, ctx->stream>>>(*smp, f->slice_id, S, C, goff2, gcap, r, it == 0, it == iters, seed,
                                                       Q, Y, group_off, target);
         LT_LAUNCH_CHECK(ctx, "k_lev_mgs");
         if (it < iters) {
-            k_lev_mult<<<dim3(rows, S), kLevRows, 0, ctx->stream>>>(*smp, S, C, G, goff2, gcap, r, Q, Y);
+            k_lev_mult<<<dim3(rows, S), kLevRows, shm, ctx->stream>>>(*smp, S, C, G, goff2, gcap, r, Q, Y);
             LT_LAUNCH_CHECK(ctx, "k_lev_mult");
             std::swap(Q, Y);
         }
