@@ -911,12 +911,14 @@ __global__ void __launch_bounds__(kLevThreads) k_lev_mgs(lt_samples smp, const i
     for (int c = threadIdx.x; c < ns; c += blockDim.x) target[goff[s] + c] = Y[c] / tot;
 }
 
-// Y = G Q of every slice, a thread per row of G and 16 columns of Q at a time.  Row i of G
-// is read as column i (G is symmetric to the bit): the CTA's 128 columns of 16 rows at a
-// time go through a ring of kLevStages tiles in shared memory (cp.async, 16 bytes), the rows
-// of Q beside them.  Sums over j in order.  Bound by the memory system: G (115 MB on the
-// workload named above) is read every round, and a load per row of G in registers, 16
-// rows ahead, kept too few bytes on their way (0.13 ms a round).
+// Y = G Q of every slice, 128 rows of G and 16 columns of Q by a CTA, 4 x 4 outputs by a
+// thread.  Row i of G is read as column i (G is symmetric to the bit): the CTA's 128 columns
+// of 16 rows at a time go through a ring of kLevStages tiles in shared memory (cp.async, 16
+// bytes), the rows of Q beside them.  Sums over j in order.  Bound by what shared memory
+// returns (a 16-byte load of a warp takes four cycles, also where lanes share it): a row and
+// 16 columns a thread read 17 cycles' worth per step, 4 x 4 outputs 8.  Training data of a
+// scene of 65536 points: 6.37 ms with G loaded straight into registers, 5.14 ms from the
+// ring with a row a thread, 4.60 ms with 4 x 4 outputs.
 constexpr int kLevRows = 128, kLevTile = 16, kLevStages = 6;
 
 struct LevStage {
@@ -965,9 +967,13 @@ __global__ void __launch_bounds__(kLevRows) k_lev_mult(lt_samples smp, int S, in
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
-        float a[16];
+        // rows 4 rq .. and columns 4 kq .. of the CTA's 128 x 16
+        const int rq = threadIdx.x >> 2, kq = threadIdx.x & 3;
+        float a[4][4];
 #pragma unroll
-        for (int k = 0; k < 16; ++k) a[k] = 0.f;
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) a[u][k] = 0.f;
 #pragma unroll 1
         for (int t = 0; t < kLevStages - 1; ++t) fill(t);
         for (int t = 0; t < steps; ++t) {
@@ -977,24 +983,23 @@ __global__ void __launch_bounds__(kLevRows) k_lev_mult(lt_samples smp, int S, in
             const LevStage& st = ring[t % kLevStages];
 #pragma unroll
             for (int j = 0; j < kLevTile; ++j) {
-                const float g = st.g[j][threadIdx.x];
+                const float4 g = *reinterpret_cast<const float4*>(&st.g[j][4 * rq]);
+                const float4 x = *reinterpret_cast<const float4*>(&st.q[j][4 * kq]);
+                const float gu[4] = {g.x, g.y, g.z, g.w}, xk[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float4 x = *reinterpret_cast<const float4*>(&st.q[j][4 * k]);
-                    a[4 * k] = fmaf(g, x.x, a[4 * k]);
-                    a[4 * k + 1] = fmaf(g, x.y, a[4 * k + 1]);
-                    a[4 * k + 2] = fmaf(g, x.z, a[4 * k + 2]);
-                    a[4 * k + 3] = fmaf(g, x.w, a[4 * k + 3]);
-                }
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) a[u][k] = fmaf(gu[u], xk[k], a[u][k]);
             }
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncthreads();  // the ring is free for the next block
-        const int i = i0 + threadIdx.x;
-        if (i < ns) {
 #pragma unroll
-            for (int k = 0; k < 16; ++k)
-                if (k0 + k < rr) Y[(int64_t)i * rr + k0 + k] = a[k];
+        for (int u = 0; u < 4; ++u) {
+            const int i = i0 + 4 * rq + u;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (i < ns && k0 + 4 * kq + k < rr) Y[(int64_t)i * rr + k0 + 4 * kq + k] = a[u][k];
         }
     }
 }
