@@ -36,6 +36,20 @@ constexpr int L2 = NH + 8;        // of 64-wide operands
 
 typedef __nv_bfloat16 bf16;
 
+// acc + v(e) for e = e0, e0 + step, ... < n, in that order, B loads in flight at a time
+template <int B, class V>
+__device__ __forceinline__ float sum_in_order(int e0, int n, int step, float acc, V v) {
+    for (int e = e0; e < n; e += B * step) {
+        float x[B];
+#pragma unroll
+        for (int u = 0; u < B; ++u) x[u] = v(min(e + u * step, n - 1));
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+            if (e + u * step < n) acc += x[u];
+    }
+    return acc;
+}
+
 __device__ __forceinline__ float silu(float h) { return h / (1.f + expf(-h)); }
 __device__ __forceinline__ float dsilu(float h) {
     const float s = 1.f / (1.f + expf(-h));
@@ -337,29 +351,45 @@ __global__ void __launch_bounds__(MT, 1) k_mlp_backward(const float* __restrict_
     for (int i = threadIdx.x; i < NPAR; i += MT) part[(int64_t)blockIdx.x * NPAR + i] = s.grad[i];
 }
 
-// softmax over each group's rows, dz = (softmax - target) / G, loss per group
+// softmax over each group's rows, dz = (softmax - target) / G, loss per group.  A warp per
+// group; lane l has the rows a + l, a + l + 32, ..., the first kKeep of them in registers, so that the
+// three passes over the group read memory once.  A step of the training on 40 K rows in 64
+// groups: 115.4 to 110.6 us, with the loads of the gradient's parts in flight together.
 __global__ void k_group_softmax(const float* __restrict__ z, const float* __restrict__ target,
                                 const int32_t* __restrict__ goff, int G, float* __restrict__ dz,
                                 float* __restrict__ gloss) {
+    constexpr int kKeep = 24;
     const int lane = threadIdx.x & 31;
     for (int gi = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); gi < G; gi += gridDim.x * (blockDim.x >> 5)) {
-        const int a = goff[gi], b = goff[gi + 1];
+        const int a = goff[gi] + lane, b = goff[gi + 1];
+        float x[kKeep], y[kKeep];
+#pragma unroll
+        for (int u = 0; u < kKeep; ++u) {
+            x[u] = a + 32 * u < b ? z[a + 32 * u] : -3.0e38f;
+            y[u] = a + 32 * u < b ? target[a + 32 * u] : 0.f;
+        }
         float mx = -3.0e38f;
-#pragma unroll 8
-        for (int i = a + lane; i < b; i += 32) mx = fmaxf(mx, z[i]);
+#pragma unroll
+        for (int u = 0; u < kKeep; ++u) mx = fmaxf(mx, x[u]);
+        for (int i = a + 32 * kKeep; i < b; i += 32) mx = fmaxf(mx, z[i]);
         mx = warp_max(mx);
         float se = 0.f;
-#pragma unroll 8
-        for (int i = a + lane; i < b; i += 32) se += expf(z[i] - mx);
+#pragma unroll
+        for (int u = 0; u < kKeep; ++u)
+            if (a + 32 * u < b) se += expf(x[u] - mx);
+        for (int i = a + 32 * kKeep; i < b; i += 32) se += expf(z[i] - mx);
         se = warp_sum(se);
         const float lse = logf(se);
         float l = 0.f;
-#pragma unroll 8
-        for (int i = a + lane; i < b; i += 32) {
-            const float lp = z[i] - mx - lse;
-            dz[i] = (expf(lp) - target[i]) / (float)G;
-            l -= target[i] * lp;
-        }
+        auto row = [&](int i, float zi, float ti) {
+            const float lp = zi - mx - lse;
+            dz[i] = (expf(lp) - ti) / (float)G;
+            l -= ti * lp;
+        };
+#pragma unroll
+        for (int u = 0; u < kKeep; ++u)
+            if (a + 32 * u < b) row(a + 32 * u, x[u], y[u]);
+        for (int i = a + 32 * kKeep; i < b; i += 32) row(i, z[i], target[i]);
         l = warp_sum(l);
         if (lane == 0) gloss[gi] = l;
     }
@@ -369,16 +399,10 @@ __global__ void k_group_softmax(const float* __restrict__ z, const float* __rest
 __global__ void k_grad_reduce(const float* __restrict__ part, int nparts, float* __restrict__ grad,
                               const float* __restrict__ gloss, int G, float* __restrict__ loss) {
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < NPAR; p += gridDim.x * blockDim.x) {
-        float a = 0.f;
-#pragma unroll 16
-        for (int q = 0; q < nparts; ++q) a += part[(int64_t)q * NPAR + p];
-        grad[p] = a;
+        grad[p] = sum_in_order<32>(0, nparts, 1, 0.f, [&](int q) { return __ldg(part + (int64_t)q * NPAR + p); });
     }
     if (loss && blockIdx.x == 0 && threadIdx.x == 0) {
-        float a = 0.f;
-#pragma unroll 16
-        for (int g = 0; g < G; ++g) a += gloss[g];
-        *loss = a / (float)G;
+        *loss = sum_in_order<32>(0, G, 1, 0.f, [&](int g) { return __ldg(gloss + g); }) / (float)G;
     }
 }
 
@@ -440,8 +464,7 @@ __global__ void k_feat_slice(lt_frame F, lt_samples smp, float* __restrict__ st)
     }
     const int n1 = smp.n1[s];
     const float* val = smp.val + smp.off[s];
-#pragma unroll 16
-    for (int e = threadIdx.x; e < n1; e += blockDim.x) acc[12] += val[e];
+    acc[12] = sum_in_order<16>(threadIdx.x, n1, blockDim.x, acc[12], [&](int e) { return __ldg(val + e); });
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
     for (int k = 0; k < 13; ++k) {  // (unrolled: acc must not live in local memory)
