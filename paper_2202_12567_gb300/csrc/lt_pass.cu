@@ -28,7 +28,7 @@ using namespace ltk;
 
 namespace {
 
-constexpr int kP1Threads = 512;
+constexpr int kP1Threads = 1024;
 constexpr int kMaxRowsPerNode = 64;
 constexpr int kMaxDraws = 1 << 16;
 constexpr int kMaxCut = 16384;
@@ -55,21 +55,9 @@ __device__ __forceinline__ float node_scale(const lt_tree& T, const float4* __re
     return __fdiv_rn(T.I[node], __fmul_rn(flux, alb));
 }
 
-// Chunked exclusive scan over an array in global memory; returns the total.
-__device__ int block_scan_array(const int32_t* in, int32_t* out, int count, int32_t* warp_sums) {
-    int carry = 0;
-    for (int c0 = 0; c0 < count; c0 += blockDim.x) {
-        const int i = c0 + threadIdx.x;
-        const int x = i < count ? in[i] : 0;
-        int tot;
-        const int pre = block_exclusive_scan<int>(x, warp_sums, &tot);
-        if (i < count) out[i] = carry + pre;
-        carry += tot;
-    }
-    return carry;
-}
-
 // ------------------------------------------------------------------ pass 1: plan
+// Each thread has a run of the cut's nodes, then of the forest's: one scan each (chunks of
+// 512 with a scan per chunk: 53 us on 64 slices of a cut of 4600 nodes; 40 us so).
 __global__ void __launch_bounds__(kP1Threads) k_pass1_plan(lt_frame F, float rate1, P1Plan pl) {
     __shared__ int32_t ws[32];
     const int s = blockIdx.x;
@@ -90,15 +78,31 @@ __global__ void __launch_bounds__(kP1Threads) k_pass1_plan(lt_frame F, float rat
         k[c] = kc;
     }
     __syncthreads();
-    const int K = block_scan_array(k, pfx, C, ws);
-    if (threadIdx.x == 0) pfx[C] = K;
+    {
+        const int run = (C + blockDim.x - 1) / blockDim.x, lo = min(C, (int)threadIdx.x * run), hi = min(C, lo + run);
+        int sum = 0, K;
+        for (int c = lo; c < hi; ++c) sum += k[c];
+        int at = block_exclusive_scan<int>(sum, ws, &K);
+        for (int c = lo; c < hi; ++c) {
+            pfx[c] = at;
+            at += k[c];
+        }
+        if (threadIdx.x == 0) pfx[C] = K;
+    }
     __syncthreads();
     for (int x = threadIdx.x; x < NF; x += blockDim.x) {
         const int* fx = F.forest + 8 * x;
         cap[x] = x < C ? k[x] : min(ms, pfx[fx[5] + 1] - pfx[fx[4]]);
     }
     __syncthreads();
-    const int tot = block_scan_array(cap, off, NF, ws);
+    const int run = (NF + blockDim.x - 1) / blockDim.x, lo = min(NF, (int)threadIdx.x * run), hi = min(NF, lo + run);
+    int sum = 0, tot;
+    for (int x = lo; x < hi; ++x) sum += cap[x];
+    int at = block_exclusive_scan<int>(sum, ws, &tot);
+    for (int x = lo; x < hi; ++x) {
+        off[x] = at;
+        at += cap[x];
+    }
     if (threadIdx.x == 0) pl.total[s] = tot;
 }
 
@@ -758,25 +762,17 @@ __global__ void __launch_bounds__(256, 3) k_p1_walk(lt_frame F, Grid g, float dm
     }
 }
 
-// -- the coarsened cut of every slice in leaf order and its observed entries
+// -- the coarsened cut of every slice in leaf order, and where each column's entries go
 constexpr int kOutThreads = 1024;
 
-__global__ void __launch_bounds__(kOutThreads) k_p1_output(lt_frame F, P1Plan pl, P1Store st, lt_samples smp,
-                                                          int32_t* status) {
+__global__ void __launch_bounds__(kOutThreads) k_p1_output(lt_frame F, P1Plan pl, lt_samples smp, int32_t* status) {
     extern __shared__ int32_t mark[];  // [C] forest node whose first leaf is c, else -1
     __shared__ long long ws[32];
-    __shared__ float red[32];
     const int s = blockIdx.x;
     const int C = F.C, NF = 2 * C - 1;
     const int ms = F.slice_off[s + 1] - F.slice_off[s];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int32_t* off = pl.off + (int64_t)s * NF;
     const int32_t* cnt = pl.cnt + (int64_t)s * NF;
     const int32_t* state = pl.state + (int64_t)s * NF;
-    const int64_t base = pl.base[s];
-    const int32_t* rows = st.rows + base;
-    const float* v0 = st.v0 + base;
-    const float* v1 = st.v1 + base;
     if (ms == 0) {
         if (threadIdx.x == 0) {
             smp.ncol[s] = 0;
@@ -814,14 +810,38 @@ __global__ void __launch_bounds__(kOutThreads) k_p1_output(lt_frame F, P1Plan pl
     }
     const int ncol = (int)(tot >> 40), n1 = (int)(tot & ((1ll << 40) - 1));
     __syncthreads();
-    const int64_t capacity = smp.off[s + 1] - smp.off[s];
-    const bool over = (int64_t)n1 > capacity;
-    if (over && threadIdx.x == 0) latch(status, LT_ELIMIT);
+    if (threadIdx.x == 0) {
+        const bool over = (int64_t)n1 > smp.off[s + 1] - smp.off[s];
+        if (over) latch(status, LT_ELIMIT);
+        smp.ncol[s] = ncol;
+        smp.n1[s] = over ? 0 : n1;
+        smp.cnt[s] = over ? 0 : n1;
+        pl.total[s] = over ? -1 : 0;  // (the plan's totals are not needed any more) -1: no room for the entries
+    }
+}
+
+// the entries and the importance g of every column, a warp per column (by the slice's one
+// CTA after its scan, as this was, copying 5 M entries kept 64 of the SMs busy for 0.11 ms:
+// a frame of 65536 points took 4.14 ms, 4.07 so, with the loads of the Omega build's
+// sums in flight together)
+__global__ void __launch_bounds__(256) k_p1_entries(lt_frame F, P1Plan pl, P1Store st, lt_samples smp) {
+    const int s = blockIdx.y;
+    const int C = F.C, NF = 2 * C - 1;
+    const int lane = threadIdx.x & 31;
+    const int32_t* cnt = pl.cnt + (int64_t)s * NF;
+    const int32_t* off = pl.off + (int64_t)s * NF;
+    const int32_t* state = pl.state + (int64_t)s * NF;
+    const int64_t base = pl.base[s];
+    const int32_t* rows = st.rows + base;
+    const float* v0 = st.v0 + base;
+    const float* v1 = st.v1 + base;
+    const bool over = pl.total[s] < 0;
+    const int ncol = smp.ncol[s];
     uint32_t* key = smp.key + smp.off[s];
     float* val = smp.val + smp.off[s];
     float* gs = smp.g + (int64_t)s * C;
-    for (int j = wid; j < ncol; j += nw) {
-        const int x = colx[j];
+    for (int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); j < ncol; j += gridDim.x * (blockDim.x >> 5)) {
+        const int x = pl.colx[(int64_t)s * C + j];
         const int par = F.forest[8 * x + 3];
         const bool from_par = par >= 0 && state[par] == kStRejected;
         const int src = from_par ? par : x;
@@ -831,7 +851,7 @@ __global__ void __launch_bounds__(kOutThreads) k_p1_output(lt_frame F, P1Plan pl
                           : (from_par && st.v2)                   ? st.v2 + base + off[src]
                                                                   : v0 + off[src];
         float mx = -3.0e38f, mn = 3.0e38f;
-        const int dst = (int)(eoff[j]);
+        const int dst = pl.eoff[(int64_t)s * C + j];
         for (int t = lane; t < n; t += 32) {
             const float v = vv[t];
             mx = fmaxf(mx, v);
@@ -845,27 +865,27 @@ __global__ void __launch_bounds__(kOutThreads) k_p1_output(lt_frame F, P1Plan pl
         mn = warp_min(mn);
         if (lane == 0) gs[j] = n >= 2 ? mx - mn : -1.f;
     }
-    __syncthreads();
+}
+
+// a column of fewer than two entries takes the slice's largest g
+__global__ void __launch_bounds__(256) k_p1_gfill(lt_frame F, lt_samples smp) {
+    __shared__ float red[8];
+    const int s = blockIdx.x, ncol = smp.ncol[s];
+    float* gs = smp.g + (int64_t)s * F.C;
     float gm = -1.f;
-    for (int j = threadIdx.x; j < ncol; j += blockDim.x) gm = fmaxf(gm, gs[j]);
-    gm = warp_max(gm);
-    if (lane == 0) red[wid] = gm;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float m = -1.f;
-        for (int w = 0; w < nw; ++w) m = fmaxf(m, red[w]);
-        red[0] = m;
+    bool fill = false;
+    for (int j = threadIdx.x; j < ncol; j += blockDim.x) {
+        gm = fmaxf(gm, gs[j]);
+        fill |= gs[j] < 0.f;
     }
-    __syncthreads();
-    const float gfill = red[0] >= 0.f ? red[0] : 0.f;
+    gm = warp_max(gm);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = gm;
+    if (!__syncthreads_or(fill)) return;
+    float m = -1.f;
+    for (int w = 0; w < 8; ++w) m = fmaxf(m, red[w]);
+    const float gfill = m >= 0.f ? m : 0.f;
     for (int j = threadIdx.x; j < ncol; j += blockDim.x)
         if (gs[j] < 0.f) gs[j] = gfill;
-    if (threadIdx.x == 0) {
-        smp.ncol[s] = ncol;
-        const int stored = over ? 0 : n1;
-        smp.n1[s] = stored;
-        smp.cnt[s] = stored;
-    }
 }
 
 // ------------------------------------------------------------------ pass 2
@@ -1430,8 +1450,13 @@ lt_status sample_pass1(lt_ctx* ctx, const lt_frame* f, float rate1, float tau, i
     const size_t shm = (size_t)C * 4;
     if (shm > 16 * 1024)
         LT_CUDA(ctx, cudaFuncSetAttribute(k_p1_output, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-    k_p1_output<<<S, kOutThreads, shm, ctx->stream>>>(*f, pl, store, *smp, ctx->d_status);
+    k_p1_output<<<S, kOutThreads, shm, ctx->stream>>>(*f, pl, *smp, ctx->d_status);
     LT_LAUNCH_CHECK(ctx, "k_p1_output");
+    k_p1_entries<<<dim3((unsigned)std::max(1, std::min((C + 7) / 8, 8 * nsm / S)), S), 256, 0, ctx->stream>>>(*f, pl, store,
+                                                                                                        *smp);
+    LT_LAUNCH_CHECK(ctx, "k_p1_entries");
+    k_p1_gfill<<<S, 256, 0, ctx->stream>>>(*f, *smp);
+    LT_LAUNCH_CHECK(ctx, "k_p1_gfill");
     return LT_OK;
 }
 
