@@ -88,10 +88,18 @@ __device__ __forceinline__ void om_sum(const lt_samples& smp, int s, int ms, int
     const uint32_t* key = smp.key + smp.off[s];
     const float* val = smp.val + smp.off[s];
     float sum = 0.f;
-#pragma unroll 8
-    for (int e = p * 256 + threadIdx.x; e < ne; e += kOmParts * 256) {
-        const uint32_t k = key[e];
-        if ((int)(k >> 16) < ms && (int)(k & 0xffffu) < ns) sum += val[e];
+    for (int e0 = p * 256 + threadIdx.x; e0 < ne; e0 += 8 * kOmParts * 256) {
+        uint32_t k[8];
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {  // the loads of eight steps in flight together
+            const int e = min(e0 + u * kOmParts * 256, ne - 1);
+            k[u] = __ldg(key + e);
+            v[u] = __ldg(val + e);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (e0 + u * kOmParts * 256 < ne && (int)(k[u] >> 16) < ms && (int)(k[u] & 0xffffu) < ns) sum += v[u];
     }
     sum = warp_sum(sum);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
@@ -1379,7 +1387,7 @@ lt_status omega_build(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, int
     LT_LAUNCH_CHECK(ctx, "k_om_bits");
     k_om_transpose<<<dim3(std::max(kOmParts, 8 * nsm / S), S), 256, 0, ctx->stream>>>(*f, *smp, om, part);
     LT_LAUNCH_CHECK(ctx, "k_om_transpose");
-    k_om_lines<<<dim3(std::max(1, 4 * nsm / S), S), 256, 0, ctx->stream>>>(*f, *smp, om);
+    k_om_lines<<<dim3(wide, S), 256, 0, ctx->stream>>>(*f, *smp, om);
     LT_LAUNCH_CHECK(ctx, "k_om_lines");
     k_om_scan<<<dim3(S, 2), 1024, 0, ctx->stream>>>(*f, *smp, om, part, kOmParts);
     LT_LAUNCH_CHECK(ctx, "k_om_scan");
