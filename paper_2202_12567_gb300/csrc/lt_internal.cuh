@@ -104,24 +104,26 @@ struct Grid {
 };
 
 // Closed-box slab test of o + t D over t in [kTMin, kTMax].
+// PAR false: the segment is parallel to no axis (par = 0).
+template <bool PAR = true>
 __device__ __forceinline__ bool slab_test(float lo0, float lo1, float lo2, float hi0, float hi1, float hi2, float3 o,
                                           float3 inv, int par) {
     float tn = kTMin, tf = kTMax;
-    if (par & 1) {
+    if (PAR && (par & 1)) {
         if (o.x < lo0 || o.x > hi0) return false;
     } else {
         const float ta = (lo0 - o.x) * inv.x, tb = (hi0 - o.x) * inv.x;
         tn = fmaxf(tn, fminf(ta, tb));
         tf = fminf(tf, fmaxf(ta, tb));
     }
-    if (par & 2) {
+    if (PAR && (par & 2)) {
         if (o.y < lo1 || o.y > hi1) return false;
     } else {
         const float ta = (lo1 - o.y) * inv.y, tb = (hi1 - o.y) * inv.y;
         tn = fmaxf(tn, fminf(ta, tb));
         tf = fminf(tf, fmaxf(ta, tb));
     }
-    if (par & 4) {
+    if (PAR && (par & 4)) {
         if (o.z < lo2 || o.z > hi2) return false;
     } else {
         const float ta = (lo2 - o.z) * inv.z, tb = (hi2 - o.z) * inv.z;
@@ -131,11 +133,12 @@ __device__ __forceinline__ bool slab_test(float lo0, float lo1, float lo2, float
     return tn <= tf;
 }
 
+template <bool PAR = true>
 __device__ __forceinline__ bool slab_hit(const float* __restrict__ b, float3 o, float3 inv, int par) {
     const float2 b01 = reinterpret_cast<const float2*>(b)[0];
     const float2 b23 = reinterpret_cast<const float2*>(b)[1];
     const float2 b45 = reinterpret_cast<const float2*>(b)[2];
-    return slab_test(b01.x, b01.y, b23.x, b23.y, b45.x, b45.y, o, inv, par);
+    return slab_test<PAR>(b01.x, b01.y, b23.x, b23.y, b45.x, b45.y, o, inv, par);
 }
 
 // Work done by the traversal (instrumentation of the ALU roofline).
@@ -241,7 +244,11 @@ __device__ __forceinline__ bool direct_blocked(const Grid& g, float3 o, float3 e
     const float3 inv = make_float3((par & 1) ? 0.f : 1.f / D.x, (par & 2) ? 0.f : 1.f / D.y,
                                    (par & 4) ? 0.f : 1.f / D.z);
     bool hit = false;
-    for (int b = 0; b < g.nb; ++b) hit |= slab_hit(g.box + 6 * b, o, inv, par);
+    if (par == 0) {
+        for (int b = 0; b < g.nb; ++b) hit |= slab_hit<false>(g.box + 6 * b, o, inv, 0);
+    } else {
+        for (int b = 0; b < g.nb; ++b) hit |= slab_hit(g.box + 6 * b, o, inv, par);
+    }
     return hit;
 }
 
@@ -272,13 +279,10 @@ __device__ __forceinline__ bool tri_hit(const float4* __restrict__ t3, float3 o,
 // from three arrays, a triangle test per step).  The tree's keys are 64-bit and distinct, so it is at
 // most 64 levels deep and the stack (one entry pushed per level) cannot overflow;
 // the walk visits each node at most once, which bounds the loops.
-__device__ inline bool bvh_blocked(const Grid& g, float3 o, float3 e) {
-    const float3 D = e - o;
-    const int par = (D.x == 0.f ? 1 : 0) | (D.y == 0.f ? 2 : 0) | (D.z == 0.f ? 4 : 0);
-    const float3 inv = make_float3((par & 1) ? 0.f : 1.f / D.x, (par & 2) ? 0.f : 1.f / D.y,
-                                   (par & 4) ? 0.f : 1.f / D.z);
+template <bool PAR>
+__device__ inline bool bvh_walk(const Grid& g, float3 o, float3 D, float3 inv, int par) {
     const int nt = g.nt, nl = nt - 1;  // leaves start at node nl
-    if (!slab_hit(g.bvh_aabb, o, inv, par)) return false;
+    if (!slab_hit<PAR>(g.bvh_aabb, o, inv, par)) return false;
     int stack[64];
     int sp = 0;
     int node = 0, left = 2 * nt;
@@ -287,8 +291,8 @@ __device__ inline bool bvh_blocked(const Grid& g, float3 o, float3 e) {
             const float4* q = g.bvh_node + 4 * (int64_t)node;
             const float4 q0 = __ldg(q), q1 = __ldg(q + 1), q2 = __ldg(q + 2), q3 = __ldg(q + 3);
             const int a = __float_as_int(q3.x), b = __float_as_int(q3.y);
-            const bool ha = slab_test(q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, o, inv, par);
-            const bool hb = slab_test(q1.z, q1.w, q2.x, q2.y, q2.z, q2.w, o, inv, par);
+            const bool ha = slab_test<PAR>(q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, o, inv, par);
+            const bool hb = slab_test<PAR>(q1.z, q1.w, q2.x, q2.y, q2.z, q2.w, o, inv, par);
             if (ha && hb) {
                 if (sp < 64) stack[sp++] = b;
                 node = a;
@@ -305,6 +309,14 @@ __device__ inline bool bvh_blocked(const Grid& g, float3 o, float3 e) {
         --left;
     }
     return false;
+}
+
+__device__ inline bool bvh_blocked(const Grid& g, float3 o, float3 e) {
+    const float3 D = e - o;
+    const int par = (D.x == 0.f ? 1 : 0) | (D.y == 0.f ? 2 : 0) | (D.z == 0.f ? 4 : 0);
+    const float3 inv = make_float3((par & 1) ? 0.f : 1.f / D.x, (par & 2) ? 0.f : 1.f / D.y,
+                                   (par & 4) ? 0.f : 1.f / D.z);
+    return par == 0 ? bvh_walk<false>(g, o, D, inv, 0) : bvh_walk<true>(g, o, D, inv, par);
 }
 
 // Any-hit test of the segment o -> e against every occluder (boxes, then triangles).
