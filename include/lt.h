@@ -390,7 +390,7 @@ lt_status lt_expand_rgb(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, c
  * apply to later calls and to later graph captures of the context. */
 typedef struct {
     int32_t eval_ctas_per_sm;   /* entry evaluation: persistent CTAs of 128 threads per SM (1..64), 16 */
-    int32_t ray_ctas_per_sm;    /* pass-1 shadow-ray kernels: the same (1..64), 16 */
+    int32_t ray_ctas_per_sm;    /* the kernel of pass 1's initial rays: the same (1..64), 16 */
     int32_t als_lane_entries;   /* ALS (r <= 16): a line gets 2^g lanes so that a lane holds at most about
                                    this many of its entries (16..1024), 96 */
     int32_t als_form;           /* ALS (r <= 16): 1 = Gram and right-hand side as dense masked products on

@@ -13,7 +13,8 @@
 //    lam_rel tr(G) / r, factors by Cholesky in float32 and solves; lines whose pivots
 //    spread beyond 1e6 are solved again in float64.  The half-step kernel is
 //    persistent: each CTA takes an equal share of all slices' warp tasks.  Above
-//    rank 16 a warp group holds a line's Gram (built on the tensor cores) row by row.
+//    rank 16 a warp sums the Grams of two lines, a block of the triangle a lane, and half
+//    a warp factors and solves each.
 //    The rank may differ per slice (factor rows keep the stride of the largest).
 //  * Render (Sec. 3 step 5): t_s = V_s^T w, pixel = max(0, u_i . t_s).
 #include <math.h>
@@ -457,18 +458,19 @@ __global__ void k_als_init(lt_frame F, lt_samples smp, Omega om, int R, const in
     }
 }
 
-// ---- One line by one warp (ranks above 16) -----------------------------------
+// ---- Two lines by one warp (ranks above 16) -----------------------------------
 // For one line (a row of U or of V) with observed entries e and factor rows x_e,
-// G = sum_e x_e x_e^T and b = sum_e a_e x_e.  Lane k accumulates row k of G (all 32
-// columns; G is symmetric) and b_k, two columns per packed multiply-add.  The entries
-// are taken 32 at a time: eight lanes copy one factor row (128 contiguous bytes, so a
-// copy instruction touches 4 lines and not 32) into the warp's stage, 16-byte chunk c
-// of row q at chunk c ^ (q & 7), and the next 32 rows are on their way (cp.async)
-// while these are added.  Rows have stride R; components at or beyond the rank are zero.  RB = 3 (ranks
-// up to 24) or 4: only the first 8 RB components are copied, added and solved for; lanes
-// past them idle.
-constexpr int kWarpStage = 32 * 32;    // floats of one stage: 32 rows of 32
-constexpr int kWarpCol = 36;           // stride of a column of L (16-byte aligned)
+// G = sum_e x_e x_e^T and b = sum_e a_e x_e.  The whole warp sums the Gram of one line after
+// the other, then half a warp solves each.  The entries are taken 32 at a time: eight lanes
+// copy one factor row (128 contiguous bytes, so a copy instruction touches 4 lines and not
+// 32) into the warp's stage with a_e behind it, and the next 32 rows are on their way
+// (cp.async) while these are added.  Rows have stride R; components at or beyond the rank
+// are zero.  RB = 3 (ranks up to 24) or 4: only the first 8 RB components are copied, added
+// and solved for.
+constexpr int kWarpRow = 36;               // floats between staged rows: 32 and a_e
+constexpr int kWarpStage = 32 * kWarpRow;  // floats of one stage: 32 rows
+constexpr int kWarpCol = 36;               // stride of a column of L (16-byte aligned)
+constexpr int kWarpGram = 36 * 16 + 32;    // a line's Gram in 4 x 4 blocks, and b
 
 __device__ __forceinline__ void copy16(float* dst, const float* src, bool full) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
@@ -487,7 +489,7 @@ __device__ __forceinline__ void stage_entries(int len, int e0, int j, const floa
         if (4 * c >= rmax) continue;
         const bool live = e0 + q < len && 4 * c < R;
         const float* p = src + (live ? (int64_t)jq * R + 4 * c : 0);
-        float* d = st + q * 32 + 4 * (c ^ (q & 7));
+        float* d = st + q * kWarpRow + 4 * c;
         if (vec) {
             copy16(d, p, live);
         } else {  // R not a multiple of 4, or rows not on 16 bytes
@@ -498,71 +500,110 @@ __device__ __forceinline__ void stage_entries(int len, int e0, int j, const floa
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
+// A line's Gram and b by one warp into `out`.  A lane holds a tile of TR x 4: RB = 3 the 21
+// 4 x 4 blocks on or below the diagonal and 6 tiles of b (a tile whose columns are a_e and
+// what lies behind it), RB = 4 the 20 tiles of 8 x 4 that reach the diagonal or below and 4
+// of b.  A row and all of its partners a lane instead read 33 floats per entry from shared
+// memory where a tile reads 8 or 12, and added both triangles.  j, av: index and value of
+// the lane's entry among the first 32.
 template <int RB>
 __device__ __forceinline__ void gram_warp(int len, const uint16_t* __restrict__ idx, const float* __restrict__ val,
-                                          const float* __restrict__ src, int R, float* st0, float (&g)[8 * RB],
-                                          float& b) {
-    const unsigned FULL = 0xffffffffu;
+                                          int j, float av, const float* __restrict__ src, int R, float* st0, float* out) {
+    constexpr int TR = RB == 3 ? 4 : 8, kTiles = RB == 3 ? 21 : 20, kVec = 8 * RB / TR;
     const int lane = threadIdx.x & 31;
     const bool vec = (R & 3) == 0 && ((uintptr_t)src & 15) == 0;
-    F32x2 g2[4 * RB];
+    int tr = 0, tc = 0;  // tile rows TR tr .., columns 4 tc ..
+    if (lane < kTiles) {
+        if (RB == 3) {
+            while ((tr + 1) * (tr + 2) / 2 <= lane) ++tr;
+            tc = lane - tr * (tr + 1) / 2;
+        } else {
+            while ((tr + 1) * (tr + 2) <= lane) ++tr;
+            tc = lane - tr * (tr + 1);
+        }
+    } else if (lane < kTiles + kVec) {
+        tr = lane - kTiles;
+        tc = 2 * RB;
+    }
+    F32x2 g2[TR / 2][4];  // two rows of the tile each
 #pragma unroll
-    for (int c = 0; c < 4 * RB; ++c) g2[c] = 0ull;
-    b = 0.f;
-    const int kc = min(lane, 8 * RB - 1) >> 2, kw = lane & 3;
-    int j = lane < len ? (int)idx[lane] : 0;
-    float av = lane < len ? val[lane] : 0.f;
+    for (int u = 0; u < TR / 2; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) g2[u][v] = 0ull;
     __syncwarp();  // the stage is free
-    if (len > 0) stage_entries(len, 0, j, src, R, 8 * RB, vec, st0);
+    if (len > 0) {
+        stage_entries(len, 0, j, src, R, 8 * RB, vec, st0);
+        st0[lane * kWarpRow + 8 * RB] = av;
+    }
     for (int e0 = 0, h = 0; e0 < len; e0 += 32, h ^= 1) {
-        const float a_now = av;
         const float* st = st0 + h * kWarpStage;
         if (e0 + 32 < len) {  // warp-uniform
             const int e = e0 + 32 + lane;
             j = e < len ? (int)idx[e] : 0;
             av = e < len ? val[e] : 0.f;
-            stage_entries(len, e0 + 32, j, src, R, 8 * RB, vec, st0 + (h ^ 1) * kWarpStage);
+            float* nx = st0 + (h ^ 1) * kWarpStage;
+            stage_entries(len, e0 + 32, j, src, R, 8 * RB, vec, nx);
+            nx[lane * kWarpRow + 8 * RB] = av;
             asm volatile("cp.async.wait_group 1;" ::: "memory");
         } else {
             asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
         __syncwarp();
         const int n = min(32, len - e0);
-#pragma unroll 2
+        const float* px = st + TR * tr;
+        const float* py = st + 4 * tc;
+#pragma unroll 4
         for (int q = 0; q < n; ++q) {
-            const float a = __shfl_sync(FULL, a_now, q);
-            const float xk = st[q * 32 + 4 * (kc ^ (q & 7)) + kw];
-            const F32x2 xx = pack2(xk, xk);
-            b = fmaf(a, xk, b);
+            const float4 y = *reinterpret_cast<const float4*>(py + q * kWarpRow);
+            const F32x2 y2[4] = {pack2(y.x, y.x), pack2(y.y, y.y), pack2(y.z, y.z), pack2(y.w, y.w)};
 #pragma unroll
-            for (int c = 0; c < 2 * RB; ++c) {
-                const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(st + q * 32 + 4 * (c ^ (q & 7)));
-                g2[2 * c] = fma2(xx, u.x, g2[2 * c]);
-                g2[2 * c + 1] = fma2(xx, u.y, g2[2 * c + 1]);
+            for (int u = 0; u < TR / 4; ++u) {
+                const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(px + q * kWarpRow + 4 * u);
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    g2[2 * u][v] = fma2(x.x, y2[v], g2[2 * u][v]);
+                    g2[2 * u + 1][v] = fma2(x.y, y2[v], g2[2 * u + 1][v]);
+                }
             }
         }
         __syncwarp();  // the stage after next is this one
     }
 #pragma unroll
-    for (int c = 0; c < 4 * RB; ++c) unpack2(g2[c], g[2 * c], g[2 * c + 1]);
+    for (int u = 0; u < TR / 2; ++u) {
+        float lo[4], hi[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) unpack2(g2[u][v], lo[v], hi[v]);
+        const int row = TR * tr + 2 * u, i = row >> 2;
+        if (lane < kTiles) {
+            if (tc <= i) {
+                float* blk = out + 16 * (i * (i + 1) / 2 + tc) + 4 * (row & 3);
+                *reinterpret_cast<float4*>(blk) = make_float4(lo[0], lo[1], lo[2], lo[3]);
+                *reinterpret_cast<float4*>(blk + 4) = make_float4(hi[0], hi[1], hi[2], hi[3]);
+            }
+        } else if (lane < kTiles + kVec) {
+            out[36 * 16 + row] = lo[0];
+            out[36 * 16 + row + 1] = hi[0];
+        }
+    }
 }
 
-// Eight columns (8 P ..) of the Cholesky of a line whose row k lane k holds, and the
-// forward substitution with them.  acc[0] is the current column and the registers move
+// Eight columns (8 P ..) of the Cholesky of half a warp's line, and the forward
+// substitution with them.  Lane l of the half has rows l (columns up to 15) and l + 16.  The
+// first register of a row is the current column and the registers move
 // down by one per column, so that one loop body serves the eight (all of them unrolled are
 // more code than the instruction caches hold: 41% of the stall cycles).  A column of L
-// goes through shared memory (one store, then 16-byte broadcast loads, a quarter as many
+// goes through shared memory (then 16-byte broadcast loads, a quarter as many
 // instructions as a shuffle per row) and stays there for the backward substitution.
 // Entries above the diagonal are not used, so every lane updates its whole row.
 template <int P, int RB>
-__device__ __forceinline__ void chol_block32(float (&acc)[8 * RB], float& y, int k, int r, bool& ok, float& dmin,
-                                             float& dmax, float& my_inv, float* Lc) {
-    constexpr int W = 8 * (RB - P);  // columns left at the start of the block
+__device__ __forceinline__ void chol_block32(float (&a1)[16], float (&a2)[8 * RB], float& y1, float& y2, int l, int r,
+                                             bool& ok, float& dmin, float& dmax, float& inv1, float& inv2, float* Lc) {
+    constexpr int W = 8 * (RB - P), W1 = 16 - 8 * P;  // columns left at the start of the block
     const unsigned FULL = 0xffffffffu;
 #pragma unroll 1
     for (int t = 0; t < 8; ++t) {
         const int J = 8 * P + t;
-        const float djj = __shfl_sync(FULL, acc[0], J);
+        const float djj = __shfl_sync(FULL, P < 2 ? a1[0] : a2[0], J & 15, 16);
         if (J < r) {
             ok &= (djj > 0.f);
             dmin = djj < dmin ? djj : dmin;
@@ -571,64 +612,122 @@ __device__ __forceinline__ void chol_block32(float (&acc)[8 * RB], float& y, int
         const float dpos = djj > 0.f ? djj : 1.f;
         const float ljj = sqrtf(dpos);
         const float inv = 1.f / ljj;
-        const float lij = (k > J) ? acc[0] * inv : (k == J ? ljj : 0.f);
         float* col = Lc + J * kWarpCol;  // row J + c of the column at col[c]
-        if (k >= J) col[k - J] = lij;
-        if (k == J) my_inv = inv;
-        const float yj = __shfl_sync(FULL, y * my_inv, J);  // L y = b: y_J is final
-        if (k == J) y = yj;
-        else if (k > J) y = fmaf(-lij, yj, y);
+        float l1 = 0.f, l2 = a2[0] * inv;
+        if (P < 2) {
+            l1 = l > J ? a1[0] * inv : (l == J ? ljj : 0.f);
+            if (l >= J) col[l - J] = l1;
+            col[l + 16 - J] = l2;
+            if (l == J) inv1 = inv;
+        } else {
+            l2 = l + 16 > J ? l2 : (l + 16 == J ? ljj : 0.f);
+            if (l + 16 >= J) col[l + 16 - J] = l2;
+            if (l + 16 == J) inv2 = inv;
+        }
+        const float yj = __shfl_sync(FULL, P < 2 ? y1 * inv1 : y2 * inv2, J & 15, 16);  // L y = b: y_J is final
+        if (P < 2) {
+            if (l == J) y1 = yj;
+            else if (l > J) y1 = fmaf(-l1, yj, y1);
+            y2 = fmaf(-l2, yj, y2);
+        } else {
+            if (l + 16 == J) y2 = yj;
+            else if (l + 16 > J) y2 = fmaf(-l2, yj, y2);
+        }
         __syncwarp();
 #pragma unroll
         for (int q = 0; q < W / 4; ++q) {  // (columns past the last hold anything and are never read)
-            const float4 l = *reinterpret_cast<const float4*>(col + 4 * q);
-            if (q > 0) acc[4 * q - 1] = fmaf(-lij, l.x, acc[4 * q]);
-            acc[4 * q] = fmaf(-lij, l.y, acc[4 * q + 1]);
-            acc[4 * q + 1] = fmaf(-lij, l.z, acc[4 * q + 2]);
-            acc[4 * q + 2] = fmaf(-lij, l.w, acc[4 * q + 3]);
+            const float4 c = *reinterpret_cast<const float4*>(col + 4 * q);
+            if (q > 0) a2[4 * q - 1] = fmaf(-l2, c.x, a2[4 * q]);
+            a2[4 * q] = fmaf(-l2, c.y, a2[4 * q + 1]);
+            a2[4 * q + 1] = fmaf(-l2, c.z, a2[4 * q + 2]);
+            a2[4 * q + 2] = fmaf(-l2, c.w, a2[4 * q + 3]);
+            if (4 * q < W1) {
+                if (q > 0) a1[4 * q - 1] = fmaf(-l1, c.x, a1[4 * q]);
+                a1[4 * q] = fmaf(-l1, c.y, a1[4 * q + 1]);
+                a1[4 * q + 1] = fmaf(-l1, c.z, a1[4 * q + 2]);
+                a1[4 * q + 2] = fmaf(-l1, c.w, a1[4 * q + 3]);
+            }
         }
     }
 }
 
-// Solves (G + ridge) u = b for one line in one warp: lane k holds row k of G in acc
-// and b_k in rhs and receives u_k.  Returns false when the float factorisation is not
-// acceptable (a non-positive pivot, or pivots spread by more than 1 / kPivotRatio).
-// Lc: 32 columns of kWarpCol floats.
+// Solves (G + ridge) u = b of one line in each half of a warp: `gram` is the half's line
+// (gram_warp), lane l of the half receives u_l and u_{l+16}.  Returns false (for the half)
+// when the float factorisation is not acceptable (a non-positive pivot, or pivots spread
+// by more than 1 / kPivotRatio).  Lc: 32 columns of kWarpCol floats a half; it may overlap
+// the Grams.
 template <int RB>
-__device__ __forceinline__ bool warp_solve32(float (&acc)[8 * RB], float rhs, int len, int r, float lam_rel, int k,
-                                             float* out_k, float* Lc) {
+__device__ __forceinline__ bool pair_solve32(const float* gram, int len, int r, float lam_rel, float* u1, float* u2,
+                                             float* Lc) {
     const unsigned FULL = 0xffffffffu;
-    float tr = 0.f;
+    const int l = threadIdx.x & 15, k2 = l + 16;
+    float a1[16], a2[8 * RB];
+    __syncwarp();  // both Grams are written
 #pragma unroll
-    for (int c = 0; c < 8 * RB; ++c)
-        if (c == k) tr = acc[c];
+    for (int c = 0; c < 4; ++c) {
+        const int i = l >> 2;
+        const float4 t = c <= i ? *reinterpret_cast<const float4*>(gram + 16 * (i * (i + 1) / 2 + c) + 4 * (l & 3))
+                                : make_float4(0.f, 0.f, 0.f, 0.f);
+        a1[4 * c] = t.x, a1[4 * c + 1] = t.y, a1[4 * c + 2] = t.z, a1[4 * c + 3] = t.w;
+    }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(FULL, tr, o);
+    for (int c = 0; c < 2 * RB; ++c) {
+        const int i = k2 >> 2;
+        const float4 t = c <= i && k2 < 8 * RB
+                             ? *reinterpret_cast<const float4*>(gram + 16 * (i * (i + 1) / 2 + c) + 4 * (l & 3))
+                             : make_float4(0.f, 0.f, 0.f, 0.f);
+        a2[4 * c] = t.x, a2[4 * c + 1] = t.y, a2[4 * c + 2] = t.z, a2[4 * c + 3] = t.w;
+    }
+    float y1 = gram[36 * 16 + l], y2 = k2 < 8 * RB ? gram[36 * 16 + k2] : 0.f;
+    __syncwarp();  // Lc is free
+    float tr = 0.f, t2 = 0.f;
+#pragma unroll
+    for (int c = 0; c < 16; ++c)
+        if (c == l) tr = a1[c];
+#pragma unroll
+    for (int c = 16; c < 8 * RB; ++c)
+        if (c == k2) t2 = a2[c];
+    tr += t2;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) tr += __shfl_xor_sync(FULL, tr, o);
     const bool zero = !(tr > 0.f) || len == 0;
     const float lam = lam_rel * tr / (float)r;
 #pragma unroll
+    for (int c = 0; c < 16; ++c)
+        if (c == l) a1[c] += lam;  // (r > 16: every first row is below the rank)
+#pragma unroll
     for (int c = 0; c < 8 * RB; ++c) {
-        const float d = (k < r) ? acc[c] + lam : 1.f;
-        acc[c] = c == k ? d : (k >= r ? 0.f : acc[c]);
+        const float d = k2 < r ? a2[c] + lam : 1.f;
+        a2[c] = c == k2 ? d : (k2 >= r ? 0.f : a2[c]);
     }
-    if (k >= r) rhs = 0.f;
-    float dmin = 3.0e38f, dmax = 0.f, inv = 1.f, y = rhs;
+    if (k2 >= r) y2 = 0.f;
+    float dmin = 3.0e38f, dmax = 0.f, inv1 = 1.f, inv2 = 1.f;
     bool ok = true;
-    chol_block32<0, RB>(acc, y, k, r, ok, dmin, dmax, inv, Lc);
-    chol_block32<1, RB>(acc, y, k, r, ok, dmin, dmax, inv, Lc);
-    chol_block32<2, RB>(acc, y, k, r, ok, dmin, dmax, inv, Lc);
-    if constexpr (RB > 3) chol_block32<3, RB>(acc, y, k, r, ok, dmin, dmax, inv, Lc);
-    if (!zero && (!ok || dmin < kPivotRatio * dmax)) return false;
-    float x = y;  // L^T x = y: lane k reads its column of L (35 k + j: no bank conflicts)
+    chol_block32<0, RB>(a1, a2, y1, y2, l, r, ok, dmin, dmax, inv1, inv2, Lc);
+    chol_block32<1, RB>(a1, a2, y1, y2, l, r, ok, dmin, dmax, inv1, inv2, Lc);
+    chol_block32<2, RB>(a1, a2, y1, y2, l, r, ok, dmin, dmax, inv1, inv2, Lc);
+    if constexpr (RB > 3) chol_block32<3, RB>(a1, a2, y1, y2, l, r, ok, dmin, dmax, inv1, inv2, Lc);
+    // L^T x = y: a lane reads its rows' columns of L (35 k + j: no bank conflicts)
+    const float* c1 = Lc + l * (kWarpCol - 1);
+    const float* c2 = Lc + k2 * (kWarpCol - 1);
 #pragma unroll 4
-    for (int j = 8 * RB - 1; j >= 0; --j) {
-        const float l = Lc[k * (kWarpCol - 1) + j];
-        const float xj = __shfl_sync(FULL, x * inv, j);
-        if (k == j) x = xj;
-        else if (k < j) x = fmaf(-l, xj, x);
+    for (int j = 8 * RB - 1; j >= 16; --j) {
+        const float m1 = c1[j], m2 = c2[j];
+        const float xj = __shfl_sync(FULL, y2 * inv2, j - 16, 16);
+        if (k2 == j) y2 = xj;
+        else if (k2 < j) y2 = fmaf(-m2, xj, y2);
+        y1 = fmaf(-m1, xj, y1);
     }
-    *out_k = (zero || k >= r) ? 0.f : x;
-    return true;
+#pragma unroll 4
+    for (int j = 15; j >= 0; --j) {
+        const float m1 = c1[j];
+        const float xj = __shfl_sync(FULL, y1 * inv1, j, 16);
+        if (l == j) y1 = xj;
+        else if (l < j) y1 = fmaf(-m1, xj, y1);
+    }
+    *u1 = zero ? 0.f : y1;
+    *u2 = zero || k2 >= r ? 0.f : y2;
+    return zero || (ok && !(dmin < kPivotRatio * dmax));
 }
 
 // ---- Float64 factor and solve of one line in one warp (the retry above rank 16) ----
@@ -715,29 +814,26 @@ __device__ __forceinline__ void factor_solve_rows(T (&acc)[G], T rhs, int len, i
     *out_k = (zero || k >= r) ? T(0) : x;
 }
 
-template <int RB>
-__device__ __forceinline__ bool warp_line(int len, const uint16_t* __restrict__ idx, const float* __restrict__ val,
-                                          const float* __restrict__ src, int R, int r, float lam_rel, float* st,
-                                          float* x) {
-    float g[8 * RB], b;
-    gram_warp<RB>(len, idx, val, src, R, st, g, b);
-    return warp_solve32<RB>(g, b, len, r, lam_rel, threadIdx.x & 31, x, st);
-}
-
-// One half-step for ranks above 16: rows of U (rows_side) or columns of V, a warp per
-// line.  A persistent grid: warps take the frame's lines in order, two at a time, from
+// One half-step for ranks above 16: rows of U (rows_side) or columns of V, two lines a
+// warp.  A persistent grid: warps take the frame's lines in order, two at a time, from
 // a counter (lines of one slice run side by side and share its factor rows in L1), so
 // that no CTA waits for another's share.  A line whose pivots fail the check goes to
 // the float64 pass (k_als_retry).
-// What bounds it: the stage reads of the Gram (9 shared-memory wavefronts per entry)
-// and the latency of the 32 dependent columns of the solve.  Completion of the 200-box
-// scene (5.7 M entries, ranks 8 to 32 per slice, 10 sweeps; the lane-group kernel has the
-// slices up to rank 16): 23.9 ms with a lane per factor row in the copies, a shuffle
-// per element in the Cholesky and 32-way bank conflicts in the solves; 14.1 ms so, 12.6
-// with the components past rank 24 left out where they are zero.
+// What bounds it: issue and the latency of shared memory at 16 warps per SM (each scheduler
+// issues in 51% of its cycles; the 24 warps that stages of 16 rows leave room for gain
+// nothing), then the dependent columns of the solve.  Completion of the 200-box scene (5.7 M
+// entries, ranks 8 to 32 per slice, 10 sweeps; the lane-group kernel has the slices up to
+// rank 16): 23.9 ms with a lane per factor row in the copies, a shuffle per element in the
+// Cholesky and 32-way bank conflicts in the solves; 12.6 ms with a row of the Gram a lane
+// and a warp per solve; 7.85 ms so.
 constexpr int kHalfWarps = 8;
-constexpr int kHalfSmem = kHalfWarps * 2 * kWarpStage * 4;  // the columns of L use the stage after the Gram
-static_assert(32 * kWarpCol <= 2 * kWarpStage, "the columns of L fit the stage");
+// a warp's floats: two stages and the first line's Gram; the second line's Gram and then the
+// columns of L of both take the same place
+constexpr int kHalfFloats = 2 * kWarpStage + kWarpGram;
+constexpr int kHalfSmem = kHalfWarps * kHalfFloats * 4;
+constexpr int kHalfCols = 32 * kWarpCol + 16;  // from the first half's columns of L to the second's: other banks
+static_assert(kHalfCols + 32 * kWarpCol <= kHalfFloats, "the columns of L fit");
+static_assert(kHalfFloats % 4 == 0 && kWarpGram % 4 == 0 && kHalfCols % 4 == 0, "16-byte accesses");
 
 __global__ void __launch_bounds__(32 * kHalfWarps, 2) k_als_half(lt_frame F, lt_samples smp, Omega om, int R,
                                                                 const int32_t* __restrict__ rk, float lam_rel,
@@ -745,8 +841,8 @@ __global__ void __launch_bounds__(32 * kHalfWarps, 2) k_als_half(lt_frame F, lt_
                                                                 float* __restrict__ Fout, AlsQueue<32> aq,
                                                                 int32_t* __restrict__ next) {
     extern __shared__ __align__(16) float wst[];
-    const int lane = threadIdx.x & 31, k = lane;
-    float* st = wst + (threadIdx.x >> 5) * 2 * kWarpStage;
+    const int lane = threadIdx.x & 31, half = lane >> 4, l = lane & 15;
+    float* st = wst + (threadIdx.x >> 5) * kHalfFloats;
     const int S = F.S;
     const int64_t total = rows_side ? (int64_t)F.slice_off[S] : om.line_pfx[S];
     int s = -1;
@@ -756,7 +852,17 @@ __global__ void __launch_bounds__(32 * kHalfWarps, 2) k_als_half(lt_frame F, lt_
         if (lane == 0) L0 = 2 * (int64_t)atomicAdd(next, 1);
         L0 = __shfl_sync(0xffffffffu, L0, 0);
         if (L0 >= total) break;
-        for (int64_t L = L0; L < min(L0 + 2, total); ++L) {
+        // the two lines (uniform in the warp; rank 0: none, or the lane-group kernel has it)
+        int rr[2], len[2], jj[2];
+        int64_t ent[2], dst[2], srow[2];
+        float vv[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int64_t L = L0 + h;
+            rr[h] = len[h] = jj[h] = 0;
+            ent[h] = dst[h] = srow[h] = 0;
+            vv[h] = 0.f;
+            if (L >= total) continue;
             if (L >= s_hi) {  // the slice with s_lo <= L < s_hi, at or after the last one's
                 int x = s < 0 ? 0 : s + 1, y = S - 1;
                 while (x < y) {
@@ -770,29 +876,54 @@ __global__ void __launch_bounds__(32 * kHalfWarps, 2) k_als_half(lt_frame F, lt_
             }
             const int r = slice_rank(rk, s, R);  // the slice's rank (factor rows have stride R)
             if (rk && r <= 16) continue;         // per-slice ranks: the lane-group kernel has these slices
+            rr[h] = r;
             const int line = (int)(L - s_lo);
             const int row0 = F.slice_off[s];
-            const int64_t o = smp.off[s];
-            const float* src = rows_side ? Fin + (int64_t)s * F.C * R : Fin + (int64_t)row0 * R;
+            srow[h] = rows_side ? (int64_t)s * F.C * R : (int64_t)row0 * R;
             const int32_t* ptr = rows_side ? om.rp + row0 + s : om.cp + (int64_t)s * (F.C + 1);
-            const int b0 = ptr[line], len = ptr[line + 1] - b0;
-            const int64_t dst = rows_side ? (int64_t)(row0 + line) * R : ((int64_t)s * F.C + line) * R;
-            const uint16_t* idx = (rows_side ? om.cidx : om.ridx) + o + b0;
-            const float* val = (rows_side ? om.cval : om.rval) + o + b0;
-            float x = 0.f;
-            const bool ok = r <= 24 ? warp_line<3>(len, idx, val, src, R, r, lam_rel, st, &x)
-                                    : warp_line<4>(len, idx, val, src, R, r, lam_rel, st, &x);
-            if (k < R) Fout[dst + k] = (ok && k < r) ? x : 0.f;
-            if (!ok && k == 0) {
+            const int b0 = ptr[line];
+            len[h] = ptr[line + 1] - b0;
+            dst[h] = rows_side ? (int64_t)(row0 + line) * R : ((int64_t)s * F.C + line) * R;
+            ent[h] = smp.off[s] + b0;
+            if (lane < len[h]) {
+                jj[h] = (int)(rows_side ? om.cidx : om.ridx)[ent[h] + lane];
+                vv[h] = (rows_side ? om.cval : om.rval)[ent[h] + lane];
+            }
+        }
+        if (rr[0] + rr[1] == 0) continue;
+        const bool three = max(rr[0], rr[1]) <= 24;
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            if ((h ? rr[1] : rr[0]) == 0) continue;
+            const int n = h ? len[1] : len[0], j = h ? jj[1] : jj[0];
+            const float av = h ? vv[1] : vv[0];
+            const uint16_t* idx = (rows_side ? om.cidx : om.ridx) + (h ? ent[1] : ent[0]);
+            const float* val = (rows_side ? om.cval : om.rval) + (h ? ent[1] : ent[0]);
+            const float* src = Fin + (h ? srow[1] : srow[0]);
+            float* out = h ? st : st + 2 * kWarpStage;
+            if (three) gram_warp<3>(n, idx, val, j, av, src, R, st, out);
+            else gram_warp<4>(n, idx, val, j, av, src, R, st, out);
+        }
+        const float* gram = half ? st : st + 2 * kWarpStage;
+        float* Lc = st + half * kHalfCols;
+        const int r = half ? rr[1] : rr[0], n = half ? len[1] : len[0];
+        float x1, x2;
+        const bool ok = three ? pair_solve32<3>(gram, n, max(r, 17), lam_rel, &x1, &x2, Lc)
+                              : pair_solve32<4>(gram, n, max(r, 17), lam_rel, &x1, &x2, Lc);
+        if (r > 0) {
+            const int64_t d = half ? dst[1] : dst[0];
+            Fout[d + l] = ok ? x1 : 0.f;
+            if (l + 16 < R) Fout[d + l + 16] = ok ? x2 : 0.f;
+            if (!ok && l == 0) {
                 // rare: the float pivots were not acceptable; k_als_retry forms the line's
                 // Gram again in float64 from the factor rows (a Gram summed in float32 would
                 // carry its rounding into the solve)
                 const int qs = atomicAdd(aq.count, 1);
                 if (qs < aq.cap) {
-                    aq.dst[qs] = dst;
-                    aq.slot[qs] = o + b0;
-                    aq.src[qs] = src - Fin;
-                    aq.len[qs] = len;
+                    aq.dst[qs] = d;
+                    aq.slot[qs] = half ? ent[1] : ent[0];
+                    aq.src[qs] = half ? srow[1] : srow[0];
+                    aq.len[qs] = n;
                     aq.grp[qs] = 0;  // contiguous in CSR / CSC
                     aq.rank[qs] = r;
                 } else {
@@ -800,6 +931,7 @@ __global__ void __launch_bounds__(32 * kHalfWarps, 2) k_als_half(lt_frame F, lt_
                 }
             }
         }
+        __syncwarp();
     }
 }
 
@@ -1461,7 +1593,7 @@ lt_status complete_impl(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, i
     const int R = uv->r;            // stride of the factor rows, the largest rank
     const int32_t* rk = uv->rank;   // per-slice ranks (NULL: R for every slice)
     // Slices of rank <= 16 go to the tensor-core form (CSR / CSC) or the lane-group
-    // SIMT kernel (sliced layout), as tuned; the warp-group ALS takes the others
+    // SIMT kernel (sliced layout), as tuned; the two-lines-a-warp ALS takes the others
     // (CSR / CSC); with per-slice ranks above 16 two of them run.
     const bool low = R <= 16 || rk != nullptr;
     const bool tc = low && ctx->tune.als_form == 1;

@@ -276,7 +276,7 @@ struct CutRecs {
 // The refinement runs on the device from the first round to the last: its kernels read the
 // size of the cut, and whether it is done, from here.  (With a copy of the errors to the host, a
 // sort there and the new cut back every round, and the forest built on the host, the setup
-// of 65536 points and 16384 lights took 5.01 ms; 2.96 ms so, 2.88 with the heights of the forest in shared memory.)
+// of 65536 points and 16384 lights took 5.01 ms; 2.96 ms so.)
 struct CutState {
     int32_t C;
     int32_t done;
