@@ -328,22 +328,35 @@ extern "C" lt_status lt_eval_pairs(lt_ctx* ctx, const float* pts, int64_t m, con
 // A CTA takes 32 shading points (a lane each) and every warp its share of each tile of
 // VPLs, which stream through shared memory; the warps' sums are added in order.  Small
 // images get CTAs of 16 warps, so that the chip is busy with few points.  Bound by the
-// instructions of the entry model (five divisions and a square root an entry): 1.07 G
-// entries in 7.24 ms, 31.5 ms with a thread per point over all VPLs and the grid walk.
+// instructions of the entry model (1.07 G entries): 31.5 ms with a thread per point over all
+// VPLs and the grid walk, 6.47 ms with every entry by entry_value.  DIRECT (few boxes, no
+// triangles; the line is kDirectBoxes): 4.79 ms.  A diffuse pair needs no unit direction,
+// n.w n'.w = n.d n'.d / d^2, so that one division stands for two and a square root; the end
+// of the ray comes with the tile; and the planes of the boxes relative to the CTA's points,
+// (lo - o, hi - o), lie in shared memory, the same differences the slab test takes.
 constexpr int kBfTile = 256;
 constexpr int kBfMaxWarps = 16;
 
-template <bool COUNT>
+template <bool COUNT, bool DIRECT>
 __global__ void __launch_bounds__(32 * kBfMaxWarps) k_bruteforce(Grid g, const float4* __restrict__ pts, int64_t m,
                                                                  const float4* __restrict__ vpls, int64_t n,
                                                                  float dmin2, float* __restrict__ img,
                                                                  unsigned long long* __restrict__ stats) {
-    __shared__ float4 tile[3][kBfTile];
+    __shared__ float4 tile[DIRECT ? 4 : 3][kBfTile];
+    __shared__ float2 slab[DIRECT ? 3 * kDirectBoxes : 1][32];  // [box][axis] (lo - o, hi - o) of every point
     __shared__ float part[kBfMaxWarps][32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int64_t i = blockIdx.x * (int64_t)32 + lane;
     const bool live = i < m;
     const PointRec P = load_rec(pts, m, live ? i : m - 1);
+    const float3 o = f3(P.a) + kRayOffset * f3(P.b);
+    const float kp = P.a.w * kInvPi;
+    if (DIRECT)
+        for (int b = wid; b < 3 * g.nb; b += nw) {
+            const int box = b / 3, axis = b % 3;
+            const float at = axis == 0 ? o.x : axis == 1 ? o.y : o.z;
+            slab[b][lane] = make_float2(__ldg(g.box + 6 * box + axis) - at, __ldg(g.box + 6 * box + 3 + axis) - at);
+        }
     float acc = 0.f;
     WorkCount wc;
     int rays = 0;
@@ -351,9 +364,14 @@ __global__ void __launch_bounds__(32 * kBfMaxWarps) k_bruteforce(Grid g, const f
         const int cnt = (int)((n - j0) < kBfTile ? (n - j0) : kBfTile);
         __syncthreads();
         for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
-            tile[0][t] = __ldg(vpls + j0 + t);
-            tile[1][t] = __ldg(vpls + n + j0 + t);
-            tile[2][t] = __ldg(vpls + 2 * n + j0 + t);
+            const float4 a = __ldg(vpls + j0 + t), b = __ldg(vpls + n + j0 + t), c = __ldg(vpls + 2 * n + j0 + t);
+            tile[0][t] = a;
+            tile[1][t] = b;
+            tile[2][t] = c;
+            if (DIRECT) {
+                const float3 e = f3(a) + kRayOffset * f3(b);
+                tile[DIRECT ? 3 : 0][t] = make_float4(e.x, e.y, e.z, c.w * (a.w * kInvPi));
+            }
         }
         __syncthreads();
         if (live) {
@@ -361,8 +379,44 @@ __global__ void __launch_bounds__(32 * kBfMaxWarps) k_bruteforce(Grid g, const f
                 PointRec L;
                 L.a = tile[0][t];
                 L.b = tile[1][t];
-                L.c = tile[2][t];
-                acc += entry_value<COUNT>(P, L, 1.f, dmin2, g, &wc, &rays);
+                if (!DIRECT) {
+                    L.c = tile[2][t];
+                    acc += entry_value<COUNT>(P, L, 1.f, dmin2, g, &wc, &rays);
+                    continue;
+                }
+                const float4 ek = tile[DIRECT ? 3 : 0][t];
+                const float3 d = f3(L.a) - f3(P.a);
+                const float dist2 = dot3(d, d);
+                const float den = dist2 * fmaxf(dist2, dmin2);
+                const bool plain = !(P.b.w > 0.f || L.b.w > 0.f) && den > 1e-24f && den < 1e30f;
+                float v;
+                if (plain) {
+                    const float cp = dot3(f3(P.b), d), cq = -dot3(f3(L.b), d);
+                    if (!(cp > 0.f && cq > 0.f)) continue;
+                    v = kp * ek.w * (cp * cq / den);
+                } else {
+                    L.c = tile[2][t];
+                    v = unoccluded(P, L, dmin2);
+                }
+                if (v > 0.f) {
+                    const float3 e = f3(ek), D = e - o;
+                    bool hit = false;
+                    if (D.x != 0.f && D.y != 0.f && D.z != 0.f) {
+                        const float3 inv = make_float3(1.f / D.x, 1.f / D.y, 1.f / D.z);
+                        for (int b = 0; b < g.nb; ++b) {
+                            const float2 x = slab[3 * b][lane], y = slab[3 * b + 1][lane], z = slab[3 * b + 2][lane];
+                            const float xa = x.x * inv.x, xb = x.y * inv.x, ya = y.x * inv.y, yb = y.y * inv.y;
+                            const float za = z.x * inv.z, zb = z.y * inv.z;
+                            const float tn = fmaxf(fmaxf(fmaxf(kTMin, fminf(xa, xb)), fminf(ya, yb)), fminf(za, zb));
+                            const float tf = fminf(fminf(fminf(kTMax, fmaxf(xa, xb)), fmaxf(ya, yb)), fmaxf(za, zb));
+                            hit |= tn <= tf;
+                        }
+                    } else {
+                        hit = direct_blocked(g, o, e);
+                    }
+                    if (hit) v = 0.f;
+                }
+                acc += v;
             }
         }
     }
@@ -393,8 +447,12 @@ extern "C" lt_status lt_bruteforce(lt_ctx* ctx, const float* pts, int64_t m, con
         return lt_fail(ctx, LT_EINVAL, "lt_bruteforce: bad arguments");
     if (!ctx->d_cell_off) return lt_fail(ctx, LT_EINVAL, "lt_bruteforce: no scene uploaded");
     const int64_t blocks = (m + 31) / 32;
-    k_bruteforce<false><<<(unsigned)blocks, bf_threads(m, ctx->num_sms), 0, ctx->stream>>>(
-        ctx->grid, (const float4*)pts, m, (const float4*)vpls, n, d_min * d_min, img, nullptr);
+    if (ctx->grid.nb <= kDirectBoxes && ctx->grid.nt == 0)
+        k_bruteforce<false, true><<<(unsigned)blocks, bf_threads(m, ctx->num_sms), 0, ctx->stream>>>(
+            ctx->grid, (const float4*)pts, m, (const float4*)vpls, n, d_min * d_min, img, nullptr);
+    else
+        k_bruteforce<false, false><<<(unsigned)blocks, bf_threads(m, ctx->num_sms), 0, ctx->stream>>>(
+            ctx->grid, (const float4*)pts, m, (const float4*)vpls, n, d_min * d_min, img, nullptr);
     LT_LAUNCH_CHECK(ctx, "k_bruteforce");
     return LT_OK;
 }
@@ -410,7 +468,7 @@ extern "C" lt_status lt_bruteforce_stats(lt_ctx* ctx, const float* pts, int64_t 
     if (!stats) return st;
     LT_CUDA(ctx, cudaMemsetAsync(stats, 0, 4 * 8, ctx->stream));
     const int64_t blocks = (m + 31) / 32;
-    k_bruteforce<true><<<(unsigned)blocks, bf_threads(m, ctx->num_sms), 0, ctx->stream>>>(
+    k_bruteforce<true, false><<<(unsigned)blocks, bf_threads(m, ctx->num_sms), 0, ctx->stream>>>(
         ctx->grid, (const float4*)pts, m, (const float4*)vpls, n, d_min * d_min, nullptr, stats);
     LT_LAUNCH_CHECK(ctx, "k_bruteforce<count>");
     unsigned long long h[4];

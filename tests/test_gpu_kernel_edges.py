@@ -93,6 +93,27 @@ def test_bruteforce_sizes(lt, ctx, m, n):
     assert np.linalg.norm(img - ref) <= 1e-5 * np.linalg.norm(ref)
 
 
+@pytest.mark.parametrize("nb,glossy,d_min", [(0, 0.0, 0.1), (2, 0.5, 0.0), (16, 0.3, 0.01)])
+def test_bruteforce_forms(lt, ctx, nb, glossy, d_min):
+    """Few boxes (diffuse pairs without a unit direction, box planes relative to the points)
+    against the walk, which copies of a box, or of one outside the room, select.  A sum of n
+    positive float32 values that differ by a few roundings: (n + 40) 2^-24 relative."""
+    n = 257
+    cfg = get_config("room256_vpl16k_200box", n_small_boxes=max(nb, 1), glossy_frac=glossy, width=16, height=9, n_vpl=n)
+    sc = make_scene(cfg)
+    boxes = sc.boxes[:nb].astype(np.float32)
+    vpls = sc.vpls.copy()
+    vpls[0, :3, :3] = sc.points[0, :3, :3]  # lights at points: no distance, no direction
+    vpls[0, 3:6, 0] = sc.points[0, 3:6, 0]  # axis-parallel rays
+    far = np.array([[9, 9, 9, 9.5, 9.5, 9.5]], np.float32)
+    imgs = []
+    for b in (boxes, np.concatenate([boxes, np.repeat(far, 17, 0)])):
+        lt.lt_scene_upload(ctx, _cuda(b))
+        imgs.append(lt.lt_bruteforce(ctx, _cuda(sc.points), _cuda(vpls), d_min).cpu().numpy().astype(np.float64))
+    assert np.isfinite(imgs[0]).all()
+    assert np.all(np.abs(imgs[0] - imgs[1]) <= (n + 40) * 2.0 ** -24 * np.abs(imgs[1]))
+
+
 @pytest.mark.parametrize("n", [2048, 4095, 4096, 4097, 8193])
 def test_sort_chunks(lt, ctx, n):
     sc = make_scene(get_config("room256_vpl16k_200box", n_vpl=n, width=8, height=8), seed=n)
