@@ -135,6 +135,7 @@ struct P1Work {
     float4* nrec;      // [NF][4] per forest node: its representative's planes, then (scale, I, 0, 0)
     int64_t* mcount;   // [Hmax] pairs of a warp per level
     int64_t* bcount;   // [Hmax] pairs of a CTA per level
+    int64_t* mnext;    // [Hmax] the next pair of a warp to take
     int64_t* mid;      // [bcap] flat pair index of a warp's pair
     int64_t* big;      // [bcap] flat pair index of a CTA's pair
     unsigned* bar;     // arrival counter of the persistent walk's grid barriers
@@ -573,8 +574,8 @@ __device__ __forceinline__ void decide_pair(const lt_frame& F, const P1Plan& pl,
 // shadow rays run side by side.
 template <int G>
 __device__ __forceinline__ void group_pair(const lt_frame& F, const Grid& g, float dmin2, const P1Plan& pl,
-                                           const P1Store& st, const P1Work& w, const PairCtx& pc, bool live,
-                                           int32_t* status) {
+                                           const P1Store& st, const P1Work& w, const PairCtx& pc, const int32_t* A,
+                                           const int32_t* B, bool live, int32_t* status) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, gl = lane & (G - 1), sh = lane & ~(G - 1);
     const unsigned gm = G == 32 ? FULL : (1u << G) - 1u, lt = (1u << gl) - 1u;
@@ -586,7 +587,7 @@ __device__ __forceinline__ void group_pair(const lt_frame& F, const Grid& g, flo
     float e = 0.f;
     for (int it = 0; it < trips; ++it) {
         const int t = it * G + gl;
-        const PairRow r = pair_row(pc.ra, na, pc.rb, nb, t);
+        const PairRow r = pair_row(A, na, B, nb, t);
         const unsigned ma = (__ballot_sync(FULL, r.in_a && r.both) >> sh) & gm;
         const unsigned mb = (__ballot_sync(FULL, r.in_b && r.both) >> sh) & gm;
         if (r.in_a || (r.in_b && !r.both)) {
@@ -630,7 +631,7 @@ __device__ __forceinline__ void p1_small_body(const lt_frame& F, const Grid& g, 
                 else latch(status, LT_ELIMIT);
             }
         }
-        group_pair<kGroup>(F, g, dmin2, pl, st, w, pc, active && rows <= kSmallPair, status);
+        group_pair<kGroup>(F, g, dmin2, pl, st, w, pc, pc.ra, pc.rb, active && rows <= kSmallPair, status);
     }
 }
 
@@ -638,13 +639,17 @@ __device__ __forceinline__ void p1_small_body(const lt_frame& F, const Grid& g, 
 // staged in shared memory when they fit), then a warp per pair; where a level has few
 // pairs (at most kFewPairs per CTA), a CTA each for those too: with a warp, a level waits
 // for eight shadow rays one after the other.  (64x64 frame 1.08 ms with kFewPairs 0, 1.01
-// with 4, 1.02 with 16.)
+// with 4, 1.02 with 16.)  Pairs differ in their rows and rays: the warps take theirs from a
+// counter and stage both row lists before they search them (sampling of the 512x512 scene
+// 4.64 ms with fixed shares and searches in memory, 4.16 so; the CTAs' pairs from a counter
+// cost the 64x64 frame 1%).
 constexpr int kBigStage = 4096;
 constexpr int kFewPairs = 4;
 
 __device__ __forceinline__ void p1_rest_body(const lt_frame& F, const Grid& g, float dmin2, const P1Plan& pl,
                                              const P1Store& st, const P1Work& w, int h, int32_t* status) {
-    __shared__ int32_t sa[kBigStage], sb[kBigStage];
+    __shared__ int32_t stage[2 * kBigStage];
+    int32_t *sa = stage, *sb = stage + kBigStage;
     __shared__ int32_t ws[32];
     __shared__ float red[32];
     // the CTA's pair: in shared memory, the registers are for the rays
@@ -694,10 +699,20 @@ __device__ __forceinline__ void p1_rest_body(const lt_frame& F, const Grid& g, f
         decide_pair(F, pl, st, w.thr, pc, pr, pc.na + pc.nb - ca, em, threadIdx.x, blockDim.x, threadIdx.x == 0);
     }
     if (few) return;
-    for (int64_t q = blockIdx.x * (int64_t)nw + wid; q < nmid; q += (int64_t)gridDim.x * nw) {
+    __syncthreads();  // the stage is free
+    int32_t* mine = stage + wid * kMidPair;  // both lists of the warp's pair
+    for (;;) {
+        unsigned long long q = 0;
+        if (lane == 0) q = atomicAdd((unsigned long long*)w.mnext + h, 1ull);
+        q = __shfl_sync(0xffffffffu, q, 0);
+        if ((int64_t)q >= nmid) break;
         PairCtx wpc;
         if (!load_pair(F, pl, st, h, w.mid[q], wpc)) continue;  // uniform in the warp
-        group_pair<32>(F, g, dmin2, pl, st, w, wpc, true, status);
+        __syncwarp();
+        for (int i = lane; i < wpc.na; i += 32) mine[i] = wpc.ra[i];
+        for (int i = lane; i < wpc.nb; i += 32) mine[wpc.na + i] = wpc.rb[i];
+        __syncwarp();
+        group_pair<32>(F, g, dmin2, pl, st, w, wpc, mine, mine + wpc.na, true, status);
     }
 }
 
@@ -1345,7 +1360,7 @@ lt_status sample_pass1(lt_ctx* ctx, const lt_frame* f, float rate1, float tau, i
     const int64_t bcap = std::max<int64_t>((int64_t)S * C, 1024);
     const size_t store_bytes = (size_t)std::max<int64_t>(acc, 1) * (target > 0 ? 16 : 12) + 1024;
     const size_t eff_bytes = target > 0 ? (size_t)S * NF * 4 : 0;
-    const size_t work_bytes = (size_t)(S + 1) * 8 + (size_t)S * C * 4 + (size_t)S * 4 + (size_t)Hn * 16 +
+    const size_t work_bytes = (size_t)(S + 1) * 8 + (size_t)S * C * 4 + (size_t)S * 4 + (size_t)Hn * 24 +
                               (size_t)bcap * 16 + (size_t)NF * 64 + eff_bytes + 18 * 256;
     char* q = (char*)lt_scratch(ctx, SCR_P1_STORE, store_bytes + work_bytes, &st);
     if (!q) return st;
@@ -1365,18 +1380,18 @@ lt_status sample_pass1(lt_ctx* ctx, const lt_frame* f, float rate1, float tau, i
     w.kpfx = (int64_t*)wtake((size_t)(S + 1) * 8);
     w.leafmean = (float*)wtake((size_t)S * C * 4);
     w.thr = (float*)wtake((size_t)S * 4);
-    w.mcount = (int64_t*)wtake((size_t)Hn * 8 + 8);
-    w.bcount = (int64_t*)wtake((size_t)Hn * 8);
+    w.mcount = (int64_t*)wtake((size_t)Hn * 24 + 8);  // the counters, zeroed together
+    w.bcount = w.mcount + Hn;
+    w.mnext = w.bcount + Hn;
     w.nrec = (float4*)wtake((size_t)NF * 64);
     w.mid = (int64_t*)wtake((size_t)bcap * 8);
     w.big = (int64_t*)wtake((size_t)bcap * 8);
-    w.bar = (unsigned*)(w.mcount + Hn);  // shares the zeroing of the level counters
+    w.bar = (unsigned*)(w.mnext + Hn);
     w.bcap = bcap;
     float* effs = target > 0 ? (float*)wtake(eff_bytes) : nullptr;
     if ((size_t)(wp - q) > ctx->scr_size[SCR_P1_STORE])
         return lt_fail(ctx, LT_ENOMEM, "lt_sample_pass1: work layout overflow");
-    LT_CUDA(ctx, cudaMemsetAsync(w.mcount, 0, (size_t)Hn * 8 + 8, ctx->stream));
-    LT_CUDA(ctx, cudaMemsetAsync(w.bcount, 0, (size_t)Hn * 8, ctx->stream));
+    LT_CUDA(ctx, cudaMemsetAsync(w.mcount, 0, (size_t)Hn * 24 + 8, ctx->stream));
     const int nsm = ctx->num_sms;
     const float dmin2 = d_min * d_min;
     auto grid_for = [&](int64_t items, int threads) {
