@@ -275,8 +275,9 @@ __device__ __forceinline__ bool tri_hit(const float4* __restrict__ t3, float3 o,
 // with an explicit stack.  A step reads one 64-byte record with both children's boxes
 // (four 16-byte loads).  The lanes of a warp descend until each has a leaf or is done
 // and test their triangles together.  Bound by the latency of the dependent node loads
-// and divergence: 5.2 M entries among 7680 triangles and 2 boxes in 0.84 ms (1.04 ms with a check for axis-parallel segments per box, 1.92 ms
-// from three arrays, a triangle test per step).  The tree's keys are 64-bit and distinct, so it is at
+// and divergence: 5.2 M entries among 7680 triangles and 2 boxes in 0.84 ms (1.04 ms with a
+// check for axis-parallel segments per box, 1.92 ms from three arrays, a triangle test per
+// step).  The tree's keys are 64-bit and distinct, so it is at
 // most 64 levels deep and the stack (one entry pushed per level) cannot overflow;
 // the walk visits each node at most once, which bounds the loops.
 template <bool PAR>

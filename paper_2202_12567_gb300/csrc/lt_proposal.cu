@@ -680,7 +680,7 @@ __global__ void k_goff(lt_samples smp, int S, int64_t* __restrict__ goff2, int64
 // shared memory 16 at a time, the next 16 loaded while these are added.  Every output
 // is one chain of multiply-adds over the rows in order.  Bound by the FP32 pipe.  With
 // this, k_slice_matrix and the split subspace iteration the training data of a scene of 65536
-// points (64 slices of about 630 columns, 30 rounds at rank 16) take 6.4 ms, 54.1 ms with
+// points (64 slices of about 630 columns, 30 rounds at rank 16) take 4.6 ms, 54.1 ms with
 // 32 x 32 tiles and one CTA per slice for the whole iteration.
 __global__ void __launch_bounds__(256, 2) k_gram(lt_frame F, lt_samples smp, const float* __restrict__ M,
                                                  const int64_t* __restrict__ moff, const int64_t* __restrict__ goff2,
