@@ -42,7 +42,7 @@ namespace cg = cooperative_groups;
 
 namespace {
 
-constexpr int kAdmMaxK = 8;                  // CTAs per slice (one cluster), at most
+constexpr int kAdmMaxK = 8;                  // Gram parts of a slice, at most (a cluster has up to twice as many CTAs)
 constexpr int kAdmThreads = 256;
 constexpr int kAdmChunk = 128;               // rows per chunk of a Gram pass
 constexpr size_t kAdmStageBytes = 96 * 1024; // Y staged in shared memory up to this size
@@ -718,20 +718,35 @@ lt_status launch_adm(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, cons
     // take their tasks from a counter (every eighth task a warp: 23.8 on the same GPU).
     int K0 = kAdmMaxK;
     while (K0 > 2 && (int64_t)f->S * K0 > 2 * (int64_t)ctx->num_sms) K0 >>= 1;
-    const int K = std::min(kAdmMaxK, 2 * K0);
+    int K = 2 * K0;
     a.parts = K0;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(f->S * K));
     cfg.blockDim = dim3(kAdmThreads);
     cfg.dynamicSmemBytes = dyn;
     cfg.stream = ctx->stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)K;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    auto cluster = [&](int k) {
+        attr[0].val.clusterDim.x = (unsigned)k;
+        cfg.gridDim = dim3((unsigned)(f->S * k));
+    };
+    cluster(K);
+    // 16 CTAs, more than the portable size, where the device can place the clusters of all
+    // slices at once: few slices leave the chip idle.  (50 iterations, clusters of 8 against 16:
+    // 7 slices of 13208 rows in all at rank 12 13.3 / 8.3 ms, 18 of 25600 at rank 16 11.8 / 8.1;
+    // where they come in turns, 35 slices of 17658 rows at rank 8, 3.8 / 6.8.)
+    if (K > kAdmMaxK) {
+        int fit = 0;
+        if (cudaFuncSetAttribute(k_adm<RP>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&fit, k_adm<RP>, &cfg) != cudaSuccess || fit < f->S) {
+            cudaGetLastError();
+            cluster(K = K0);
+        }
+    }
     LT_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_adm<RP>, *f, *smp, om, a, sr));
     LT_LAUNCH_CHECK(ctx, "k_adm");
     return LT_OK;

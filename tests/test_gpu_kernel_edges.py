@@ -242,9 +242,10 @@ def test_completion_sizes(lt, rank, slices):
         assert _completed(lt, R, s, Uo, Vo) <= 1e-3, s
 
 
-@pytest.mark.parametrize("rank,slices", [(8, 40), (16, 40), (20, 80)])
+@pytest.mark.parametrize("rank,slices", [(8, 40), (16, 40), (20, 80), (12, 3), (24, 12), (16, 20)])
 def test_adm_clusters(lt, rank, slices):
-    """More than 38 slices: clusters of 8 CTAs over 4 Gram parts (80: 4 over 2)."""
+    """More than 38 slices: clusters of 8 CTAs over 4 Gram parts (80: 4 over 2); few: clusters of
+    16 over 8 where all of them can run at once, else of 8."""
     from paper_2202_12567_gb300.renderer import Renderer
     cfg = get_config("room64_vpl1k_2box", max_cut=128, n_slices=slices, rank=rank, rate=0.3, rate1=0.002,
                      completion="adm", adm_iters=7)
