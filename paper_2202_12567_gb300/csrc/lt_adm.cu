@@ -14,14 +14,14 @@
 // the Y step, so the state per slice is X (two buffers: the Y step needs X_k and
 // X_{k+1}), U, Lambda, Y, V, Pi and the |Omega| residuals.
 //
-// One cluster of K CTAs (K = 2, 4 or 8, so that the whole grid is resident at
-// two CTAs per SM where possible) completes one slice and runs all iterations in
-// one launch.  Per iteration: (1) the X step, a group of G lanes per row of the CTA's
+// One cluster of K CTAs completes one slice and runs all iterations in one launch (K is
+// twice the number of parts its Gram matrices are summed in, 2, 4 or 8 by the number of
+// slices, where clusters of that size can be had; launch_adm has the rule).  Per iteration: (1) the X step, a group of G lanes per row of the CTA's
 // rows (G a power of two sized by the slice's mean row length; the lanes split the
 // row's entries two at a time, reduce with shuffles and split the r output
 // components), with the U and Lambda updates fused and no barrier between rows;
-// then the CTA's part of B and C from its rows staged through shared memory;
-// cluster barrier; (2) every CTA sums the K partial Gram matrices from distributed
+// then a part of B or C from its rows staged through shared memory;
+// cluster barrier; (2) every CTA sums the partial Gram matrices from distributed
 // shared memory in rank order (so every CTA holds the same bits), inverts
 // B + beta I by Gauss-Jordan in one warp and forms D = (B + beta I)^-1 C; the Y step
 // per column of the CTA's columns (residual through the CSC -> CSR slot map, row of
