@@ -1101,13 +1101,14 @@ extern "C" lt_status lt_leverage_targets(lt_ctx* ctx, const lt_frame* f, const l
     const int64_t nmax = std::min<int64_t>(C, 4096);
     const int64_t gcap = (int64_t)S * nmax * gram_ld((int)nmax);
     lt_status st;
-    char* p = (char*)lt_scratch(ctx, SCR_PROPOSAL_T,
-                                (size_t)gcap * 4 + (size_t)2 * S * C * r * 4 + (size_t)(S + 1) * 16 + 4 * 256, &st);
+    auto up = [](size_t n) { return (n + 255) & ~(size_t)255; };  // each part starts on 256 bytes
+    const size_t b_g = up((size_t)gcap * 4), b_q = up((size_t)S * C * r * 4);
+    char* p = (char*)lt_scratch(ctx, SCR_PROPOSAL_T, b_g + 2 * b_q + (size_t)(S + 1) * 16, &st);
     if (!p) return st;
     float* G = (float*)p;
-    float* Q = (float*)(p + (((size_t)gcap * 4 + 255) & ~(size_t)255));
-    float* Y = Q + (size_t)S * C * r;
-    int64_t* goff2 = (int64_t*)((char*)Y + (((size_t)S * C * r * 4 + 255) & ~(size_t)255));
+    float* Q = (float*)(p + b_g);
+    float* Y = (float*)(p + b_g + b_q);
+    int64_t* goff2 = (int64_t*)(p + b_g + 2 * b_q);
     int64_t* tpfx = goff2 + S + 1;
     k_goff<<<1, 1024, 0, ctx->stream>>>(*smp, S, goff2, tpfx);
     LT_LAUNCH_CHECK(ctx, "k_goff");

@@ -1,0 +1,51 @@
+"""Forms of the calls that the parity tests do not reach: sizes, orders and refusals at which
+a layout, a launch or a check of the library decides.  Tolerances are those of the parity tests.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from ltinputs import get_config, make_scene
+from oracle import proposal as o_prop
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lt():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2202_12567_gb300 import lt as _lt
+    _lt.load()
+    return _lt
+
+
+def _targets_renderer(**over):
+    from paper_2202_12567_gb300.renderer import Renderer
+    cfg = get_config("room64_vpl1k_2box", **{**dict(width=24, height=24, eps_cut=1e-4, rate1=0.002), **over})
+    R = Renderer(make_scene(cfg), cfg, device=0).setup()
+    R.pass1(3)
+    return R
+
+
+def _check_targets(R, M, moff, goff, ncol, t, rank, iters, seed):
+    M, moff, goff, t = (x.cpu().numpy() for x in (M, moff, goff, t))
+    for s in range(R.frame.S):
+        A = M[moff[s]:moff[s + 1]].reshape(-1, ncol[s]).astype(np.float64)
+        want = o_prop.targets(o_prop.leverage(A, rank, iters, seed, s))
+        got = t[goff[s]:goff[s + 1]]
+        assert np.linalg.norm(got - want) <= 1e-3 * np.linalg.norm(want), (s, ncol[s])
+
+
+@pytest.mark.parametrize("slices,cut,rank,iters", [(17, 631, 5, 0), (17, 631, 1, 1), (3, 257, 7, 0)])
+def test_targets_odd_layout(lt, slices, cut, rank, iters):
+    """Slices, cut and rank all odd: the parts of the scratch hold an odd number of floats."""
+    R = _targets_renderer(n_slices=slices, max_cut=cut, rank=rank)
+    assert R.frame.C == cut and R.frame.S == slices
+    _, goff = lt.lt_proposal_features(R.ctx, R.frame, R.smp)
+    ncol = R.smp.ncol.cpu().numpy()
+    M, moff = lt.lt_slice_matrices(R.ctx, R.frame, R.smp, R.cfg["d_min"], int(np.sum(R.frame.sizes * ncol)))
+    t = lt.lt_leverage_targets(R.ctx, R.frame, R.smp, M, moff, goff, rank, iters, 9)
+    lt.lt_sync(R.ctx)
+    _check_targets(R, M, moff, goff, ncol, t, rank, iters, 9)
