@@ -654,8 +654,12 @@ __host__ __device__ __forceinline__ int gram_ld(int n) { return (n + 3) & ~3; }
 constexpr int kGramTile = 128;
 constexpr int kGramStep = 16;
 
-// goff2 and the prefix of the tiles on or above the diagonal of every G_s
-__global__ void k_goff(lt_samples smp, int S, int64_t* __restrict__ goff2, int64_t* __restrict__ tpfx) {
+// goff2 and the prefix of the tiles on or above the diagonal of every G_s.  A latched
+// LT_ELIMIT may be that of the slice matrices (a total beyond the caller's capacity): M then
+// holds less than the slices' rows and columns say, and goff2[S] tells the kernels that
+// follow to read none of it.
+__global__ void k_goff(lt_samples smp, int S, int64_t* __restrict__ goff2, int64_t* __restrict__ tpfx,
+                       const int32_t* status) {
     __shared__ int64_t ws[32];
     int64_t carry = 0, tcarry = 0;
     for (int c0 = 0; c0 < S; c0 += blockDim.x) {
@@ -670,7 +674,7 @@ __global__ void k_goff(lt_samples smp, int S, int64_t* __restrict__ goff2, int64
         tcarry += tot;
     }
     if (threadIdx.x == 0) {
-        goff2[S] = carry;
+        goff2[S] = *status == LT_ELIMIT ? INT64_MAX : carry;
         tpfx[S] = tcarry;
     }
 }
@@ -1110,7 +1114,7 @@ extern "C" lt_status lt_leverage_targets(lt_ctx* ctx, const lt_frame* f, const l
     float* Y = (float*)(p + b_g + b_q);
     int64_t* goff2 = (int64_t*)(p + b_g + 2 * b_q);
     int64_t* tpfx = goff2 + S + 1;
-    k_goff<<<1, 1024, 0, ctx->stream>>>(*smp, S, goff2, tpfx);
+    k_goff<<<1, 1024, 0, ctx->stream>>>(*smp, S, goff2, tpfx, ctx->d_status);
     LT_LAUNCH_CHECK(ctx, "k_goff");
     k_gram<<<2 * ctx->num_sms, 256, 0, ctx->stream>>>(*f, *smp, M, moff, goff2, tpfx, gcap, G);
     LT_LAUNCH_CHECK(ctx, "k_gram");

@@ -49,3 +49,21 @@ def test_targets_odd_layout(lt, slices, cut, rank, iters):
     t = lt.lt_leverage_targets(R.ctx, R.frame, R.smp, M, moff, goff, rank, iters, 9)
     lt.lt_sync(R.ctx)
     _check_targets(R, M, moff, goff, ncol, t, rank, iters, 9)
+
+
+def test_targets_after_refused_matrices(lt):
+    """Matrices beyond the caller's capacity are refused at the next sync; the targets queued
+    behind them read nothing of the buffer and write nothing."""
+    R = _targets_renderer(n_slices=4, max_cut=256, rank=4)
+    _, goff = lt.lt_proposal_features(R.ctx, R.frame, R.smp)
+    M, moff = lt.lt_slice_matrices(R.ctx, R.frame, R.smp, R.cfg["d_min"], 1000)
+    t = torch.full((R.frame.S * R.frame.C,), -7.0, device="cuda")
+    lt.lt_leverage_targets(R.ctx, R.frame, R.smp, M, moff, goff, 4, 2, 9, t)
+    with pytest.raises(lt.LtError):
+        lt.lt_sync(R.ctx)
+    assert int(moff[-1]) > 1000 and torch.all(t == -7.0) and torch.all(M == 0)
+    ncol = R.smp.ncol.cpu().numpy()  # the sync cleared the status: the same calls with room
+    M, moff = lt.lt_slice_matrices(R.ctx, R.frame, R.smp, R.cfg["d_min"], int(np.sum(R.frame.sizes * ncol)))
+    lt.lt_leverage_targets(R.ctx, R.frame, R.smp, M, moff, goff, 4, 0, 9, t)
+    lt.lt_sync(R.ctx)
+    _check_targets(R, M, moff, goff, ncol, t, 4, 0, 9)
