@@ -1100,10 +1100,11 @@ extern "C" lt_status lt_leverage_targets(lt_ctx* ctx, const lt_frame* f, const l
         return lt_fail(ctx, LT_EINVAL, "lt_leverage_targets: bad arguments");
     cudaSetDevice(ctx->device);
     const int S = f->S, C = f->C;
-    // Gram capacity: sum of n'^2 <= S * min(C, 4096)^2 floats is bounded by the
-    // largest coarsened cut the slices can have; slices beyond it are skipped
+    // Gram capacity: slices of any n' whose squares add up to at most S min(C, 4096)^2
+    // floats, and the padding of their rows (at most 3 floats each); with more no target is
+    // written.
     const int64_t nmax = std::min<int64_t>(C, 4096);
-    const int64_t gcap = (int64_t)S * nmax * gram_ld((int)nmax);
+    const int64_t gcap = (int64_t)S * (nmax * nmax + 3 * (int64_t)C);
     lt_status st;
     auto up = [](size_t n) { return (n + 255) & ~(size_t)255; };  // each part starts on 256 bytes
     const size_t b_g = up((size_t)gcap * 4), b_q = up((size_t)S * C * r * 4);

@@ -67,3 +67,26 @@ def test_targets_after_refused_matrices(lt):
     lt.lt_leverage_targets(R.ctx, R.frame, R.smp, M, moff, goff, 4, 0, 9, t)
     lt.lt_sync(R.ctx)
     _check_targets(R, M, moff, goff, ncol, t, 4, 0, 9)
+
+
+def _wide_slices(lt, ncol):
+    """Slices of ncol columns each, all of one coarsened cut of more than 4096 nodes."""
+    S, most = len(ncol), max(ncol)
+    R = _targets_renderer(n_slices=S, n_vpl=8192, max_cut=8192, target_cut=most, rank=2, width=20, height=16)
+    assert R.smp.ncol.cpu().tolist() == [most] * S
+    R.smp.ncol.copy_(torch.tensor(ncol, dtype=torch.int32))
+    goff = torch.tensor(np.concatenate([[0], np.cumsum(ncol)]).astype(np.int32), device="cuda")
+    M, moff = lt.lt_slice_matrices(R.ctx, R.frame, R.smp, R.cfg["d_min"], int(np.sum(R.frame.sizes * np.array(ncol))))
+    t = torch.full((R.frame.S * R.frame.C,), -7.0, device="cuda")
+    lt.lt_leverage_targets(R.ctx, R.frame, R.smp, M, moff, goff, 2, 1, 9, t)
+    return R, M, moff, goff, t
+
+
+def test_targets_within_capacity(lt):
+    """Above 4096 columns in one slice, the squares of all within two times 4096 squared, though
+    not with every row of the products padded to four floats."""
+    ncol = [5001, 2923]
+    assert sum(n * n for n in ncol) <= 2 * 4096 ** 2 < sum(n * ((n + 3) & ~3) for n in ncol)
+    R, M, moff, goff, t = _wide_slices(lt, ncol)
+    lt.lt_sync(R.ctx)
+    _check_targets(R, M, moff, goff, ncol, t, 2, 1, 9)
