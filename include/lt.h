@@ -441,8 +441,9 @@ lt_status lt_slice_matrices(lt_ctx* ctx, const lt_frame* f, const lt_samples* sm
 /* Training targets, in row order: p_j = (l_j + 1/n') / sum, l_j the squared norm of
  * row j of the basis after `iters` rounds of subspace iteration Q <- mgs(M^T M Q)
  * (modified Gram-Schmidt) from a Philox start (counter (k, j, slice, 4)), rank
- * min(r, n').  Slices with n' > 4096 are skipped.  While LT_ELIMIT is latched (the
- * matrices may not have been written) M is not read and no target is written. */
+ * min(r, n').  Slices whose n'^2 add up to more than S min(C, 4096)^2 (about: the rows of
+ * M^T M are padded) latch LT_ELIMIT.  While LT_ELIMIT is latched (the matrices may not
+ * have been written) M is not read and no target is written. */
 lt_status lt_leverage_targets(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, const float* M,
                               const int64_t* moff, const int32_t* group_off, int32_t r, int32_t iters,
                               uint64_t seed, float* target);

@@ -659,7 +659,7 @@ constexpr int kGramStep = 16;
 // holds less than the slices' rows and columns say, and goff2[S] tells the kernels that
 // follow to read none of it.
 __global__ void k_goff(lt_samples smp, int S, int64_t* __restrict__ goff2, int64_t* __restrict__ tpfx,
-                       const int32_t* status) {
+                       int64_t gcap, int32_t* status) {
     __shared__ int64_t ws[32];
     int64_t carry = 0, tcarry = 0;
     for (int c0 = 0; c0 < S; c0 += blockDim.x) {
@@ -675,6 +675,7 @@ __global__ void k_goff(lt_samples smp, int S, int64_t* __restrict__ goff2, int64
     }
     if (threadIdx.x == 0) {
         goff2[S] = *status == LT_ELIMIT ? INT64_MAX : carry;
+        if (carry > gcap) latch(status, LT_ELIMIT);
         tpfx[S] = tcarry;
     }
 }
@@ -1101,8 +1102,8 @@ extern "C" lt_status lt_leverage_targets(lt_ctx* ctx, const lt_frame* f, const l
     cudaSetDevice(ctx->device);
     const int S = f->S, C = f->C;
     // Gram capacity: slices of any n' whose squares add up to at most S min(C, 4096)^2
-    // floats, and the padding of their rows (at most 3 floats each); with more no target is
-    // written.
+    // floats, and the padding of their rows (at most 3 floats each).  More latches LT_ELIMIT
+    // and no target is written.
     const int64_t nmax = std::min<int64_t>(C, 4096);
     const int64_t gcap = (int64_t)S * (nmax * nmax + 3 * (int64_t)C);
     lt_status st;
@@ -1115,7 +1116,7 @@ extern "C" lt_status lt_leverage_targets(lt_ctx* ctx, const lt_frame* f, const l
     float* Y = (float*)(p + b_g + b_q);
     int64_t* goff2 = (int64_t*)(p + b_g + 2 * b_q);
     int64_t* tpfx = goff2 + S + 1;
-    k_goff<<<1, 1024, 0, ctx->stream>>>(*smp, S, goff2, tpfx, ctx->d_status);
+    k_goff<<<1, 1024, 0, ctx->stream>>>(*smp, S, goff2, tpfx, gcap, ctx->d_status);
     LT_LAUNCH_CHECK(ctx, "k_goff");
     k_gram<<<2 * ctx->num_sms, 256, 0, ctx->stream>>>(*f, *smp, M, moff, goff2, tpfx, gcap, G);
     LT_LAUNCH_CHECK(ctx, "k_gram");

@@ -90,3 +90,11 @@ def test_targets_within_capacity(lt):
     R, M, moff, goff, t = _wide_slices(lt, ncol)
     lt.lt_sync(R.ctx)
     _check_targets(R, M, moff, goff, ncol, t, 2, 1, 9)
+
+
+def test_targets_beyond_capacity(lt):
+    """Products that do not fit are an error, not targets left as they were."""
+    R, _, _, _, t = _wide_slices(lt, [4200])
+    with pytest.raises(lt.LtError):
+        lt.lt_sync(R.ctx)
+    assert torch.all(t == -7.0)
