@@ -840,7 +840,7 @@ __global__ void __launch_bounds__(kOutThreads) k_p1_output(lt_frame F, P1Plan pl
 // a frame of 65536 points took 4.14 ms, 4.07 so, with the loads of the Omega build's
 // sums in flight together)
 __global__ void __launch_bounds__(256) k_p1_entries(lt_frame F, P1Plan pl, P1Store st, lt_samples smp) {
-    const int s = blockIdx.y;
+    const int s = blockIdx.x;  // (grid.y ends at 65535)
     const int C = F.C, NF = 2 * C - 1;
     const int lane = threadIdx.x & 31;
     const int32_t* cnt = pl.cnt + (int64_t)s * NF;
@@ -855,7 +855,7 @@ __global__ void __launch_bounds__(256) k_p1_entries(lt_frame F, P1Plan pl, P1Sto
     uint32_t* key = smp.key + smp.off[s];
     float* val = smp.val + smp.off[s];
     float* gs = smp.g + (int64_t)s * C;
-    for (int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); j < ncol; j += gridDim.x * (blockDim.x >> 5)) {
+    for (int j = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5); j < ncol; j += gridDim.y * (blockDim.x >> 5)) {
         const int x = pl.colx[(int64_t)s * C + j];
         const int par = F.forest[8 * x + 3];
         const bool from_par = par >= 0 && state[par] == kStRejected;
@@ -1467,8 +1467,8 @@ lt_status sample_pass1(lt_ctx* ctx, const lt_frame* f, float rate1, float tau, i
         LT_CUDA(ctx, cudaFuncSetAttribute(k_p1_output, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
     k_p1_output<<<S, kOutThreads, shm, ctx->stream>>>(*f, pl, *smp, ctx->d_status);
     LT_LAUNCH_CHECK(ctx, "k_p1_output");
-    k_p1_entries<<<dim3((unsigned)std::max(1, std::min((C + 7) / 8, 8 * nsm / S)), S), 256, 0, ctx->stream>>>(*f, pl, store,
-                                                                                                        *smp);
+    k_p1_entries<<<dim3(S, (unsigned)std::max(1, std::min((C + 7) / 8, 8 * nsm / S))), 256, 0, ctx->stream>>>(
+        *f, pl, store, *smp);
     LT_LAUNCH_CHECK(ctx, "k_p1_entries");
     k_p1_gfill<<<S, 256, 0, ctx->stream>>>(*f, *smp);
     LT_LAUNCH_CHECK(ctx, "k_p1_gfill");

@@ -7,7 +7,7 @@ import pytest
 torch = pytest.importorskip("torch")
 
 from ltinputs import get_config, make_scene
-from oracle import proposal as o_prop
+from oracle import pipeline, proposal as o_prop
 
 pytestmark = pytest.mark.gpu
 
@@ -98,3 +98,21 @@ def test_targets_beyond_capacity(lt):
     with pytest.raises(lt.LtError):
         lt.lt_sync(R.ctx)
     assert torch.all(t == -7.0)
+
+
+def test_pass1_many_slices(lt):
+    """More slices than a grid has in its second dimension: 66560 of no rows, then 1024 of one."""
+    from paper_2202_12567_gb300.renderer import Renderer
+    cfg = get_config("room64_vpl1k_2box", width=32, height=32, n_vpl=64, max_cut=8)
+    sc = make_scene(cfg)
+    st = pipeline.setup(sc, cfg, slicing=(np.arange(sc.m), np.maximum(np.arange(66560 + sc.m + 1) - 66560, 0)))
+    R = Renderer(sc, cfg, device=0).setup(cut=st["cut"], row_perm=st["row_perm"], slice_off=st["slice_off"])
+    assert R.frame.S == 67584
+    R.pass1(11)
+    lt.lt_sync(R.ctx)
+    assert int(R.smp.cnt[:66560].abs().max()) == 0 and int(R.smp.ncol[:66560].abs().max()) == 0
+    for s in (66560, 67000, 67583):
+        rows, cols, vals, col_node, _ = R.smp.slice(s)
+        o = pipeline.run_slice(st, sc, cfg, s, 11).p1
+        assert np.array_equal(col_node, o.col_node) and np.array_equal(rows, o.rows) and np.array_equal(cols, o.cols)
+        assert np.all(np.abs(vals - o.vals) <= 1e-5 * np.abs(o.vals) + 1e-12)
