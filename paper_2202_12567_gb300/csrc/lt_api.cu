@@ -88,7 +88,7 @@ extern "C" lt_status lt_create(lt_ctx** out, int device, void* stream) {
     ctx->stream = (cudaStream_t)stream;  // NULL: the CUDA default stream
     ctx->own_stream = false;
     if (cudaMalloc(&ctx->d_status, sizeof(int32_t)) != cudaSuccess ||
-        cudaMallocHost(&ctx->h_status, sizeof(int32_t)) != cudaSuccess) {
+        cudaMallocHost(&ctx->h_status, 8 * sizeof(int32_t)) != cudaSuccess) {
         delete ctx;
         return LT_ENOMEM;
     }

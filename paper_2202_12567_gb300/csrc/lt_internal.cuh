@@ -520,7 +520,7 @@ struct lt_ctx {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     int32_t* d_status = nullptr;
-    int32_t* h_status = nullptr;
+    int32_t* h_status = nullptr;         // [8] pinned: the status word as read back; rounds of a cut, its state
     std::string err;
     // occluder grid
     float* d_boxes = nullptr;

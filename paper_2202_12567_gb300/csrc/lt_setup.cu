@@ -391,14 +391,15 @@ __global__ void __launch_bounds__(kCutThreads) k_cut_error(const float4* __restr
 // One refinement round: of the internal nodes of error above eps the `take` largest errors
 // (ties: the lower node) are split in place, so that the cut stays in leaf order.  take is
 // all of them, at most floor(growth C) (at least one) and at most max_cut - C.  One CTA: a
-// radix select of the take-th key (error descending, node ascending) and one scan.
+// radix select of the take-th key (error descending, node ascending) and one scan.  told, in
+// host memory: the rounds so far, INT32_MAX after the last.
 constexpr int kRefineThreads = 1024;
 constexpr int kMaxRounds = 4096;
 
 __global__ void __launch_bounds__(kRefineThreads) k_cut_refine(const int32_t* __restrict__ child, int64_t n, float eps,
                                                                int32_t max_cut, float growth, int32_t* __restrict__ cut,
                                                                int32_t* __restrict__ nxt, const float* __restrict__ err,
-                                                               CutState* st) {
+                                                               CutState* st, volatile int32_t* told) {
     __shared__ int32_t ws[32];
     __shared__ int32_t hist[256];
     __shared__ unsigned long long sel[2];
@@ -420,7 +421,10 @@ __global__ void __launch_bounds__(kRefineThreads) k_cut_refine(const int32_t* __
     room = min(room, grow > 1 ? grow : (int64_t)1);
     const int take = cand > room ? (int)(room > 0 ? room : 0) : cand;
     if (take == 0) {
-        if (threadIdx.x == 0) st->done = 1;
+        if (threadIdx.x == 0) {
+            st->done = 1;
+            *told = INT32_MAX;
+        }
         return;
     }
     unsigned long long pivot = ~0ull;
@@ -484,7 +488,9 @@ __global__ void __launch_bounds__(kRefineThreads) k_cut_refine(const int32_t* __
     if (threadIdx.x == 0) {
         st->C = total;
         const int rounds = ++st->rounds;
-        if ((take < cand && total >= max_cut) || rounds >= kMaxRounds) st->done = 1;
+        const bool end = (take < cand && total >= max_cut) || rounds >= kMaxRounds;
+        if (end) st->done = 1;
+        *told = end ? INT32_MAX : rounds;
     }
 }
 
@@ -959,19 +965,29 @@ extern "C" lt_status lt_build_global_cut(lt_ctx* ctx, const lt_tree* tree, const
     LT_CUDA(ctx, cudaMemsetAsync(cut, 0, sizeof(int32_t), ctx->stream));  // the root
     k_cut_state<<<1, 1, 0, ctx->stream>>>(w.st, 1);
     LT_LAUNCH_CHECK(ctx, "k_cut_state");
-    // Rounds follow one another without the host, which looks at the state after the 20th and
-    // then after every sixth (a cut that grows by half a round has 8192 nodes after 23; a
-    // round past the end is four kernels that return at once)
-    CutState h{};
-    for (int round = 0; !h.done; ++round) {
+    // The host launches one round beyond the one that it waits for, from a word in its memory,
+    // so that the device goes on without it and at most two rounds are launched past the end
+    // (four kernels each that return at once).  us a cut with no round ahead / one / two / four,
+    // and with 20 rounds before the first look: ended with its first round 98 / 101 / 107 / 115, 310;
+    // 64 lights, 10 rounds, 348 / 314 / 325 / 370, 445; 16384 lights, 21 rounds, 671 / 576 / 589 / 625,
+    // 650.  (A word that does not come ends the wait when the stream is idle or failed.)
+    constexpr int kAhead = 1, kLook = 64;
+    volatile int32_t* told = ctx->h_status + 1;
+    CutState* h = reinterpret_cast<CutState*>(ctx->h_status + 2);
+    *told = 0;
+    h->done = 0;
+    for (int round = 1; !h->done; ++round) {
         if ((st = cut_errors(ctx, tree, vpls, nr, cut, d_min, w, w.err)) != LT_OK) return st;
-        k_cut_refine<<<1, kRefineThreads, 0, ctx->stream>>>(tree->child, n, eps, max_cut, growth, cut, w.nxt, w.err, w.st);
+        k_cut_refine<<<1, kRefineThreads, 0, ctx->stream>>>(tree->child, n, eps, max_cut, growth, cut, w.nxt, w.err, w.st,
+                                                            told);
         LT_LAUNCH_CHECK(ctx, "k_cut_refine");
-        if (round < 19 || (round - 19) % 6 != 0) continue;
-        LT_CUDA(ctx, cudaMemcpyAsync(&h, w.st, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
+        while (*told < round - kAhead && cudaStreamQuery(ctx->stream) == cudaErrorNotReady) {
+        }
+        if (*told != INT32_MAX && round % kLook) continue;
+        LT_CUDA(ctx, cudaMemcpyAsync(h, w.st, sizeof(*h), cudaMemcpyDeviceToHost, ctx->stream));
         LT_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     }
-    *cut_size_host = h.C;
+    *cut_size_host = h->C;
     return LT_OK;
 }
 

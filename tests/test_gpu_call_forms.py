@@ -116,3 +116,21 @@ def test_pass1_many_slices(lt):
         o = pipeline.run_slice(st, sc, cfg, s, 11).p1
         assert np.array_equal(col_node, o.col_node) and np.array_equal(rows, o.rows) and np.array_equal(cols, o.cols)
         assert np.all(np.abs(vals - o.vals) <= 1e-5 * np.abs(o.vals) + 1e-12)
+
+
+@pytest.mark.parametrize("n,eps", [(1, 0.02), (64, 1e9), (1024, 1e9)])
+def test_cut_that_ends_at_once(lt, n, eps):
+    """The cut is the root after one round; the rounds that are launched before the host hears
+    of it are few (four kernels each)."""
+    sc = make_scene(get_config("room64_vpl1k_2box", n_vpl=n))
+    ctx = lt.Context(0)
+    vp, pts = torch.from_numpy(sc.vpls).cuda(), torch.from_numpy(np.ascontiguousarray(sc.points)).cuda()
+    tree = lt.lt_build_tree(ctx, vp)
+    rows = torch.arange(0, sc.m, 64, dtype=torch.int32, device="cuda")
+    launches = []
+    for _ in range(5):  # the first call also loads the kernels
+        before = lt.lt_launch_count(ctx)
+        cut = lt.lt_build_global_cut(ctx, tree, pts, vp, rows, eps, 8192, 0.5, 0.1)
+        launches.append(lt.lt_launch_count(ctx) - before)
+        assert cut.tolist() == [0]
+    assert sorted(launches)[2] <= 42, launches
