@@ -396,7 +396,8 @@ __global__ void __launch_bounds__(kCutThreads) k_cut_error(const float4* __restr
 constexpr int kRefineThreads = 1024;
 constexpr int kMaxRounds = 4096;
 
-__global__ void __launch_bounds__(kRefineThreads) k_cut_refine(const int32_t* __restrict__ child, int64_t n, float eps,
+__global__ void __launch_bounds__(kRefineThreads) k_cut_refine(const int32_t* __restrict__ child,
+                                                               const int32_t* __restrict__ range, int64_t n, float eps,
                                                                int32_t max_cut, float growth, int32_t* __restrict__ cut,
                                                                int32_t* __restrict__ nxt, const float* __restrict__ err,
                                                                CutState* st, volatile int32_t* told) {
@@ -477,8 +478,10 @@ __global__ void __launch_bounds__(kRefineThreads) k_cut_refine(const int32_t* __
     int at = block_exclusive_scan<int>(grown, ws, &total);
     for (int i = lo; i < hi; ++i) {
         if (split(i)) {
-            nxt[at++] = child[2 * (int64_t)cut[i]];
-            nxt[at++] = child[2 * (int64_t)cut[i] + 1];
+            const int64_t a = child[2 * (int64_t)cut[i]], b = child[2 * (int64_t)cut[i] + 1];
+            const bool swap = range[2 * b] < range[2 * a];  // a caller's tree may name the right child first
+            nxt[at++] = (int32_t)(swap ? b : a);
+            nxt[at++] = (int32_t)(swap ? a : b);
         } else {
             nxt[at++] = cut[i];
         }
@@ -978,8 +981,8 @@ extern "C" lt_status lt_build_global_cut(lt_ctx* ctx, const lt_tree* tree, const
     h->done = 0;
     for (int round = 1; !h->done; ++round) {
         if ((st = cut_errors(ctx, tree, vpls, nr, cut, d_min, w, w.err)) != LT_OK) return st;
-        k_cut_refine<<<1, kRefineThreads, 0, ctx->stream>>>(tree->child, n, eps, max_cut, growth, cut, w.nxt, w.err, w.st,
-                                                            told);
+        k_cut_refine<<<1, kRefineThreads, 0, ctx->stream>>>(tree->child, tree->range, n, eps, max_cut, growth, cut, w.nxt,
+                                                            w.err, w.st, told);
         LT_LAUNCH_CHECK(ctx, "k_cut_refine");
         while (*told < round - kAhead && cudaStreamQuery(ctx->stream) == cudaErrorNotReady) {
         }

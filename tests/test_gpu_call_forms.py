@@ -134,3 +134,20 @@ def test_cut_that_ends_at_once(lt, n, eps):
         launches.append(lt.lt_launch_count(ctx) - before)
         assert cut.tolist() == [0]
     assert sorted(launches)[2] <= 42, launches
+
+
+def test_cut_of_a_tree_with_children_exchanged(lt):
+    """The cut is in leaf order whichever child a tree names first."""
+    sc = make_scene(get_config("room64_vpl1k_2box", n_vpl=1000))
+    ctx = lt.Context(0)
+    vp, pts = torch.from_numpy(sc.vpls).cuda(), torch.from_numpy(np.ascontiguousarray(sc.points)).cuda()
+    tree = lt.lt_build_tree(ctx, vp)
+    rows = torch.arange(0, sc.m, 64, dtype=torch.int32, device="cuda")
+    cut = lt.lt_build_global_cut(ctx, tree, pts, vp, rows, 0.02, 300, 0.5, 0.1)
+    child = tree.child.view(-1, 2)
+    swap = torch.arange(child.shape[0], device="cuda") % 3 != 0
+    child[swap] = child[swap].flip(1)
+    again = lt.lt_build_global_cut(ctx, tree, pts, vp, rows, 0.02, 300, 0.5, 0.1)
+    assert cut.numel() > 200 and torch.equal(cut, again)
+    first = tree.range.view(-1, 2)[cut.long(), 0]
+    assert torch.all(first[1:] > first[:-1])
