@@ -508,14 +508,13 @@ struct ForestState {
 constexpr int kMaxHeight = 2046;
 
 __global__ void k_fo_init(int64_t NN, int C, int32_t* __restrict__ local, int32_t* __restrict__ anc,
-                          int32_t* __restrict__ arrived, int32_t* __restrict__ fo, ForestState* st) {
+                          int32_t* __restrict__ arrived, ForestState* st) {
     const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
     for (int64_t x = i0; x < NN; x += step) {
         local[x] = -1;
         anc[x] = 0;
     }
     for (int64_t x = i0; x < C; x += step) arrived[x] = 0;
-    for (int64_t x = i0; x < 2 * (int64_t)C - 1; x += step) fo[8 * x + 3] = -1;
     if (i0 == 0) *st = ForestState{0, 0, 0};
 }
 
@@ -553,72 +552,85 @@ __global__ void __launch_bounds__(1024) k_fo_scan(int64_t NN, int C, const int32
         }
 }
 
-__global__ void k_fo_nodes(const int32_t* __restrict__ child, const int32_t* __restrict__ cut, int C,
-                           const int32_t* __restrict__ local, const int32_t* __restrict__ inner, int32_t* __restrict__ fo,
+// children of every ancestor, parents of all nodes (par: the root has none)
+__global__ void k_fo_nodes(const int32_t* __restrict__ child, int C, const int32_t* __restrict__ local,
+                           const int32_t* __restrict__ inner, int2* __restrict__ kid, int32_t* __restrict__ par,
                            ForestState* st) {
     if (st->err) return;
-    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < 2 * C - 1; x += gridDim.x * blockDim.x) {
-        int32_t* f = fo + 8 * (int64_t)x;
-        const int t = x < C ? cut[x] : inner[x - C];
-        int a = -1, b = -1;
-        if (x >= C) {
-            a = local[child[2 * (int64_t)t]];
-            b = local[child[2 * (int64_t)t + 1]];
-            if (a < 0 || b < 0) {
-                atomicMax(&st->err, 2);
-                a = b = -1;
-            } else {
-                fo[8 * (int64_t)a + 3] = x;
-                fo[8 * (int64_t)b + 3] = x;
-            }
+    const int i0 = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i0 == 0) par[C > 1 ? C : 0] = -1;
+    for (int i = i0; i < C - 1; i += gridDim.x * blockDim.x) {
+        const int a = local[child[2 * (int64_t)inner[i]]], b = local[child[2 * (int64_t)inner[i] + 1]];
+        kid[i] = make_int2(a, b);
+        if (a < 0 || b < 0) {
+            atomicMax(&st->err, 2);
+        } else {
+            par[a] = C + i;
+            par[b] = C + i;
         }
-        f[0] = t;
-        f[1] = a;
-        f[2] = b;
-        f[4] = x < C ? x : 0;
-        f[5] = x < C ? x : 0;
-        f[6] = 0;
-        f[7] = 0;
     }
 }
 
-// leaf ranges and heights: the second child to arrive at a node combines both
-__global__ void k_fo_up(int C, int32_t* fo, int32_t* arrived, ForestState* st) {
+// leaf ranges and heights (span: first leaf, last leaf, height): the second child to arrive
+// at a node combines both
+__global__ void k_fo_up(int C, const int2* __restrict__ kid, const int32_t* __restrict__ par, int32_t* span,
+                        int32_t* arrived, ForestState* st) {
     if (st->err) return;
-    volatile int32_t* v = fo;
+    volatile int32_t* v = span;
+    auto get = [&](int x, int k) { return x < C ? (k < 2 ? x : 0) : v[4 * (int64_t)(x - C) + k]; };
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x) {
-        int x = fo[8 * (int64_t)c + 3];
+        int x = par[c];
         for (int it = 0; x >= C && it <= kMaxHeight; ++it) {
             __threadfence();
             if (atomicAdd(&arrived[x - C], 1) == 0) break;
             __threadfence();
-            const int64_t a = 8 * (int64_t)v[8 * (int64_t)x + 1], b = 8 * (int64_t)v[8 * (int64_t)x + 2], f = 8 * (int64_t)x;
-            v[f + 4] = min(v[a + 4], v[b + 4]);
-            v[f + 5] = max(v[a + 5], v[b + 5]);
-            const int h = 1 + max(v[a + 6], v[b + 6]);
-            v[f + 6] = h;
+            const int2 k = kid[x - C];
+            const int64_t f = 4 * (int64_t)(x - C);
+            v[f] = min(get(k.x, 0), get(k.y, 0));
+            v[f + 1] = max(get(k.x, 1), get(k.y, 1));
+            const int h = 1 + max(get(k.x, 2), get(k.y, 2));
+            v[f + 2] = h;
             atomicMax(&st->height, h);
-            x = v[f + 3];
+            x = par[x];
         }
     }
 }
 
+// The caller's arrays, which are written only when nothing is refused.  The first CTA lists
 // the internal nodes of every height by id, and where each height starts: a run of the
 // nodes per thread, one scan per height, the heights of the first kHeightStage nodes in
 // shared memory (one CTA waits on each read; read from memory once per height, the setup
-// of 65536 points and 16384 lights took 3.00 ms instead of 2.88)
+// of 65536 points and 16384 lights took 3.00 ms instead of 2.88).  The others write the forest.
 constexpr int kHeightStage = 16384;
 
-__global__ void __launch_bounds__(1024) k_fo_levels(int C, const int32_t* __restrict__ fo, int32_t max_levels,
-                                                    int32_t* __restrict__ level_off, int32_t* __restrict__ level_nodes,
-                                                    const ForestState* __restrict__ st) {
+__global__ void __launch_bounds__(1024) k_fo_out(int C, const int32_t* __restrict__ cut, const int32_t* __restrict__ inner,
+                                                 const int2* __restrict__ kid, const int32_t* __restrict__ par,
+                                                 const int32_t* __restrict__ span, int32_t max_levels,
+                                                 int32_t* __restrict__ forest, int32_t* __restrict__ level_off,
+                                                 int32_t* __restrict__ level_nodes, const ForestState* __restrict__ st) {
     __shared__ int32_t ws[32];
     __shared__ uint16_t hs[kHeightStage];
     const int H = st->height;
     if (st->err || H > max_levels || H > kMaxHeight) return;
-    for (int i = threadIdx.x; i < min(C - 1, kHeightStage); i += 1024) hs[i] = (uint16_t)fo[8 * (int64_t)(C + i) + 6];
+    if (blockIdx.x > 0) {
+        for (int x = (blockIdx.x - 1) * 1024 + threadIdx.x; x < 2 * C - 1; x += (gridDim.x - 1) * 1024) {
+            int32_t* f = forest + 8 * (int64_t)x;
+            const int32_t* sp = span + 4 * (int64_t)(x - C);
+            const int2 k = x < C ? make_int2(-1, -1) : kid[x - C];
+            f[0] = x < C ? cut[x] : inner[x - C];
+            f[1] = k.x;
+            f[2] = k.y;
+            f[3] = par[x];
+            f[4] = x < C ? x : sp[0];
+            f[5] = x < C ? x : sp[1];
+            f[6] = x < C ? 0 : sp[2];
+            f[7] = 0;
+        }
+        return;
+    }
+    for (int i = threadIdx.x; i < min(C - 1, kHeightStage); i += 1024) hs[i] = (uint16_t)span[4 * (int64_t)i + 2];
     __syncthreads();
-    auto height = [&](int i) { return i < kHeightStage ? (int)hs[i] : fo[8 * (int64_t)(C + i) + 6]; };
+    auto height = [&](int i) { return i < kHeightStage ? (int)hs[i] : span[4 * (int64_t)i + 2]; };
     const int run = (C - 1 + 1023) / 1024, lo = min(C - 1, (int)threadIdx.x * run), hi = min(C - 1, lo + run);
     int start = 0;
     if (threadIdx.x == 0) level_off[0] = 0;
@@ -1006,28 +1018,32 @@ extern "C" lt_status lt_cut_forest(lt_ctx* ctx, const lt_tree* tree, const int32
     if (C > tree->n) return lt_fail(ctx, LT_EINVAL, "lt_cut_forest: cut nodes out of range or repeated");
     auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
     lt_status st;
-    char* p = (char*)lt_scratch(ctx, SCR_CUT, 2 * up((size_t)NN * 4) + 2 * up((size_t)C * 4) + 256, &st);
+    const size_t b_nn = up((size_t)NN * 4), b_c = up((size_t)C * 4);
+    char* p = (char*)lt_scratch(ctx, SCR_CUT, 2 * b_nn + 4 * b_c + up((size_t)C * 16) + 256, &st);
     if (!p) return st;
     int32_t* local = (int32_t*)p;
-    int32_t* anc = (int32_t*)(p + up((size_t)NN * 4));
-    int32_t* arrived = (int32_t*)(p + 2 * up((size_t)NN * 4));
-    int32_t* inner = (int32_t*)(p + 2 * up((size_t)NN * 4) + up((size_t)C * 4));
-    ForestState* fs = (ForestState*)(p + 2 * up((size_t)NN * 4) + 2 * up((size_t)C * 4));
+    int32_t* anc = (int32_t*)(p + b_nn);
+    int32_t* par = anc;  // (the marks are not read any more when the parents are written)
+    p += 2 * b_nn;
+    int32_t* arrived = (int32_t*)p;
+    int32_t* inner = (int32_t*)(p + b_c);
+    int2* kid = (int2*)(p + 2 * b_c);
+    int32_t* span = (int32_t*)(p + 4 * b_c);
+    ForestState* fs = (ForestState*)(p + 4 * b_c + up((size_t)C * 16));
     const int most = 8 * ctx->num_sms;
-    k_fo_init<<<(unsigned)std::min<int64_t>((NN + 255) / 256, most), 256, 0, ctx->stream>>>(NN, C, local, anc, arrived,
-                                                                                            forest, fs);
+    k_fo_init<<<(unsigned)std::min<int64_t>((NN + 255) / 256, most), 256, 0, ctx->stream>>>(NN, C, local, anc, arrived, fs);
     LT_LAUNCH_CHECK(ctx, "k_fo_init");
     k_fo_mark<<<std::min((C + 127) / 128, most), 128, 0, ctx->stream>>>(NN, tree->parent, cut, C, local, anc, fs);
     LT_LAUNCH_CHECK(ctx, "k_fo_mark");
     k_fo_scan<<<1, 1024, 0, ctx->stream>>>(NN, C, anc, local, inner, fs);
     LT_LAUNCH_CHECK(ctx, "k_fo_scan");
-    k_fo_nodes<<<std::min((2 * C + 254) / 256, most), 256, 0, ctx->stream>>>(tree->child, cut, C, local, inner, forest,
-                                                                             fs);
+    k_fo_nodes<<<std::min((C + 255) / 256, most), 256, 0, ctx->stream>>>(tree->child, C, local, inner, kid, par, fs);
     LT_LAUNCH_CHECK(ctx, "k_fo_nodes");
-    k_fo_up<<<std::min((C + 127) / 128, most), 128, 0, ctx->stream>>>(C, forest, arrived, fs);
+    k_fo_up<<<std::min((C + 127) / 128, most), 128, 0, ctx->stream>>>(C, kid, par, span, arrived, fs);
     LT_LAUNCH_CHECK(ctx, "k_fo_up");
-    k_fo_levels<<<1, 1024, 0, ctx->stream>>>(C, forest, max_levels, level_off, level_nodes, fs);
-    LT_LAUNCH_CHECK(ctx, "k_fo_levels");
+    k_fo_out<<<1 + std::min((2 * C + 1023) / 1024, most), 1024, 0, ctx->stream>>>(C, cut, inner, kid, par, span, max_levels,
+                                                                                 forest, level_off, level_nodes, fs);
+    LT_LAUNCH_CHECK(ctx, "k_fo_out");
     ForestState h{};
     LT_CUDA(ctx, cudaMemcpyAsync(&h, fs, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
     LT_CUDA(ctx, cudaStreamSynchronize(ctx->stream));

@@ -151,3 +151,49 @@ def test_cut_of_a_tree_with_children_exchanged(lt):
     assert cut.numel() > 200 and torch.equal(cut, again)
     first = tree.range.view(-1, 2)[cut.long(), 0]
     assert torch.all(first[1:] > first[:-1])
+
+
+@pytest.mark.parametrize("kind", ["repeated", "negative", "past_the_tree", "short", "nested", "too_many", "levels"])
+def test_forest_refusals_write_nothing(lt, kind):
+    """A cut that is no partition, or higher than the caller's levels, is an error and leaves the
+    caller's arrays as they were; the cut itself is accepted with room for exactly its levels."""
+    import ctypes
+    n = 300
+    sc = make_scene(get_config("room64_vpl1k_2box", n_vpl=n, width=16, height=16))
+    ctx = lt.Context(0)
+    tree = lt.lt_build_tree(ctx, torch.from_numpy(sc.vpls).cuda())
+    child = tree.child.cpu().numpy().reshape(-1, 2)
+    good = [0]
+    for _ in range(100):  # the first internal node is split
+        i = next(k for k, x in enumerate(good) if x < n - 1)
+        good[i:i + 1] = child[good[i]].tolist()
+    _, _, _, H = lt.lt_cut_forest(ctx, tree, torch.tensor(good, dtype=torch.int32, device="cuda"))
+    assert H > 1
+    cut, levels = list(good), H
+    if kind == "repeated":
+        cut[5] = cut[50]
+    elif kind == "negative":
+        cut[5] = -1
+    elif kind == "past_the_tree":
+        cut[5] = 2 * n - 1
+    elif kind == "short":
+        del cut[5]
+    elif kind == "nested":
+        i = next(k for k, x in enumerate(cut) if x < n - 1)
+        cut.insert(i, int(child[cut[i]][0]))
+    elif kind == "too_many":
+        cut = list(range(n + 1))
+    else:
+        levels = H - 1
+
+    def call(cut, levels):
+        C = len(cut)
+        c = torch.tensor(cut, dtype=torch.int32, device="cuda")
+        out = [torch.full((k,), -7, dtype=torch.int32, device="cuda") for k in (8 * (2 * C - 1), levels + 2, C)]
+        h, s = ctypes.c_int32(-7), tree.struct()
+        status = ctx.lib.lt_cut_forest(ctx.h, ctypes.byref(s), c.data_ptr(), C, out[0].data_ptr(), out[1].data_ptr(),
+                                       levels, out[2].data_ptr(), ctypes.byref(h))
+        return status, h.value, all(bool(torch.all(x == -7)) for x in out)
+
+    assert call(cut, levels) == (1, -7, True)  # LT_EINVAL
+    assert call(good, H) == (0, H, False)
