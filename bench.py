@@ -238,7 +238,13 @@ class ClockSampler:
 # Algorithmic FP32 operations of one evaluated entry (counted from the source of
 # the entry model and the traversal): shading of the unoccluded value 40, ray set-up
 # and grid clipping 40 per shadow ray, 6 per grid cell visited, 24 per box slab test.
+# Where every ray tests every box (no cell is visited) the set-up alone takes 18; the
+# brute force of a diffuse scene then takes 20 an entry up to the cosines, 11 more a ray
+# (the value, direction and its inverses) and 18 a box, whose planes relative to the
+# point it keeps.
 OPS_ENTRY, OPS_RAY, OPS_CELL, OPS_BOX = 40, 40, 6, 24
+OPS_RAY_DIRECT = 18
+OPS_SHORT_ENTRY, OPS_SHORT_RAY, OPS_SHORT_BOX = 20, 11, 18
 SMS, FP32_LANES, MAX_SM_MHZ = 152, 128, 2070.0
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch from one ncu
@@ -261,10 +267,20 @@ def fp32_peak(clk) -> dict:
                             f"no measured FP32 peak); at the sampled median {mhz:.0f} MHz in peak_at_sampled_clock")
 
 
+def entry_ops(st, short=False) -> int:
+    """FP32 operations of the entries that the counters describe (short: the brute force of a
+    diffuse scene without triangles)."""
+    if st["cells"]:
+        return OPS_ENTRY * st["entries"] + OPS_RAY * st["rays"] + OPS_CELL * st["cells"] + OPS_BOX * st["boxes"]
+    if short:
+        return OPS_SHORT_ENTRY * st["entries"] + OPS_SHORT_RAY * st["rays"] + OPS_SHORT_BOX * st["boxes"]
+    return OPS_ENTRY * st["entries"] + OPS_RAY_DIRECT * st["rays"] + OPS_BOX * st["boxes"]
+
+
 def eval_roofline(lt, ctx, R, eval_ms, clk):
     """ALU roofline of the entry-evaluation kernel (the shadow-ray kernel)."""
     st = lt.lt_eval_stats(ctx, R.frame, R.smp, R.cfg["d_min"])
-    ops = OPS_ENTRY * st["entries"] + OPS_RAY * st["rays"] + OPS_CELL * st["cells"] + OPS_BOX * st["boxes"]
+    ops = entry_ops(st)
     secs = eval_ms * 1e-3
     achieved = ops / secs / 1e12 if secs > 0 else 0.0
     pk = fp32_peak(clk)
@@ -296,7 +312,8 @@ def bruteforce_roofline(lt, ctx, R, bf_ms, clk):
     """ALU roofline of the brute-force column sum (the baseline of the speed-up): the
     entry-model operations of all m n entries, their shadow rays, cells and boxes."""
     st = lt.lt_bruteforce_stats(ctx, R.pts, R.vpls, R.cfg["d_min"])
-    ops = OPS_ENTRY * st["entries"] + OPS_RAY * st["rays"] + OPS_CELL * st["cells"] + OPS_BOX * st["boxes"]
+    short = R.cfg["glossy_frac"] == 0 and getattr(R.scene, "tris", None) is None
+    ops = entry_ops(st, short)
     achieved = ops / (bf_ms * 1e-3) / 1e12
     pk = fp32_peak(clk)
     return dict(bound="alu", kernel="k_bruteforce", achieved=round(achieved, 3), unit="TFLOP/s",

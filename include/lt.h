@@ -172,7 +172,8 @@ lt_status lt_bruteforce(lt_ctx* ctx, const float* pts, int64_t m, const float* v
 /* Instrumentation (no counterpart in the paper): re-runs the brute force of the same
  * points and VPLs without storing the image and returns in stats_host[4] the entries
  * (m n), the shadow rays cast (entries with a positive unoccluded value), the grid
- * cells visited and the box slab tests made.  Synchronous. */
+ * cells visited and the box slab tests made.  It takes the path of the call that it
+ * describes: up to 16 boxes every ray tests every box and no cell is visited.  Synchronous. */
 lt_status lt_bruteforce_stats(lt_ctx* ctx, const float* pts, int64_t m, const float* vpls, int64_t n,
                               float d_min, int64_t* stats_host);
 
@@ -287,7 +288,7 @@ lt_status lt_eval_entries_noalloc(lt_ctx* ctx, const lt_frame* f, float d_min, l
 /* Instrumentation (no counterpart in the paper): re-runs the evaluation of the same
  * entries without storing values and returns in stats_host[4] the entries, the shadow
  * rays cast (entries with a positive unoccluded value), the grid cells visited and
- * the box slab tests made.  Synchronous. */
+ * the box slab tests made (as in lt_bruteforce_stats).  Synchronous. */
 lt_status lt_eval_stats(lt_ctx* ctx, const lt_frame* f, float d_min, const lt_samples* smp,
                         int64_t* stats_host);
 /* Masked ALS at rank r (uv->rank[s] per slice when given), `iters` sweeps (U-step

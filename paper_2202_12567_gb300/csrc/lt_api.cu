@@ -399,6 +399,10 @@ __global__ void __launch_bounds__(32 * kBfMaxWarps) k_bruteforce(Grid g, const f
                     v = unoccluded(P, L, dmin2);
                 }
                 if (v > 0.f) {
+                    if (COUNT) {
+                        ++rays;
+                        wc.boxes += g.nb;
+                    }
                     const float3 e = f3(ek), D = e - o;
                     bool hit = false;
                     if (D.x != 0.f && D.y != 0.f && D.z != 0.f) {
@@ -468,8 +472,12 @@ extern "C" lt_status lt_bruteforce_stats(lt_ctx* ctx, const float* pts, int64_t 
     if (!stats) return st;
     LT_CUDA(ctx, cudaMemsetAsync(stats, 0, 4 * 8, ctx->stream));
     const int64_t blocks = (m + 31) / 32;
-    k_bruteforce<true, false><<<(unsigned)blocks, bf_threads(m, ctx->num_sms), 0, ctx->stream>>>(
-        ctx->grid, (const float4*)pts, m, (const float4*)vpls, n, d_min * d_min, nullptr, stats);
+    if (ctx->grid.nb <= kDirectBoxes && ctx->grid.nt == 0)
+        k_bruteforce<true, true><<<(unsigned)blocks, bf_threads(m, ctx->num_sms), 0, ctx->stream>>>(
+            ctx->grid, (const float4*)pts, m, (const float4*)vpls, n, d_min * d_min, nullptr, stats);
+    else
+        k_bruteforce<true, false><<<(unsigned)blocks, bf_threads(m, ctx->num_sms), 0, ctx->stream>>>(
+            ctx->grid, (const float4*)pts, m, (const float4*)vpls, n, d_min * d_min, nullptr, stats);
     LT_LAUNCH_CHECK(ctx, "k_bruteforce<count>");
     unsigned long long h[4];
     LT_CUDA(ctx, cudaMemcpyAsync(h, stats, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));

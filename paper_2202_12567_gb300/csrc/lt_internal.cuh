@@ -323,7 +323,8 @@ __device__ inline bool bvh_blocked(const Grid& g, float3 o, float3 e) {
 // Any-hit test of the segment o -> e against every occluder (boxes, then triangles).
 template <bool COUNT = false>
 __device__ inline bool seg_blocked(const Grid& g, float3 o, float3 e, WorkCount* wc = nullptr) {
-    if (!COUNT && g.nb <= kDirectBoxes) {
+    if (g.nb <= kDirectBoxes) {
+        if (COUNT) wc->boxes += g.nb;
         if (g.nb > 0 && direct_blocked(g, o, e)) return true;
     } else if (g.nb > 0 && grid_blocked<COUNT>(g, o, e, wc)) {
         return true;

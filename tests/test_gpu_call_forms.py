@@ -197,3 +197,31 @@ def test_forest_refusals_write_nothing(lt, kind):
 
     assert call(cut, levels) == (1, -7, True)  # LT_EINVAL
     assert call(good, H) == (0, H, False)
+
+
+@pytest.mark.parametrize("nb,extra", [(2, 0), (2, 15), (0, 0)])
+def test_counters_follow_the_path(lt, nb, extra):
+    """Up to 16 boxes every ray of the evaluation and of the brute force tests every box and visits
+    no cell; more boxes (here: outside the room) are found through the grid by the same rays."""
+    from paper_2202_12567_gb300.renderer import Renderer
+    cfg = get_config("room64_vpl1k_2box", n_vpl=300, max_cut=128)
+    sc = make_scene(cfg)
+    R = Renderer(sc, cfg, device=0).setup()
+    far = np.array([[9, 9, 9, 9.5, 9.5, 9.5]], np.float32)
+    lt.lt_scene_upload(R.ctx, torch.from_numpy(np.concatenate([sc.boxes[:nb], np.repeat(far, extra, 0)])).cuda())
+    R.pass1(5)
+    R.pass2(5)
+    R.evaluate()
+    lt.lt_sync(R.ctx)
+    ev = lt.lt_eval_stats(R.ctx, R.frame, R.smp, cfg["d_min"])
+    bf = lt.lt_bruteforce_stats(R.ctx, R.pts, R.vpls, cfg["d_min"])
+    assert bf["entries"] == sc.m * sc.n and ev["entries"] == int((R.smp.cnt - R.smp.n1).sum())
+    assert bf["rays"] > 0 and (ev["rays"] > 0 or ev["entries"] == 0)  # (a coarse cut leaves pass 2 nothing)
+    for st in (ev, bf):
+        assert st["rays"] <= st["entries"]
+        if extra == 0:
+            assert st["cells"] == 0 and st["boxes"] == nb * st["rays"]
+        else:
+            assert st["cells"] > 0 or st["entries"] == 0
+    lt.lt_scene_upload(R.ctx, torch.from_numpy(np.repeat(far, 17, 0)).cuda())
+    assert lt.lt_bruteforce_stats(R.ctx, R.pts, R.vpls, cfg["d_min"])["rays"] == bf["rays"]
