@@ -360,12 +360,18 @@ __device__ __forceinline__ void load_f(bool staged, const float* sm, const float
     }
 }
 
-constexpr int kAdmBatch = 4;  // entries whose indices a lane loads at once, one batch ahead
+// Entries whose indices a lane loads at once, one batch ahead.  A lane has about a dozen
+// entries of a line and stops behind its last.  20 iterations in ms, batches of 4 with two dot
+// products side by side and the rest of a batch filled up with zeros against this: 160 x 160
+// points, 80 slices, rank 8 2.44 / 2.19; 192 x 192, 100 slices, rank 8 3.09 / 2.96; 256 x 256, 64 slices,
+// rank 16 4.85 / 4.81, 120 slices 5.01 / 5.12.
+// Above rank 16 one CTA fills an SM's shared memory, so its threads may have 255 registers
+// (bound to 128, 584 bytes of them were spilled: rank 24, 36 slices 7.82 / 6.68 ms; rank 32 7.30 / 6.19).
+constexpr int kAdmBatch = 8;
 
 template <int RP>
-__global__ void __launch_bounds__(kAdmThreads, 2) k_adm(lt_frame F, lt_samples smp, Omega om, AdmArgs a, SeedRef sr) {
+__global__ void __launch_bounds__(kAdmThreads, RP <= 16 ? 2 : 1) k_adm(lt_frame F, lt_samples smp, Omega om, AdmArgs a, SeedRef sr) {
     constexpr int NE = (RP * RP + kAdmThreads - 1) / kAdmThreads;
-    constexpr int PU = RP <= 16 ? 2 : 1;  // entries whose dot products run side by side
     __shared__ __align__(16) float sInv[RP * RP];   // (A + alpha I)^-1, then (B + beta I)^-1
     __shared__ __align__(16) float sD[RP * RP];     // (B + beta I)^-1 C
     __shared__ __align__(16) float sM[2 * RP * RP]; // reduced A, or B and C
@@ -505,8 +511,7 @@ __global__ void __launch_bounds__(kAdmThreads, 2) k_adm(lt_frame F, lt_samples s
 #pragma unroll
             for (int c = 0; c < RP; ++c) acc[c] = 0.f;
             const int e1 = rp[i + 1];
-            // batches of kAdmBatch entries, the next batch's indices on their way; past the end
-            // an entry repeats the batch's first row with a zero residual
+            // batches of kAdmBatch entries, the next batch's indices on their way
             int e0 = rp[i] + lane;
             int jj[kAdmBatch], ss[kAdmBatch];
             float mm[kAdmBatch];
@@ -525,24 +530,16 @@ __global__ void __launch_bounds__(kAdmThreads, 2) k_adm(lt_frame F, lt_samples s
                 float mn[kAdmBatch];
                 fetch(e0 + kAdmBatch * G, jn, sn, mn);
 #pragma unroll
-                for (int u = 0; u < kAdmBatch; u += PU) {
-                    float y[PU][RP], d[PU];
+                for (int u = 0; u < kAdmBatch; ++u) {
+                    if (jj[u] < 0) break;
+                    float y[RP];
+                    load_f<RP>(staged, sY, Yb, jj[u], R, y);
+                    float d = mm[u];
 #pragma unroll
-                    for (int v = 0; v < PU; ++v) {
-                        load_f<RP>(staged, sY, Yb, jj[u + v] >= 0 ? jj[u + v] : jj[0], R, y[v]);
-                        d[v] = mm[u + v];
-                    }
+                    for (int c = 0; c < RP; ++c) d = fmaf(-xo[c], y[c], d);
+                    Sr[ss[u]] = d;
 #pragma unroll
-                    for (int c = 0; c < RP; ++c)
-#pragma unroll
-                        for (int v = 0; v < PU; ++v) d[v] = fmaf(-xo[c], y[v][c], d[v]);
-#pragma unroll
-                    for (int v = 0; v < PU; ++v) {
-                        if (jj[u + v] >= 0) Sr[ss[u + v]] = d[v];
-                        else d[v] = 0.f;
-#pragma unroll
-                        for (int c = 0; c < RP; ++c) acc[c] = fmaf(d[v], y[v][c], acc[c]);
-                    }
+                    for (int c = 0; c < RP; ++c) acc[c] = fmaf(d, y[c], acc[c]);
                 }
 #pragma unroll
                 for (int u = 0; u < kAdmBatch; ++u) {
@@ -640,8 +637,9 @@ __global__ void __launch_bounds__(kAdmThreads, 2) k_adm(lt_frame F, lt_samples s
                 fetch(e0 + kAdmBatch * G, in, vn);
 #pragma unroll
                 for (int u = 0; u < kAdmBatch; ++u) {
+                    if (ii[u] < 0) break;
                     float x[RP];
-                    load_f<RP>(staged_x, sY, Xs, ii[u] >= 0 ? ii[u] : ii[0], R, x);
+                    load_f<RP>(staged_x, sY, Xs, ii[u], R, x);
 #pragma unroll
                     for (int c = 0; c < RP; ++c) acc[c] = fmaf(sv[u], x[c], acc[c]);
                 }
