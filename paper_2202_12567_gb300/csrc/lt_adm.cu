@@ -361,17 +361,20 @@ __device__ __forceinline__ void load_f(bool staged, const float* sm, const float
 }
 
 // Entries whose indices a lane loads at once, one batch ahead.  A lane has about a dozen
-// entries of a line and stops behind its last.  20 iterations in ms, batches of 4 with two dot
-// products side by side and the rest of a batch filled up with zeros against this: 160 x 160
-// points, 80 slices, rank 8 2.44 / 2.19; 192 x 192, 100 slices, rank 8 3.09 / 2.96; 256 x 256, 64 slices,
-// rank 16 4.85 / 4.81, 120 slices 5.01 / 5.12.
+// entries of a line and stops behind its last.  20 iterations in ms with batches of 4, two dot products
+// side by side and the rest of a batch filled up with zeros, then 4 / 5 / 6 / 8 without: 160 x 160 points,
+// 80 slices, rank 8 2.44, 2.20 / 1.97 / 2.01 / 2.00, 120 slices 2.87, 2.07 / 1.94 / 1.96 / 1.87; 256 x 256,
+// 120 slices, rank 16 5.00, 4.97 / 4.90 / 5.01 / 5.22, 7 slices, rank 12 39.4, 37.6 / 37.4 / 38.1 / 41.9
+// (at 8, 128 registers do not hold a row of 16 and its batches).
 // Above rank 16 one CTA fills an SM's shared memory, so its threads may have 255 registers
 // (bound to 128, 584 bytes of them were spilled: rank 24, 36 slices 7.82 / 6.68 ms; rank 32 7.30 / 6.19).
-constexpr int kAdmBatch = 8;
+template <int RP>
+__host__ __device__ constexpr int adm_batch() { return RP == 16 ? 5 : 8; }
 
 template <int RP>
 __global__ void __launch_bounds__(kAdmThreads, RP <= 16 ? 2 : 1) k_adm(lt_frame F, lt_samples smp, Omega om, AdmArgs a, SeedRef sr) {
     constexpr int NE = (RP * RP + kAdmThreads - 1) / kAdmThreads;
+    constexpr int kAdmBatch = adm_batch<RP>();
     __shared__ __align__(16) float sInv[RP * RP];   // (A + alpha I)^-1, then (B + beta I)^-1
     __shared__ __align__(16) float sD[RP * RP];     // (B + beta I)^-1 C
     __shared__ __align__(16) float sM[2 * RP * RP]; // reduced A, or B and C
