@@ -15,10 +15,10 @@
 // X_{k+1}), U, Lambda, Y, V, Pi and the |Omega| residuals.
 //
 // One cluster of K CTAs completes one slice and runs all iterations in one launch (K is
-// twice the number of parts its Gram matrices are summed in, 2, 4 or 8 by the number of
-// slices, where clusters of that size can be had; launch_adm has the rule).  Per iteration: (1) the X step, a group of G lanes per row of the CTA's
-// rows (G a power of two sized by the slice's mean row length; the lanes split the
-// row's entries two at a time, reduce with shuffles and split the r output
+// the number of parts its Gram matrices are summed in, 2, 4 or 8 by the number of slices,
+// or twice that; adm_shape has the rule).  Per iteration: (1) the X step, a group of G lanes
+// per row of the CTA's rows (G a power of two sized by the slice's mean row length; the
+// lanes split the row's entries, reduce with shuffles and split the r output
 // components), with the U and Lambda updates fused and no barrier between rows;
 // then a part of B or C from its rows staged through shared memory;
 // cluster barrier; (2) every CTA sums the partial Gram matrices from distributed
@@ -33,6 +33,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <vector>
 
 #include "lt_internal.cuh"
 #include "lt_omega.cuh"
@@ -98,8 +99,11 @@ __device__ __forceinline__ int adm_class(int len) {
 // Lines of every slice and side ordered by class, largest class first and by line
 // index within a class (a stable counting sort, so the order is deterministic), and
 // the count of each class.  Block (s, side): side 0 the rows, 1 the columns.
+// The slices in launch order: by decreasing entry count; with first > 0 (adm_shape) the longest
+// in the middle, where they have an SM to themselves.
 __global__ void k_adm_order(lt_frame F, lt_samples smp, Omega om, int32_t* __restrict__ ordr,
-                            int32_t* __restrict__ ordc, int32_t* __restrict__ ncls, int32_t* __restrict__ sord) {
+                            int32_t* __restrict__ ordc, int32_t* __restrict__ ncls, int32_t* __restrict__ sord,
+                            int first) {
     __shared__ int32_t ws[32];
     __shared__ int32_t cnt[kAdmClasses], base[kAdmClasses];
     const int s = blockIdx.x, side = blockIdx.y;
@@ -110,7 +114,12 @@ __global__ void k_adm_order(lt_frame F, lt_samples smp, Omega om, int32_t* __res
             before += smp.cnt[q] > mine || (smp.cnt[q] == mine && q < s);
         int32_t tot;
         block_exclusive_scan<int32_t>(before, ws, &tot);
-        if (threadIdx.x == 0) sord[tot] = s;
+        if (threadIdx.x == 0) {
+            int at = tot;
+            const int shared = F.S - first;  // clusters that come after the first fill
+            if (first > 0 && tot < first) at = tot < first - shared ? shared + tot : tot - (first - shared);
+            sord[at] = s;
+        }
     }
     const int row0 = F.slice_off[s];
     const int n = side ? smp.ncol[s] : F.slice_off[s + 1] - row0;
@@ -706,48 +715,85 @@ __global__ void __launch_bounds__(kAdmThreads, RP <= 16 ? 2 : 1) k_adm(lt_frame 
     cl.sync();  // no CTA leaves while another may still read its shared memory
 }
 
-template <int RP>
-lt_status launch_adm(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, const Omega& om, AdmArgs a, SeedRef sr) {
-    const size_t dyn = (size_t)std::max(2 * kAdmChunk, a.stage_cap) * RP * 4;
-    LT_CUDA(ctx, cudaFuncSetAttribute(k_adm<RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
-    // Gram parts: 8, 4 or 2, as many as let all slices run at once at two CTAs per SM.
-    // The cluster is twice as large where it can be: slices are uneven (a factor of four in
-    // entries on the bench workload), every slice runs all iterations, and with all
-    // of them resident the chip waits for the longest.  100 iterations at rank 16 on 6 M
-    // entries: 33.9 ms with clusters of the parts' size in slice order, a batch of indices
-    // loaded when the one before is done and one dot product at a time; 24.3 ms so, and 22.5 when the warps of a CTA
-    // take their tasks from a counter (every eighth task a warp: 23.8 on the same GPU).
-    int K0 = kAdmMaxK;
-    while (K0 > 2 && (int64_t)f->S * K0 > 2 * (int64_t)ctx->num_sms) K0 >>= 1;
-    int K = 2 * K0;
-    a.parts = K0;
+cudaLaunchConfig_t adm_config(lt_ctx* ctx, int S, int K, size_t dyn, cudaLaunchAttribute* attr) {
     cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(S * K));
     cfg.blockDim = dim3(kAdmThreads);
     cfg.dynamicSmemBytes = dyn;
     cfg.stream = ctx->stream;
-    cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)K;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    auto cluster = [&](int k) {
-        attr[0].val.clusterDim.x = (unsigned)k;
-        cfg.gridDim = dim3((unsigned)(f->S * k));
-    };
-    cluster(K);
-    // 16 CTAs, more than the portable size, where the device can place the clusters of all
-    // slices at once: few slices leave the chip idle.  (50 iterations, clusters of 8 against 16:
-    // 7 slices of 13208 rows in all at rank 12 13.3 / 8.3 ms, 18 of 25600 at rank 16 11.8 / 8.1;
-    // where they come in turns, 35 slices of 17658 rows at rank 8, 3.8 / 6.8.)
-    if (K > kAdmMaxK) {
-        int fit = 0;
-        if (cudaFuncSetAttribute(k_adm<RP>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&fit, k_adm<RP>, &cfg) != cudaSuccess || fit < f->S) {
-            cudaGetLastError();
-            cluster(K = K0);
+    return cfg;
+}
+
+// Shape of a launch: Gram parts, CTAs of a slice's cluster (the same number or twice as
+// many), and for k_adm_order how many clusters fill the chip before others share their SMs.
+struct AdmShape {
+    int parts, K, first;
+};
+
+// Gram parts: 8, 4 or 2, as many as let all slices run at once at two CTAs per SM (their sums
+// are added in rank order, so the parts say what the bits are and the cluster does not).
+// Every slice runs all iterations and slices are uneven (the longest has two to three times the
+// mean's entries), so the chip waits for the longest.  Twice the CTAs a slice halve its time but
+// cost two more cluster barriers an iteration, and more clusters come in turns (S / fit, fit the
+// clusters that the device places at once).  They pay where the slices have the entries for it:
+// the line is linear in the cluster's CTAs and in the turns.  20 iterations in ms, clusters of the
+// parts' size against doubled ones, with the mean entries of a slice:
+//   16 CTAs, one turn: 8 slices 16 K 0.74 / 0.76, 34 K 1.30 / 1.10; 4 of 74 K 1.64 / 1.32;
+//   16, up to 2 turns: 18 slices 89 K 2.37 / 2.53, 165 K 4.58 / 3.27; 28 of 89 K 2.59 / 3.02, 141 K 4.71 / 4.45;
+//   8, up to 2: 40 slices 33 K 2.20 / 2.52, 58 K 3.13 / 2.85; 64 of 51 K 3.52 / 3.56, 72 K 5.52 / 4.12;
+//   4, up to 2: 80 slices 25 K 2.96 / 3.03, 39 K 3.94 / 3.62; 100 of 30 K 3.71 / 3.99, 43 K 4.62 / 4.26;
+//   4 in 5 turns for 2: 300 slices 20 K 5.63 / 7.92; rank 24, 8 in 5 turns for 2: 64 of 93 K 14.1 / 21.1.
+// Where all clusters are resident and some share an SM, the clusters launched first
+// share theirs with the last: the longest slices go in between (120 slices of 17 K in clusters of
+// 2: 3.34 ms longest first, 3.08 in their own order, 2.72 so).
+constexpr int64_t kAdmOneTurn = 1024;                       // entries a CTA
+constexpr int64_t kAdmTurns = 3800, kAdmTurnsBase = 9400;   // entries a CTA and a slice, for each turn
+
+template <int RP>
+lt_status adm_shape(lt_ctx* ctx, const lt_frame* f, int64_t entries, size_t dyn, AdmShape* sh) {
+    LT_CUDA(ctx, cudaFuncSetAttribute(k_adm<RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+    const int64_t S = f->S;
+    auto fits = [&](int k) -> int64_t {  // clusters of k CTAs that the device runs at once, 0: none or unknown
+        int& known = ctx->adm_fit[RP == 8 ? 0 : RP == 16 ? 1 : 2][k == 2 ? 0 : k == 4 ? 1 : k == 8 ? 2 : 3];
+        if (known < 0) {
+            cudaLaunchAttribute attr[1];
+            const cudaLaunchConfig_t cfg = adm_config(ctx, f->S, k, dyn, attr);
+            if (cudaOccupancyMaxActiveClusters(&known, k_adm<RP>, &cfg) != cudaSuccess) {
+                cudaGetLastError();
+                known = 0;
+            }
         }
-    }
+        return known;
+    };
+    if (cudaFuncSetAttribute(k_adm<RP>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+        cudaGetLastError();  // clusters of 16 do not fit then
+    int K = kAdmMaxK;
+    while (K > 2 && S * K > 2 * (int64_t)ctx->num_sms) K >>= 1;
+    sh->parts = K;
+    const int64_t fit1 = fits(K), fit2 = fits(2 * K);
+    auto turns = [&](int64_t fit) { return fit > 0 ? (S + fit - 1) / fit : S; };
+    const bool pays = S <= fit2 ? entries >= kAdmOneTurn * 2 * K * S
+                                : turns(fit2) <= 2 * turns(fit1) &&
+                                      entries * fit2 >= (kAdmTurns * 2 * K + kAdmTurnsBase) * S * S;
+    const int64_t fit = fit2 > 0 && pays ? fit2 : fit1;
+    if (fit2 > 0 && pays) K *= 2;
+    sh->K = K;
+    const int64_t n1 = fit / 2;  // (two clusters share their SMs)
+    sh->first = S <= fit && S * K > ctx->num_sms && n1 < S && S < 2 * n1 ? (int)n1 : 0;
+    return LT_OK;
+}
+
+template <int RP>
+lt_status launch_adm(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, const Omega& om, const AdmArgs& a, int K,
+                     size_t dyn, SeedRef sr) {
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = adm_config(ctx, f->S, K, dyn, attr);
     LT_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_adm<RP>, *f, *smp, om, a, sr));
     LT_LAUNCH_CHECK(ctx, "k_adm");
     return LT_OK;
@@ -763,13 +809,20 @@ extern "C" lt_status lt_complete_adm(lt_ctx* ctx, const lt_frame* f, const lt_sa
         return lt_fail(ctx, LT_EINVAL, "lt_complete_adm: bad arguments");
     cudaSetDevice(ctx->device);
     const int S = f->S, C = f->C, R = uv->r;
-    int64_t E = 0;
+    // capacity of the entry arrays; the entries in them, for the launch's shape (a captured
+    // frame has those of its warm run)
+    int64_t E = 0, entries = 0;
     if (ctx->use_plan) {
         E = ctx->plan.entries;
+        entries = ctx->plan.adm_entries;
     } else {
+        std::vector<int32_t> cnt(S);
         LT_CUDA(ctx, cudaMemcpyAsync(&E, smp->off + S, sizeof(int64_t), cudaMemcpyDeviceToHost, ctx->stream));
+        LT_CUDA(ctx, cudaMemcpyAsync(cnt.data(), smp->cnt, (size_t)S * 4, cudaMemcpyDeviceToHost, ctx->stream));
         LT_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+        for (int s = 0; s < S; ++s) entries += cnt[s];
         ctx->plan.entries = E;
+        ctx->plan.adm_entries = entries;
     }
     Omega om;
     lt_status st = omega_build(ctx, f, smp, E, false, true, false, uv->rank, R, &om);
@@ -798,8 +851,6 @@ extern "C" lt_status lt_complete_adm(lt_ctx* ctx, const lt_frame* f, const lt_sa
     a.ncls = ncls;
     int32_t* sord = (int32_t*)((char*)ncls + up((size_t)S * 16));
     a.sord = sord;
-    k_adm_order<<<dim3(S, 2), 1024, 0, ctx->stream>>>(*f, *smp, om, ordr, ordc, ncls, sord);
-    LT_LAUNCH_CHECK(ctx, "k_adm_order");
     a.R = R;
     a.rk = uv->rank;
     a.iters = iters;
@@ -807,8 +858,17 @@ extern "C" lt_status lt_complete_adm(lt_ctx* ctx, const lt_frame* f, const lt_sa
     a.gamma = gamma;
     const int RP = R <= 8 ? 8 : R <= 16 ? 16 : 32;
     a.stage_cap = (int)(kAdmStageBytes / ((size_t)RP * 4));
+    const size_t dyn = (size_t)std::max(2 * kAdmChunk, a.stage_cap) * RP * 4;
+    AdmShape sh{};
+    st = RP == 8    ? adm_shape<8>(ctx, f, entries, dyn, &sh)
+         : RP == 16 ? adm_shape<16>(ctx, f, entries, dyn, &sh)
+                    : adm_shape<32>(ctx, f, entries, dyn, &sh);
+    if (st != LT_OK) return st;
+    a.parts = sh.parts;
+    k_adm_order<<<dim3(S, 2), 1024, 0, ctx->stream>>>(*f, *smp, om, ordr, ordc, ncls, sord, sh.first);
+    LT_LAUNCH_CHECK(ctx, "k_adm_order");
     const SeedRef sr = seed_ref(ctx, seed);
-    if (RP == 8) return launch_adm<8>(ctx, f, smp, om, a, sr);
-    if (RP == 16) return launch_adm<16>(ctx, f, smp, om, a, sr);
-    return launch_adm<32>(ctx, f, smp, om, a, sr);
+    if (RP == 8) return launch_adm<8>(ctx, f, smp, om, a, sh.K, dyn, sr);
+    if (RP == 16) return launch_adm<16>(ctx, f, smp, om, a, sh.K, dyn, sr);
+    return launch_adm<32>(ctx, f, smp, om, a, sh.K, dyn, sr);
 }

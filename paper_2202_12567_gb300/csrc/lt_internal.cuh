@@ -541,8 +541,10 @@ struct lt_ctx {
         int64_t p1_total = 0;              // pass-1 row slots of all slices
         std::vector<int32_t> level_off;    // forest level offsets [H + 2]
         int64_t entries = 0;               // sampling capacity off[S]
+        int64_t adm_entries = 0;           // sampled entries (of the seed of the warm run), for a launch's shape
     } plan;
     bool use_plan = false;                 // set while a frame is captured
+    int adm_fit[3][4] = {{-1, -1, -1, -1}, {-1, -1, -1, -1}, {-1, -1, -1, -1}};  // ADM clusters that run at once
     const uint64_t* seed_dev = nullptr;    // device seed word of the graph being captured
     std::vector<void*> retired;            // scratch that live graphs may still reference
     int graphs = 0;                        // graphs alive on this context

@@ -7,7 +7,7 @@ import pytest
 torch = pytest.importorskip("torch")
 
 from ltinputs import get_config, make_scene
-from oracle import pipeline, proposal as o_prop
+from oracle import adm as o_adm, pipeline, proposal as o_prop
 
 pytestmark = pytest.mark.gpu
 
@@ -225,3 +225,28 @@ def test_counters_follow_the_path(lt, nb, extra):
             assert st["cells"] > 0 or st["entries"] == 0
     lt.lt_scene_upload(R.ctx, torch.from_numpy(np.repeat(far, 17, 0)).cuda())
     assert lt.lt_bruteforce_stats(R.ctx, R.pts, R.vpls, cfg["d_min"])["rays"] == bf["rays"]
+
+
+@pytest.mark.parametrize("slices,rank,least", [(40, 16, 45_000), (80, 8, 27_000), (20, 10, 102_000)])
+def test_adm_clusters_in_turns(lt, slices, rank, least):
+    """Slices of many entries on clusters of twice the Gram parts that run in two turns: 8 CTAs over 4
+    parts, 4 over 2, 16 over 8.  (Smaller slices keep to clusters of the parts.)"""
+    from paper_2202_12567_gb300.renderer import Renderer
+    cfg = get_config("room64_vpl1k_2box", width=96, height=96, n_vpl=4096, max_cut=1024, eps_cut=1e-4, n_slices=slices,
+                     rank=rank, rate=0.7, rate1=0.002, tau=1e-4, completion="adm", adm_iters=5)
+    R = Renderer(make_scene(cfg), cfg, device=0).setup()
+    R.render(seed=4)
+    assert float(R.smp.cnt.double().mean()) >= least
+    img = R.img.clone()
+    for s in range(0, slices, 13):
+        rows, cols, vals, col_node, _ = R.smp.slice(s)
+        a, b, n = int(R.frame.slice_off_host[s]), int(R.frame.slice_off_host[s + 1]), int(R.smp.ncol[s])
+        Xo, Yo = o_adm.complete_slice_adm(rows, cols, vals.astype(np.float64), b - a, n, rank, 5, cfg["adm_alpha_rel"],
+                                          cfg["adm_gamma"], 4, s)
+        U = R.uv.U.cpu().numpy().reshape(-1, rank)[a:b].astype(np.float64)
+        V = R.uv.V.cpu().numpy().reshape(R.frame.S, R.frame.C, rank)[s, :n].astype(np.float64)
+        assert np.linalg.norm(U @ V.T - Xo @ Yo.T) <= 1e-3 * np.linalg.norm(Xo @ Yo.T), s
+    R.complete(4)
+    R.render_image()
+    lt.lt_sync(R.ctx)
+    assert torch.equal(R.img, img)
