@@ -7,7 +7,7 @@ import pytest
 torch = pytest.importorskip("torch")
 
 from ltinputs import get_config, make_scene
-from oracle import adm as o_adm, pipeline, proposal as o_prop
+from oracle import adm as o_adm, pipeline, proposal as o_prop, slices as o_slices
 
 pytestmark = pytest.mark.gpu
 
@@ -250,3 +250,17 @@ def test_adm_clusters_in_turns(lt, slices, rank, least):
     R.render_image()
     lt.lt_sync(R.ctx)
     assert torch.equal(R.img, img)
+
+
+@pytest.mark.parametrize("order", ["image", "random"])
+@pytest.mark.parametrize("S", [5, 64, 500])
+def test_slices_of_points_in_any_order(lt, S, order):
+    """A warp's points in one cluster, in a few and in 32 clusters: the oracle's labels."""
+    pts = np.ascontiguousarray(make_scene(get_config("room64_vpl1k_2box", width=63, height=61)).points)
+    if order == "random":
+        pts = np.ascontiguousarray(pts[:, np.random.default_rng(S).permutation(pts.shape[1])])
+    perm, off = lt.lt_make_slices(lt.Context(0), torch.from_numpy(pts).cuda(), S, 10, 0.3)
+    perm, off = perm.cpu().numpy(), off.cpu().numpy()
+    lab = np.empty(pts.shape[1], np.int64)
+    lab[perm] = np.repeat(np.arange(S), np.diff(off))
+    assert np.mean(lab == o_slices.kmeans_slices(pts, S, 10, 0.3)[2]) >= 0.99
