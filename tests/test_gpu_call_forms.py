@@ -7,7 +7,7 @@ import pytest
 torch = pytest.importorskip("torch")
 
 from ltinputs import get_config, make_scene
-from oracle import adm as o_adm, pipeline, proposal as o_prop, slices as o_slices
+from oracle import adm as o_adm, pipeline, proposal as o_prop, shading, slices as o_slices
 
 pytestmark = pytest.mark.gpu
 
@@ -264,3 +264,68 @@ def test_slices_of_points_in_any_order(lt, S, order):
     lab = np.empty(pts.shape[1], np.int64)
     lab[perm] = np.repeat(np.arange(S), np.diff(off))
     assert np.mean(lab == o_slices.kmeans_slices(pts, S, 10, 0.3)[2]) >= 0.99
+
+
+@pytest.mark.parametrize("nr,C", [(1, 1), (33, 7), (64, 1215), (64, 1300), (64, 5000)])
+def test_cut_errors_of_every_row(lt, nr, C):
+    """One round's errors at cuts on both sides of the rules for warps per node, on rows that the
+    cut lights (each is compared) and with a row that it leaves dark (every bound infinite)."""
+    n = 8192
+    sc = make_scene(get_config("room256_vpl16k_200box", n_vpl=n, width=16, height=16))
+    ctx, vp = lt.Context(0), torch.from_numpy(sc.vpls).cuda()
+    t = lt.lt_build_tree(ctx, vp)
+    rng = np.random.default_rng(C)
+    I, B, rep, bb = (x.cpu().numpy() for x in (t.I, t.B, t.rep, t.aabb))
+    cut = np.sort(rng.choice(2 * n - 1, C, replace=False)).astype(np.int32) if C > 1 else np.zeros(1, np.int32)
+    rc, pts = rep[cut], sc.points.copy()
+    scale = I[cut].astype(np.float64) / (sc.vpls[2, rc, 3].astype(np.float64) * sc.vpls[0, rc, 3])
+    rr, cc = np.repeat(np.arange(sc.m), C), np.tile(np.arange(C), sc.m)
+    est = (shading.unoccluded(pts, sc.vpls, rr, rc[cc], 0.1) * scale[cc]).reshape(sc.m, C).sum(1)
+    rows = np.argsort(-est, kind="stable")[rng.permutation(np.arange(max(nr, 64)))[:nr]].astype(np.int32)
+    assert (est[rows] > 0).all()
+
+    def errors(pts, rows):
+        p, r = (torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (pts, rows))
+        return lt.lt_cut_errors(ctx, t, p, vp, r, torch.from_numpy(cut).cuda(), 0.1).cpu().numpy()
+
+    P = pts[0, rows].astype(np.float64)
+    lo, hi = bb.reshape(-1, 6)[cut, :3].astype(np.float64), bb.reshape(-1, 6)[cut, 3:].astype(np.float64)
+    gap = np.maximum(0, np.maximum(lo[None] - P[:, None, :3], P[:, None, :3] - hi[None]))
+    bound = (I * B)[cut].astype(np.float64) * (P[:, 3] / np.pi)[:, None] / np.maximum((gap ** 2).sum(2), 0.01)
+    np.testing.assert_allclose(errors(pts, rows), (bound / est[rows][:, None]).max(0), rtol=1e-4)
+    dark = pts.copy()
+    dark[0, rows[0], :3], dark[1, rows[0], :3] = (0.5, 2.0, 0.5), (0.0, 1.0, 0.0)  # above the room, facing up
+    assert np.all(np.isinf(errors(dark, rows)))
+
+
+@pytest.mark.parametrize("form", [0, 1])
+@pytest.mark.parametrize("rate1,slices", [(0.002, 2), (0.03, 1)])
+def test_pass1_decides_as_the_oracle(lt, rate1, slices, form):
+    """Every pair whose children both coarsenings reached: merged by both or by neither, unless its
+    cost is within 1e-4 of the threshold."""
+    from paper_2202_12567_gb300.renderer import Renderer
+    cfg = get_config("room64_vpl1k_2box", max_cut=256, n_slices=slices, rate1=rate1, tau=0.2)
+    sc = make_scene(cfg)
+    st = pipeline.setup(sc, cfg)
+    fo = st["forest"]
+    R = Renderer(sc, cfg, device=0).setup(cut=st["cut"], row_perm=st["row_perm"], slice_off=st["slice_off"])
+    lt.lt_set_tuning(R.ctx, p1_form=form)
+    R.pass1(11)
+    lt.lt_sync(R.ctx)
+    for s in range(slices):
+        col_node = set(R.smp.slice(s)[3].tolist())
+        ours = np.zeros(len(fo.node), bool)  # the node is a column or lies under one
+        for x in range(len(fo.node)):
+            y = x
+            while y >= 0 and int(fo.node[y]) not in col_node:
+                y = int(fo.parent[y])
+            ours[x] = y >= 0
+        o = pipeline.run_slice(st, sc, cfg, s, 11).p1
+        reached = lambda x: x < fo.C or ours[x]
+        ties = [f for f, _, cf, thr, merged, *_ in o.log
+                if ours[f] != merged and reached(fo.child[f, 0]) and reached(fo.child[f, 1]) and
+                abs(cf - thr) <= 1e-4 * thr]
+        wrong = [f for f, _, cf, thr, merged, *_ in o.log
+                 if ours[f] != merged and reached(fo.child[f, 0]) and reached(fo.child[f, 1]) and f not in ties]
+        assert len(o.log) > 50 and not wrong, (s, wrong)
+        assert ties or col_node == set(o.col_node.tolist())
