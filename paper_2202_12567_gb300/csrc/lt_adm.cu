@@ -60,7 +60,8 @@ struct AdmArgs {
     const int32_t* ordr;  // [m]        rows of each slice ordered by class (k_adm_order)
     const int32_t* ordc;  // [S][C]     columns of each slice ordered by class
     const int32_t* ncls;  // [S][2][8]  lines per class, rows then columns
-    const int32_t* sord;  // [S]        slices by decreasing entry count
+    const int32_t* sord;  // [S]        slices in launch order
+    int32_t* shape;       // [2]        CTAs of a cluster, Gram parts
     int parts;            // CTAs of a slice whose Gram parts are added (the cluster has 1 or 2 times as many)
     int R;
     const int32_t* rk;
@@ -402,6 +403,7 @@ __global__ void __launch_bounds__(kAdmThreads, RP <= 16 ? 2 : 1) k_adm(lt_frame 
     // for X'^T X' and Y^T Y, the others for X'^T X.
     const int K0 = a.parts, kg = k % K0, second = k / K0;
     const bool split = K > K0;
+    if (blockIdx.x == 0 && threadIdx.x < 2) a.shape[threadIdx.x] = threadIdx.x ? K0 : K;
     const int s = a.sord[blockIdx.x / K];  // the longest slices start first
     const int tid = threadIdx.x;
     const int R = a.R;
@@ -830,10 +832,12 @@ extern "C" lt_status lt_complete_adm(lt_ctx* ctx, const lt_frame* f, const lt_sa
     const size_t nx = (size_t)f->m * R, ny = (size_t)S * C * R;
     auto up = [](size_t n) { return (n * 4 + 255) & ~(size_t)255; };
     char* p = (char*)lt_scratch(ctx, SCR_ADM,
-                                3 * up(nx) + 2 * up(ny) + up((size_t)E) + up((size_t)f->m) + up((size_t)S * C) +
+                                256 + 3 * up(nx) + 2 * up(ny) + up((size_t)E) + up((size_t)f->m) + up((size_t)S * C) +
                                     up((size_t)S * 16) + up((size_t)S),
                                 &st);
     if (!p) return st;
+    int32_t* shape = (int32_t*)p;  // CTAs of a cluster and Gram parts, as launched (for inspection)
+    p += 256;
     AdmArgs a;
     a.X0 = uv->U;
     a.X1 = (float*)p;
@@ -851,6 +855,7 @@ extern "C" lt_status lt_complete_adm(lt_ctx* ctx, const lt_frame* f, const lt_sa
     a.ncls = ncls;
     int32_t* sord = (int32_t*)((char*)ncls + up((size_t)S * 16));
     a.sord = sord;
+    a.shape = shape;
     a.R = R;
     a.rk = uv->rank;
     a.iters = iters;

@@ -329,3 +329,19 @@ def test_pass1_decides_as_the_oracle(lt, rate1, slices, form):
                  if ours[f] != merged and reached(fo.child[f, 0]) and reached(fo.child[f, 1]) and f not in ties]
         assert len(o.log) > 50 and not wrong, (s, wrong)
         assert ties or col_node == set(o.col_node.tolist())
+
+
+@pytest.mark.parametrize("rank,slices,side,rate,K,parts",
+                         [(8, 40, 64, 0.3, 4, 4), (16, 40, 64, 0.3, 4, 4), (20, 80, 64, 0.3, 2, 2), (12, 3, 64, 0.3, 16, 8),
+                          (24, 12, 64, 0.3, 8, 8), (16, 20, 64, 0.3, 8, 8), (16, 40, 96, 0.7, 8, 4), (8, 80, 96, 0.7, 4, 2),
+                          (10, 20, 96, 0.7, 16, 8)])
+def test_adm_shapes(lt, rank, slices, side, rate, K, parts):
+    """The clusters that the cases of the ADM tests run on (with fewer entries a slice those of the
+    Gram parts, with more twice as many CTAs), as the kernel itself reports them."""
+    from paper_2202_12567_gb300.renderer import Renderer
+    over = dict(max_cut=128) if side == 64 else dict(n_vpl=4096, max_cut=1024, eps_cut=1e-4, tau=1e-4)
+    cfg = get_config("room64_vpl1k_2box", width=side, height=side, n_slices=slices, rank=rank, rate=rate, rate1=0.002,
+                     completion="adm", adm_iters=2, **over)
+    R = Renderer(make_scene(cfg), cfg, device=0).setup()
+    R.render(seed=4)
+    assert lt.lt_debug_scratch(R.ctx, 14)[:8].view(torch.int32).tolist() == [K, parts]
