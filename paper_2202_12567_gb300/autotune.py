@@ -5,10 +5,14 @@ Each tunable value is tried over its candidates with the others fixed
 acts on with CUDA events on the context's stream (median of `reps` frames after a
 warm frame).  Results are cached in a JSON file keyed by the workload:
 (config name, rank, power-of-two bucket of the median slice rows m', and of the
-median coarsened cut n').  `apply` loads a cached entry or tunes and stores one.
+median coarsened cut n').  An entry names the kernel sources and the GPU that it was
+measured on and counts for those alone.  `apply` loads such an entry or tunes and
+stores one.
 """
 from __future__ import annotations
 
+import glob
+import hashlib
 import json
 import os
 import statistics
@@ -40,6 +44,15 @@ def bucket(x: float) -> int:
 
 def workload_key(name: str, rank: int, slice_rows, ncol) -> str:
     return f"{name}|r{int(rank)}|m{bucket(np.median(slice_rows))}|n{bucket(np.median(ncol))}"
+
+
+def made_for(R) -> dict:
+    """What a measurement holds for: the kernel sources (a hash) and the GPU's name."""
+    h = hashlib.sha256()
+    for p in sorted(glob.glob(os.path.join(HERE, "csrc", "*.cu*")), key=os.path.basename):
+        with open(p, "rb") as f:
+            h.update(os.path.basename(p).encode() + b"\0" + f.read())
+    return dict(kernels=h.hexdigest()[:16], gpu=torch.cuda.get_device_name(R.dev))
 
 
 def stage_times(R, seed: int) -> dict:
@@ -95,11 +108,12 @@ def apply(R, name: str, path: str = DEFAULT_CACHE, retune: bool = False, log=Non
     if os.path.exists(path):
         with open(path) as f:
             cache = json.load(f)
-    if key in cache and not retune:
+    current = made_for(R)
+    if key in cache and cache[key].get("made_for") == current and not retune:
         lt.lt_set_tuning(R.ctx, **cache[key]["values"])
         return key, cache[key]["values"], True
     res = tune(R, log=log)
-    cache[key] = res
+    cache[key] = dict(res, made_for=current)
     with open(path, "w") as f:
         json.dump(cache, f, indent=1, sort_keys=True)
     return key, res["values"], False
