@@ -935,15 +935,13 @@ __global__ void __launch_bounds__(32 * kHalfWarps, 2) k_als_half(lt_frame F, lt_
     }
 }
 
-// ---- rank <= 16: Gram on the tensor cores, then one thread per line ------------
-// The in-warp Cholesky of the line solve costs as many warp instructions as the
-// whole tensor-core Gram; a 16 x 16 Cholesky fits one thread's registers instead.
-// ---- Masked ALS, one thread per line (r <= 16) --------------------------------
-// A line is a row of U_s (U-step, its entries in CSR) or a column of V_s (V-step,
-// CSC).  The thread gathers the factor row x_j of each observed entry from the
-// slice's factor rows staged in shared memory and accumulates the lower triangle of
-// G = sum x_j x_j^T and b = sum a_j x_j in registers (RP(RP+1)/2 + RP values),
-// adds the ridge lam_rel tr(G)/r, factors G by Cholesky in float32 and solves.
+// ---- Masked ALS, a group of lanes per line (r <= 16) ---------------------------
+// A line is a row of U_s (U-step) or a column of V_s (V-step); its 2^g lanes have its
+// entries in turn, each as a stream of the sliced layout.  A lane gathers the factor row
+// x_j of each of its entries from the slice's factor rows staged in shared memory and
+// accumulates the lower triangle of G = sum x_j x_j^T and b = sum a_j x_j in registers
+// (RP(RP+1)/2 + RP values); the group's sums go to its first lane, which adds the ridge
+// lam_rel tr(G)/r, factors G by Cholesky in float32 and solves.
 // Lines whose pivots fail the check go to a queue; a second kernel forms their
 // Gram again in float64 (products of the float32 factors are exact in float64) and
 // solves it in float64, so an ill-conditioned line carries no float32 rounding.
@@ -1184,7 +1182,7 @@ __global__ void __launch_bounds__(256, RP == 8 ? 2 : 1) k_als_line(lt_frame F, l
     const int64_t total = wk[S];
     const int64_t lo = total * blockIdx.x / gridDim.x;
     const int64_t hi = blockIdx.x + 1 == gridDim.x ? INT64_MAX : total * (blockIdx.x + 1) / gridDim.x;
-    // tasks of slice x (none where its rank is the warp-per-line kernel's) and the work before task t
+    // tasks of slice x (none where its rank is k_als_half's) and the work before task t
     auto tasks_of = [&](int x) {
         return slice_rank(rk, x, R) <= RP ? cls_all[(int64_t)x * 16 + 8 + kClasses] : 0;
     };
@@ -1610,7 +1608,7 @@ lt_status complete_impl(lt_ctx* ctx, const lt_frame* f, const lt_samples* smp, i
     int32_t* n64 = (int32_t*)sp;
     int32_t* qcount = n64 + 64;
     int32_t* qcount_hi = qcount + nq;
-    int32_t* next_hi = qcount + 2 * nq;  // line counters of the warp-per-line kernel
+    int32_t* next_hi = qcount + 2 * nq;  // line counters of k_als_half
     LT_CUDA(ctx, cudaMemsetAsync(n64, 0, (size_t)(3 * nq + 64) * 4, ctx->stream));
     const int nsm = ctx->num_sms;
     k_als_init<<<dim3(8, S), 256, 0, ctx->stream>>>(*f, *smp, om, R, rk, seed_ref(ctx, seed), uv->V);

@@ -225,7 +225,7 @@ __device__ __forceinline__ int tc_exp(float m) {
 
 // -------------------------------------------------------------------- per lt_complete
 // One block: the four per-slice prefixes (slices of rank above RP get no tiles and
-// no image blocks: the warp-per-line kernel has them).
+// no image blocks: k_als_half has them).
 __global__ void __launch_bounds__(1024) k_tc_prefix(lt_frame F, lt_samples smp, int R, const int32_t* rk, int RP,
                                                     TcPlan P) {
     __shared__ int32_t ws[32];

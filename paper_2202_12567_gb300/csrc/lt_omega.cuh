@@ -56,7 +56,7 @@ struct Omega {
     int tcap;
     int lane_entries;   // class threshold (line_class)
     bool sell;          // fill the sliced layout
-    bool csr;           // fill CSR / CSC (the warp-per-line ALS for r > 16)
+    bool csr;           // fill CSR / CSC (the ALS above rank 16, two lines a warp)
 };
 
 // Builds Omega for the frame's samples (E = total entry count, known to the host):

@@ -2,12 +2,12 @@
 //
 //  * Pass 1 and light coarsening (Sec. 4, Eq. 2): the cut nodes of every slice draw
 //    their k_c rows and evaluate them (one kernel over all slices), then the cut's
-//    ancestor forest is walked level by level with a few kernels per level over all
-//    slices: sibling pairs are laid out as the union zeta_f = zeta_a U zeta_b (one
-//    thread per small pair, one CTA per big pair), the entries missing from either
-//    child are queued and evaluated one shadow ray per thread, and each pair merges
-//    when cost = eps + cost(q) < tau * S_hat, eps = max |V_q - V_p I_q / I_p| (in a dark
-//    slice, S_hat = 0, when the cost is exactly zero).
+//    ancestor forest is walked level by level with two kernels per level over all
+//    slices.  One group of lanes (8, a warp or a CTA by the pair's rows) handles a
+//    sibling pair from end to end: the union zeta_f = zeta_a U zeta_b, the entries
+//    missing from either child, and the merge when cost = eps + cost(q) < tau * S_hat,
+//    eps = max |V_q - V_p I_q / I_p| (in a dark slice, S_hat = 0, when the cost is
+//    exactly zero).
 //  * Pass 2 (Sec. 5, Eq. 3): per slice one cluster of eight CTAs draws (column from
 //    the integer CDF of g or of given weights, row uniform) in rounds, keeps the
 //    first occurrence of every new entry in draw order, and stops at
