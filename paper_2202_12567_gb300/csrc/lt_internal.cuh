@@ -231,8 +231,9 @@ __device__ inline bool grid_blocked(const Grid& g, float3 o, float3 e, WorkCount
 // Up to this many boxes every segment tests every box: the loads are the same for the
 // whole warp, while the walk above spends its time on divergent cell look-ups.  With this
 // and the walk's state out of local memory, the brute force of 65536 points and 16384
-// VPLs among 2 boxes took 7.24 ms where it had taken 31.5.  The answer is the walk's (a cell
-// lists every box within a margin of it, so the walk misses none that the test meets).
+// VPLs among 2 boxes took 7.24 ms where it had taken 31.5.  For finite segments and boxes with
+// lo <= hi the answer is the walk's (a cell lists every box within a margin of it, so the walk
+// misses none that the test meets).
 // The line: brute force of 16384 points and 4096 lights, boxes one by one against the walk,
 // 0.56 / 0.93 ms at 2 boxes, 1.41 / 1.80 at 8, 2.21 / 2.50 at 16, 2.86 / 2.60 at 24;
 // evaluation of the pass-2 entries of such a scene 0.074 / 0.100 ms at 16, 0.097 / 0.120 at 24.

@@ -1102,10 +1102,10 @@ extern "C" lt_status lt_leverage_targets(lt_ctx* ctx, const lt_frame* f, const l
     cudaSetDevice(ctx->device);
     const int S = f->S, C = f->C;
     // Gram capacity: slices of any n' whose squares add up to at most S min(C, 4096)^2
-    // floats, and the padding of their rows (at most 3 floats each).  More latches LT_ELIMIT
-    // and no target is written.
+    // floats, and the padding of their rows, at most 3 floats each (S slices whose squares add
+    // up to S nmax^2 have at most S nmax rows).  More latches LT_ELIMIT and no target is written.
     const int64_t nmax = std::min<int64_t>(C, 4096);
-    const int64_t gcap = (int64_t)S * (nmax * nmax + 3 * (int64_t)C);
+    const int64_t gcap = (int64_t)S * (nmax * nmax + 3 * nmax);
     lt_status st;
     auto up = [](size_t n) { return (n + 255) & ~(size_t)255; };  // each part starts on 256 bytes
     const size_t b_g = up((size_t)gcap * 4), b_q = up((size_t)S * C * r * 4);
