@@ -252,9 +252,17 @@ SMS, FP32_LANES, MAX_SM_MHZ = 152, 128, 2070.0
 # learned pdf), the median over the captured launches; profiles/traffic_room256_vpl16k_2box.md
 # gives the command.  A kernel changed since its capture has no entry here.
 MEASURED_TRAFFIC = {
-    "k_render": 7_067_392,
-    "k_als_line": 49_546_240,  # U-steps and V-steps of the captured frames
+    "k_render": 7_064_320,
+    "k_als_line": 50_754_688,  # U-steps and V-steps of the captured frames
+    "k_eval_entries": 27_806_464,
 }
+
+
+def measured_traffic(R, kernel):
+    """The captured bytes where R renders the scene and rank that they were captured on."""
+    same = all(R.cfg.get(k) == v for k, v in dict(width=256, height=256, n_vpl=16384, n_big_boxes=2, n_small_boxes=0,
+                                                  rank=16).items()) and getattr(R.scene, "tris", None) is None
+    return MEASURED_TRAFFIC.get(kernel) if same else None
 
 
 def fp32_peak(clk) -> dict:
@@ -285,7 +293,7 @@ def eval_roofline(lt, ctx, R, eval_ms, clk):
     achieved = ops / secs / 1e12 if secs > 0 else 0.0
     pk = fp32_peak(clk)
     return dict(bound="alu", kernel="k_eval_entries", achieved=round(achieved, 3), unit="TFLOP/s",
-                frac=round(achieved / pk["peak"], 4), traffic=MEASURED_TRAFFIC.get("k_eval_entries"),
+                frac=round(achieved / pk["peak"], 4), traffic=measured_traffic(R, "k_eval_entries"),
                 launch_ms=round(eval_ms, 4), **pk,
                 work=dict(entries=st["entries"], rays=st["rays"], cells=st["cells"], boxes=st["boxes"],
                           ops_per_launch=int(ops)))
@@ -303,7 +311,7 @@ def als_roofline(lt, ctx, R, half_ms, clk):
     pk = fp32_peak(clk)
     return dict(bound="alu", kernel="k_als_line (ALS half-step)", achieved=round(achieved, 3), unit="TFLOP/s",
                 frac=round(achieved / pk["peak"], 4),
-                traffic=MEASURED_TRAFFIC.get("k_als_line") if R.cfg["rank"] == 16 else None,
+                traffic=measured_traffic(R, "k_als_line"),
                 launch_ms=round(half_ms, 4), **pk,
                 work=dict(entries=E, lines_per_half_step=lines, flops_per_launch=int(flops)))
 
@@ -330,7 +338,7 @@ def render_roofline(R, render_ms, peaks):
     achieved = byts / (render_ms * 1e-3) / 1e9
     peak = peaks.get("hbm_gbs", 6800.0)
     return dict(bound="hbm", kernel="k_render", achieved=round(achieved, 1), peak=peak, unit="GB/s",
-                frac=round(achieved / peak, 4), traffic=MEASURED_TRAFFIC.get("k_render"),
+                frac=round(achieved / peak, 4), traffic=measured_traffic(R, "k_render"),
                 launch_ms=round(render_ms, 4), bytes_per_launch=int(byts),
                 peak_source="measured copy bandwidth (MEASURED_PEAKS.json hbm_gbs)" if "hbm_gbs" in peaks
                 else "fallback 6.8 TB/s")
